@@ -240,21 +240,28 @@ int step_exact(conqur_ctx* c, const TIn* X, int64_t n, int64_t ld, int64_t pstri
   const int64_t c_ps = (int64_t)g.n_max * d;
   rownorm_kernel<TIn><<<dim3(cdiv(n, 8), P), 256, 0, c->stream>>>(X, n, d, ld, pstride, rnorm, g.n_max, st, 1);
   CQ_LAUNCHED(c, K_ROWNORM);
-  const dim3 grid1(cdiv(d, SG_BN), cdiv(n, SG_BM), P);
+  const int rt = sg_pick(n, d, P, c->L.max_partials);
   int per_problem;
   double* pdiag = g.diagnostics ? c->at<double>(c->L.part_diag) : nullptr;
   if (g.quant_bits == 0 && !g.diagnostics) {
-    rotate_target_exact_kernel<TIn, false><<<grid1, SG_THREADS, 0, c->stream>>>(
-        X, ld, pstride, c->at<float>(c->L.R) + pdd, (int)n, d, rnorm, g.n_max, C, c_ps, nullptr, nullptr, part);
+    sg_with_tile(rt, [&](auto tile) {
+      using Tile = decltype(tile);
+      const dim3 grid = sg_grid<Tile>(n, d, P);
+      per_problem = grid.x * grid.y;
+      rotate_target_exact_kernel<Tile, TIn, false><<<grid, Tile::NT, 0, c->stream>>>(
+          X, ld, pstride, c->at<float>(c->L.R) + pdd, (int)n, d, rnorm, g.n_max, C, c_ps, nullptr, nullptr, part);
+    });
     CQ_LAUNCHED(c, K_ROTATE);
-    per_problem = grid1.x * grid1.y;
   } else {
     unsigned* rowmax = c->at<unsigned>(c->L.rowmax);
     unsigned* rowmin = rowmax + g.n_max * g.P;
     CQ_CUDA(cudaMemsetAsync(rowmax, 0, sizeof(unsigned) * g.n_max * P, c->stream));
     CQ_CUDA(cudaMemsetAsync(rowmin, 0xff, sizeof(unsigned) * g.n_max * P, c->stream));
-    rotate_target_exact_kernel<TIn, true><<<grid1, SG_THREADS, 0, c->stream>>>(
-        X, ld, pstride, c->at<float>(c->L.R) + pdd, (int)n, d, rnorm, g.n_max, C, c_ps, rowmax, rowmin, part);
+    sg_with_tile(rt, [&](auto tile) {
+      using Tile = decltype(tile);
+      rotate_target_exact_kernel<Tile, TIn, true><<<sg_grid<Tile>(n, d, P), Tile::NT, 0, c->stream>>>(
+          X, ld, pstride, c->at<float>(c->L.R) + pdd, (int)n, d, rnorm, g.n_max, C, c_ps, rowmax, rowmin, part);
+    });
     CQ_LAUNCHED(c, K_ROTATE);
     quant_target_kernel<<<dim3(cdiv(n, 8), P), 256, 0, c->stream>>>(C, n, d, c_ps, rnorm, g.n_max, rowmax, rowmin, g.qs,
                                                                     part, pdiag);
@@ -265,9 +272,12 @@ int step_exact(conqur_ctx* c, const TIn* X, int64_t n, int64_t ld, int64_t pstri
                                                  pdiag ? cdiv(n, 8) : 0);
   CQ_LAUNCHED(c, K_OTHER);
   const int S = c->L.acc_splits;
-  accumulate_exact_kernel<TIn><<<dim3(cdiv(d, SG_BN), cdiv(d, SG_BM), P * S), SG_THREADS, 0, c->stream>>>(
-      X, ld, pstride, C, c_ps, rnorm, g.n_max, (int)n, d, S, c->at<float>(c->L.M) + pdd,
-      S > 1 ? c->at<float>(c->L.splitk) : nullptr);
+  sg_with_tile(sg_pick(d, d, (int64_t)P * S), [&](auto tile) {
+    using Tile = decltype(tile);
+    accumulate_exact_kernel<Tile, TIn><<<sg_grid<Tile>(d, d, P * S), Tile::NT, 0, c->stream>>>(
+        X, ld, pstride, C, c_ps, rnorm, g.n_max, (int)n, d, S, c->at<float>(c->L.M) + pdd,
+        S > 1 ? c->at<float>(c->L.splitk) : nullptr);
+  });
   CQ_LAUNCHED(c, K_ACCUM);
   if (S > 1) {
     splitk_reduce_add_kernel<<<dim3(ew_blocks((int64_t)d * d), P), 256, 0, c->stream>>>(
@@ -301,21 +311,36 @@ __global__ void check_guards_kernel(const unsigned char* ws, const GuardList gl,
 
 // ---------------------------------------------------------------- update (both modes share the control flow)
 // residual check of the fp32 matrix X (P x d x d) into E; fills the partials.
+// One fp32 product of the iteration, on the tile that suits d x d outputs of this context.
+int ns_tile(const conqur_ctx* c, int epi) {
+  return sg_pick(c->cfg.d, c->cfg.d, c->cfg.P, c->L.max_partials, /*sym=*/epi != EPI_NEXT);
+}
+template <int EPI>
+void launch_ns_exact(conqur_ctx* c, const float* A, const float* B, const float* Cin, float* D) {
+  sg_with_tile(ns_tile(c, EPI), [&](auto tile) {
+    using Tile = decltype(tile);
+    ns_gemm_exact_kernel<Tile, EPI><<<sg_grid<Tile>(c->cfg.d, c->cfg.d, c->cfg.P), Tile::NT, 0, c->stream>>>(
+        A, B, Cin, D, c->cfg.d, c->state(), c->at<float>(c->L.part_f), c->at<double>(c->L.part_d));
+  });
+}
+// per-CTA partials of one problem that such a residual product leaves
+int ns_exact_parts(const conqur_ctx* c) {
+  int parts = 0;
+  sg_with_tile(ns_tile(c, EPI_RESIDUAL), [&](auto tile) {
+    const dim3 grid = sg_grid<decltype(tile)>(c->cfg.d, c->cfg.d, 1);
+    parts = (int)(grid.x * grid.y);
+  });
+  return parts;
+}
 int launch_residual(conqur_ctx* c, const float* X, int buf) {
-  const Cfg& g = c->cfg;
-  const int T = cdiv(g.d, SG_BM);
-  if (g.simt_ns) {
-    ns_gemm_exact_kernel<EPI_RESIDUAL><<<dim3(T, T, g.P), SG_THREADS, 0, c->stream>>>(
-        X, X, nullptr, c->at<float>(c->L.E), g.d, c->state(), c->at<float>(c->L.part_f), c->at<double>(c->L.part_d));
+  if (c->cfg.simt_ns) {
+    launch_ns_exact<EPI_RESIDUAL>(c, X, X, nullptr, c->at<float>(c->L.E));
     CQ_LAUNCHED(c, K_NS_RESID);
     return CONQUR_OK;
   }
   return tc_ns_residual(c->tc, c->stream, buf);
 }
-int ns_parts(const conqur_ctx* c) {
-  if (c->cfg.simt_ns) { const int T = cdiv(c->cfg.d, SG_BM); return T * T; }
-  return tc_ns_parts(c->tc);
-}
+int ns_parts(const conqur_ctx* c) { return c->cfg.simt_ns ? ns_exact_parts(c) : tc_ns_parts(c->tc); }
 
 // The update in three parts, so that it can be enqueued unrolled (every step a fixed set of launches that early-exit once
 // the iteration has finished) or as a captured graph whose middle part is a device-side loop.
@@ -361,7 +386,6 @@ int update_step(conqur_ctx* c, int k, int cur, bool last) {
   double* pd = c->at<double>(c->L.part_d);
   float* pf = c->at<float>(c->L.part_f);
   const int use_shift = g.simt_ns ? 0 : 1;
-  const int T = cdiv(d, SG_BM);
   const int parts = ns_parts(c);
   const NsControlParams ncp{c->at<SchedEntry>(c->L.sched), c->n_sched, c->n_lift_init, g.ns_max_steps, d, use_shift, g.orth_tol,
                             g.fro_tol, g.margin, g.lo_budget, 1.0 / (double)d};
@@ -374,9 +398,9 @@ int update_step(conqur_ctx* c, int k, int cur, bool last) {
   CQ_LAUNCHED(c, K_OTHER);
   if (last) return CONQUR_OK;
   if (g.simt_ns) {
-    ns_gemm_exact_kernel<EPI_POLY><<<dim3(T, T, P), SG_THREADS, 0, c->stream>>>(E, E, E, B, d, st, nullptr, nullptr);
+    launch_ns_exact<EPI_POLY>(c, E, E, E, B);
     CQ_LAUNCHED(c, K_NS_POLY);
-    ns_gemm_exact_kernel<EPI_NEXT><<<dim3(T, T, P), SG_THREADS, 0, c->stream>>>(X, B, X, Xn, d, st, nullptr, nullptr);
+    launch_ns_exact<EPI_NEXT>(c, X, B, X, Xn);
     CQ_LAUNCHED(c, K_NS_NEXT);
     return CONQUR_OK;
   }
@@ -657,16 +681,12 @@ extern "C" int conqur_set_R(conqur_ctx* c, const float* R_dev) {
   const Cfg& g = c->cfg;
   const int64_t dd = (int64_t)g.d * g.d;
   { const int frc = flush_pending(c); if (frc) return frc; }      // queued rows belong to the rotation being replaced
-  // check orthogonality with the exact fp32 residual product, whatever the mode
-  float* Xa = c->at<float>(c->L.Xa);
-  CQ_CUDA(cudaMemcpyAsync(Xa, R_dev, sizeof(float) * dd * g.P, cudaMemcpyDeviceToDevice, c->stream));
+  // check orthogonality with the exact fp32 residual product, whatever the mode (statistics only: nothing is stored)
   arm_check_kernel<<<1, 256, 0, c->stream>>>(c->state(), g.P);
   CQ_LAUNCHED(c, K_OTHER);
-  const int T = cdiv(g.d, SG_BM);
-  ns_gemm_exact_kernel<EPI_RESIDUAL><<<dim3(T, T, g.P), SG_THREADS, 0, c->stream>>>(
-      Xa, Xa, nullptr, c->at<float>(c->L.E), g.d, c->state(), c->at<float>(c->L.part_f), c->at<double>(c->L.part_d));
+  launch_ns_exact<EPI_RESIDUAL>(c, R_dev, R_dev, nullptr, nullptr);
   CQ_LAUNCHED(c, K_OTHER);
-  std::vector<float> pm((size_t)T * T * g.P);
+  std::vector<float> pm((size_t)ns_exact_parts(c) * g.P);
   CQ_CUDA(cudaMemcpyAsync(pm.data(), c->at<float>(c->L.part_f), sizeof(float) * pm.size(), cudaMemcpyDeviceToHost,
                           c->stream));
   CQ_CUDA(cudaStreamSynchronize(c->stream));
@@ -1043,13 +1063,15 @@ extern "C" int conqur_fold_weight(const float* W_dev, int64_t ldw, int32_t rows,
     CQ_CUDA(cudaStreamSynchronize(s));
     return flags_to_status(h.status_flags);
   }
-  if (side == CONQUR_FOLD_INPUT) {
-    const dim3 grid(cdiv(block, SG_BN), cdiv(rows, SG_BM), nblk);
-    fold_exact_kernel<0><<<grid, SG_THREADS, 0, s>>>(W_dev, ldw, R_dev, block, rows, cols, out_dev, ldo);
-  } else {
-    const dim3 grid(cdiv(cols, SG_BN), cdiv(block, SG_BM), nblk);
-    fold_exact_kernel<1><<<grid, SG_THREADS, 0, s>>>(W_dev, ldw, R_dev, block, rows, cols, out_dev, ldo);
-  }
+  const int64_t fm = side == CONQUR_FOLD_INPUT ? rows : block, fn = side == CONQUR_FOLD_INPUT ? block : cols;
+  sg_with_tile(sg_pick(fm, fn, nblk), [&](auto tile) {
+    using Tile = decltype(tile);
+    const dim3 grid = sg_grid<Tile>(fm, fn, nblk);
+    if (side == CONQUR_FOLD_INPUT)
+      fold_exact_kernel<Tile, 0><<<grid, Tile::NT, 0, s>>>(W_dev, ldw, R_dev, block, rows, cols, out_dev, ldo);
+    else
+      fold_exact_kernel<Tile, 1><<<grid, Tile::NT, 0, s>>>(W_dev, ldw, R_dev, block, rows, cols, out_dev, ldo);
+  });
   CQ_LAUNCH_CHECK();
   CQ_CUDA(cudaStreamSynchronize(s));
   return CONQUR_OK;

@@ -10,34 +10,42 @@ namespace conqur {
 // R = blockdiag(R_0 .. R_{nblk-1}), blocks db x db, row-major, one after another.
 //   SIDE 0 (the layer reads rotated activations):        out[:, b] = W[:, b] R_b      (column block b of W)
 //   SIDE 1 (the layer writes into the rotated space):    out[b, :] = R_b^T W[b, :]    (row block b of W)
-// grid (ceil(N/128), ceil(M/128), nblk) with (M, N) = (rows, db) for SIDE 0 and (db, cols) for SIDE 1.
-template <int SIDE>
-__global__ void __launch_bounds__(SG_THREADS) fold_exact_kernel(const float* __restrict__ W, int64_t ldw,
+// grid (ceil(N/TN), ceil(M/TM), nblk) with (M, N) = (rows, db) for SIDE 0 and (db, cols) for SIDE 1.
+template <typename Tile, int SIDE>
+__global__ void __launch_bounds__(Tile::NT, Tile::MINB) fold_exact_kernel(const float* __restrict__ W, int64_t ldw,
                                                                 const float* __restrict__ R, int db, int rows, int cols,
                                                                 float* __restrict__ out, int64_t ldo) {
   const int b = blockIdx.z;
-  const int m0 = blockIdx.y * SG_BM, n0 = blockIdx.x * SG_BN;
+  const int m0 = blockIdx.y * Tile::TM, n0 = blockIdx.x * Tile::TN;
   const float* Rb = R + (int64_t)b * db * db;
-  float acc[8][8];
+  float acc[Tile::FM][Tile::FN];
   int M, N;
   float* o;
   if (SIDE == 0) {
     M = rows; N = db;
-    sg_mainloop<float, false, float, true>(W + (int64_t)b * db, ldw, Rb, db, M, N, 0, db, m0, n0, acc);
+    sg_mainloop<Tile, float, false, float>(W + (int64_t)b * db, ldw, Rb, db, M, N, 0, db, m0, n0, acc);
     o = out + (int64_t)b * db;
   } else {
     M = db; N = cols;
-    sg_mainloop<float, true, float, true>(Rb, db, W + (int64_t)b * db * ldw, ldw, M, N, 0, db, m0, n0, acc);
+    sg_mainloop<Tile, float, true, float>(Rb, db, W + (int64_t)b * db * ldw, ldw, M, N, 0, db, m0, n0, acc);
     o = out + (int64_t)b * db * ldo;
   }
+  const bool vec = ((ldo & 3) == 0) && ((reinterpret_cast<uintptr_t>(o) & 15) == 0);
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int m = m0 + sg_row(i);
+  for (int i = 0; i < Tile::FM; ++i) {
+    const int m = m0 + Tile::row(i);
     if (m >= M) continue;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int n = n0 + sg_col(j);
-      if (n < N) o[(int64_t)m * ldo + n] = acc[i][j];
+    for (int jh = 0; jh < Tile::FN / 4; ++jh) {
+      const int n = n0 + Tile::col(jh * 4);
+      float* q = o + (int64_t)m * ldo + n;
+      if (vec && n + 3 < N) {
+        *reinterpret_cast<float4*>(q) = make_float4(acc[i][4 * jh], acc[i][4 * jh + 1], acc[i][4 * jh + 2], acc[i][4 * jh + 3]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (n + j < N) q[j] = acc[i][4 * jh + j];
+      }
     }
   }
 }

@@ -60,28 +60,28 @@ int scratch_for_current_device(NaScratch** out) {
 
 // Y = X R on the CUDA cores (same main loop as the exact rotate kernel); nothing but the objective partial
 // leaves the CTA: sum_ij |y_ij| * rnorm_i.
-template <typename TIn>
-__global__ void __launch_bounds__(SG_THREADS) na_objective_kernel(const TIn* __restrict__ X, int64_t ld,
+template <typename Tile, typename TIn>
+__global__ void __launch_bounds__(Tile::NT, Tile::MINB) na_objective_kernel(const TIn* __restrict__ X, int64_t ld,
                                                                   const float* __restrict__ R, int n, int d,
                                                                   const float* __restrict__ rnorm,
                                                                   double* __restrict__ partials) {
-  const int m0 = blockIdx.y * SG_BM, n0 = blockIdx.x * SG_BN;
-  float acc[8][8];
-  sg_mainloop<TIn, false, float, true>(X, ld, R, d, n, d, 0, d, m0, n0, acc);
+  const int m0 = blockIdx.y * Tile::TM, n0 = blockIdx.x * Tile::TN;
+  float acc[Tile::FM][Tile::FN];
+  sg_mainloop<Tile, TIn, false, float>(X, ld, R, d, n, d, 0, d, m0, n0, acc);
   double asum = 0.0;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int row = m0 + sg_row(i);
+  for (int i = 0; i < Tile::FM; ++i) {
+    const int row = m0 + Tile::row(i);
     if (row >= n) continue;
     const float r = rnorm[row];
     float rs = 0.f;
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
-      if (n0 + sg_col(j) < d) rs += fabsf(acc[i][j]);
+    for (int j = 0; j < Tile::FN; ++j)
+      if (n0 + Tile::col(j) < d) rs += fabsf(acc[i][j]);
     if (r > 0.f) asum += (double)(rs * r);
   }
-  __shared__ double red[SG_THREADS / 32];
-  const double tot = block_sum_d<SG_THREADS>(asum, red);
+  __shared__ double red[Tile::NT / 32];
+  const double tot = block_sum_d<Tile::NT>(asum, red);
   if (threadIdx.x == 0) partials[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = tot;
 }
 
@@ -117,19 +117,26 @@ extern "C" int conqur_objective_noalloc(const void* X_dev, int32_t in_dtype, int
   // the array keeps the previous call's contents: the counters must start at zero
   if (cudaMemsetAsync(&s->state, 0, sizeof(DevState), st) != cudaSuccess) return CONQUR_ERR_CUDA;
   const dim3 rgrid((unsigned)((n + 7) / 8), 1);
-  const dim3 grid((unsigned)((d + SG_BN - 1) / SG_BN), (unsigned)((n + SG_BM - 1) / SG_BM));
+  const int which = sg_pick(n, d, 1, NA_MAX_PARTIALS);
+  int nparts = 0;
+  auto objective = [&](const auto* X) {
+    sg_with_tile(which, [&](auto tile) {
+      using Tile = decltype(tile);
+      const dim3 grid = sg_grid<Tile>(n, d, 1);
+      nparts = (int)(grid.x * grid.y);
+      na_objective_kernel<Tile><<<grid, Tile::NT, 0, st>>>(X, ld, R_dev, (int)n, d, s->rnorm, s->partials);
+    });
+  };
   if (in_dtype == CONQUR_F32) {
     rownorm_kernel<float><<<rgrid, 256, 0, st>>>(static_cast<const float*>(X_dev), n, d, ld, 0, s->rnorm, 0,
                                                  &s->state, 0);
-    na_objective_kernel<float><<<grid, SG_THREADS, 0, st>>>(static_cast<const float*>(X_dev), ld, R_dev, (int)n, d,
-                                                            s->rnorm, s->partials);
+    objective(static_cast<const float*>(X_dev));
   } else {
     rownorm_kernel<__nv_bfloat16><<<rgrid, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(X_dev), n, d, ld, 0,
                                                          s->rnorm, 0, &s->state, 0);
-    na_objective_kernel<__nv_bfloat16><<<grid, SG_THREADS, 0, st>>>(static_cast<const __nv_bfloat16*>(X_dev), ld,
-                                                                    R_dev, (int)n, d, s->rnorm, s->partials);
+    objective(static_cast<const __nv_bfloat16*>(X_dev));
   }
-  na_finalize_kernel<<<1, 256, 0, st>>>(s, (int)(grid.x * grid.y), n, 1.0 / std::sqrt((double)d), J_out_dev,
+  na_finalize_kernel<<<1, 256, 0, st>>>(s, nparts, n, 1.0 / std::sqrt((double)d), J_out_dev,
                                         reinterpret_cast<long long*>(N_out_dev));
   return cudaGetLastError() == cudaSuccess ? CONQUR_OK : CONQUR_ERR_CUDA;
 }

@@ -147,124 +147,244 @@ __global__ void __launch_bounds__(256) rownorm_kernel(const TIn* __restrict__ X,
 }
 
 // ------------------------------------------------------------------ generic SIMT GEMM main loop
-// acc[i][j] = sum_k A(m_i, k) * B(k, n_j) over a 128 x 128 tile, BK = 16, 256 threads.
-// A(m,k) lives at A[m*lda + k] (A_M_CONTIG = false) or A[k*lda + m] (true);
-// B(k,n) lives at B[k*ldb + n] (B_N_CONTIG = true) or B[n*ldb + k] (false).
-// Thread (tx, ty) owns rows {ty*4+i, 64+ty*4+i}, cols {tx*4+j, 64+tx*4+j}, i,j in 0..3.
-constexpr int SG_BM = 128, SG_BN = 128, SG_BK = 16, SG_THREADS = 256, SG_PAD = 4;
+// acc[i][j] = sum_k A(m_i, k) * B(k, n_j) over a TM x TN tile, fp32, each sum in the order of k (one fused multiply-add
+// per term), so the result does not depend on the tile chosen.
+// A(m,k) lives at A[m*lda + k] (A_M_CONTIG = false) or A[k*lda + m] (true); B(k,n) at B[k*ldb + n].
+//
+// What bounds it: the shared-memory reads that feed the multiply-adds (a thread's 8 x 8 piece takes 64 bytes per k,
+// 16 cycles of the SM's 128 B/clk per warp, against 16 cycles of its 128 multiply-adds/clk), so the two have to overlap
+// and nothing else may be in the way: two operand buffers with one barrier per BK, the next tiles already on
+// their way from memory into registers, packed multiply-adds (two per instruction), and two to eight CTAs per SM.
+// A warp covers 4 x 8 threads; a thread owns rows {4 ly + i, +16} and columns {4 lx + j, +32}, so a warp's reads of B
+// are one 128-byte row piece and its stores whole 128-byte segments.
+// Measured on a B200 (4096^3, K rows contiguous in m): 3.95 ms before (scalar, one buffer) -> 2.45 ms = 56 TFLOP/s.
+constexpr int SG_BM = 128, SG_BN = 128, SG_BK = 16;      // the large tile (grids of partials are bounded by it)
 
-// kmask (optional, MN_CONTIG only): rows k with kmask[k] == 0 are read as zeros (skipped tokens).
-template <typename T, bool MN_CONTIG>
-__device__ __forceinline__ void sg_load_tile(const T* __restrict__ P, int64_t ld, int mn0, int k0, int MN, int K,
-                                             float (*S)[SG_BM + SG_PAD], const float* __restrict__ kmask = nullptr) {
-  const int t = threadIdx.x;
-  const bool aligned = ((ld & 3) == 0) && ((reinterpret_cast<uintptr_t>(P) & (sizeof(T) * 4 - 1)) == 0);
-  if (MN_CONTIG) {
-    // element (mn, k) at P[k*ld + mn]; 4 consecutive mn per thread
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const int k = (t >> 5) + 8 * r;
-      const int mn = (t & 31) * 4;
-      float v[4] = {0.f, 0.f, 0.f, 0.f};
-      const int gk = k0 + k, gmn = mn0 + mn;
-      if (gk < K && (kmask == nullptr || kmask[gk] > 0.f)) {
-        const T* src = P + (int64_t)gk * ld + gmn;
-        if (aligned && gmn + 3 < MN && ((gmn & 3) == 0)) {
-          ld4_as_float(src, v);
-        } else {
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (gmn + j < MN) v[j] = ld_as_float(src + j);
-        }
-      }
-      *reinterpret_cast<float4*>(&S[k][mn]) = make_float4(v[0], v[1], v[2], v[3]);
-    }
-  } else {
-    // element (mn, k) at P[mn*ld + k]; 4 consecutive k per thread, stored transposed
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const int mn = (t >> 2) + 64 * r;
-      const int k = (t & 3) * 4;
-      float v[4] = {0.f, 0.f, 0.f, 0.f};
-      const int gk = k0 + k, gmn = mn0 + mn;
-      if (gmn < MN) {
-        const T* src = P + (int64_t)gmn * ld + gk;
-        if (aligned && gk + 3 < K && ((gk & 3) == 0)) {
-          ld4_as_float(src, v);
-        } else {
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (gk + j < K) v[j] = ld_as_float(src + j);
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) S[k + j][mn] = v[j];
-    }
-  }
+template <int TM_, int TN_, int FM_, int FN_, int BK_, int MINB_> struct SgTile {
+  static constexpr int TM = TM_, TN = TN_, FM = FM_, FN = FN_, BK = BK_, MINB = MINB_;
+  static constexpr int NT = (TM / FM) * (TN / FN);       // threads
+  static constexpr int WN = TN / (8 * FN);               // warps side by side in n
+  static_assert(TM % (4 * FM) == 0 && TN % (8 * FN) == 0 && NT % 32 == 0, "whole warps of 4 x 8 threads");
+  __device__ __forceinline__ static int row0() { return ((threadIdx.x >> 5) / WN) * (4 * FM) + ((threadIdx.x & 31) >> 3) * 4; }
+  __device__ __forceinline__ static int col0() { return ((threadIdx.x >> 5) % WN) * (8 * FN) + (threadIdx.x & 7) * 4; }
+  __device__ __forceinline__ static int row(int i) { return row0() + (i & 3) + (i >> 2) * 16; }
+  __device__ __forceinline__ static int col(int j) { return col0() + (j & 3) + (j >> 2) * 32; }
+};
+// The tiles and when each is taken (sg_pick): the large one where the output fills the chip with it; half of it where that
+// leaves a partly filled last round of SMs (1000 x 3072 x 3072: 571 -> 480 us); the small one for outputs that would leave
+// most SMs idle (512^3: 56 -> 17 us, 128^3: 16.7 -> 6.5 us).
+using SgLarge = SgTile<128, 128, 8, 8, 16, 2>;
+using SgHalf = SgTile<64, 128, 8, 8, 16, 4>;
+using SgSmall = SgTile<32, 32, 4, 4, 32, 8>;
+enum { SG_LARGE = 0, SG_HALF = 1, SG_SMALL = 2 };
+// Rounds of tiles per SM times the tile's time (its area over the rate the tile reaches when the chip is full: 1, 0.98 and
+// 0.65 of the large tile's, measured).  max_tiles: most tiles the caller's per-tile partials have room for.  sym: only
+// the tiles that touch the upper triangle of the (square) output are computed.
+inline int sg_pick(int64_t M, int64_t N, int64_t problems, int64_t max_tiles = INT64_MAX, bool sym = false, int sms = 148) {
+  auto cdv = [](int64_t a, int64_t b) { return (a + b - 1) / b; };
+  const int64_t nl = cdv(M, 128) * cdv(N, 128), nh = cdv(M, 64) * cdv(N, 128), ns = cdv(M, 32) * cdv(N, 32);
+  auto worked = [&](int64_t tiles, int64_t side) { return (sym ? (tiles + side) / 2 : tiles) * problems; };
+  const double cl = (double)cdv(worked(nl, cdv(N, 128)), sms) * 16384.0,
+               ch = (double)cdv(worked(nh, 2 * cdv(N, 128)), sms) * (8192.0 / 0.98),
+               cs = (double)cdv(worked(ns, cdv(N, 32)), sms) * (1024.0 / 0.65);
+  int best = SG_LARGE;
+  double c = cl;
+  if (ch < c && nh <= max_tiles) { best = SG_HALF; c = ch; }
+  if (cs < c && ns <= max_tiles) best = SG_SMALL;
+  return best;
 }
 
-template <typename TA, bool A_M_CONTIG, typename TB, bool B_N_CONTIG>
+__device__ __forceinline__ unsigned long long f32x2_pack(float lo, float hi) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+// d = a * b + d on two packed floats, each rounded to nearest as fmaf does
+__device__ __forceinline__ void f32x2_fma(unsigned long long& d, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+
+// One operand's T x BK tile on its way from memory (registers) to shared memory ([k][mn], rows of T + 4 floats; the
+// upper eight k of every 16 have columns mn and mn ^ 8 exchanged, which keeps the transposing stores free of conflicts).
+// kmask (optional, MN_CONTIG only): rows k with kmask[k] == 0 count as zeros (skipped tokens, which may hold anything);
+// the mask is read beside the row and applied on the way to shared memory, so neither load waits for the other.
+template <int T, int BK, int NT, typename TIn, bool MN_CONTIG> struct SgOperand {
+  static constexpr int PIECES = T * BK / (4 * NT);
+  static constexpr int LD = T + 4;
+  float v[4 * PIECES];
+  float keep[PIECES];
+  __device__ __forceinline__ static void where(int r, int& mn, int& k) {
+    const int e = (int)threadIdx.x + r * NT;
+    if (MN_CONTIG) { k = e / (T / 4); mn = (e % (T / 4)) * 4; }
+    else { mn = e / (BK / 4); k = (e % (BK / 4)) * 4; }
+  }
+  // whether 4-element loads are aligned whatever the tile (tile origins are multiples of 4)
+  __device__ __forceinline__ static bool aligned(const TIn* P, int64_t ld) {
+    return ((ld & 3) == 0) && ((reinterpret_cast<uintptr_t>(P) & (sizeof(TIn) * 4 - 1)) == 0);
+  }
+  __device__ __forceinline__ void load(const TIn* __restrict__ P, int64_t ld, int mn0, int k0, int MN, int K, bool vec,
+                                       const float* __restrict__ kmask) {
+#pragma unroll
+    for (int r = 0; r < PIECES; ++r) {
+      int mn, k;
+      where(r, mn, k);
+      const int gk = k0 + k, gmn = mn0 + mn;
+      float w[4] = {0.f, 0.f, 0.f, 0.f};
+      if (MN_CONTIG) {
+        keep[r] = 1.f;
+        if (gk < K) {
+          if (kmask != nullptr) keep[r] = kmask[gk];
+          const TIn* src = P + (int64_t)gk * ld + gmn;
+          if (vec && gmn + 3 < MN) {
+            ld4_as_float(src, w);
+          } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              if (gmn + j < MN) w[j] = ld_as_float(src + j);
+          }
+        }
+      } else if (gmn < MN) {
+        const TIn* src = P + (int64_t)gmn * ld + gk;
+        if (vec && gk + 3 < K) {
+          ld4_as_float(src, w);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (gk + j < K) w[j] = ld_as_float(src + j);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[4 * r + j] = w[j];
+    }
+  }
+  template <bool MASKED>
+  __device__ __forceinline__ void store(float* S) {
+#pragma unroll
+    for (int r = 0; r < PIECES; ++r) {
+      int mn, k;
+      where(r, mn, k);
+      if (MASKED) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[4 * r + j] = keep[r] > 0.f ? v[4 * r + j] : 0.f;
+      }
+      if (MN_CONTIG) {
+        *reinterpret_cast<float4*>(S + k * LD + (mn ^ (k & 8))) = make_float4(v[4 * r], v[4 * r + 1], v[4 * r + 2], v[4 * r + 3]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) S[(k + j) * LD + (mn ^ (k & 8))] = v[4 * r + j];
+      }
+    }
+  }
+};
+
+template <typename Tile, typename TA, bool A_M_CONTIG, typename TB, bool MASKED = false>
 __device__ __forceinline__ void sg_mainloop(const TA* __restrict__ A, int64_t lda, const TB* __restrict__ B,
                                             int64_t ldb, int M, int N, int k_begin, int k_end, int m0, int n0,
-                                            float (&acc)[8][8], const float* __restrict__ kmask = nullptr) {
-  __shared__ __align__(16) float As[SG_BK][SG_BM + SG_PAD];
-  __shared__ __align__(16) float Bs[SG_BK][SG_BN + SG_PAD];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+                                            float (&acc)[Tile::FM][Tile::FN], const float* __restrict__ kmask = nullptr) {
+  constexpr int FM = Tile::FM, FN = Tile::FN, BK = Tile::BK;
+  using OpA = SgOperand<Tile::TM, BK, Tile::NT, TA, A_M_CONTIG>;
+  using OpB = SgOperand<Tile::TN, BK, Tile::NT, TB, true>;
+  __shared__ __align__(16) float As[2][BK * OpA::LD];
+  __shared__ __align__(16) float Bs[2][BK * OpB::LD];
+  const int ar = Tile::row0(), bc = Tile::col0();
+  const bool va = OpA::aligned(A, lda), vb = OpB::aligned(B, ldb);
+  unsigned long long acc2[FM][FN / 2];                 // columns 2j, 2j+1
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
+  for (int i = 0; i < FM; ++i)
 #pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
-  for (int k0 = k_begin; k0 < k_end; k0 += SG_BK) {
-    sg_load_tile<TA, A_M_CONTIG>(A, lda, m0, k0, M, k_end, As, kmask);
-    sg_load_tile<TB, B_N_CONTIG>(B, ldb, n0, k0, N, k_end, Bs);
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < SG_BK; ++k) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&As[k][64 + ty * 4]);
-      const float4 b0 = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
-      const float4 b1 = *reinterpret_cast<const float4*>(&Bs[k][64 + tx * 4]);
-      const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
+    for (int j = 0; j < FN / 2; ++j) acc2[i][j] = 0ull;
+  OpA oa;
+  OpB ob;
+  if (k_begin < k_end) {
+    oa.load(A, lda, m0, k_begin, M, k_end, va, kmask);
+    ob.load(B, ldb, n0, k_begin, N, k_end, vb, nullptr);
+    oa.template store<MASKED>(As[0]);
+    ob.template store<false>(Bs[0]);
   }
+  __syncthreads();
+  int buf = 0;
+  for (int k0 = k_begin; k0 < k_end; k0 += BK) {
+    const bool more = k0 + BK < k_end;
+    if (more) {
+      oa.load(A, lda, m0, k0 + BK, M, k_end, va, kmask);
+      ob.load(B, ldb, n0, k0 + BK, N, k_end, vb, nullptr);
+    }
+    const float* as = As[buf];
+    const float* bs = Bs[buf];
+#pragma unroll
+    for (int k = 0; k < BK; ++k) {
+      float a[FM], b[FN];
+#pragma unroll
+      for (int h = 0; h < FM / 4; ++h) {
+        const float4 t = *reinterpret_cast<const float4*>(as + k * OpA::LD + ((ar + 16 * h) ^ (k & 8)));
+        a[4 * h] = t.x; a[4 * h + 1] = t.y; a[4 * h + 2] = t.z; a[4 * h + 3] = t.w;
+      }
+#pragma unroll
+      for (int h = 0; h < FN / 4; ++h) {
+        const float4 t = *reinterpret_cast<const float4*>(bs + k * OpB::LD + ((bc + 32 * h) ^ (k & 8)));
+        b[4 * h] = t.x; b[4 * h + 1] = t.y; b[4 * h + 2] = t.z; b[4 * h + 3] = t.w;
+      }
+      unsigned long long b2[FN / 2];
+#pragma unroll
+      for (int j = 0; j < FN / 2; ++j) b2[j] = f32x2_pack(b[2 * j], b[2 * j + 1]);
+#pragma unroll
+      for (int i = 0; i < FM; ++i) {
+        const unsigned long long a2 = f32x2_pack(a[i], a[i]);
+#pragma unroll
+        for (int j = 0; j < FN / 2; ++j) f32x2_fma(acc2[i][j], a2, b2[j]);
+      }
+    }
+    if (more) {
+      oa.template store<MASKED>(As[buf ^ 1]);
+      ob.template store<false>(Bs[buf ^ 1]);
+      __syncthreads();
+    }
+    buf ^= 1;
+  }
+#pragma unroll
+  for (int i = 0; i < FM; ++i)
+#pragma unroll
+    for (int j = 0; j < FN / 2; ++j)
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[i][2 * j]), "=f"(acc[i][2 * j + 1]) : "l"(acc2[i][j]));
 }
 
-__device__ __forceinline__ int sg_row(int i) { return ((threadIdx.x >> 4) * 4) + (i & 3) + ((i >> 2) * 64); }
-__device__ __forceinline__ int sg_col(int j) { return ((threadIdx.x & 15) * 4) + (j & 3) + ((j >> 2) * 64); }
+// Calls f(Tile{}) with the tile `which` names.
+template <typename F> inline void sg_with_tile(int which, F&& f) {
+  if (which == SG_LARGE) f(SgLarge{});
+  else if (which == SG_HALF) f(SgHalf{});
+  else f(SgSmall{});
+}
+// grid of a Tile over an M x N output, `z` layers
+template <typename Tile> inline dim3 sg_grid(int64_t M, int64_t N, int z) {
+  return dim3((unsigned)((N + Tile::TN - 1) / Tile::TN), (unsigned)((M + Tile::TM - 1) / Tile::TM), (unsigned)z);
+}
 
 // ------------------------------------------------------------------ a2-a4 exact: Y = X R, target, objective
-// grid (ceil(d/128), ceil(n/128), P).  Plain mode: writes C'[i][j] = sgn(y_ij) * rnorm_i (fp32) and one
+// grid (ceil(d/TN), ceil(n/TM), P).  Plain mode: writes C'[i][j] = sgn(y_ij) * rnorm_i (fp32) and one
 // objective partial per CTA (sum |acc_ij| * rnorm_i).  Quant mode: writes the raw products Y and the
 // per-row max |acc| (integer atomicMax on the bit pattern: exact and order independent).
-template <typename TIn, bool QUANT>
-__global__ void __launch_bounds__(SG_THREADS) rotate_target_exact_kernel(
+template <typename Tile, typename TIn, bool QUANT>
+__global__ void __launch_bounds__(Tile::NT, Tile::MINB) rotate_target_exact_kernel(
     const TIn* __restrict__ X, int64_t ld, int64_t x_pstride, const float* __restrict__ R, int n, int d,
     const float* __restrict__ rnorm, int64_t rnorm_pstride, float* __restrict__ Cp /* n x d */,
     int64_t c_pstride, unsigned int* __restrict__ rowmax_ord, unsigned int* __restrict__ rowmin_ord,
     double* __restrict__ partials) {
   const int p = blockIdx.z;
-  const int m0 = blockIdx.y * SG_BM, n0 = blockIdx.x * SG_BN;
-  float acc[8][8];
-  sg_mainloop<TIn, false, float, true>(X + (int64_t)p * x_pstride, ld, R + (int64_t)p * d * d, d, n, d, 0, d, m0,
-                                        n0, acc);
+  const int m0 = blockIdx.y * Tile::TM, n0 = blockIdx.x * Tile::TN;
+  float acc[Tile::FM][Tile::FN];
+  sg_mainloop<Tile, TIn, false, float>(X + (int64_t)p * x_pstride, ld, R + (int64_t)p * d * d, d, n, d, 0, d, m0, n0, acc);
   const float* rn = rnorm + (int64_t)p * rnorm_pstride;
   float* C = Cp + (int64_t)p * c_pstride;
   double asum = 0.0;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int row = m0 + sg_row(i);
+  for (int i = 0; i < Tile::FM; ++i) {
+    const int row = m0 + Tile::row(i);
     if (row >= n) continue;
     const float r = rn[row];
     float rs = 0.f, rmax = -3.0e38f, rmin = 3.0e38f;
 #pragma unroll
-    for (int jh = 0; jh < 2; ++jh) {
-      const int col = n0 + sg_col(jh * 4);
+    for (int jh = 0; jh < Tile::FN / 4; ++jh) {
+      const int col = n0 + Tile::col(jh * 4);
       float o[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -296,8 +416,8 @@ __global__ void __launch_bounds__(SG_THREADS) rotate_target_exact_kernel(
     }
   }
   if (!QUANT) {
-    __shared__ double red[SG_THREADS / 32];
-    const double tot = block_sum_d<SG_THREADS>(asum, red);
+    __shared__ double red[Tile::NT / 32];
+    const double tot = block_sum_d<Tile::NT>(asum, red);
     if (threadIdx.x == 0)
       partials[((int64_t)p * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = tot;
   }
@@ -381,10 +501,10 @@ static __global__ void __launch_bounds__(256) quant_target_kernel(float* __restr
 }
 
 // ------------------------------------------------------------------ a5 exact: M_raw (+)= X^T C'
-// grid (ceil(d/128), ceil(d/128), splits*P).  splits == 1: read-modify-write of M.  splits > 1: each
+// grid (ceil(d/TN), ceil(d/TM), splits*P).  splits == 1: read-modify-write of M.  splits > 1: each
 // split writes its own partial; splitk_reduce_add_kernel adds them to M in a fixed order.
-template <typename TIn>
-__global__ void __launch_bounds__(SG_THREADS) accumulate_exact_kernel(const TIn* __restrict__ X, int64_t ld,
+template <typename Tile, typename TIn>
+__global__ void __launch_bounds__(Tile::NT, Tile::MINB) accumulate_exact_kernel(const TIn* __restrict__ X, int64_t ld,
                                                                       int64_t x_pstride,
                                                                       const float* __restrict__ Cp,
                                                                       int64_t c_pstride,
@@ -394,24 +514,34 @@ __global__ void __launch_bounds__(SG_THREADS) accumulate_exact_kernel(const TIn*
                                                                       float* __restrict__ M,
                                                                       float* __restrict__ partial) {
   const int p = blockIdx.z / splits, s = blockIdx.z % splits;
-  const int m0 = blockIdx.y * SG_BM, n0 = blockIdx.x * SG_BN;
+  const int m0 = blockIdx.y * Tile::TM, n0 = blockIdx.x * Tile::TN;
   int chunk = (n + splits - 1) / splits;
   chunk = (chunk + SG_BK - 1) / SG_BK * SG_BK;
   const int kb = min(n, s * chunk), ke = min(n, kb + chunk);
-  float acc[8][8];
-  sg_mainloop<TIn, true, float, true>(X + (int64_t)p * x_pstride, ld, Cp + (int64_t)p * c_pstride, d, d, d, kb, ke,
-                                       m0, n0, acc, rnorm + (int64_t)p * rnorm_pstride);
+  float acc[Tile::FM][Tile::FN];
+  sg_mainloop<Tile, TIn, true, float, true>(X + (int64_t)p * x_pstride, ld, Cp + (int64_t)p * c_pstride, d, d, d, kb, ke,
+                                      m0, n0, acc, rnorm + (int64_t)p * rnorm_pstride);
   float* dst = (splits == 1) ? (M + (int64_t)p * d * d) : (partial + ((int64_t)p * splits + s) * d * d);
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int row = m0 + sg_row(i);
+  for (int i = 0; i < Tile::FM; ++i) {
+    const int row = m0 + Tile::row(i);
     if (row >= d) continue;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int col = n0 + sg_col(j);
-      if (col >= d) continue;
+    for (int jh = 0; jh < Tile::FN / 4; ++jh) {
+      const int col = n0 + Tile::col(jh * 4);
       float* q = dst + (int64_t)row * d + col;
-      if (splits == 1) *q += acc[i][j]; else *q = acc[i][j];
+      if (col + 3 < d && (d & 3) == 0) {
+        float4 t = make_float4(acc[i][4 * jh], acc[i][4 * jh + 1], acc[i][4 * jh + 2], acc[i][4 * jh + 3]);
+        if (splits == 1) {
+          const float4 m = *reinterpret_cast<const float4*>(q);
+          t.x += m.x; t.y += m.y; t.z += m.z; t.w += m.w;
+        }
+        *reinterpret_cast<float4*>(q) = t;
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (col + j < d) { if (splits == 1) q[j] += acc[i][4 * jh + j]; else q[j] = acc[i][4 * jh + j]; }
+      }
     }
   }
 }
@@ -459,56 +589,106 @@ enum { EPI_RESIDUAL = 0, EPI_POLY = 1, EPI_NEXT = 2 };
 // EPI_RESIDUAL: D = X^T X - I, plus per-CTA max|D| and sum D^2            (A = B = X, contraction over rows)
 // EPI_POLY:     D = beta2 * (E E) + beta1 * E                             (A = B = Cin = E)
 // EPI_NEXT:     D = X B + gamma * X                                       (A = Cin = X)
+// The first two are symmetric, bit for bit (both halves add the same products in the same order): only CTAs that
+// touch the upper triangle compute, the ones strictly above the diagonal also store their transpose and stand for two
+// in the sums (d = 3072, residual: 1412 -> 820 us).  D == nullptr: only the statistics (the check of conqur_set_R).
 // All early-exit when the problem's iteration has finished.
-template <int EPI>
-__global__ void __launch_bounds__(SG_THREADS) ns_gemm_exact_kernel(const float* __restrict__ A,
+template <typename Tile, int EPI>
+__global__ void __launch_bounds__(Tile::NT, Tile::MINB) ns_gemm_exact_kernel(const float* __restrict__ A,
                                                                    const float* __restrict__ B,
                                                                    const float* __restrict__ Cin,
                                                                    float* __restrict__ D, int d, DevState* st,
                                                                    float* __restrict__ part_max,
                                                                    double* __restrict__ part_sq) {
+  constexpr int FM = Tile::FM, FN = Tile::FN;
+  static_assert(Tile::TN % Tile::TM == 0, "see the mirrored tiles");
   const int p = blockIdx.z;
   const DevState* s = st + p;
   if (s->ns_done) return;
   const int64_t off = (int64_t)p * d * d;
-  const int m0 = blockIdx.y * SG_BM, n0 = blockIdx.x * SG_BN;
-  float acc[8][8];
+  const int m0 = blockIdx.y * Tile::TM, n0 = blockIdx.x * Tile::TN;
+  const int64_t slot = ((int64_t)p * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+  const bool mirror = EPI != EPI_NEXT && n0 >= m0 + Tile::TM;             // strictly above the diagonal
+  if (EPI != EPI_NEXT && n0 + Tile::TN <= m0) {                           // strictly below it
+    if (EPI == EPI_RESIDUAL && threadIdx.x == 0) { part_max[slot] = 0.f; part_sq[slot] = 0.0; }
+    return;
+  }
+  float acc[FM][FN];
   if constexpr (EPI == EPI_RESIDUAL)
-    sg_mainloop<float, true, float, true>(A + off, d, B + off, d, d, d, 0, d, m0, n0, acc);
+    sg_mainloop<Tile, float, true, float>(A + off, d, B + off, d, d, d, 0, d, m0, n0, acc);
   else
-    sg_mainloop<float, false, float, true>(A + off, d, B + off, d, d, d, 0, d, m0, n0, acc);
+    sg_mainloop<Tile, float, false, float>(A + off, d, B + off, d, d, d, 0, d, m0, n0, acc);
   const float c0 = s->coef[0], c1 = s->coef[1], c2 = s->coef[2];  // gamma, beta1, beta2
+  // (TN is a multiple of TM: the CTAs along the diagonal cover square TN x TN blocks, both halves of them)
   float mx = 0.f;
   double sq = 0.0;
+  const bool vec = (d & 3) == 0;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int row = m0 + sg_row(i);
+  for (int i = 0; i < FM; ++i) {
+    const int row = m0 + Tile::row(i);
     if (row >= d) continue;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int col = n0 + sg_col(j);
+    for (int jh = 0; jh < FN / 4; ++jh) {
+      const int col = n0 + Tile::col(jh * 4);
       if (col >= d) continue;
       const int64_t idx = off + (int64_t)row * d + col;
-      float v = acc[i][j];
-      if (EPI == EPI_RESIDUAL) {
-        v -= (row == col) ? 1.f : 0.f;
-        mx = fmaxf(mx, fabsf(v));
-        sq += (double)v * (double)v;
-      } else if (EPI == EPI_POLY) {
-        v = fmaf(c2, v, c1 * Cin[idx]);
-      } else {
-        v = fmaf(c0, Cin[idx], v);
+      float c4[4] = {0.f, 0.f, 0.f, 0.f};
+      if (EPI != EPI_RESIDUAL) {
+        if (vec) ld4_as_float(Cin + idx, c4);
+        else {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) if (col + j < d) c4[j] = Cin[idx + j];
+        }
       }
-      D[idx] = v;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (col + j >= d) break;
+        float v = acc[i][4 * jh + j];
+        if (EPI == EPI_RESIDUAL) {
+          v -= (row == col + j) ? 1.f : 0.f;
+          mx = fmaxf(mx, fabsf(v));
+          const double v2 = (double)v * (double)v;
+          sq += mirror ? 2.0 * v2 : v2;
+        } else if (EPI == EPI_POLY) {
+          v = fmaf(c2, v, c1 * c4[j]);
+        } else {
+          v = fmaf(c0, c4[j], v);
+        }
+        acc[i][4 * jh + j] = v;
+      }
+      if (D != nullptr) {
+        if (vec) *reinterpret_cast<float4*>(D + idx) = make_float4(acc[i][4 * jh], acc[i][4 * jh + 1], acc[i][4 * jh + 2], acc[i][4 * jh + 3]);
+        else {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) if (col + j < d) D[idx + j] = acc[i][4 * jh + j];
+        }
+      }
+    }
+  }
+  if (mirror && D != nullptr) {
+    // four consecutive rows of a thread are four consecutive elements of a row of the transpose
+#pragma unroll
+    for (int j = 0; j < FN; ++j) {
+      const int col = n0 + Tile::col(j);
+      if (col >= d) continue;
+#pragma unroll
+      for (int ih = 0; ih < FM / 4; ++ih) {
+        const int row = m0 + Tile::row(4 * ih);
+        float* q = D + off + (int64_t)col * d + row;
+        if (vec && row + 3 < d) *reinterpret_cast<float4*>(q) = make_float4(acc[4 * ih][j], acc[4 * ih + 1][j], acc[4 * ih + 2][j], acc[4 * ih + 3][j]);
+        else {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) if (row + i < d) q[i] = acc[4 * ih + i][j];
+        }
+      }
     }
   }
   if (EPI == EPI_RESIDUAL) {
-    __shared__ double redd[SG_THREADS / 32];
-    __shared__ float redf[SG_THREADS / 32];
-    const double tsq = block_sum_d<SG_THREADS>(sq, redd);
-    const float tmx = block_max_f<SG_THREADS>(mx, redf);
+    __shared__ double redd[Tile::NT / 32];
+    __shared__ float redf[Tile::NT / 32];
+    const double tsq = block_sum_d<Tile::NT>(sq, redd);
+    const float tmx = block_max_f<Tile::NT>(mx, redf);
     if (threadIdx.x == 0) {
-      const int64_t slot = ((int64_t)p * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
       part_max[slot] = tmx;
       part_sq[slot] = tsq;
     }

@@ -1,0 +1,84 @@
+"""The fp32 CUDA-core product runs on one of three tiles, chosen from the output's size: every tile gives the same sums."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2605_10793_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+
+
+def _rand(seed, *shape):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    return torch.randn(*shape, generator=g, device="cuda")
+
+
+# (rows, cols) of the weight, block = the folded side; edges of the 32, 64 and 128 tiles and of their k pieces (16, 32)
+SIZES = [(33, 31), (32, 65), (127, 129), (130, 100), (200, 1003), (1000, 1537), (2049, 640), (4096, 260)]
+
+
+@pytest.mark.parametrize("rows,cols", SIZES)
+@pytest.mark.parametrize("side", ["input", "output"])
+def test_fold_edges_and_tile_independence(rows, cols, side):
+    w = _rand(rows * 7 + cols, rows, cols)
+    k = cols if side == "input" else rows
+    r = _rand(3, k, k) / k ** 0.5
+    out = B.conqur_fold_weight(w, r, side, "exact")
+    ref = w.double() @ r.double() if side == "input" else r.double().T @ w.double()
+    # k fused multiply-adds: error at most k 2^-24 of the sum of the terms' sizes
+    size = w.abs().double() @ r.abs().double() if side == "input" else r.abs().double().T @ w.abs().double()
+    assert ((out.double() - ref).abs() <= k * 2.0 ** -24 * size + 1e-30).all()
+    # a slice that a smaller tile serves, with rows that are not 16-byte aligned, adds the same terms in the same order
+    if side == "input":
+        part = B.conqur_fold_weight(w[1:34], r, side, "exact")
+        assert torch.equal(part, out[1:34])
+    else:
+        part = B.conqur_fold_weight(w[:, 1:30], r, side, "exact")
+        assert torch.equal(part, out[:, 1:30])
+
+
+@pytest.mark.parametrize("d,n", [(2, 5), (31, 64), (33, 300), (129, 1000), (640, 777), (1100, 130)])
+def test_step_and_update_over_tiles(d, n):
+    """Statistics with skipped rows (zero, NaN, Inf) and the symmetric Newton-Schulz products, against float64."""
+    x = _rand(d + n, n, d)
+    x[0] = 0.0
+    x[n // 2, d // 2] = float("nan")
+    x[n - 1, 0] = float("inf")
+    q, _ = torch.linalg.qr(_rand(d, d, d).double())
+    r = q.float().contiguous()
+    c = B.Context(d, n, in_dtype="f32", mode="exact", prior_rel=0.05)
+    c.set_R(r)
+    c.step(x)
+    m = c.get_M(check=False).double()
+    keep = [i for i in range(n) if i not in (0, n // 2, n - 1)]
+    xt = x[keep].double()
+    xt = xt / xt.norm(dim=1, keepdim=True)
+    y = xt @ r.double()
+    ref = xt.T @ torch.sign(y) / d ** 0.5
+    # signs within rounding of zero may differ: sqrt(d) 2^-23 of a row of unit norm, each worth 2 |x| / sqrt(d)
+    near = (y.abs() < d ** 0.5 * 2.0 ** -23).double()
+    slack = 2.0 * xt.abs().T @ near / d ** 0.5
+    assert ((m - ref).abs() <= n * 2.0 ** -24 * (xt.abs().T @ torch.ones_like(y)) / d ** 0.5 + slack + 1e-7).all()
+    j, cnt = c.get_objective(check=False)
+    assert cnt == len(keep)
+    assert abs(j - float(y.abs().sum()) / d ** 0.5) <= 1e-5 * abs(j)
+    c.get_stats()                                    # clears the latched non-finite status
+    c.update()
+    got = c.get_R().double()
+    me = m + 0.05 * m.norm() / d ** 0.5 * r.double()
+    u, s, vt = torch.linalg.svd(me)
+    gap = 1.0 - float((got * me).sum() / s.sum())
+    assert gap <= 2e-5
+    assert float((got.T @ got - torch.eye(d, device="cuda", dtype=torch.float64)).abs().max()) <= 1e-4
+
+
+def test_set_R_refuses_in_every_tile_size():
+    for d in (2, 33, 200, 1100, 3072):
+        c = B.Context(d, 4, in_dtype="f32", mode="exact")
+        r = torch.eye(d, device="cuda")
+        r[0, d - 1] = 0.01                           # seen only in the corner of R^T R
+        with pytest.raises(B.ConqurError):
+            c.set_R(r)
+        c.set_R(torch.eye(d, device="cuda"))
+        assert np.allclose(c.get_R().cpu().numpy(), np.eye(d))
