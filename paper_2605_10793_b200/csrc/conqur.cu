@@ -452,12 +452,17 @@ int update_impl(conqur_ctx* c) {
   return CONQUR_OK;
 }
 
-// Ends one pass of the graph's loop body (two Newton-Schulz steps): go round again while the iteration is running.
-// The pass counter bounds the loop whatever the data (the control kernel ends the iteration at ns_max_steps anyway).
-__global__ void ns_loop_condition_kernel(DevState* st, cudaGraphConditionalHandle handle, int max_passes) {
+// Ends one pass of the graph's loop body (two Newton-Schulz steps): go round again while any problem's iteration is
+// running.  The pass counter bounds the loop whatever the data (the control kernel ends the iteration at ns_max_steps
+// anyway).  One block.
+__global__ void ns_loop_condition_kernel(DevState* st, int P, cudaGraphConditionalHandle handle, int max_passes) {
+  int running = 0;
+  for (int p = threadIdx.x; p < P; p += blockDim.x) running |= st[p].ns_done == 0;
+  running = __syncthreads_or(running);
+  if (threadIdx.x != 0) return;
   const int passes = ++st->loop_passes;
   st->loop_passes_total += 1;
-  cudaGraphSetConditional(handle, (st->ns_done == 0 && passes < max_passes) ? 1u : 0u);
+  cudaGraphSetConditional(handle, (running && passes < max_passes) ? 1u : 0u);
 }
 
 // The update as a graph: prologue, a WHILE node whose body is two steps (the iterate ping-pongs between two buffers,
@@ -497,7 +502,8 @@ bool build_looped_update_graph(conqur_ctx* c) {
     capturing_body = true;
     c->stream = body_stream;
     if (update_step(c, -1, 0, false) != CONQUR_OK || update_step(c, -1, 1, false) != CONQUR_OK) break;
-    ns_loop_condition_kernel<<<1, 1, 0, body_stream>>>(c->state(), handle, c->cfg.ns_max_steps / 2 + 2);
+    ns_loop_condition_kernel<<<1, c->cfg.P > 32 ? 256 : 32, 0, body_stream>>>(c->state(), c->cfg.P, handle,
+                                                                             c->cfg.ns_max_steps / 2 + 2);
     if (cudaGetLastError() != cudaSuccess) break;
     c->prof.count(K_OTHER);
     cudaGraph_t body_out = nullptr;
@@ -532,11 +538,16 @@ bool build_looped_update_graph(conqur_ctx* c) {
   return ok;
 }
 
-// Enqueue one update: directly the first time (kernel attributes get set), then through a captured graph.
+// Enqueue one update: directly the first time (kernel attributes get set), then through a captured graph, in either mode:
+// of the steps enqueued directly only those the iteration needs do work, and at small d the rest of the ~160 launches
+// took longer than the work (exact mode, d = 128: 704 -> 340 us for set_R, step, update and get_R).  (Many tensor-core problems: one kernel.)
 int update_enqueue(conqur_ctx* c) {
   const bool no_graph = (c->cfg.debug_flags & CONQUR_DEBUG_NO_GRAPH) != 0;
-  const bool eligible = !no_graph && c->cfg.mode == CONQUR_TC_BF16 && c->cfg.P == 1 && !c->prof.enabled;
-  if (!eligible || c->updates_enqueued++ == 0) return update_impl(c);
+  const bool eligible = !no_graph && (c->cfg.mode == CONQUR_EXACT_F32 || c->cfg.P == 1) && !c->prof.enabled;
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  if (eligible && cudaStreamIsCapturing(c->stream, &capturing) != cudaSuccess) { cudaGetLastError(); capturing = cudaStreamCaptureStatusNone; }
+  // (a caller that captures the stream gets the launches themselves: an instantiated graph cannot be captured)
+  if (!eligible || capturing != cudaStreamCaptureStatusNone || c->updates_enqueued++ == 0) return update_impl(c);
   if (!c->upd_graph) {
     if (!c->cap_stream && cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
       cudaGetLastError();

@@ -82,3 +82,49 @@ def test_set_R_refuses_in_every_tile_size():
             c.set_R(r)
         c.set_R(torch.eye(d, device="cuda"))
         assert np.allclose(c.get_R().cpu().numpy(), np.eye(d))
+
+
+@pytest.mark.parametrize("batch", [1, 3, 40])
+def test_exact_update_graph_equals_direct_launches(batch):
+    """From a context's second update on, the fp32 iteration is replayed as a graph with a device-side loop: the same bits
+    as the launches enqueued one by one, problems that converge after different numbers of steps among them."""
+    d, n = 48, 200
+    out = []
+    for flags in (0, B.CONQUR_DEBUG_NO_GRAPH):
+        c = B.Context(d, n, in_dtype="f32", mode="exact", batch=batch, debug_flags=flags)
+        for rep in range(3):
+            x = _rand(rep, batch, n, d)
+            x *= torch.logspace(0, -2, batch, device="cuda")[:, None, None] ** torch.linspace(0, 1, d, device="cuda")
+            if batch == 1:
+                c.step(x[0])
+            else:
+                c.step_batched(x, n, d, n * d)
+            c.update()
+        st = c.get_stats()
+        assert st.status == 0 and st.updates == 3
+        out.append((c.get_R(), st.ns_steps_used))
+    assert torch.equal(out[0][0], out[1][0]) and out[0][1] == out[1][1]
+
+
+def test_exact_update_inside_a_callers_capture():
+    d, n = 64, 256
+    x = _rand(1, n, d)
+    ref = B.Context(d, n, in_dtype="f32", mode="exact")
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        c = B.Context(d, n, in_dtype="f32", mode="exact")
+        for _ in range(2):
+            c.step(x)
+            c.update()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        c.step(x)
+        c.update()
+    g.replay()
+    torch.cuda.synchronize()
+    for _ in range(3):
+        ref.step(x)
+        ref.update()
+    assert torch.equal(c.get_R(), ref.get_R())
