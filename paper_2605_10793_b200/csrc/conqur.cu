@@ -357,13 +357,13 @@ int update_prologue(conqur_ctx* c) {
   const float isd = (float)(1.0 / std::sqrt((double)d));
   sumsq_kernel<<<dim3(nb, P), 256, 0, c->stream>>>(M, R, dd, st, 0, pd);
   CQ_LAUNCHED(c, K_OTHER);
-  ns_setup_kernel<<<P, 256, 0, c->stream>>>(st, pd, nb, 0, g.prior_rel, isd, g.margin, d, use_shift, c->tc.e1_tau, c->n_lift_init);
+  ns_setup_kernel<<<P, 256, 0, c->stream>>>(st, pd, nb, 0, g.prior_rel, isd, g.margin, d, use_shift, c->n_lift_init);
   CQ_LAUNCHED(c, K_OTHER);
   if (g.prior_rel > 0.f) {
     sumsq_kernel<<<dim3(nb, P), 256, 0, c->stream>>>(M, R, dd, st, 1, pd);
     CQ_LAUNCHED(c, K_OTHER);
   }
-  ns_setup_kernel<<<P, 256, 0, c->stream>>>(st, pd, nb, 1, g.prior_rel, isd, g.margin, d, use_shift, c->tc.e1_tau, c->n_lift_init);
+  ns_setup_kernel<<<P, 256, 0, c->stream>>>(st, pd, nb, 1, g.prior_rel, isd, g.margin, d, use_shift, c->n_lift_init);
   CQ_LAUNCHED(c, K_OTHER);
   if (g.simt_ns) {
     ns_x0_kernel<<<dim3(ew_blocks(dd), P), 256, 0, c->stream>>>(M, R, c->at<float>(c->L.Xa), dd, st);
@@ -388,7 +388,8 @@ int update_step(conqur_ctx* c, int k, int cur, bool last) {
   const int use_shift = g.simt_ns ? 0 : 1;
   const int parts = ns_parts(c);
   const NsControlParams ncp{c->at<SchedEntry>(c->L.sched), c->n_sched, c->n_lift_init, g.ns_max_steps, d, use_shift, g.orth_tol,
-                            g.fro_tol, g.margin, g.lo_budget, 1.0 / (double)d};
+                            g.fro_tol, g.margin, g.lo_budget, 1.0 / (double)d, use_shift,
+                            1.f / 2048.f};
   float* X = cur ? Xb : Xa;
   float* Xn = cur ? Xa : Xb;
   c->tc.ns_k = k;
@@ -404,7 +405,7 @@ int update_step(conqur_ctx* c, int k, int cur, bool last) {
     CQ_LAUNCHED(c, K_NS_NEXT);
     return CONQUR_OK;
   }
-  return tc_ns_poly_next(c->tc, c->stream, cur);
+  return tc_ns_poly_next(c->tc, c->stream, cur, c->n_sched, g.ns_max_steps, g.orth_tol);
 }
 
 int update_epilogue(conqur_ctx* c) {
@@ -431,7 +432,7 @@ int update_impl(conqur_ctx* c) {
   if (g.mode == CONQUR_TC_BF16 && g.P > 1) {
     // many small problems: the whole iteration of a problem runs inside one CTA
     const NsControlParams ncp{c->at<SchedEntry>(c->L.sched), c->n_sched, c->n_lift_init, g.ns_max_steps, g.d, 1,
-                              g.orth_tol, g.fro_tol, g.margin, g.lo_budget, 1.0 / (double)g.d};
+                              g.orth_tol, g.fro_tol, g.margin, g.lo_budget, 1.0 / (double)g.d, 0, 1.f / 256.f};
     return tcb_update(c->tc, c->stream, ncp, g.prior_rel, g.margin);
   }
   int rc = update_prologue(c);
@@ -668,7 +669,7 @@ extern "C" int conqur_init(conqur_ctx** out, int32_t d, const conqur_config* cfg
                      c->at<float>(L.rnorm), c->state(), c->at<double>(L.part_d), c->at<float>(L.part_f),
                      (cfg->quant_bits || cfg->diagnostics) ? c->at<float>(L.C) : nullptr, c->at<unsigned>(L.rowmax), g.qs,
                      g.diagnostics, g.diagnostics ? c->at<double>(L.part_diag) : nullptr, &c->prof,
-                     (g.debug_flags & CONQUR_DEBUG_SINGLE_CTA) != 0, cfg->ns_gram_single_pass_tau, g.lo_budget);
+                     (g.debug_flags & CONQUR_DEBUG_SINGLE_CTA) != 0, cfg->ns_gram_single_pass_tau);
     if (rc) return fail(rc);
     rc = tc_refresh_R(c->tc, c->stream, 0);
     if (rc) return fail(rc);

@@ -779,7 +779,7 @@ __device__ __forceinline__ void ns_adapt_lift_plan(DevState* s, int n_endgame, i
 // phase 0: lam = prior_rel * ||M_raw||_F / sqrt(d)      (reads partials of sumsq over M)
 // phase 1: scale = ||M_raw + lam R||_F ; arms the iteration
 static __global__ void ns_setup_kernel(DevState* st, const double* __restrict__ partials, int nblocks, int phase,
-                                float prior_rel, float inv_sqrt_d, float margin, int d, int use_shift, float e1_tau,
+                                float prior_rel, float inv_sqrt_d, float margin, int d, int use_shift,
                                 int n_lift_init) {
   const int p = blockIdx.x;
   __shared__ double red[8];
@@ -802,7 +802,7 @@ static __global__ void ns_setup_kernel(DevState* st, const double* __restrict__ 
       s->seg_x = 2;
       // ||X_0||_F = 1/(1+margin): mean sigma^2 of the first iterate (the tensor-core mode shifts by it)
       s->tau = use_shift ? 1.0f / ((1.0f + margin) * (1.0f + margin) * (float)d) : 1.0f;
-      s->seg_e = (use_shift && s->tau < e1_tau) ? 1 : 3;
+      s->seg_e = use_shift ? 1 : 3;
     }
   }
 }
@@ -837,8 +837,10 @@ struct NsControlParams {
   const SchedEntry* sched;
   int n_sched, n_lift_init, max_steps, d, use_shift;
   float tol, fro_tol, margin;
-  float lo_budget;          // tensor-core mode: the iterate enters the last product as hi + lo while d 2^-8 / growth exceeds this
+  float lo_budget;          // tensor-core mode: the iterate enters the last product as hi + lo while d lo_unit / growth exceeds this
   double inv_d;             // 1 / d (the decision runs on one thread between two products: no divisions there)
+  int full_check;           // 1: a rotation is accepted only on a residual of all three passes (seg_e == 3)
+  float lo_unit;            // rounding of the one-pass form's operand: 2^-8 where it is the bf16 hi part, 2^-11 for the fp16 copy
 };
 
 // The decision itself (one thread): tmx = max|G - I|, tsq = ||G - I||_F^2, ttr = tr G of step k.
@@ -871,7 +873,7 @@ __device__ __forceinline__ unsigned char ns_control_decide(NsCtl* s, float tmx, 
   s->e_fro = fro;
   if (!(tmx == tmx) || !(fro == fro)) {
     s->ns_done = NS_DONE_FAILED;
-  } else if (tmx <= c.tol && fro <= c.fro_tol) {
+  } else if (tmx <= c.tol && fro <= c.fro_tol && (!c.full_check || s->seg_e == 3)) {
     s->ns_done = NS_DONE_CONVERGED;
     s->ns_final_buf = cur_buf;
   } else if (k >= c.max_steps) {
@@ -922,9 +924,9 @@ __device__ __forceinline__ unsigned char ns_control_decide(NsCtl* s, float tmx, 
     s->coef[1] = (float)b1;
     s->coef[2] = (float)cc;
     s->coef[3] = (float)kappa;
-    // bf16 rounding of X adds noise of spectral size about 2^-8; after a cumulative growth G of the small singular
-    // values the directions it can scramble had sigma_0 <= 2^-8 / G, at most d of them: Procrustes gap <= d 2^-8 / G
-    const int seg_x = (!c.use_shift || (float)c.d * (1.0f / 256.0f) / s->growth > c.lo_budget) ? 2 : 1;
+    // rounding X adds noise of spectral size about u = lo_unit; after a cumulative growth G of the small singular
+    // values the directions it can scramble had sigma_0 <= u / G, at most d of them: Procrustes gap <= d u / G
+    const int seg_x = (!c.use_shift || (float)c.d * c.lo_unit / s->growth > c.lo_budget) ? 2 : 1;
     s->growth *= (float)a;
     s->seg_x = seg_x;
     log_entry = (unsigned char)(seg_x | (s->seg_e << 4));           // seg_e: what this step's residual product used
@@ -963,15 +965,13 @@ static __global__ void ns_control_kernel(DevState* st, const float* __restrict__
 }
 
 // tau of the next residual product = mean sigma^2 of the new iterate = ||X||_F^2 / d (tensor-core mode), and how
-// many bf16 passes that product takes.  Dropping the iterate's lo part changes G = X^T X by about
-// 4.4e-3 sqrt(tau) sigma_max (a symmetric perturbation).  One pass is enough
-//   * while the iterate is tiny (tau below e1_tau): the perturbation is small in absolute terms;
-//   * for a late lifting step, once the small singular values have grown so far (same bound as for the iterate's
-//     lo part in the last product: d 2^-8 / growth <= lo_budget) that the directions such noise can still scramble
-//     carry no weight.  Endgame steps and the acceptance check always take three passes: there a perturbation of
-//     G by a few 1e-3 costs a whole extra step.
+// many passes that product takes: three over the bf16 pair when it may accept the rotation, i.e. once the last endgame
+// entry has been applied or no step is left; one over the fp16 copy otherwise (see tc_ns_residual).  One pass leaves about
+// 0.8 2^-12 / sqrt(d) in an entry of G and the last endgame step hands that on to X^T X - I, so that step's G takes three
+// passes as well where the largest of d^2 such entries (4.5 times as much) would come near the tolerance (d <= 1240 at 1e-4:
+// at d = 512 every update spent a step more).
 static __global__ void ns_tau_kernel(DevState* st, const double* __restrict__ part_x2, int nparts, int d, float e1_tau,
-                                     float lo_budget) {
+                                     int n_sched, int max_steps, float tol) {
   DevState* s = st + blockIdx.x;
   if (s->ns_done) return;
   __shared__ double redd[8];
@@ -980,9 +980,10 @@ static __global__ void ns_tau_kernel(DevState* st, const double* __restrict__ pa
   const double tot = block_sum_d<256>(v, redd);
   if (threadIdx.x == 0) {
     s->tau = (float)(tot / (double)d);
-    const bool grown = (float)d * (1.0f / 256.0f) / s->growth <= lo_budget;
-    const bool next_is_lifting = s->lift_left > 0 && s->e_fro >= 0.7f;     // (control drops the rest of the lifting below 0.7)
-    s->seg_e = (s->tau < e1_tau || (grown && next_is_lifting)) ? 1 : 3;
+    const float left = 4.5f * 0.8f / 4096.f * rsqrtf((float)d);
+    const int first_full = left <= 0.25f * tol ? n_sched : n_sched - 1;
+    const bool may_accept = s->ns_idx >= first_full || s->ns_steps_used >= max_steps;
+    s->seg_e = (may_accept && s->tau >= e1_tau) ? 3 : 1;
   }
 }
 

@@ -235,6 +235,7 @@ struct TcGemmArgs {
                                 //    computed; tiles strictly above the diagonal also write their transpose
   float* outF; long long ldo;   // fp32 output (M read-modify-write, E, X_next, Y)
   __nv_bfloat16* outH; long long ldh; long long lo_elems;   // bf16 output hi part (+ lo part at +lo_elems)
+  uint16_t* out16;              // next iterate: its fp16 copy (times TC_F16_SCALE), operand of the one-pass Gram product
   const __nv_bfloat16* inH;                                 // bf16 pair epilogue input (the old iterate; same ld / lo_elems as outH)
   const float* rnorm;
   unsigned* rowmax; unsigned* rowmin;   // per-row ordered max / min of the raw products (quant modes)
@@ -317,6 +318,25 @@ __device__ __forceinline__ void bf16x2_split(float a, float b, uint32_t& wh, uin
   wl = bf16x2_pack(a - __uint_as_float(wh << 16), b - __uint_as_float(wh & 0xffff0000u));
 }
 
+// Two floats -> packed fp16 pair (first in the low half).
+__device__ __forceinline__ uint32_t f16x2_pack(float lo, float hi) {
+  uint32_t r;
+  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+  return r;
+}
+__device__ __forceinline__ float2 f16x2_unpack(uint32_t w) {
+  float2 r;
+  asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %2;\n\tcvt.f32.f16 %0, l;\n\tcvt.f32.f16 %1, h;\n\t}" : "=f"(r.x), "=f"(r.y) : "r"(w));
+  return r;
+}
+// Scale of the fp16 operands of the Newton-Schulz products (the iterate's copy X and the residual E = X^T X - tau I):
+// their entries are at most a little above 1 (singular values are); those below 2^-26 lose bits, and what they contribute
+// is far below the rounding of the larger ones.
+constexpr float TC_F16_SCALE = 4096.f;
+// Scale of the polynomial B where the last product runs on fp16 operands.  |B| <= a / s with the lifting quintic's a = 3.98
+// and the first step's rescaling s >= d^(-1/4): at most 54 for any d taken.
+constexpr float TC_B16_SCALE = 256.f;
+
 // Epilogue stores.  A thread holds 32 consecutive columns of ONE row (TMEM lane = row), so a direct 16-byte store
 // per thread touches 32 different lines per instruction and only half a sector of each.  The warp's 32 x 32 block
 // goes through a private, swizzled shared-memory buffer instead and leaves as full 128-byte (fp32) or 64-byte (bf16)
@@ -388,7 +408,8 @@ static __global__ void tc_wait_probe_kernel(DevState* st, long long limit_cycles
 
 template <int BN, bool A_MN, bool B_MN, int EPI, bool PAIR, int NA = 1, int NB = 1>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const TcGemmArgs g) {
+tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+               const __grid_constant__ CUtensorMap tmF, const TcGemmArgs g) {
   using Cfg = TcCfg<BN, PAIR, NA, NB>;
   constexpr int TM = Cfg::TILE_M;
   constexpr int R = BN / TM;                        // tiles per column step of a symmetric product
@@ -416,16 +437,30 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const int num_kb = (g.K + TC_BK - 1) / TC_BK;
   const int nseg = g.nseg_from_state ? max(1, min(g.nseg, g.nseg_from_state == 2 ? g.st->seg_e : g.st->seg_x)) : g.nseg;
   const int k_iters = PAIR ? num_kb : num_kb * nseg;     // a pair runs all passes of a k block from one stage
+  // fp16 operands: the residual squared, and the one-pass forms of the Gram and of the last product, which read the fp16
+  // copy of the iterate
+  const bool one16 = (EPI == TC_EPI_RESID || EPI == TC_EPI_NEXT) && nseg == 1;
+  const bool f16 = one16 || EPI == TC_EPI_POLY;
+  const CUtensorMap* const mapA = one16 ? &tmF : &tmA;
+  const CUtensorMap* const mapB = (one16 && EPI == TC_EPI_RESID) ? &tmF : &tmB;
+  // operand tiles the passes in use need; the shared memory holds as many stages of them as fit
+  int na = 1, nb = 1;
+  if (PAIR) {
+    for (int sg = 0; sg < nseg; ++sg) { na = max(na, g.a_tile[sg] + 1); nb = max(nb, g.b_tile[sg] + 1); }
+    na = min(na, NA); nb = min(nb, NB);
+  }
+  const int stage_bytes = PAIR ? na * Cfg::A_BYTES + nb * Cfg::B_BYTES : Cfg::STAGE_BYTES;
+  const int n_stages = PAIR ? min(8, Cfg::STAGES * Cfg::STAGE_BYTES / stage_bytes) : Cfg::STAGES;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < Cfg::STAGES; ++s) { ptx::mbar_init(&aux->full[s], 1); ptx::mbar_init(&aux->empty[s], 1); }
+    for (int s = 0; s < n_stages; ++s) { ptx::mbar_init(&aux->full[s], 1); ptx::mbar_init(&aux->empty[s], 1); }
     // the accumulator is handed back by every epilogue thread (of both CTAs of a pair)
     for (int b = 0; b < 2; ++b) { ptx::mbar_init(&aux->tfull[b], 1); ptx::mbar_init(&aux->tempty[b], PAIR ? 2 * TC_EPI_THREADS : TC_EPI_THREADS); }
     aux->abort_flag = 0;
     ptx::fence_barrier_init();
     ptx::fence_proxy_async();
-    ptx::prefetch_tmap(&tmA);
-    ptx::prefetch_tmap(&tmB);
+    ptx::prefetch_tmap(mapA);
+    ptx::prefetch_tmap(mapB);
   }
   if (warp == 1) {
     if (PAIR) { ptx::tmem_alloc_pair(&aux->tmem_base, Cfg::TMEM_COLS); ptx::tmem_relinquish_pair(); }
@@ -455,14 +490,11 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           const int seg = it / num_kb, k0 = (it - seg * num_kb) * TC_BK;
           const int a_off = g.a_off[seg], b_off = g.b_off[seg];
           if (!tc_wait(&aux->empty[stage], phase ^ 1u, abort_flag)) { ok = false; timeout_site = 1; break; }
-          uint8_t* sa = smem + stage * Cfg::STAGE_BYTES;
+          uint8_t* sa = smem + stage * stage_bytes;
           uint8_t* sb = sa + Cfg::A_BYTES;
           if (PAIR) {
             // both CTAs' copies are counted on the barrier of CTA 0, whose MMA thread consumes the stage
             const uint32_t bar = ptx::mapa_u32(ptx::smem_u32(&aux->full[stage]), 0);
-            int na = 1, nb = 1;                          // tiles the passes in use need
-            for (int sg = 0; sg < nseg; ++sg) { na = max(na, g.a_tile[sg] + 1); nb = max(nb, g.b_tile[sg] + 1); }
-            na = min(na, NA); nb = min(nb, NB);
             if (rank == 0) ptx::mbar_expect_tx(&aux->full[stage], 2 * (na * Cfg::A_BYTES + nb * b_rows * TC_BK * 2));
             const int kk = it * TC_BK;
 #pragma unroll
@@ -471,23 +503,23 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
               uint8_t* ta = sa + ia * Cfg::A_BYTES;
               if (A_MN) {
 #pragma unroll
-                for (int h = 0; h < TC_BM / 64; ++h) ptx::tma_load_2d_pair(ta + h * 8192, &tmA, bar, m0 + 64 * h, kk + g.a_toff[ia]);
+                for (int h = 0; h < TC_BM / 64; ++h) ptx::tma_load_2d_pair(ta + h * 8192, mapA, bar, m0 + 64 * h, kk + g.a_toff[ia]);
               } else {
-                ptx::tma_load_2d_pair(ta, &tmA, bar, kk, m0 + g.a_toff[ia]);
+                ptx::tma_load_2d_pair(ta, mapA, bar, kk, m0 + g.a_toff[ia]);
               }
             }
 #pragma unroll
             for (int ib = 0; ib < NB; ++ib) {
               if (ib >= nb) break;
-              uint8_t* tb = sa + NA * Cfg::A_BYTES + ib * Cfg::B_BYTES;
+              uint8_t* tb = sa + na * Cfg::A_BYTES + ib * Cfg::B_BYTES;
               if (B_MN) {
 #pragma unroll
                 for (int h = 0; h < Cfg::B_ROWS / 64; ++h) {
                   if (h * 64 >= b_rows) break;
-                  ptx::tma_load_2d_pair(tb + h * 8192, &tmB, bar, n0 + 64 * h, kk + g.b_toff[ib]);
+                  ptx::tma_load_2d_pair(tb + h * 8192, mapB, bar, n0 + 64 * h, kk + g.b_toff[ib]);
                 }
               } else {
-                ptx::tma_load_2d_pair(tb, &tmB, bar, kk, n0 + g.b_toff[ib]);
+                ptx::tma_load_2d_pair(tb, mapB, bar, kk, n0 + g.b_toff[ib]);
               }
             }
           } else {
@@ -495,20 +527,20 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             if (A_MN) {
 #pragma unroll
               for (int h = 0; h < TC_BM / 64; ++h)
-                ptx::tma_load_2d(sa + h * 8192, &tmA, &aux->full[stage], m0 + 64 * h, k0 + a_off);
+                ptx::tma_load_2d(sa + h * 8192, mapA, &aux->full[stage], m0 + 64 * h, k0 + a_off);
             } else {
-              ptx::tma_load_2d(sa, &tmA, &aux->full[stage], k0, m0 + a_off);
+              ptx::tma_load_2d(sa, mapA, &aux->full[stage], k0, m0 + a_off);
             }
             if (B_MN) {
 #pragma unroll
               for (int h = 0; h < BN / 64; ++h)
-                ptx::tma_load_2d(sb + h * 8192, &tmB, &aux->full[stage], n0 + 64 * h, k0 + b_off);
+                ptx::tma_load_2d(sb + h * 8192, mapB, &aux->full[stage], n0 + 64 * h, k0 + b_off);
             } else {
-              ptx::tma_load_2d(sb, &tmB, &aux->full[stage], k0, n0 + b_off);
+              ptx::tma_load_2d(sb, mapB, &aux->full[stage], k0, n0 + b_off);
             }
           }
           ++issued;
-          if (++stage == Cfg::STAGES) { stage = 0; phase ^= 1u; }
+          if (++stage == n_stages) { stage = 0; phase ^= 1u; }
         }
       }
       if (!ok) {
@@ -532,7 +564,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer (CTA 0 of a pair issues for both)
     if (lane == 0 && rank == 0) {
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((A_MN ? 1u : 0u) << 15) | ((B_MN ? 1u : 0u) << 16) |
+      const uint32_t types = f16 ? 0u : ((1u << 7) | (1u << 10));          // fp16 or bf16 operands
+      const uint32_t idesc = (1u << 4) | types | ((A_MN ? 1u : 0u) << 15) | ((B_MN ? 1u : 0u) << 16) |
                              ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
       int stage = 0;
       uint32_t phase = 0;
@@ -548,14 +581,14 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         for (int it = 0; it < k_iters; ++it) {
           if (!tc_wait(&aux->full[stage], phase, abort_flag)) { ok = false; timeout_site = 3; break; }
           ptx::tc_fence_after();
-          const uint32_t sa = ptx::smem_u32(smem + stage * Cfg::STAGE_BYTES);
+          const uint32_t sa = ptx::smem_u32(smem + stage * stage_bytes);
           // K-major: 16 k = 32 bytes inside the swizzled 128-byte row; 8-row groups 1024 bytes apart.
           // MN-major: 16 k = two 8-row groups of 1024 bytes; 64-wide m|n chunks 8192 bytes apart.
           // For a pair the descriptors name this CTA's tiles; the peer's halves sit at the same offsets in its memory.
           if (PAIR) {
             for (int sg = 0; sg < nseg; ++sg) {
               const uint32_t ta = sa + (uint32_t)(g.a_tile[sg] * Cfg::A_BYTES);
-              const uint32_t tb = sa + (uint32_t)(NA * Cfg::A_BYTES + g.b_tile[sg] * Cfg::B_BYTES);
+              const uint32_t tb = sa + (uint32_t)(na * Cfg::A_BYTES + g.b_tile[sg] * Cfg::B_BYTES);
 #pragma unroll
               for (int j = 0; j < TC_BK / 16; ++j) {
                 const uint64_t ad = A_MN ? tc_smem_desc(ta + j * 2048, 8192, 1024) : tc_smem_desc(ta + j * 32, 16, 1024);
@@ -574,7 +607,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           }
           // frees the shared-memory stage (in both CTAs of a pair) once these MMAs retire
           if (PAIR) ptx::umma_commit_pair(&aux->empty[stage]); else ptx::umma_commit(&aux->empty[stage]);
-          if (++stage == Cfg::STAGES) { stage = 0; phase ^= 1u; }
+          if (++stage == n_stages) { stage = 0; phase ^= 1u; }
         }
         if (ok) {                                         // accumulator complete
           if (PAIR) ptx::umma_commit_pair(&aux->tfull[buf]); else ptx::umma_commit(&aux->tfull[buf]);
@@ -592,6 +625,11 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     if (EPI == TC_EPI_POLY || EPI == TC_EPI_NEXT) {
       c_gamma = g.st->coef[0]; c_b1 = g.st->coef[1]; c_b2 = g.st->coef[2]; c_kappa = g.st->coef[3];
     }
+    if (EPI == TC_EPI_POLY) {                             // in units of the scaled fp16 operands
+      c_b2 *= 1.f / (TC_F16_SCALE * TC_F16_SCALE);
+      c_b1 *= 1.f / TC_F16_SCALE;
+    }
+    const bool b16 = EPI == TC_EPI_POLY && g.st->seg_x == 1;       // B goes into a product on fp16 operands
     if (EPI == TC_EPI_RESID) c_tau = g.st->tau;
     int local = 0;
     bool ok = true;
@@ -658,6 +696,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           if (EPI == TC_EPI_RESID) {
             // statistics of G - I and of tr G; the stored residual is E = G - tau I
             float sq32 = 0.f;                              // 32 terms in fp32, then one double add per chunk
+            if (one16) {
+#pragma unroll
+              for (int i = 0; i < 32; ++i) v[i] *= 1.f / (TC_F16_SCALE * TC_F16_SCALE);
+            }
 #pragma unroll
             for (int i = 0; i < 32; ++i) {
               float e1 = v[i];
@@ -668,8 +710,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             acc_sq += (double)sq32;
           } else {
             if (EPI == TC_EPI_POLY) {
-              // beta1 E from the bf16 copy of E this product streams as its operands: the difference to fp32 E is a
-              // symmetric relative perturbation of the size of B's own rounding to bf16
+              // beta1 E from the fp16 copy of E this product streams as its operands: the difference to fp32 E is a
+              // symmetric relative perturbation below the size of B's own rounding to bf16
               const uint4* se = reinterpret_cast<const uint4*>(g.inH + (long long)(row_ok ? row : wrow0) * g.ldh + col0);
 #pragma unroll
               for (int i = 0; i < 4; ++i) {
@@ -677,12 +719,17 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 const uint32_t ee[4] = {e4.x, e4.y, e4.z, e4.w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                  v[8 * i + 2 * e] = fmaf(c_b2, v[8 * i + 2 * e], c_b1 * __uint_as_float(ee[e] << 16));
-                  v[8 * i + 2 * e + 1] = fmaf(c_b2, v[8 * i + 2 * e + 1], c_b1 * __uint_as_float(ee[e] & 0xffff0000u));
+                  const float2 e2 = f16x2_unpack(ee[e]);
+                  v[8 * i + 2 * e] = fmaf(c_b2, v[8 * i + 2 * e], c_b1 * e2.x);
+                  v[8 * i + 2 * e + 1] = fmaf(c_b2, v[8 * i + 2 * e + 1], c_b1 * e2.y);
                 }
               }
             } else {
-              // the old iterate is its bf16 pair hi + lo (the same tiles this product streams as operand A)
+              // the old iterate is its bf16 pair hi + lo (the tiles that the two-pass product streams as operand A)
+              if (one16) {
+#pragma unroll
+                for (int i = 0; i < 32; ++i) v[i] *= 1.f / (TC_F16_SCALE * TC_B16_SCALE);
+              }
               const long long at = (long long)(row_ok ? row : wrow0) * g.ldh + col0;
               const uint4* sh = reinterpret_cast<const uint4*>(g.inH + at);
               const uint4* sl = reinterpret_cast<const uint4*>(g.inH + g.lo_elems + at);
@@ -714,11 +761,18 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             if (EPI == TC_EPI_NEXT) bf16x2_split(v[2 * i], v[2 * i + 1], wh[i], wl[i]);
+            else if (EPI == TC_EPI_RESID) wh[i] = f16x2_pack(v[2 * i] * TC_F16_SCALE, v[2 * i + 1] * TC_F16_SCALE);
+            else if (b16) wh[i] = f16x2_pack(v[2 * i] * TC_B16_SCALE, v[2 * i + 1] * TC_B16_SCALE);
             else wh[i] = bf16x2_pack(v[2 * i], v[2 * i + 1]);
           }
           tc_store_block_bf16(stg, lane, wh, g.outH + (long long)wrow0 * g.ldh + col0, g.ldh, rows_ok);
-          if (EPI == TC_EPI_NEXT)
+          if (EPI == TC_EPI_NEXT) {
             tc_store_block_bf16(stg, lane, wl, g.outH + g.lo_elems + (long long)wrow0 * g.ldh + col0, g.ldh, rows_ok);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) wh[i] = f16x2_pack(v[2 * i] * TC_F16_SCALE, v[2 * i + 1] * TC_F16_SCALE);
+            tc_store_block_bf16(stg, lane, wh, reinterpret_cast<__nv_bfloat16*>(g.out16) + (long long)wrow0 * g.ldh + col0, g.ldh,
+                                rows_ok);
+          }
           if (EPI != TC_EPI_NEXT && mirror && row_ok) {
             // transpose of the tile: lane t holds row (m0 + 32 q + t), so for a fixed column the 32 lanes write
             // 32 consecutive elements of one output row
@@ -953,8 +1007,7 @@ struct TcHost {
   int d, P, quant_bits, num_sms;
   int device;                                // CUDA device the context was created on
   int pair_clusters;                         // CTA pairs that can be co-resident (0: single-CTA kernels only)
-  float e1_tau;                              // residual product runs one pass while mean sigma^2 of the iterate is below this
-  float lo_budget;                           // ... and in mid-iteration, see ns_tau_kernel
+  float e1_tau;                              // residual product runs one pass while mean sigma^2 of the iterate is below this, see ns_tau_kernel
   int64_t n_max;
   char* ws;
   TcLayout L;
@@ -970,6 +1023,8 @@ struct TcHost {
   CUtensorMap tmRb_mn;                       // R bf16 as MN-major B of the rotate product
   CUtensorMap tmM_blk, tmMpart_blk;          // per-head case: fp32 M of all problems / the partials, 32 x 32 boxes
   CUtensorMap tmXh_mn[2], tmXh_k[2];         // iterate, stacked [hi; lo]
+  CUtensorMap tmX16_mn[2], tmX16_k[2];       // ... its fp16 copy
+  const CUtensorMap* f16_map;                // the one that the next launch's one-pass form reads
   CUtensorMap tmEh_k, tmEh_mn, tmBh_mn;
   Prof* prof;
   int ns_k;                                  // Newton-Schulz step index of the launches being enqueued (-1 outside)
@@ -1109,6 +1164,7 @@ inline void tc_fuse_passes(TcGemmArgs* g) {
 
 template <int BN, bool A_MN, bool B_MN, int EPI, bool PAIR, int NA = 1, int NB = 1>
 inline int tc_launch(TcHost& h, cudaStream_t s, const CUtensorMap& a, const CUtensorMap& b, const TcGemmArgs& g) {
+  const CUtensorMap& f = (EPI == TC_EPI_RESID || EPI == TC_EPI_NEXT) ? *h.f16_map : a;
   using Cfg = TcCfg<BN, PAIR, NA, NB>;
   auto kern = tc_gemm_kernel<BN, A_MN, B_MN, EPI, PAIR, NA, NB>;
   // the attribute is per device; setting it twice from two threads is harmless, so an atomic mask is enough
@@ -1144,9 +1200,9 @@ inline int tc_launch(TcHost& h, cudaStream_t s, const CUtensorMap& a, const CUte
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.attrs = at; cfg.numAttrs = 1;
-    err = cudaLaunchKernelEx(&cfg, kern, a, b, gl);
+    err = cudaLaunchKernelEx(&cfg, kern, a, b, f, gl);
   } else {
-    kern<<<grid, TC_THREADS, Cfg::SMEM_BYTES, s>>>(a, b, gl);
+    kern<<<grid, TC_THREADS, Cfg::SMEM_BYTES, s>>>(a, b, f, gl);
     err = cudaGetLastError();
   }
   if (timed) { cudaEventRecord(rec.e1, s); h.prof->open.push_back(rec); }
@@ -1209,7 +1265,7 @@ inline int tc_device_facts(int dev, TcDevFacts* out) {
 inline int tc_init(TcHost* h, char* ws, const TcLayout& L, int d, int P, int64_t n_max, int quant_bits, float* R,
                    float* M, float* Xa, float* Xb, float* E, float* B, float* rnorm, DevState* st, double* part_d,
                    float* part_f, float* Y, unsigned* rowmax, QuantSpec qs, int diagnostics, double* part_diag, Prof* prof,
-                   int single_cta, float gram_single_pass_tau, float lo_budget) {
+                   int single_cta, float gram_single_pass_tau) {
   h->d = d; h->P = P; h->n_max = n_max; h->quant_bits = quant_bits; h->ws = ws; h->L = L;
   h->R = R; h->M = M; h->Xa = Xa; h->Xb = Xb; h->E = E; h->B = B; h->rnorm = rnorm; h->st = st;
   h->part_d = part_d; h->part_f = part_f; h->Y = Y; h->rowmax = rowmax; h->qs = qs; h->diagnostics = diagnostics; h->part_diag = part_diag; h->prof = prof; h->ns_k = -1;
@@ -1225,7 +1281,6 @@ inline int tc_init(TcHost* h, char* ws, const TcLayout& L, int d, int P, int64_t
   h->device = dev;
   h->pair_clusters = single_cta ? 0 : f.pair_clusters;
   h->e1_tau = gram_single_pass_tau > 0.f ? gram_single_pass_tau : 2e-3f;
-  h->lo_budget = lo_budget;
   const uint64_t D = (uint64_t)d;
   int rc = 0;
   if (P > 1) {
@@ -1241,6 +1296,10 @@ inline int tc_init(TcHost* h, char* ws, const TcLayout& L, int d, int P, int64_t
   for (int i = 0; i < 2; ++i) {
     rc |= tc_make_tmap(&h->tmXh_mn[i], ws + L.Xh[i], 2 * D, D, D, 64);
     rc |= tc_make_tmap(&h->tmXh_k[i], ws + L.Xh[i], 2 * D, D, D, 128);
+  }
+  for (int i = 0; i < 2; ++i) {                             // (the fp32 iterate's regions: this mode has no fp32 iterate)
+    rc |= tc_make_tmap(&h->tmX16_mn[i], i ? Xb : Xa, D, D, D, 64);
+    rc |= tc_make_tmap(&h->tmX16_k[i], i ? Xb : Xa, D, D, D, 128);
   }
   rc |= tc_make_tmap(&h->tmEh_k, ws + L.Eh, D, D, D, 128);
   rc |= tc_make_tmap(&h->tmEh_mn, ws + L.Eh, D, D, D, 64);
@@ -1324,22 +1383,29 @@ inline int tc_process(TcHost& h, cudaStream_t s, int64_t n) {
   return tc_launch_n<true, true, TC_EPI_ACCUM>(h, s, tmXs_mn, tmCp_mn, a);
 }
 
-// X0 = (M_raw + lam R) * x0_scale, written straight as the stacked bf16 split [hi; lo] (no fp32 copy of X0)
+// X0 = (M_raw + lam R) * x0_scale, written straight as the stacked bf16 split [hi; lo] and the scaled fp16 copy
+// (no fp32 copy of X0)
 static __global__ void tc_x0_split_kernel(const float* __restrict__ M, const float* __restrict__ R,
-                                          __nv_bfloat16* __restrict__ dst, int64_t dd, const DevState* st) {
+                                          __nv_bfloat16* __restrict__ dst, uint16_t* __restrict__ x16, int64_t dd,
+                                          const DevState* st) {
   const float lam = st->lam, sc = st->x0_scale;
   for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; i < dd; i += (int64_t)gridDim.x * blockDim.x * 4) {
     const float4 m = *reinterpret_cast<const float4*>(M + i), r = *reinterpret_cast<const float4*>(R + i);
     uint2 o, l;
-    bf16x2_split(fmaf(lam, r.x, m.x) * sc, fmaf(lam, r.y, m.y) * sc, o.x, l.x);
-    bf16x2_split(fmaf(lam, r.z, m.z) * sc, fmaf(lam, r.w, m.w) * sc, o.y, l.y);
+    const float a0 = fmaf(lam, r.x, m.x) * sc, a1 = fmaf(lam, r.y, m.y) * sc, a2 = fmaf(lam, r.z, m.z) * sc,
+                a3 = fmaf(lam, r.w, m.w) * sc;
+    bf16x2_split(a0, a1, o.x, l.x);
+    bf16x2_split(a2, a3, o.y, l.y);
+    *reinterpret_cast<uint2*>(x16 + i) = make_uint2(f16x2_pack(a0 * TC_F16_SCALE, a1 * TC_F16_SCALE),
+                                                    f16x2_pack(a2 * TC_F16_SCALE, a3 * TC_F16_SCALE));
     *reinterpret_cast<uint2*>(dst + i) = o;
     *reinterpret_cast<uint2*>(dst + dd + i) = l;
   }
 }
 inline int tc_ns_begin(TcHost& h, cudaStream_t s) {
   const int64_t dd = (int64_t)h.d * h.d;
-  tc_x0_split_kernel<<<tc_ew_blocks(dd / 4), 256, 0, s>>>(h.M, h.R, reinterpret_cast<__nv_bfloat16*>(h.ws + h.L.Xh[0]), dd, h.st);
+  tc_x0_split_kernel<<<tc_ew_blocks(dd / 4), 256, 0, s>>>(h.M, h.R, reinterpret_cast<__nv_bfloat16*>(h.ws + h.L.Xh[0]),
+                                                             reinterpret_cast<uint16_t*>(h.Xa), dd, h.st);
   if (h.prof) h.prof->count(K_OTHER);
   return cudaGetLastError() == cudaSuccess ? CONQUR_OK : CONQUR_ERR_CUDA;
 }
@@ -1349,20 +1415,25 @@ inline int tc_ns_begin(TcHost& h, cudaStream_t s) {
 inline int tc_ns_parts(const TcHost& h) { return tc_part_slots(h, tc_variant(h, h.d), h.d, h.d, 1); }
 inline int tc_ns_next_parts(const TcHost& h) { return tc_part_slots(h, tc_variant(h, h.d), h.d, h.d, 0); }
 
-// G = X^T X from the split iterate in Xh[buf] (three passes: hi hi, hi lo, lo hi; symmetric tiles only);
-// stores E = G - tau I as fp32 and bf16, and the statistics of G - I.
+// G = X^T X (symmetric tiles only), stored as E = G - tau I in (scaled) fp16, and the statistics of G - I.  Between the
+// steps G only has to be about as good as its rounding (2^-12): one pass over the iterate's fp16 copy does.  The check
+// that may accept the rotation takes three passes over the bf16 pair in Xh[buf]: hi hi, hi lo, lo hi.
+// (d = 4096: 60 us against 150; with a one-pass product of the bf16 hi part instead, early steps lost the directions
+// below 1e-4 of the largest and endgame steps had to be repeated.)
 inline int tc_ns_residual(TcHost& h, cudaStream_t s, int buf) {
   const int d = h.d;
   TcGemmArgs g = tc_args(h, d, d, d);
   g.nseg = 3; g.nseg_from_state = 2; g.a_off[2] = d; g.b_off[1] = d; g.check_done = 1; g.sym = 1;
   g.outH = reinterpret_cast<__nv_bfloat16*>(h.ws + h.L.Eh); g.ldh = d;
   g.part_t = h.part_d + tc_ns_parts(h);
+  h.f16_map = &h.tmX16_mn[buf];
   return tc_launch_n<true, true, TC_EPI_RESID>(h, s, h.tmXh_mn[buf], h.tmXh_mn[buf], g);
 }
 
-// B = beta2 E E + beta1 E - kappa I (one bf16 pass, symmetric tiles only) ;  X_next = X B + (gamma + kappa) X
-// (the iterate enters as hi, or hi + lo while small singular values are still being lifted).
-inline int tc_ns_poly_next(TcHost& h, cudaStream_t s, int cur) {
+// B = beta2 E E + beta1 E - kappa I (one fp16 pass, symmetric tiles only) ;  X_next = X B + (gamma + kappa) X.  The iterate
+// enters the last product as the bf16 pair hi + lo while small singular values are still being lifted (B is then stored in
+// bf16, as an instruction's operands have one type), after that as its fp16 copy in one pass (B in scaled fp16).
+inline int tc_ns_poly_next(TcHost& h, cudaStream_t s, int cur, int n_sched, int max_steps, float tol) {
   const int d = h.d;
   const long long dd = (long long)d * d;
   TcGemmArgs g = tc_args(h, d, d, d);
@@ -1375,10 +1446,12 @@ inline int tc_ns_poly_next(TcHost& h, cudaStream_t s, int cur) {
   x.nseg = 2; x.nseg_from_state = 1; x.a_off[1] = d; x.check_done = 1;
   x.inH = reinterpret_cast<const __nv_bfloat16*>(h.ws + h.L.Xh[cur]);
   x.outH = reinterpret_cast<__nv_bfloat16*>(h.ws + h.L.Xh[1 - cur]); x.ldh = d; x.lo_elems = dd;
+  x.out16 = reinterpret_cast<uint16_t*>(cur ? h.Xa : h.Xb);
+  h.f16_map = &h.tmX16_k[cur];
   x.part_t = h.part_d + tc_ns_parts(h);
   rc = tc_launch_n<false, true, TC_EPI_NEXT>(h, s, h.tmXh_k[cur], h.tmBh_mn, x);
   if (rc) return rc;
-  ns_tau_kernel<<<1, 256, 0, s>>>(h.st, h.part_d + tc_ns_parts(h), tc_ns_next_parts(h), d, h.e1_tau, h.lo_budget);
+  ns_tau_kernel<<<1, 256, 0, s>>>(h.st, h.part_d + tc_ns_parts(h), tc_ns_next_parts(h), d, h.e1_tau, n_sched, max_steps, tol);
   if (h.prof) h.prof->count(K_OTHER);
   return cudaGetLastError() == cudaSuccess ? CONQUR_OK : CONQUR_ERR_CUDA;
 }
