@@ -170,7 +170,7 @@ int conqur_step(conqur_ctx* ctx, const void* X_dev, int64_t n, int64_t ld);
  * cfg.batch reads its n rows at X_dev + p*problem_stride + i*ld (elements), each
  * row normalised by its own d-slice norm.  problem_stride = d, ld = P*d is the
  * head-interleaved layout; problem_stride = n*ld is stacked problems.
- * In tensor-core mode (d = 128) the fused kernel takes a row's norm from the rotated row, ||x R~|| with R~ the bf16
+ * In tensor-core mode with fake-quantisation the fused kernel takes a row's norm from the rotated row, ||x R~|| with R~ the bf16
  * copy of R its product uses: equal to ||x|| for an orthogonal R, here within ||R~ R~^T - I||_2 / 2 of it (about
  * 1e-4 relative; the scale then enters the target tile rounded to bf16, 2^-9).  A uniform factor on the rows' scales
  * does not change the rotation an update returns.

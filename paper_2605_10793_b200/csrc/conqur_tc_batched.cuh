@@ -77,9 +77,12 @@ struct TcbStepArgs {
   int8_t* signs;              // test hook: when set, the sign decisions (-1/0/+1) of this call, (P * n) x 128 row-major
 };
 
+// A box of the input, which is read once: first in line to leave the L2, where M and R are worth more (1.4 % of the step
+// at 1024 x 4096 rows).
 __device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* tmap, uint64_t* bar, int x, int y, int z) {
   asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+      "{\n\t.reg .b64 pol;\n\tcreatepolicy.fractional.L2::evict_first.b64 pol, 1.0;\n\t"
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %5}], [%2], pol;\n\t}"
       ::"r"(ptx::smem_u32(smem_dst)), "l"(tmap), "r"(ptx::smem_u32(bar)), "r"(x), "r"(y), "r"(z)
       : "memory");
 }
@@ -281,7 +284,7 @@ tcb_step_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     const int ew = (warp - 2) & 7;                 // 0..7 inside the group
     const int half = ew >> 2;                      // which 64 of the 128 columns this warp handles
     const int r = q * 32 + lane;                   // token inside the tile; later: row of M
-    int it = 0, lp = 0;
+    int it = 0, lp = 0, wo_grp = 0;
     uint32_t wo_count = 0;                         // write-outs this warp's group has done
     bool ok = true;
     for (int item = blockIdx.x; item < g.P * g.S && ok; item += gridDim.x, ++lp) {
@@ -427,7 +430,9 @@ tcb_step_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       // groups, the one that owned the problem's last tile writes all of it out (each warp 32 rows x 64 columns) while
       // the other goes straight on to the next problem's first tile, so the second products resume as soon as the
       // accumulator has been read.
-      const int wo_grp = (TCB_EPI_GROUPS == 2) ? ((it - 1) & 1) : 0;
+      // (the same group for all items of this CTA, so that its waits on the accumulator see every phase, however short
+      // the items are: the one that owned the first item's last tile)
+      if (lp == 0) wo_grp = (TCB_EPI_GROUPS == 2) ? ((it - 1) & 1) : 0;
       if (grp == wo_grp) {
         const int mb = lp % TCB_MBUF;
         if (ew == 0) TCB_TR(it - 1, TCB_EV_OUT_WAIT);
@@ -455,6 +460,376 @@ tcb_step_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         const double wsum = warp_sum_d(acc);
         if (lane == 0) g.part_d[(long long)item * TCB_PARTS + grp * 8 + ew] = wsum;
       }
+    }
+  }
+
+  if (timeout_site != 0) {
+    atomicOr(&g.st[0].status_flags, STATUS_FLAG_TIMEOUT);
+    g.st[0].timeout_site = timeout_site;
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc(tmem_base, 512);
+  }
+}
+
+// ------------------------------------------------------------------ the step without fake-quantisation
+// The same fused step, transposed, for the plain corner target (Eq. 2), whose decisions need nothing of the rest of the
+// row but its norm.  Two tiles (256 tokens) at a time:
+//   tcgen05.mma    Y^T = R^T X^T              (N = 256 tokens)    -> TMEM (lane = rotated coordinate, column = token)
+//   epilogue       C'^T = sgn(Y^T) * rnorm(token), packed bf16    -> TMEM (a group of eight warps per tile)
+//   tcgen05.mma    M^T += C'^T X      (A operand from TMEM)       -> TMEM accumulator of the problem
+// so the targets never pass through shared memory, whose bandwidth bounds tcb_step_kernel: per tile 192 KB (TMA 32, first
+// product 64, targets 32, second product 64 KB: 1500 cycles at 128 B/clk), here 144 KB (TMA 32, first product 32 and half
+// of R's 32, second product 32, row norms 32).  The row norms come from the input tile (four warps): the rotated tile has
+// a token's coordinates in 128 different lanes.
+// TMEM: Y^T 256 columns, C'^T 2 x 64, M^T 128: all 512.
+// What bounds it: power.  Streaming the input and the two products draw the board's 1000 W limit between them (a plain copy
+// of the same bytes does, too), so the SM clock settles at 1.38-1.5 GHz and fewer bytes moved inside the SM count, not
+// fewer cycles: 1024 problems x 4096 rows in 341 us sustained, 282-330 us in bursts of 20-150 ms; tcb_step_kernel 371 and
+// 312-366 us, single tiles with a second R and five stages 345 and 293-335 us.
+// With fake-quantisation the row's range is needed as well, and tcb_step_kernel, where a thread owns a token, stays.
+constexpr int TCBT_STAGES = 3;                                  // input stages of two tiles
+constexpr int TCBT_STAGE_BYTES = 2 * TCB_TILE_BYTES;            // two 64-column chunks of 256 rows x 128 bytes
+constexpr int TCBT_CHUNK_BYTES = TCB_TILE_BYTES;
+constexpr int TCBT_NORM_WARP0 = 3, TCBT_EPI_WARP0 = 7;
+constexpr int TCBT_THREADS = (TCBT_EPI_WARP0 + 16) * 32;       // TMA, first product, second product, 4 norm, 2 x 8 epilogue warps
+constexpr uint32_t TCBT_C_COL = 256, TCBT_M_COL = 384;         // Y^T from column 0
+
+struct TcbtAux {
+  uint64_t rfull, rempty, mfull, mempty, yfull, yempty;
+  uint64_t xfull[TCBT_STAGES], xempty[TCBT_STAGES], nready[TCBT_STAGES];
+  uint64_t cready[2], cfree[2];
+  uint32_t tmem_base;
+  int abort_flag;
+  __align__(16) uint16_t rn[TCBT_STAGES][256];                 // bf16 row scales of the tokens in each stage
+};
+static_assert(sizeof(TcbtAux) <= TCB_AUX_BYTES, "the barrier / exchange block must fit its reserved shared memory");
+constexpr int TCBT_SMEM_BYTES = TCB_TILE_BYTES + TCBT_STAGES * TCBT_STAGE_BYTES + TCB_AUX_BYTES + 1024;
+static_assert(TCBT_SMEM_BYTES <= 232448, "227 KB of dynamic shared memory per CTA");
+
+namespace ptx {
+// D(tmem) (+)= A(tmem: lane = row, two consecutive 16-bit k per column) * B(smem desc)
+__device__ __forceinline__ void umma_bf16_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      ::"r"(tmem_d), "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// 32 lanes x 16 consecutive columns: thread t of the warp writes row (lane base + t); complete after tmem_st_wait.
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&w)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+      ::"r"(taddr), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]), "r"(w[8]),
+        "r"(w[9]), "r"(w[10]), "r"(w[11]), "r"(w[12]), "r"(w[13]), "r"(w[14]), "r"(w[15])
+      : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+}  // namespace ptx
+
+// A wait of a whole warp: every lane waits (bounded), and all of them agree on the outcome.
+__device__ __forceinline__ bool tc_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  return __all_sync(0xffffffffu, tc_wait(bar, parity, abort_flag) ? 1 : 0) != 0;
+}
+// Byte offset of the 16-byte piece `c16` (0..15) of row `r` (0..255) inside a stage.
+__device__ __forceinline__ uint32_t tcbt_piece(int r, int c16) {
+  return (uint32_t)((c16 >> 3) * TCBT_CHUNK_BYTES + r * 128 + (((c16 & 7) ^ (r & 7)) << 4));
+}
+
+__global__ void __launch_bounds__(TCBT_THREADS, 1)
+tcb_step_plain_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmR, const TcbStepArgs g) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* sR = smem;
+  uint8_t* sX = smem + TCB_TILE_BYTES;
+  TcbtAux* aux = reinterpret_cast<TcbtAux*>(sX + TCBT_STAGES * TCBT_STAGE_BYTES);
+  volatile int* abort_flag = &aux->abort_flag;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int T = (g.n + 255) / 256;                 // double tiles per problem
+
+  if (threadIdx.x == 0) {
+    ptx::mbar_init(&aux->rfull, 1); ptx::mbar_init(&aux->rempty, 1);
+    ptx::mbar_init(&aux->mfull, 1); ptx::mbar_init(&aux->mempty, 2 * TCB_EPI_WARPS);
+    ptx::mbar_init(&aux->yfull, 1); ptx::mbar_init(&aux->yempty, 2 * TCB_EPI_WARPS);
+    for (int s = 0; s < TCBT_STAGES; ++s) {
+      ptx::mbar_init(&aux->xfull[s], 1); ptx::mbar_init(&aux->xempty[s], 1); ptx::mbar_init(&aux->nready[s], 4);
+    }
+    for (int b = 0; b < 2; ++b) { ptx::mbar_init(&aux->cready[b], TCB_EPI_WARPS); ptx::mbar_init(&aux->cfree[b], 1); }
+    aux->abort_flag = 0;
+    ptx::fence_barrier_init();
+    ptx::fence_proxy_async();
+    ptx::prefetch_tmap(&tmX);
+    ptx::prefetch_tmap(&tmR);
+  }
+  if (warp == 1) { ptx::tmem_alloc(&aux->tmem_base, 512); ptx::tmem_relinquish(); }
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem_base = aux->tmem_base;
+  const uint32_t sR_a = ptx::smem_u32(sR), sX_a = ptx::smem_u32(sX);
+  const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 4) << 24);    // bf16, fp32 accumulation, M = 128
+  int timeout_site = 0;
+  const bool tracing = g.trace != nullptr && blockIdx.x == 0 && lane == 0;
+
+  // Every role walks the same sequence of work items (problem, range of double tiles); `it` counts the double tiles of
+  // this CTA, `lp` its items.
+  if (warp == 0) {
+    if (lane == 0) {
+      int xs = 0; uint32_t xph = 0;
+      int it = 0, lp = 0;
+      bool ok = true;
+      for (int item = blockIdx.x; item < g.P * g.S && ok; item += gridDim.x, ++lp) {
+        int p, t_begin, t_end;
+        tcb_item(item, T, g.S, p, t_begin, t_end);
+        for (int t = t_begin; t < t_end; ++t, ++it) {
+          if (!tc_wait(&aux->xempty[xs], xph ^ 1u, abort_flag)) { ok = false; timeout_site = 12; break; }
+          uint8_t* dst = sX + xs * TCBT_STAGE_BYTES;
+          ptx::mbar_expect_tx(&aux->xfull[xs], TCBT_STAGE_BYTES);
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {            // boxes of 128 tokens x 64 features
+            const int tok = t * 256 + h * 128;
+            const int c1 = g.xp_outer_tokens ? p : tok, c2 = g.xp_outer_tokens ? tok : p;
+            tma_load_3d(dst + h * 16384, &tmX, &aux->xfull[xs], 0, c1, c2);
+            tma_load_3d(dst + TCBT_CHUNK_BYTES + h * 16384, &tmX, &aux->xfull[xs], 64, c1, c2);
+          }
+          TCB_TR(2 * it, TCB_EV_TMA); TCB_TR(2 * it + 1, TCB_EV_TMA);
+          if (++xs == TCBT_STAGES) { xs = 0; xph ^= 1u; }
+        }
+      }
+      if (!ok) {                                   // let the copies in flight land before the CTA exits
+        const long long t0 = clock64();
+        while (clock64() - t0 < 4000000ll) {}
+      }
+    }
+  } else if (warp == 1) {
+    // ---------------------------------------------------------------- first product: Y^T = R^T X^T
+    if (lane == 0) {
+      const uint32_t idesc1 = idesc0 | (1u << 15) | ((uint32_t)(256 >> 3) << 17);    // A (R, read transposed) MN-major, B (X) K-major
+      int xs = 0; uint32_t xph = 0;
+      int it = 0, lp = 0;
+      bool ok = true;
+      for (int item = blockIdx.x; item < g.P * g.S && ok; item += gridDim.x, ++lp) {
+        int p, t_begin, t_end;
+        tcb_item(item, T, g.S, p, t_begin, t_end);
+        // the rotation: this thread's own products are the only readers of its buffer
+        if (!tc_wait(&aux->rempty, ((uint32_t)lp & 1u) ^ 1u, abort_flag)) { ok = false; timeout_site = 11; break; }
+        ptx::mbar_expect_tx(&aux->rfull, TCB_TILE_BYTES);
+        ptx::tma_load_2d(sR, &tmR, &aux->rfull, 0, (g.p0 + p) * TCB_D);
+        ptx::tma_load_2d(sR + 16384, &tmR, &aux->rfull, 64, (g.p0 + p) * TCB_D);
+        if (!tc_wait(&aux->rfull, (uint32_t)lp & 1u, abort_flag)) { ok = false; timeout_site = 20; break; }
+        for (int t = t_begin; t < t_end && ok; ++t, ++it) {
+          if (!tc_wait(&aux->xfull[xs], xph, abort_flag)) { ok = false; timeout_site = 22; break; }
+          if (!tc_wait(&aux->yempty, ((uint32_t)it & 1u) ^ 1u, abort_flag)) { ok = false; timeout_site = 24; break; }
+          ptx::tc_fence_after();
+          TCB_TR(2 * it, TCB_EV_MMA1); TCB_TR(2 * it + 1, TCB_EV_MMA1);
+          const uint32_t xa = sX_a + xs * TCBT_STAGE_BYTES;
+#pragma unroll
+          for (int j = 0; j < 8; ++j)              // 16 features per instruction
+            ptx::umma_bf16(tmem_base, tc_smem_desc(sR_a + j * 2048, 16384, 1024),
+                           tc_smem_desc(xa + (j >> 2) * TCBT_CHUNK_BYTES + (j & 3) * 32, 16, 1024), idesc1, j > 0 ? 1u : 0u);
+          ptx::umma_commit(&aux->yfull);
+          if (t == t_end - 1) ptx::umma_commit(&aux->rempty);
+          if (++xs == TCBT_STAGES) { xs = 0; xph ^= 1u; }
+        }
+      }
+      if (!ok) {
+        const long long t0 = clock64();
+        while (clock64() - t0 < 4000000ll) {}
+      }
+    }
+  } else if (warp == 2) {
+    // ---------------------------------------------------------------- second product: M^T += C'^T X
+    if (lane == 0) {
+      const uint32_t idesc2 = idesc0 | (1u << 16) | ((uint32_t)(128 >> 3) << 17);    // A from TMEM, B (X, contraction over the tokens) MN-major
+      int xs = 0; uint32_t xph = 0;
+      int it = 0, lp = 0;
+      bool ok = true;
+      for (int item = blockIdx.x; item < g.P * g.S && ok; item += gridDim.x, ++lp) {
+        int p, t_begin, t_end;
+        tcb_item(item, T, g.S, p, t_begin, t_end);
+        if (!tc_wait(&aux->mempty, ((uint32_t)lp & 1u) ^ 1u, abort_flag)) { ok = false; timeout_site = 21; break; }
+        for (int t = t_begin; t < t_end && ok; ++t, ++it) {
+          if (!tc_wait(&aux->xfull[xs], xph, abort_flag)) { ok = false; timeout_site = 25; break; }
+          const uint32_t xa = sX_a + xs * TCBT_STAGE_BYTES;
+          for (int h = 0; h < 2; ++h) {
+            if (!tc_wait(&aux->cready[h], (uint32_t)it & 1u, abort_flag)) { ok = false; timeout_site = 23; break; }
+            ptx::tc_fence_after();
+            TCB_TR(2 * it + h, TCB_EV_MMA2);
+#pragma unroll
+            for (int j = 0; j < 8; ++j)            // 16 tokens per instruction, 8 columns of C'^T
+              ptx::umma_bf16_ta(tmem_base + TCBT_M_COL, tmem_base + TCBT_C_COL + h * 64 + j * 8,
+                                tc_smem_desc(xa + h * 16384 + j * 2048, TCBT_CHUNK_BYTES, 1024), idesc2,
+                                (t > t_begin || h > 0 || j > 0) ? 1u : 0u);
+            ptx::umma_commit(&aux->cfree[h]);
+          }
+          if (!ok) break;
+          ptx::umma_commit(&aux->xempty[xs]);
+          if (++xs == TCBT_STAGES) { xs = 0; xph ^= 1u; }
+        }
+        if (ok) ptx::umma_commit(&aux->mfull);
+      }
+    }
+  } else if (warp < TCBT_EPI_WARP0) {
+    // ---------------------------------------------------------------- row norms: two tokens per thread
+    const int r0 = (warp - TCBT_NORM_WARP0) * 32 + lane;
+    int xs = 0; uint32_t xph = 0;
+    int it = 0;
+    bool ok = true;
+    for (int item = blockIdx.x; item < g.P * g.S && ok; item += gridDim.x) {
+      int p, t_begin, t_end;
+      tcb_item(item, T, g.S, p, t_begin, t_end);
+      int skipped = 0, nonfinite = 0;
+      for (int t = t_begin; t < t_end; ++t, ++it) {
+        if (!tc_wait_warp(&aux->xfull[xs], xph, abort_flag)) { ok = false; timeout_site = 34; break; }
+        uint8_t* xt = sX + xs * TCBT_STAGE_BYTES;
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+          const int r = h * 128 + r0;
+          if (warp == TCBT_NORM_WARP0) TCB_TR(2 * it + h, TCB_EV_NORM_BEGIN);
+          float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;        // four chains, added in a fixed order
+#pragma unroll 8
+          for (int c = 0; c < 16; ++c) {
+            const uint4 u = *reinterpret_cast<const uint4*>(xt + tcbt_piece(r, c));
+            const float a0 = __uint_as_float(u.x << 16), b0 = __uint_as_float(u.x & 0xffff0000u);
+            const float a1 = __uint_as_float(u.y << 16), b1 = __uint_as_float(u.y & 0xffff0000u);
+            const float a2 = __uint_as_float(u.z << 16), b2 = __uint_as_float(u.z & 0xffff0000u);
+            const float a3 = __uint_as_float(u.w << 16), b3 = __uint_as_float(u.w & 0xffff0000u);
+            s0 = fmaf(a0, a0, s0); s1 = fmaf(a1, a1, s1); s2 = fmaf(a2, a2, s2); s3 = fmaf(a3, a3, s3);
+            s0 = fmaf(b0, b0, s0); s1 = fmaf(b1, b1, s1); s2 = fmaf(b2, b2, s2); s3 = fmaf(b3, b3, s3);
+          }
+          const float ss = (s0 + s1) + (s2 + s3);
+          const bool valid = (t * 256 + r) < g.n;              // rows past the end were filled with zeros by the copy
+          const bool good = (ss > 0.f) && (ss <= 3.0e38f);
+          if (!good) {
+            if (valid) { ++skipped; if (!(ss == 0.f)) nonfinite = 1; }
+            // a row that takes no part must not reach M: its target is +-0, its input (which may hold NaN) becomes zero
+            if (!(ss == 0.f)) {
+#pragma unroll
+              for (int c = 0; c < 16; ++c) *reinterpret_cast<uint4*>(xt + tcbt_piece(r, c)) = make_uint4(0, 0, 0, 0);
+              ptx::fence_proxy_async();                        // seen by the second product (the first one's column is masked)
+            }
+          }
+          aux->rn[xs][r] = good ? (uint16_t)bf16_bits(1.0f / sqrtf(ss)) : (uint16_t)0;
+          if (warp == TCBT_NORM_WARP0) TCB_TR(2 * it + h, TCB_EV_NORM_END);
+        }
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(&aux->nready[xs]);
+        if (++xs == TCBT_STAGES) { xs = 0; xph ^= 1u; }
+      }
+      if (!ok) break;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        skipped += __shfl_xor_sync(0xffffffffu, skipped, o);
+        nonfinite |= __shfl_xor_sync(0xffffffffu, nonfinite, o);
+      }
+      if (lane == 0) {
+        if (skipped) atomicAdd(reinterpret_cast<unsigned long long*>(&g.st[p].step_skipped), (unsigned long long)skipped);
+        if (nonfinite) atomicOr(&g.st[p].status_flags, STATUS_FLAG_NONFINITE);
+      }
+    }
+  } else {
+    // ---------------------------------------------------------------- epilogue: a group of eight warps per tile of the pair
+    const int ew = (warp - TCBT_EPI_WARP0) & 7, grp = (warp - TCBT_EPI_WARP0) >> 3;
+    const int q = warp & 3;                        // TMEM lane quarter this warp may read
+    const int half = ew >> 2;                      // which 64 of the tile's 128 tokens
+    const int j = q * 32 + lane;                   // rotated coordinate
+    const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
+    const uint32_t y_addr = lane_addr + (uint32_t)(grp * 128 + half * 64);
+    const uint32_t c_addr = lane_addr + TCBT_C_COL + (uint32_t)(grp * 64 + half * 32);
+    const uint32_t m_col = (uint32_t)((grp * 2 + half) * 32);        // write-out: this warp's 32 rows of M
+    const bool tr_epi = ew == 0;                   // the first warp of a tile's group stamps its epilogue
+    int it = 0, lp = 0, xs = 0;
+    uint32_t xph = 0;
+    bool ok = true;
+    for (int item = blockIdx.x; item < g.P * g.S && ok; item += gridDim.x, ++lp) {
+      int p, t_begin, t_end;
+      tcb_item(item, T, g.S, p, t_begin, t_end);
+      for (int t = t_begin; t < t_end; ++t, ++it) {
+        const uint32_t par = (uint32_t)it & 1u;
+        if (tr_epi) TCB_TR(2 * it + grp, TCB_EV_EPI_BEGIN);
+        if (!tc_wait_warp(&aux->yfull, par, abort_flag)) { ok = false; timeout_site = 32; break; }
+        ptx::tc_fence_after();
+        if (tr_epi) TCB_TR(2 * it + grp, TCB_EV_EPI_Y);
+        // two tokens per word: the sign bit over 0x7fff where the value (as bf16) is not +-0, else 0
+        uint32_t m[2][16];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          float v[32];
+          ptx::tmem_ld32(y_addr + (uint32_t)(c * 32), v);
+          if (tr_epi) TCB_TR(2 * it + grp, c == 0 ? TCB_EV_EPI_LD0 : TCB_EV_EPI_LD1);
+#pragma unroll
+          for (int e = 0; e < 16; ++e) {
+            const uint32_t pk = bf16x2_pack(v[2 * e], v[2 * e + 1]);
+            uint32_t nz;
+            asm("set.neu.u32.bf16x2 %0, %1, %2;" : "=r"(nz) : "r"(pk), "r"(0u));
+            m[c][e] = (pk | 0x7fff7fffu) & nz;
+          }
+        }
+        ptx::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(&aux->yempty);         // the next first product may overwrite Y^T
+        if (!tc_wait_warp(&aux->nready[xs], xph, abort_flag)) { ok = false; timeout_site = 35; break; }
+        if (tr_epi) TCB_TR(2 * it + grp, TCB_EV_EPI_NORMS);
+        if (!tc_wait_warp(&aux->cfree[grp], par ^ 1u, abort_flag)) { ok = false; timeout_site = 31; break; }
+        ptx::tc_fence_after();
+        if (tr_epi) TCB_TR(2 * it + grp, TCB_EV_EPI_CFREE);
+        const uint4* rn4 = reinterpret_cast<const uint4*>(&aux->rn[xs][grp * 128 + half * 64]);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const uint4 r4 = rn4[c * 4 + k];       // the same 8 tokens for every lane
+            m[c][4 * k] &= r4.x | 0x80008000u; m[c][4 * k + 1] &= r4.y | 0x80008000u;
+            m[c][4 * k + 2] &= r4.z | 0x80008000u; m[c][4 * k + 3] &= r4.w | 0x80008000u;
+          }
+          ptx::tmem_st16(c_addr + (uint32_t)(c * 16), m[c]);
+          if (tr_epi && c == 0) TCB_TR(2 * it + grp, TCB_EV_EPI_ST0);
+          if (g.signs != nullptr) {
+            const int tok0 = t * 256 + grp * 128 + half * 64 + c * 32;
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+              const uint32_t h16 = (m[c][i >> 1] >> (16 * (i & 1))) & 0xffffu;
+              if (tok0 + i < g.n)
+                g.signs[((long long)p * g.n + tok0 + i) * TCB_D + j] = (h16 & 0x7fffu) ? ((h16 & 0x8000u) ? -1 : 1) : 0;
+            }
+          }
+        }
+        ptx::tmem_st_wait();
+        ptx::tc_fence_before();
+        __syncwarp();                              // one arrival per warp: every lane's fences precede it
+        if (tr_epi) TCB_TR(2 * it + grp, TCB_EV_EPI_END);
+        if (lane == 0) ptx::mbar_arrive(&aux->cready[grp]);
+        if (++xs == TCBT_STAGES) { xs = 0; xph ^= 1u; }
+      }
+      if (!ok) break;
+      // The problem's cross-covariance, transposed: lane = column of M, TMEM column = its row; each of the 16 warps takes
+      // 32 columns x 32 rows, and the accumulator is free once they are in registers.  One item per problem: added into M
+      // (one addition per element and launch, so the result does not depend on any order); several: stored to the item's
+      // partial, summed in item order afterwards.  128 contiguous bytes per warp and row.
+      if (tr_epi && grp == 1) TCB_TR(2 * it - 1, TCB_EV_OUT_WAIT);
+      if (!tc_wait_warp(&aux->mfull, (uint32_t)lp & 1u, abort_flag)) { ok = false; timeout_site = 33; break; }
+      ptx::tc_fence_after();
+      if (tr_epi && grp == 1) TCB_TR(2 * it - 1, TCB_EV_OUT_BEGIN);
+      {
+        float v[32];
+        ptx::tmem_ld32(lane_addr + TCBT_M_COL + m_col, v);
+        ptx::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(&aux->mempty);
+        float* out = (g.S == 1 ? g.M + (size_t)p * TCB_D * TCB_D : g.Mpart + (size_t)item * TCB_D * TCB_D) + m_col * TCB_D + j;
+        if (g.S == 1) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) asm volatile("red.global.add.f32 [%0], %1;" ::"l"(out + i * TCB_D), "f"(v[i]) : "memory");
+        } else {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) out[i * TCB_D] = v[i];
+        }
+      }
+      if (tr_epi && grp == 1) TCB_TR(2 * it - 1, TCB_EV_OUT_END);
     }
   }
 
@@ -556,10 +931,11 @@ inline int tcb_make_x_tmap(CUtensorMap* tm, const void* ptr, uint64_t n, uint64_
 // Problems [p0, p0 + np) of the context; X holds those np problems.
 inline int tcb_step(TcHost& h, cudaStream_t s, const void* X, int in_dtype, int64_t n, int64_t ld, int64_t pstride, int p0,
                     int np, int8_t* signs_out = nullptr, long long* trace = nullptr) {
-  static std::atomic<unsigned long long> attr_dev_mask{0};      // the attribute is per device
+  static std::atomic<unsigned long long> attr_dev_mask{0};      // the attributes are per device
   const unsigned long long dev_bit = 1ull << (h.device & 63);
   if (!(attr_dev_mask.load(std::memory_order_acquire) & dev_bit)) {
-    if (cudaFuncSetAttribute(tcb_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TCB_SMEM_BYTES) != cudaSuccess)
+    if (cudaFuncSetAttribute(tcb_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TCB_SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(tcb_step_plain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TCBT_SMEM_BYTES) != cudaSuccess)
       return CONQUR_ERR_CUDA;
     attr_dev_mask.fetch_or(dev_bit, std::memory_order_release);
   }
@@ -585,7 +961,7 @@ inline int tcb_step(TcHost& h, cudaStream_t s, const void* X, int in_dtype, int6
   g.trace = trace;
   // few problems: split each problem's tokens over several CTAs (partials land in the idle Newton-Schulz buffers,
   // 4 P matrices of 128 x 128 starting at Xa, and are summed in a fixed order)
-  const int T = (int)((n + 127) / 128);
+  const int T = h.qs.bits == 0 ? (int)((n + 255) / 256) : (int)((n + 127) / 128);      // units the kernel works in
   int S = 1;
   if (np < h.num_sms) S = std::max(1, std::min(std::min(h.num_sms / np, T), 4 * h.P / np));
   g.S = S; g.Mpart = h.Xa;
@@ -598,7 +974,8 @@ inline int tcb_step(TcHost& h, cudaStream_t s, const void* X, int in_dtype, int6
     rec.e0 = h.prof->get_event(); rec.e1 = h.prof->get_event();
     cudaEventRecord(rec.e0, s);
   }
-  tcb_step_kernel<<<grid, TCB_THREADS, TCB_SMEM_BYTES, s>>>(tmX, h.tmRb_mn, S == 1 ? h.tmM_blk : h.tmMpart_blk, g);
+  if (h.qs.bits == 0) tcb_step_plain_kernel<<<grid, TCBT_THREADS, TCBT_SMEM_BYTES, s>>>(tmX, h.tmRb_mn, g);
+  else tcb_step_kernel<<<grid, TCB_THREADS, TCB_SMEM_BYTES, s>>>(tmX, h.tmRb_mn, S == 1 ? h.tmM_blk : h.tmMpart_blk, g);
   if (timed) { cudaEventRecord(rec.e1, s); h.prof->open.push_back(rec); }
   if (cudaGetLastError() != cudaSuccess) return CONQUR_ERR_CUDA;
   if (h.prof) h.prof->count(K_ROTATE);
