@@ -184,11 +184,20 @@ int cuda_fail(const char* what, cudaError_t e) {
     (c)->prof.count(cls);            \
   } while (0)
 
-__global__ void or_flags_kernel(const DevState* st, int P, int* agg) {
+// The latched status of all problems (one block) and, where J is given, their sums: what a read-out copies to the host.
+__global__ void read_out_kernel(const DevState* st, int P, int* agg, double* J, long long* N) {
+  __shared__ int all;
+  if (threadIdx.x == 0) all = 0;
+  __syncthreads();
   int f = 0;
-  for (int i = threadIdx.x; i < P; i += blockDim.x) f |= st[i].status_flags;
-  for (int o = 16; o > 0; o >>= 1) f |= __shfl_xor_sync(0xffffffffu, f, o);
-  if ((threadIdx.x & 31) == 0 && f) atomicOr(agg, f);
+  for (int i = threadIdx.x; i < P; i += blockDim.x) {
+    f |= st[i].status_flags;
+    if (J) { J[i] = st[i].J; N[i] = st[i].N; }
+  }
+  f = __reduce_or_sync(0xffffffffu, f);
+  if ((threadIdx.x & 31) == 0 && f) atomicOr(&all, f);
+  __syncthreads();
+  if (threadIdx.x == 0) *agg = all;
 }
 __global__ void clear_flags_kernel(DevState* st, int P, int* agg) {
   for (int i = threadIdx.x; i < P; i += blockDim.x) st[i].status_flags = 0;
@@ -203,6 +212,7 @@ __global__ void export_sums_kernel(const DevState* st, double* J, long long* N, 
 __global__ void set_sums_kernel(DevState* st, const double* J, const long long* N, int P) {
   for (int i = threadIdx.x; i < P; i += blockDim.x) { st[i].J = J[i]; st[i].N = N[i]; }
 }
+__global__ void set_sum_kernel(DevState* st, double J, long long N) { st->J = J; st->N = N; }
 
 int flags_to_status(int f) {
   if (f & STATUS_FLAG_TIMEOUT) return CONQUR_ERR_TIMEOUT;
@@ -214,8 +224,7 @@ int flags_to_status(int f) {
 // Synchronise and return the latched device status (not cleared).
 int sync_status(conqur_ctx* c) {
   int* agg = c->at<int>(c->L.flags_agg);
-  CQ_CUDA(cudaMemsetAsync(agg, 0, sizeof(int), c->stream));
-  or_flags_kernel<<<1, 256, 0, c->stream>>>(c->state(), c->cfg.P, agg);
+  read_out_kernel<<<1, c->cfg.P > 32 ? 256 : 32, 0, c->stream>>>(c->state(), c->cfg.P, agg, nullptr, nullptr);
   CQ_LAUNCHED(c, K_OTHER);
   int f = 0;
   CQ_CUDA(cudaMemcpyAsync(&f, agg, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
@@ -786,11 +795,20 @@ extern "C" int conqur_get_objective(conqur_ctx* c, double* J_sum, int64_t* n_tok
   { const int frc = flush_pending(c); if (frc) return frc; }
   const int P = c->cfg.P;
   if (c->cfg.mode == CONQUR_TC_BF16) { const int orc = tcb_refresh_objective(c->tc, c->stream); if (orc) return orc; }
-  std::vector<DevState> h(P);
-  CQ_CUDA(cudaMemcpyAsync(h.data(), c->state(), sizeof(DevState) * P, cudaMemcpyDeviceToHost, c->stream));
-  const int rc = sync_status(c);
-  for (int p = 0; p < P; ++p) { J_sum[p] = h[p].J; n_tokens[p] = h[p].N; }
-  return rc;
+  // J, N and the status leave together through the (idle) partials: one launch and one copy of 16 bytes a problem
+  double* dJ = c->at<double>(c->L.part_d);
+  long long* dN = reinterpret_cast<long long*>(dJ + P);
+  int* df = reinterpret_cast<int*>(dN + P);
+  read_out_kernel<<<1, P > 32 ? 256 : 32, 0, c->stream>>>(c->state(), P, df, dJ, dN);
+  CQ_LAUNCHED(c, K_OTHER);
+  std::vector<unsigned char> h(16 * (size_t)P + sizeof(int));
+  CQ_CUDA(cudaMemcpyAsync(h.data(), dJ, h.size(), cudaMemcpyDeviceToHost, c->stream));
+  CQ_CUDA(cudaStreamSynchronize(c->stream));
+  std::memcpy(J_sum, h.data(), 8 * (size_t)P);
+  std::memcpy(n_tokens, h.data() + 8 * (size_t)P, 8 * (size_t)P);
+  int f;
+  std::memcpy(&f, h.data() + 16 * (size_t)P, sizeof(int));
+  return flags_to_status(f);
 }
 
 extern "C" int conqur_get_objective_async(conqur_ctx* c, double* J_sum_host, int64_t* n_tokens_host) {
@@ -841,14 +859,20 @@ extern "C" int conqur_set_M(conqur_ctx* c, const float* M_dev, const double* J_s
   scale_copy_kernel<<<ew_blocks(count), 256, 0, c->stream>>>(M_dev, c->at<float>(c->L.M), count,
                                                              (float)std::sqrt((double)c->cfg.d));
   CQ_LAUNCHED(c, K_OTHER);
-  // stage the sums through the partials buffer
-  double* dJ = c->at<double>(c->L.part_d);
-  long long* dN = reinterpret_cast<long long*>(dJ + P);
-  std::vector<long long> n64(n_tokens, n_tokens + P);
-  CQ_CUDA(cudaMemcpyAsync(dJ, J_sum, sizeof(double) * P, cudaMemcpyHostToDevice, c->stream));
-  CQ_CUDA(cudaMemcpyAsync(dN, n64.data(), sizeof(long long) * P, cudaMemcpyHostToDevice, c->stream));
-  set_sums_kernel<<<1, 256, 0, c->stream>>>(c->state(), dJ, dN, P);
-  CQ_LAUNCHED(c, K_OTHER);
+  std::vector<unsigned char> h;                       // (outlives the copy: the stream is synchronised below)
+  if (P == 1) {
+    set_sum_kernel<<<1, 1, 0, c->stream>>>(c->state(), J_sum[0], (long long)n_tokens[0]);
+    CQ_LAUNCHED(c, K_OTHER);
+  } else {
+    // stage the sums through the partials buffer, in one copy
+    double* dJ = c->at<double>(c->L.part_d);
+    h.resize(16 * (size_t)P);
+    std::memcpy(h.data(), J_sum, 8 * (size_t)P);
+    std::memcpy(h.data() + 8 * (size_t)P, n_tokens, 8 * (size_t)P);
+    CQ_CUDA(cudaMemcpyAsync(dJ, h.data(), h.size(), cudaMemcpyHostToDevice, c->stream));
+    set_sums_kernel<<<1, 256, 0, c->stream>>>(c->state(), dJ, reinterpret_cast<const long long*>(dJ + P), P);
+    CQ_LAUNCHED(c, K_OTHER);
+  }
   CQ_CUDA(cudaStreamSynchronize(c->stream));
   for (int p = 0; p < P; ++p) c->tokens[p] = n_tokens[p];
   return CONQUR_OK;
