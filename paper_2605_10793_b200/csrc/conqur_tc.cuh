@@ -1478,6 +1478,7 @@ inline int tc_ns_commit(TcHost& h, cudaStream_t s) {
   return cudaGetLastError() == cudaSuccess ? CONQUR_OK : CONQUR_ERR_CUDA;
 }
 
+inline __nv_bfloat16* tc_iterate_ptr(const TcHost& h, int i) { return reinterpret_cast<__nv_bfloat16*>(h.ws + h.L.Xh[i]); }
 inline const __nv_bfloat16* tc_cp_ptr(const TcHost& h) { return reinterpret_cast<const __nv_bfloat16*>(h.ws + h.L.Cp); }
 
 // Stand-alone product (tests, weight folding): D (fp32, M x N, row stride ldo; 0 = N) = A * B^T-style contraction with

@@ -128,3 +128,42 @@ def test_exact_update_inside_a_callers_capture():
         ref.step(x)
         ref.update()
     assert torch.equal(c.get_R(), ref.get_R())
+
+
+@pytest.mark.parametrize("d", [128, 512, 640, 1024])
+def test_set_R_decides_alike_in_both_modes(d):
+    """The tensor-core contexts decide on a bf16-pair product and go to the fp32 one near the limit of 1e-3: the same
+    rotations pass, on both sides of the limit, close to it, and with infinities in them."""
+    q = torch.linalg.qr(_rand(d, d, d).double())[0]
+    tc = B.Context(d, 8, mode="tc")
+    ex = B.Context(d, 8, in_dtype="f32", mode="exact")
+
+    def takes(ctx, r):
+        try:
+            ctx.set_R(r)
+            return True
+        except B.ConqurError as e:
+            assert e.status == -3
+            return False
+
+    cases = []
+    for err in (0.0, 2e-4, 8e-4, 9.7e-4, 9.97e-4, 9.997e-4, 1.0003e-3, 1.003e-3, 1.03e-3, 1.3e-3, 0.1):
+        r = q.clone()
+        r[:, d // 3] *= (1.0 + err) ** 0.5                 # one diagonal element of R^T R off by err
+        # (fp32 sums of d terms of size up to 1: within 1e-6 of the limit either answer is right, but the same one)
+        want = err < 1e-3 if abs(err - 1e-3) > 2e-6 else None
+        cases.append((r.float().contiguous(), want))
+        r = q.clone()
+        r[:, 1] = (r[:, 1] + err * r[:, d - 1])            # one off-diagonal pair
+        cases.append((r.float().contiguous(), want))
+    for bad in (float("inf"), 1e30):
+        r = q.float().contiguous()
+        r[d // 2, 3] = bad
+        cases.append((r, False))
+    for r, want in cases:
+        got = takes(tc, r)
+        assert got == takes(ex, r) and want in (None, got)
+    big = torch.zeros(d * d + 1, device="cuda")
+    big[1:] = q.float().flatten()                          # not 16-byte aligned
+    assert takes(tc, big[1:].view(d, d))
+    assert torch.equal(tc.get_R(), q.float())
