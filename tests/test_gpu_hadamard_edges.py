@@ -1,0 +1,29 @@
+"""The tensor-core transform's bf16 write-out at the ends of its 32-chunk groups and 256-chunk tiles."""
+import pytest
+import torch
+
+from paper_2605_10793_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("d,n", [(128, 1), (128, 31), (128, 33), (128, 255), (128, 257), (256, 17), (64, 66), (4, 96), (1024, 5),
+                                 (4096, 9), (8192, 3), (8192, 150), (4096, 1201)])
+def test_bf16_rows_match_fp64_and_leave_the_rest_alone(d, n):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d + n)
+    x = torch.randn(n, d, generator=g, device="cuda").to(torch.bfloat16)
+    buf = torch.full((n + 2, d), 7.0, dtype=torch.bfloat16, device="cuda")
+    B.conqur_hadamard_rows(x, out=buf[1:n + 1])
+    assert B.conqur_hadamard_status() == 0
+    y = x.double()
+    h = 1
+    while h < d:
+        v = y.view(n, d // (2 * h), 2, h)
+        y = torch.stack((v[:, :, 0] + v[:, :, 1], v[:, :, 0] - v[:, :, 1]), dim=2).reshape(n, d)
+        h *= 2
+    ref = y / d ** 0.5
+    # log2(d) levels of fp32 additions of partial sums bounded by ||x||_2, then one rounding to bf16
+    bound = max(d.bit_length() - 1, 1) * 2.0 ** -24 * x.double().norm(dim=1, keepdim=True) + 2.0 ** -8 * ref.abs()
+    assert ((buf[1:n + 1].double() - ref).abs() <= bound).all()
+    assert (buf[0] == 7.0).all() and (buf[n + 1] == 7.0).all()
