@@ -29,6 +29,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <mutex>
+#include <type_traits>
 
 #include "../../include/conqur.h"
 #include "conqur_internal.h"
@@ -836,26 +837,42 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 
 // ------------------------------------------------------------------ element-wise kernels of the mode
 
-// a1 for the tensor-core mode: one warp per row.  rnorm_i = 1/||x_i||_2 (fp32, from the bf16-rounded values the
+// a1 for the tensor-core mode: W warps per row.  rnorm_i = 1/||x_i||_2 (fp32, from the bf16-rounded values the
 // MMA will see) and a bf16 copy of the row in the workspace; skipped rows are written as zeros so that they
-// cannot reach the accumulators.
-template <typename TIn>
+// cannot reach the accumulators.  A warp's share of a row (up to 4096 elements) sits in its registers as packed bf16, all
+// 16-byte loads in flight at once, so a row is read from memory once: bound by memory (4093 x 8192 bf16: 65 -> 28 us
+// against two passes over rows longer than 4096).  Rows that do not start on 16-byte boundaries take two passes of
+// narrow loads.
+template <typename TIn, int W>
 __global__ void __launch_bounds__(256) rownorm_stage_kernel(const TIn* __restrict__ X, int64_t n, int d, int64_t ld,
                                                             float* __restrict__ rnorm,
                                                             __nv_bfloat16* __restrict__ Xs, DevState* st) {
-  const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (row >= n) return;
-  const TIn* x = X + row * ld;
+  __shared__ float part_ss[8];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t row = (int64_t)blockIdx.x * (8 / W) + warp / W;
+  const bool live = row < n;
+  if (W == 1 && !live) return;
+  const int slice = ((d + W * 256 - 1) / (W * 256)) * 256;
+  const int k0 = (warp % W) * slice, k1 = min(d, k0 + slice);           // this warp's columns
+  const TIn* x = X + (live ? row : 0) * ld;
   __nv_bfloat16* dst = Xs + row * (int64_t)d;
-  if (sizeof(TIn) == 2 && d <= 4096 && (d & 255) == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0) {
-    // bf16 rows of up to 4096 elements: the whole row sits in the warp's registers (16-byte pieces, all loads in
-    // flight at once), is read from memory once and written out from the registers
-    const int nchunk = d >> 8;                          // 256 elements = 32 lanes x 16 bytes
-    uint4 buf[16];
+  const bool vec = (reinterpret_cast<uintptr_t>(x) & 15) == 0;          // (d and the slices are multiples of 8)
+  uint4 buf[16];
+  float ss = 0.f;
+  if (live && vec) {
 #pragma unroll
-    for (int c = 0; c < 16; ++c)
-      buf[c] = (c < nchunk) ? __ldg(reinterpret_cast<const uint4*>(x + c * 256 + lane * 8)) : make_uint4(0u, 0u, 0u, 0u);
+    for (int c = 0; c < 16; ++c) {
+      const int k = k0 + c * 256 + lane * 8;
+      buf[c] = make_uint4(0u, 0u, 0u, 0u);
+      if (k < k1) {
+        if (sizeof(TIn) == 2) {
+          buf[c] = __ldg(reinterpret_cast<const uint4*>(x + k));
+        } else {
+          const float4 a = __ldg(reinterpret_cast<const float4*>(x + k)), b = __ldg(reinterpret_cast<const float4*>(x + k + 4));
+          buf[c] = make_uint4(bf16x2_pack(a.x, a.y), bf16x2_pack(a.z, a.w), bf16x2_pack(b.x, b.y), bf16x2_pack(b.z, b.w));
+        }
+      }
+    }
     float s4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int c = 0; c < 16; ++c) {
@@ -866,56 +883,33 @@ __global__ void __launch_bounds__(256) rownorm_stage_kernel(const TIn* __restric
         s4[e] = fmaf(a, a, s4[e]); s4[e] = fmaf(b, b, s4[e]);
       }
     }
-    const float ssr = warp_sum((s4[0] + s4[1]) + (s4[2] + s4[3]));
-    const bool goodr = (ssr > 0.f) && (ssr <= 3.0e38f);
-#pragma unroll
-    for (int c = 0; c < 16; ++c)
-      if (c < nchunk) *reinterpret_cast<uint4*>(dst + c * 256 + lane * 8) = goodr ? buf[c] : make_uint4(0u, 0u, 0u, 0u);
-    if (lane == 0) {
-      if (!goodr) {
-        atomicAdd(reinterpret_cast<unsigned long long*>(&st->step_skipped), 1ull);
-        if (!(ssr == 0.f)) atomicOr(&st->status_flags, STATUS_FLAG_NONFINITE);
-      }
-      rnorm[row] = goodr ? 1.0f / sqrtf(ssr) : 0.f;
+    ss = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+  } else if (live) {
+    for (int k = k0 + lane; k < k1; k += 32) {
+      const float v = bf16_round(ld_as_float(x + k));                   // (bf16 values are exact already)
+      ss = fmaf(v, v, ss);
     }
-    return;
-  }
-  const bool vec = (reinterpret_cast<uintptr_t>(x) & (sizeof(TIn) * 4 - 1)) == 0;    // d is a multiple of 128
-  float ss = 0.f;
-  for (int k = lane * 4; k < d; k += 128) {
-    float v[4];
-    if (vec) {
-      ld4_as_float(x + k, v);
-    } else {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) v[j] = ld_as_float(x + k + j);
-    }
-    if (sizeof(TIn) == 4) {                            // fp32 input: the norm of what the MMA will see (bf16 values are exact already)
-      const uint32_t p0 = bf16x2_pack(v[0], v[1]), p1 = bf16x2_pack(v[2], v[3]);
-      v[0] = __uint_as_float(p0 << 16); v[1] = __uint_as_float(p0 & 0xffff0000u);
-      v[2] = __uint_as_float(p1 << 16); v[3] = __uint_as_float(p1 & 0xffff0000u);
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) ss = fmaf(v[j], v[j], ss);
   }
   ss = warp_sum(ss);
-  const bool good = (ss > 0.f) && (ss <= 3.0e38f);
-  for (int k = lane * 4; k < d; k += 128) {
-    float v[4] = {0.f, 0.f, 0.f, 0.f};
-    if (good) {
-      if (vec) {
-        ld4_as_float(x + k, v);
-      } else {
+  if (W > 1) {                                                          // the row's parts, added in order
+    if (lane == 0) part_ss[warp] = ss;
+    __syncthreads();
+    ss = 0.f;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) v[j] = ld_as_float(x + k + j);
-      }
-    }
-    uint2 o;
-    o.x = bf16x2_pack(v[0], v[1]);
-    o.y = bf16x2_pack(v[2], v[3]);
-    *reinterpret_cast<uint2*>(dst + k) = o;
+    for (int i = 0; i < W; ++i) ss += part_ss[warp / W * W + i];
+    if (!live) return;
   }
-  if (lane == 0) {
+  const bool good = (ss > 0.f) && (ss <= 3.0e38f);
+  if (vec) {
+#pragma unroll
+    for (int c = 0; c < 16; ++c) {
+      const int k = k0 + c * 256 + lane * 8;
+      if (k < k1) *reinterpret_cast<uint4*>(dst + k) = good ? buf[c] : make_uint4(0u, 0u, 0u, 0u);
+    }
+  } else {
+    for (int k = k0 + lane; k < k1; k += 32) dst[k] = __float2bfloat16(good ? ld_as_float(x + k) : 0.f);
+  }
+  if (lane == 0 && warp % W == 0) {
     if (!good) {
       atomicAdd(reinterpret_cast<unsigned long long*>(&st->step_skipped), 1ull);
       if (!(ss == 0.f)) atomicOr(&st->status_flags, STATUS_FLAG_NONFINITE);
@@ -1330,11 +1324,18 @@ inline TcGemmArgs tc_args(const TcHost& h, int M, int N, int K) {
 inline int tc_stage(TcHost& h, cudaStream_t s, const void* X, int in_dtype, int64_t n, int64_t ld, int64_t row0) {
   const int d = h.d;
   __nv_bfloat16* Xs = reinterpret_cast<__nv_bfloat16*>(h.ws + h.L.Xs) + row0 * d;
-  const int rb = (int)((n + 7) / 8);
-  if (in_dtype == CONQUR_F32)
-    rownorm_stage_kernel<float><<<rb, 256, 0, s>>>(static_cast<const float*>(X), n, d, ld, h.rnorm + row0, Xs, h.st);
-  else
-    rownorm_stage_kernel<__nv_bfloat16><<<rb, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(X), n, d, ld, h.rnorm + row0, Xs, h.st);
+  auto launch = [&](auto w) {                              // W warps a row: at most 4096 elements each
+    constexpr int W = decltype(w)::value;
+    const int rb = (int)((n + 8 / W - 1) / (8 / W));
+    if (in_dtype == CONQUR_F32)
+      rownorm_stage_kernel<float, W><<<rb, 256, 0, s>>>(static_cast<const float*>(X), n, d, ld, h.rnorm + row0, Xs, h.st);
+    else
+      rownorm_stage_kernel<__nv_bfloat16, W><<<rb, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(X), n, d, ld, h.rnorm + row0, Xs, h.st);
+  };
+  if (d <= 4096) launch(std::integral_constant<int, 1>{});
+  else if (d <= 8192) launch(std::integral_constant<int, 2>{});
+  else if (d <= 16384) launch(std::integral_constant<int, 4>{});
+  else launch(std::integral_constant<int, 8>{});
   if (cudaGetLastError() != cudaSuccess) return CONQUR_ERR_CUDA;
   if (h.prof) h.prof->count(K_ROWNORM);
   return CONQUR_OK;
