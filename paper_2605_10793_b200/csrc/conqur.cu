@@ -1166,12 +1166,13 @@ extern "C" int conqur_hadamard_rows(const void* X_dev, int32_t in_dtype, int64_t
   while ((1 << logd) < d) ++logd;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   using bf = __nv_bfloat16;
-  // bf16 rows that lie back to back: the 128-point sub-transforms run on the tensor cores
+  // bf16 rows whose layout the copy engine takes: the 128-point sub-transforms run on the tensor cores
   const bool simt_only = (flags & CONQUR_HADAMARD_CUDA_CORES_ONLY) != 0;
-  if (!simt_only && in_dtype == CONQUR_BF16 && ldx == d && ldy == d && (reinterpret_cast<uintptr_t>(X_dev) & 15) == 0 &&
-      (reinterpret_cast<uintptr_t>(Y_dev) & 15) == 0 && (n * d) % 128 == 0) {
-    const int rc = (out_dtype == CONQUR_F32) ? hadamard_tc_launch(static_cast<const bf*>(X_dev), static_cast<float*>(Y_dev), n, logd, s)
-                                             : hadamard_tc_launch(static_cast<const bf*>(X_dev), static_cast<bf*>(Y_dev), n, logd, s);
+  if (!simt_only && in_dtype == CONQUR_BF16 &&
+      hadamard_tc_takes(X_dev, ldx, Y_dev, ldy, out_dtype == CONQUR_F32 ? 4 : 2, n, d)) {
+    const int rc = (out_dtype == CONQUR_F32)
+                       ? hadamard_tc_launch(static_cast<const bf*>(X_dev), ldx, static_cast<float*>(Y_dev), ldy, n, logd, s)
+                       : hadamard_tc_launch(static_cast<const bf*>(X_dev), ldx, static_cast<bf*>(Y_dev), ldy, n, logd, s);
     if (rc != CONQUR_ERR_UNSUPPORTED) return rc;
   }
   if (in_dtype == CONQUR_F32 && out_dtype == CONQUR_F32)

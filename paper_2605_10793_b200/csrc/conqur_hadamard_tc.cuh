@@ -41,9 +41,12 @@ struct HtcAux {
 };
 static_assert(sizeof(HtcAux) <= HTC_AUX_BYTES, "the barrier block must fit its reserved shared memory");
 
-template <typename TOut>
+template <typename TOut, bool FLAT>
 __global__ void __launch_bounds__(HTC_THREADS, 1)
-hadamard_tc_kernel(const __grid_constant__ CUtensorMap tmX, TOut* Y, long long NC, int logd, float scale) {
+hadamard_tc_kernel(const __grid_constant__ CUtensorMap tmX, TOut* Y, long long NC, int logd, float scale, int lr, long long ldr) {
+  // FLAT: rows that lie back to back, one run of NC chunks (a kernel of its own: the address arithmetic of the general form
+  // costs 6 % there).  Otherwise chunk ch belongs to row ch >> lr, columns 128 (ch mod 2^lr).., of the output, whose rows are
+  // ldr elements apart.
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = smem;
@@ -100,8 +103,14 @@ hadamard_tc_kernel(const __grid_constant__ CUtensorMap tmX, TOut* Y, long long N
         if (!tc_wait(&aux->xempty[s], ph ^ 1u, abort_flag)) { ok = false; timeout_site = 1; break; }
         uint8_t* dst = sX + s * HTC_X_BYTES;
         ptx::mbar_expect_tx(&aux->xfull[s], HTC_X_BYTES);
-        ptx::tma_load_2d(dst, &tmX, &aux->xfull[s], 0, (int)(t * HTC_N));
-        ptx::tma_load_2d(dst + HTC_X_BYTES / 2, &tmX, &aux->xfull[s], 64, (int)(t * HTC_N));
+        // the tile's 256 chunks: a run of one flat row, or whole rows
+        if (FLAT) {
+          ptx::tma_load_2d(dst, &tmX, &aux->xfull[s], 0, (int)(t * HTC_N));
+          ptx::tma_load_2d(dst + HTC_X_BYTES / 2, &tmX, &aux->xfull[s], 64, (int)(t * HTC_N));
+        } else {
+          tma_load_3d(dst, &tmX, &aux->xfull[s], 0, 0, (int)(t * (HTC_N >> lr)));
+          tma_load_3d(dst + HTC_X_BYTES / 2, &tmX, &aux->xfull[s], 64, 0, (int)(t * (HTC_N >> lr)));
+        }
         ++issued;
         if (++s == HTC_STAGES) { s = 0; ph ^= 1u; }
       }
@@ -140,6 +149,8 @@ hadamard_tc_kernel(const __grid_constant__ CUtensorMap tmX, TOut* Y, long long N
     float* stg = reinterpret_cast<float*>(sStg + ew * HTC_STG_BYTES);
     const int lc = (logd > 7) ? (logd - 7) : 0;    // level-2 butterfly levels (c = 2^lc chunks per row)
     int it = 0;
+    const long long cmask = (1ll << lr) - 1;
+    auto out_at = [&](long long ch) { return FLAT ? Y + ch * 128 : Y + (ch >> lr) * ldr + (ch & cmask) * 128; };
     // one 32-column group: level-2 levels < 5, scale, transpose, store
     auto finish32 = [&](float (&v)[32], long long chunk0) {
       had_butterflies(v, lc < 5 ? lc : 5);
@@ -158,12 +169,11 @@ hadamard_tc_kernel(const __grid_constant__ CUtensorMap tmX, TOut* Y, long long N
           const uint4 b = *reinterpret_cast<const uint4*>(&stw[kp * 32 + e0 + 4 - sw]);
           const uint4 lo = sw ? b : a, hi = sw ? a : b;
           const long long r = chunk0 + 2 * kp;
-          TOut* at = Y + r * 128 + q * 32 + e0;
           if (r < NC)
-            *reinterpret_cast<uint4*>(at) = make_uint4(__byte_perm(lo.x, lo.y, 0x5410), __byte_perm(lo.z, lo.w, 0x5410),
+            *reinterpret_cast<uint4*>(out_at(r) + q * 32 + e0) = make_uint4(__byte_perm(lo.x, lo.y, 0x5410), __byte_perm(lo.z, lo.w, 0x5410),
                                                        __byte_perm(hi.x, hi.y, 0x5410), __byte_perm(hi.z, hi.w, 0x5410));
           if (r + 1 < NC)
-            *reinterpret_cast<uint4*>(at + 128) = make_uint4(__byte_perm(lo.x, lo.y, 0x7632), __byte_perm(lo.z, lo.w, 0x7632),
+            *reinterpret_cast<uint4*>(out_at(r + 1) + q * 32 + e0) = make_uint4(__byte_perm(lo.x, lo.y, 0x7632), __byte_perm(lo.z, lo.w, 0x7632),
                                                              __byte_perm(hi.x, hi.y, 0x7632), __byte_perm(hi.z, hi.w, 0x7632));
         }
         __syncwarp();
@@ -176,7 +186,7 @@ hadamard_tc_kernel(const __grid_constant__ CUtensorMap tmX, TOut* Y, long long N
       for (int i = 0; i < 8; ++i) {
         const int r = i * 4 + (lane >> 3), p4 = (lane & 7) * 4;
         const float4 o = *reinterpret_cast<const float4*>(&stg[r * 32 + p4]);
-        if (chunk0 + r < NC) st4_from_float(Y + (chunk0 + r) * 128 + q * 32 + p4, o);
+        if (chunk0 + r < NC) st4_from_float(out_at(chunk0 + r) + q * 32 + p4, o);
       }
       __syncwarp();
     };
@@ -217,30 +227,61 @@ hadamard_tc_kernel(const __grid_constant__ CUtensorMap tmX, TOut* Y, long long N
   }
 }
 
-// n rows of d bf16 elements, contiguous (row stride d), 16-byte aligned base, n * d a multiple of 128.
+// Input rows ldx elements apart as chunks of 128 elements, (128, d / 128, n); a box is 64 columns of a tile's 256 chunks.
+inline int hadamard_make_tmap(CUtensorMap* tm, const void* X, uint64_t chunks, uint64_t rows, uint64_t ldx, uint32_t box_rows) {
+  PFN_encodeTiled fn = tc_encode_fn();
+  if (!fn) return CONQUR_ERR_CUDA;
+  const cuuint64_t dims[3] = {128, chunks, rows};
+  const cuuint64_t strides[2] = {256, ldx * 2};
+  const cuuint32_t box[3] = {64, (cuuint32_t)HTC_N / box_rows, box_rows};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  const CUresult r = fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(X), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) {
+    std::fprintf(stderr, "conqur: cuTensorMapEncodeTiled (transform input) failed (%d)\n", (int)r);
+    return CONQUR_ERR_CUDA;
+  }
+  return CONQUR_OK;
+}
+
+// Whether the tensor-core kernel takes these rows.  Back to back, 16-byte aligned, n d a multiple of 128; or d >= 128 and
+// rows that start on 16-byte boundaries on both sides (32768 x 4096 bf16 with 8 elements between rows: 168 us on the CUDA
+// cores, 126 here; 8192-element rows to fp32 199 -> 169; d = 128 184 -> 181).
+inline bool hadamard_tc_takes(const void* X, int64_t ldx, const void* Y, int64_t ldy, size_t out_size, int64_t n, int d) {
+  if ((reinterpret_cast<uintptr_t>(X) & 15) || (reinterpret_cast<uintptr_t>(Y) & 15)) return false;
+  if (ldx == d && ldy == d) return (n * d) % 128 == 0;
+  return d >= 128 && (ldx * 2) % 16 == 0 && ((size_t)ldy * out_size) % 16 == 0 && ldx < (1ll << 38) && n <= 0x7fffffffll;
+}
+
 template <typename TOut>
-inline int hadamard_tc_launch(const __nv_bfloat16* X, TOut* Y, int64_t n, int logd, cudaStream_t s) {
+inline int hadamard_tc_launch(const __nv_bfloat16* X, int64_t ldx, TOut* Y, int64_t ldy, int64_t n, int logd, cudaStream_t s) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return CONQUR_ERR_CUDA;
   TcDevFacts f;
   if (tc_device_facts(dev, &f) != CONQUR_OK) return CONQUR_ERR_CUDA;
-  auto kern = hadamard_tc_kernel<TOut>;
   if (f.major != 10) return CONQUR_ERR_UNSUPPORTED;
-  static std::atomic<unsigned long long> attr_dev_mask{0};      // the attribute is per device
+  static std::atomic<unsigned long long> attr_dev_mask{0};      // the attributes are per device
   const unsigned long long dev_bit = 1ull << (dev & 63);
   if (!(attr_dev_mask.load(std::memory_order_acquire) & dev_bit)) {
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, HTC_SMEM_BYTES) != cudaSuccess) return CONQUR_ERR_CUDA;
+    if (cudaFuncSetAttribute(hadamard_tc_kernel<TOut, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, HTC_SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(hadamard_tc_kernel<TOut, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, HTC_SMEM_BYTES) != cudaSuccess)
+      return CONQUR_ERR_CUDA;
     attr_dev_mask.fetch_or(dev_bit, std::memory_order_release);
   }
   const long long NC = (long long)n * (1ll << logd) / 128;
   if (NC < 1 || NC > 0x7fffff00ll) return CONQUR_ERR_INVALID_ARG;
+  const bool flat = ldx == (1ll << logd) && ldy == (1ll << logd);
+  const int lr = flat ? 0 : logd - 7;
   CUtensorMap tm;
-  int rc = tc_make_tmap(&tm, X, (uint64_t)NC, 128, 128, HTC_N);
+  int rc = flat ? tc_make_tmap(&tm, X, (uint64_t)NC, 128, 128, HTC_N)
+                : hadamard_make_tmap(&tm, X, 1ull << lr, (uint64_t)n, (uint64_t)ldx, (uint32_t)(HTC_N >> lr));
   if (rc) return rc;
   const long long tiles = (NC + HTC_N - 1) / HTC_N;
   const int grid = (int)(tiles < f.sms ? tiles : f.sms);
   const float scale = (float)(1.0 / sqrt((double)(1 << logd)));
-  kern<<<grid, HTC_THREADS, HTC_SMEM_BYTES, s>>>(tm, Y, NC, logd, scale);
+  if (flat) hadamard_tc_kernel<TOut, true><<<grid, HTC_THREADS, HTC_SMEM_BYTES, s>>>(tm, Y, NC, logd, scale, lr, (long long)ldy);
+  else hadamard_tc_kernel<TOut, false><<<grid, HTC_THREADS, HTC_SMEM_BYTES, s>>>(tm, Y, NC, logd, scale, lr, (long long)ldy);
   return cudaGetLastError() == cudaSuccess ? CONQUR_OK : CONQUR_ERR_CUDA;
 }
 
