@@ -717,19 +717,27 @@ extern "C" int conqur_set_R(conqur_ctx* c, const float* R_dev) {
   arm_check_kernel<<<1, 256, 0, c->stream>>>(c->state(), g.P);
   CQ_LAUNCHED(c, K_OTHER);
   bool decided = false;
-  if (g.mode == CONQUR_TC_BF16 && g.P == 1 && g.d >= 512 && (reinterpret_cast<uintptr_t>(R_dev) & 15) == 0) {
+  const bool aligned = (reinterpret_cast<uintptr_t>(R_dev) & 15) == 0;
+  if (g.mode == CONQUR_TC_BF16 && aligned && (g.P > 1 || g.d >= 512)) {
     // The decision max|R^T R - I| <= 1e-3 on the tensor cores first: the three-pass product of R's bf16 pair, whose
     // entries are off by at most 2 2^-17 (the split) + (3 d / 16) 2^-23 (the accumulation) times the columns' norms, which
     // are 1 within 1e-3 wherever a decision is close.  Only a result within that bound of the limit, or one that is not
     // finite, goes on to the fp32 product below, so what is accepted and what is refused does not change
     // (whole call at d = 4096: 1650 -> 213 us, 3072: 865 -> 154, 1024: 111 -> 66; at 256 the extra launches cost 7 us).
     const double bound = 2.0e-5 + 2.5e-8 * g.d;
-    split_bf16_kernel<<<ew_blocks(dd / 4), 256, 0, c->stream>>>(R_dev, tc_iterate_ptr(c->tc, 0), dd, dd);
-    CQ_LAUNCHED(c, K_OTHER);
-    const int rc = tc_ns_residual(c->tc, c->stream, 0);
+    float* pf = c->at<float>(c->L.part_f);
+    double* pd = c->at<double>(c->L.part_d);
+    int rc;
+    if (g.P > 1) {
+      rc = tcb_check(c->tc, c->stream, R_dev, pf, pd);
+    } else {
+      split_bf16_kernel<<<ew_blocks(dd / 4), 256, 0, c->stream>>>(R_dev, tc_iterate_ptr(c->tc, 0), dd, dd);
+      CQ_LAUNCHED(c, K_OTHER);
+      rc = tc_ns_residual(c->tc, c->stream, 0);
+    }
     if (rc) return rc;
     double* out = c->at<double>(c->L.obj_out);
-    check_reduce_kernel<<<1, 256, 0, c->stream>>>(c->state(), c->at<float>(c->L.part_f), c->at<double>(c->L.part_d), ns_parts(c), out);
+    check_reduce_kernel<<<1, 256, 0, c->stream>>>(c->state(), pf, pd, g.P > 1 ? g.P : ns_parts(c), out);
     CQ_LAUNCHED(c, K_OTHER);
     double h[2];
     CQ_CUDA(cudaMemcpyAsync(h, out, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
@@ -751,6 +759,7 @@ extern "C" int conqur_set_R(conqur_ctx* c, const float* R_dev) {
     for (float v : pm) mx = (v == v) ? std::max(mx, v) : INFINITY;
     if (!(mx <= 1e-3f)) return CONQUR_ERR_NOT_ORTHOGONAL_INPUT;
   }
+  if (g.mode == CONQUR_TC_BF16 && aligned) return tc_take_R(c->tc, c->stream, R_dev);
   CQ_CUDA(cudaMemcpyAsync(c->at<float>(c->L.R), R_dev, sizeof(float) * dd * g.P, cudaMemcpyDeviceToDevice, c->stream));
   if (g.mode == CONQUR_TC_BF16) return tc_refresh_R(c->tc, c->stream, 0);
   return CONQUR_OK;

@@ -932,6 +932,16 @@ __global__ void split_bf16_kernel(const float* __restrict__ src, __nv_bfloat16* 
   }
 }
 
+// A rotation taken over: fp32 copy and its bf16 rounding in one pass.
+static __global__ void copy_split_kernel(const float* __restrict__ src, float* __restrict__ dst, __nv_bfloat16* __restrict__ dst16,
+                                         int64_t count) {
+  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; i < count; i += (int64_t)gridDim.x * blockDim.x * 4) {
+    const float4 t = *reinterpret_cast<const float4*>(src + i);
+    *reinterpret_cast<float4*>(dst + i) = t;
+    *reinterpret_cast<uint2*>(dst16 + i) = make_uint2(bf16x2_pack(t.x, t.y), bf16x2_pack(t.z, t.w));
+  }
+}
+
 // Second pass of the two-pass step in tensor-core mode (quant modes, or diagnostics): Y (fp32, row-major) ->
 // C' (bf16, row-major) + objective partials (+ diagnostics partials).
 __global__ void __launch_bounds__(256) quant_target_bf16_kernel(const float* __restrict__ Y, int64_t n, int d,
@@ -1309,6 +1319,14 @@ inline int tc_ew_blocks(int64_t count4) {
 inline int tc_refresh_R(TcHost& h, cudaStream_t s, int) {
   const int64_t dd = (int64_t)h.d * h.d * h.P;
   split_bf16_kernel<<<tc_ew_blocks(dd / 4), 256, 0, s>>>(h.R, reinterpret_cast<__nv_bfloat16*>(h.ws + h.L.Rb), dd, 0);
+  if (h.prof) h.prof->count(K_OTHER);
+  return cudaGetLastError() == cudaSuccess ? CONQUR_OK : CONQUR_ERR_CUDA;
+}
+
+// R <- src (16-byte aligned), with the bf16 copy the products read
+inline int tc_take_R(TcHost& h, cudaStream_t s, const float* src) {
+  const int64_t dd = (int64_t)h.d * h.d * h.P;
+  copy_split_kernel<<<tc_ew_blocks(dd / 4), 256, 0, s>>>(src, h.R, reinterpret_cast<__nv_bfloat16*>(h.ws + h.L.Rb), dd);
   if (h.prof) h.prof->count(K_OTHER);
   return cudaGetLastError() == cudaSuccess ? CONQUR_OK : CONQUR_ERR_CUDA;
 }

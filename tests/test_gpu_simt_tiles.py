@@ -167,3 +167,30 @@ def test_set_R_decides_alike_in_both_modes(d):
     big[1:] = q.float().flatten()                          # not 16-byte aligned
     assert takes(tc, big[1:].view(d, d))
     assert torch.equal(tc.get_R(), q.float())
+
+
+@pytest.mark.parametrize("P", [2, 5, 500])
+def test_set_R_of_many_heads_refuses_when_one_is_off(P):
+    d = 128
+    q = torch.linalg.qr(_rand(P, P, d, d).double())[0]
+    tc = B.Context(d, 8, mode="tc", batch=P)
+    ex = B.Context(d, 8, in_dtype="f32", mode="exact", batch=P)
+    for err, want in ((0.0, True), (9.0e-4, True), (9.95e-4, True), (1.005e-3, False), (1.1e-3, False), (float("inf"), False)):
+        for p in sorted({0, P // 2, P - 1}):
+            r = q.clone()
+            r[p, :, 77] *= (1.0 + err) ** 0.5
+            if err == float("inf"):
+                r[p] = q[p]
+                r[p, 3, 4] = err
+            r = r.float().contiguous()
+            got = []
+            for c in (tc, ex):
+                try:
+                    c.set_R(r)
+                    got.append(True)
+                except B.ConqurError as e:
+                    assert e.status == -3
+                    got.append(False)
+            assert got == [want, want], (err, p)
+            if want:
+                assert torch.equal(tc.get_R(), r)
