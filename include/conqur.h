@@ -58,8 +58,9 @@ enum { CONQUR_QUANT_SYMMETRIC = 0, CONQUR_QUANT_ZEROPOINT = 1 };   /* fake-quant
  * mode CONQUR_TC_BF16:   bf16 operands, fp32 accumulation on the tcgen05 tensor
  *                        cores; fp32 X is rounded to bf16 on the way in; the
  *                        Newton-Schulz iterate is held as a two-term bf16 split hi + lo
- *                        and each of its products takes one to three bf16 passes
- *                        (hi hi, hi lo, lo hi), chosen per step on the device.
+ *                        and, for a single problem, as a scaled fp16 copy; each of its
+ *                        products takes one pass over fp16 operands or two to three
+ *                        bf16 passes (hi hi, hi lo, lo hi), chosen per step on the device.
  */
 typedef struct {
   uint32_t struct_size;     /* = sizeof(conqur_config) */
@@ -93,11 +94,11 @@ typedef struct {
                                the cross-covariance is accumulated with R fixed, so the grouping changes no result
                                beyond fp32 summation order).  Use the update cadence; the workspace grows by
                                4*d*n_max bytes per deferred batch.  0 or 1: every step runs its products at once */
-  float    ns_gram_single_pass_tau;  /* tensor-core mode tuning: the Gram product of a Newton-Schulz step runs one bf16
-                               pass instead of three while the iterate's mean squared singular value is below this;
-                               0 = default */
-  float    ns_lo_gap_budget;/* tensor-core mode tuning: bound on the Procrustes gap given up by dropping the low bf16
-                               half of the iterate in the products of late steps (a worst-case bound: d directions at the
+  float    ns_gram_single_pass_tau;  /* tensor-core mode tuning: a Gram product that may accept the rotation runs one
+                               pass instead of three while the iterate's mean squared singular value is below this
+                               (the others run one pass anyway); 0 = default */
+  float    ns_lo_gap_budget;/* tensor-core mode tuning: bound on the Procrustes gap given up by dropping the low
+                               bits of the iterate in the products of late steps (a worst-case bound: d directions at the
                                noise floor under one dominant one; measured gaps are 20-50x smaller); 0 = default 5e-4 */
   int32_t  debug_flags;     /* test hooks, 0 in production: CONQUR_DEBUG_CANARIES | CONQUR_DEBUG_SINGLE_CTA |
                                CONQUR_DEBUG_NO_GRAPH */
