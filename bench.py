@@ -702,8 +702,8 @@ def main():
         "data": "synthetic",
         "config": {"workload": _workload_desc(w), "tokens_per_step": cyc * w.n, "mode": "tc (bf16 operands, fp32 accumulate; "
                    "the two step products run once per cycle over its 8 queued batches; Newton-Schulz: residual product "
-                   "as 1- or 3-term bf16 split on symmetric tiles, polynomial product 1 term, iterate product 2 terms "
-                   "then 1)", "l2": f"inputs larger than L2: {resident_bytes / 1e6:.0f} MB "
+                   "in one fp16 pass (the accepting check as 3-term bf16 split) and polynomial product in one fp16 pass on "
+                   "symmetric tiles, iterate product 2 bf16 terms then one fp16 pass)", "l2": f"inputs larger than L2: {resident_bytes / 1e6:.0f} MB "
                    f"of distinct batches resident, each read once per cycle", "replicas": g.world,
                    "input_gen_s": round(t_gen, 1)},
         "clocks": clocks, "e2e": e2e, "gpu_launches": int(launches),
