@@ -187,10 +187,12 @@ inline int sg_pick(int64_t M, int64_t N, int64_t problems, int64_t max_tiles = I
   const double cl = (double)cdv(worked(nl, cdv(N, 128)), sms) * 16384.0,
                ch = (double)cdv(worked(nh, 2 * cdv(N, 128)), sms) * (8192.0 / 0.98),
                cs = (double)cdv(worked(ns, cdv(N, 32)), sms) * (1024.0 / 0.65);
+  // rows of tiles are blocks in y, of which a launch takes 65535
+  auto fits = [&](int64_t tm, int64_t tiles) { return tiles <= max_tiles && cdv(M, tm) <= 65535; };
   int best = SG_LARGE;
   double c = cl;
-  if (ch < c && nh <= max_tiles) { best = SG_HALF; c = ch; }
-  if (cs < c && ns <= max_tiles) best = SG_SMALL;
+  if (ch < c && fits(64, nh)) { best = SG_HALF; c = ch; }
+  if (cs < c && fits(32, ns)) best = SG_SMALL;
   return best;
 }
 

@@ -194,3 +194,25 @@ def test_set_R_of_many_heads_refuses_when_one_is_off(P):
             assert got == [want, want], (err, p)
             if want:
                 assert torch.equal(tc.get_R(), r)
+
+
+@pytest.mark.parametrize("n,d", [(2097120, 2), (2097121, 2), (4194240, 33), (4194241, 2), (8388480, 2)])
+def test_more_rows_than_a_launch_has_blocks_of_the_smaller_tiles(n, d):
+    """65535 rows of tiles at most: 2097120 rows of the 32-row tile, 4194240 of the 64-row one, 8388480 of the 128-row one."""
+    x = _rand(n, n, d)
+    c = B.Context(d, n, in_dtype="f32", mode="exact")
+    r = torch.linalg.qr(_rand(1, d, d))[0].contiguous()
+    c.set_R(r)
+    c.step(x)
+    j, cnt = c.get_objective()
+    assert cnt == n
+    ref = 0.0
+    for part in x.split(1 << 20):
+        y = part.double() / part.double().norm(dim=1, keepdim=True)
+        ref += float((y @ r.double()).abs().sum()) / d ** 0.5
+    # per row of norm 1: fp32 errors of the d sums of d products and of the norm, against a sum of at least 1
+    assert abs(j - ref) <= d * (d + 4) * 2.0 ** -24 * ref
+    out = B.conqur_fold_weight(x, r, "input", "exact")
+    for a in (0, n // 2, n - 1000):                  # first, middle and last tiles
+        want = x[a:a + 1000].double() @ r.double()
+        assert ((out[a:a + 1000].double() - want).abs() <= d * 2.0 ** -24 * (x[a:a + 1000].abs() @ r.abs()).double() + 1e-30).all()
