@@ -206,7 +206,8 @@ __global__ void clear_flags_kernel(DevState* st, int P, int* agg) {
 __global__ void arm_check_kernel(DevState* st, int P) {
   for (int i = threadIdx.x; i < P; i += blockDim.x) { st[i].ns_done = 0; st[i].ns_steps_used = 0; st[i].seg_e = 3; }
 }
-// max|G - I| and sum (G - I)^2 over the partials of a residual product (one block).
+// max|G - I| and sum (G - I)^2 over the partials of a residual product (one block).  st: state of the tensor-core product
+// that left them, or null.
 __global__ void check_reduce_kernel(const DevState* st, const float* pmax, const double* psq, int n, double* out) {
   __shared__ double redd[8];
   __shared__ float redf[8];
@@ -215,7 +216,7 @@ __global__ void check_reduce_kernel(const DevState* st, const float* pmax, const
   for (int i = threadIdx.x; i < n; i += 256) { mx = fmaxf(mx, pmax[i]); sq += psq[i]; }
   const double tsq = block_sum_d<256>(sq, redd);
   const float tmx = block_max_f<256>(mx, redf);
-  const bool gave_up = (st->status_flags & STATUS_FLAG_TIMEOUT) != 0;            // the product is not to be trusted
+  const bool gave_up = st != nullptr && (st->status_flags & STATUS_FLAG_TIMEOUT) != 0;   // the product is not to be trusted
   if (threadIdx.x == 0) { out[0] = (double)tmx; out[1] = gave_up ? (double)INFINITY : tsq; }
 }
 __global__ void export_sums_kernel(const DevState* st, double* J, long long* N, int P) {
@@ -709,6 +710,17 @@ extern "C" int conqur_destroy(conqur_ctx* ctx) {
   return CONQUR_OK;
 }
 
+// What a residual product left in `n` partials, on the host: h[0] = max|G - I| without NaN, h[1] = sum (G - I)^2 (NaN where
+// any entry is; infinite where the tensor-core product of state `st` gave up).
+static int check_read(conqur_ctx* c, const DevState* st, int n, double (&h)[2]) {
+  double* out = c->at<double>(c->L.obj_out);
+  check_reduce_kernel<<<1, 256, 0, c->stream>>>(st, c->at<float>(c->L.part_f), c->at<double>(c->L.part_d), n, out);
+  CQ_LAUNCHED(c, K_OTHER);
+  CQ_CUDA(cudaMemcpyAsync(h, out, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
+  CQ_CUDA(cudaStreamSynchronize(c->stream));
+  return CONQUR_OK;
+}
+
 extern "C" int conqur_set_R(conqur_ctx* c, const float* R_dev) {
   if (!c || !R_dev) return CONQUR_ERR_INVALID_ARG;
   const Cfg& g = c->cfg;
@@ -736,12 +748,9 @@ extern "C" int conqur_set_R(conqur_ctx* c, const float* R_dev) {
       rc = tc_ns_residual(c->tc, c->stream, 0);
     }
     if (rc) return rc;
-    double* out = c->at<double>(c->L.obj_out);
-    check_reduce_kernel<<<1, 256, 0, c->stream>>>(c->state(), pf, pd, g.P > 1 ? g.P : ns_parts(c), out);
-    CQ_LAUNCHED(c, K_OTHER);
     double h[2];
-    CQ_CUDA(cudaMemcpyAsync(h, out, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
-    CQ_CUDA(cudaStreamSynchronize(c->stream));
+    rc = check_read(c, c->state(), g.P > 1 ? g.P : ns_parts(c), h);
+    if (rc) return rc;
     if (std::isfinite(h[1]) && std::fabs(h[0] - 1e-3) > bound) {
       if (h[0] > 1e-3) return CONQUR_ERR_NOT_ORTHOGONAL_INPUT;
       decided = true;
@@ -751,13 +760,11 @@ extern "C" int conqur_set_R(conqur_ctx* c, const float* R_dev) {
   if (!decided) {
     launch_ns_exact<EPI_RESIDUAL>(c, R_dev, R_dev, nullptr, nullptr);
     CQ_LAUNCHED(c, K_OTHER);
-    std::vector<float> pm((size_t)ns_exact_parts(c) * g.P);
-    CQ_CUDA(cudaMemcpyAsync(pm.data(), c->at<float>(c->L.part_f), sizeof(float) * pm.size(), cudaMemcpyDeviceToHost,
-                            c->stream));
-    CQ_CUDA(cudaStreamSynchronize(c->stream));
-    float mx = 0.f;
-    for (float v : pm) mx = (v == v) ? std::max(mx, v) : INFINITY;
-    if (!(mx <= 1e-3f)) return CONQUR_ERR_NOT_ORTHOGONAL_INPUT;
+    double h[2];
+    const int rc = check_read(c, nullptr, ns_exact_parts(c) * g.P, h);
+    if (rc) return rc;
+    // (the maximum drops NaN, the sum keeps it)
+    if (!((float)h[0] <= 1e-3f) || !std::isfinite(h[1])) return CONQUR_ERR_NOT_ORTHOGONAL_INPUT;
   }
   if (g.mode == CONQUR_TC_BF16 && aligned) return tc_take_R(c->tc, c->stream, R_dev);
   CQ_CUDA(cudaMemcpyAsync(c->at<float>(c->L.R), R_dev, sizeof(float) * dd * g.P, cudaMemcpyDeviceToDevice, c->stream));

@@ -216,3 +216,19 @@ def test_more_rows_than_a_launch_has_blocks_of_the_smaller_tiles(n, d):
     for a in (0, n // 2, n - 1000):                  # first, middle and last tiles
         want = x[a:a + 1000].double() @ r.double()
         assert ((out[a:a + 1000].double() - want).abs() <= d * 2.0 ** -24 * (x[a:a + 1000].abs() @ r.abs()).double() + 1e-30).all()
+
+
+@pytest.mark.parametrize("mode,d,P", [("exact", 33, 1), ("exact", 600, 1), ("exact", 48, 3), ("tc", 256, 1), ("tc", 640, 1), ("tc", 128, 2),
+                                      ("tc", 128, 200)])
+def test_set_R_refuses_nan(mode, d, P):
+    """A NaN reaches one row and one column of R^T R only; the rotation in place stays."""
+    q = torch.linalg.qr(_rand(d, P, d, d).double())[0].float().contiguous()
+    c = B.Context(d, 8, in_dtype="f32" if mode == "exact" else "bf16", mode=mode, batch=P)
+    c.set_R(q[0] if P == 1 else q)
+    for p, i, j in ((0, 0, 0), (P - 1, d - 1, 3), (P // 2, d // 2, d - 1)):
+        r = q.clone()
+        r[p, i, j] = float("nan")
+        with pytest.raises(B.ConqurError) as e:
+            c.set_R(r[0] if P == 1 else r)
+        assert e.value.status == -3
+        assert torch.equal(c.get_R(), q[0] if P == 1 else q)
