@@ -94,9 +94,10 @@ typedef struct {
                                the cross-covariance is accumulated with R fixed, so the grouping changes no result
                                beyond fp32 summation order).  Use the update cadence; the workspace grows by
                                4*d*n_max bytes per deferred batch.  0 or 1: every step runs its products at once */
-  float    ns_gram_single_pass_tau;  /* tensor-core mode tuning: a Gram product that may accept the rotation runs one
-                               pass instead of three while the iterate's mean squared singular value is below this
-                               (the others run one pass anyway); 0 = default */
+  float    ns_gram_single_pass_tau;  /* tensor-core mode tuning, single problem: Gram products between the steps run one
+                               pass over the iterate's fp16 copy while its mean squared singular value is below this
+                               and three passes over the bf16 pair from there on; 0 = one pass throughout.  A product
+                               that may accept the rotation always takes three */
   float    ns_lo_gap_budget;/* tensor-core mode tuning: bound on the Procrustes gap given up by dropping the low
                                bits of the iterate in the products of late steps (a worst-case bound: d directions at the
                                noise floor under one dominant one; measured gaps are 20-50x smaller); 0 = default 5e-4 */

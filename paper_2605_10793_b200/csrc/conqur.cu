@@ -379,13 +379,13 @@ int update_prologue(conqur_ctx* c) {
   const float isd = (float)(1.0 / std::sqrt((double)d));
   sumsq_kernel<<<dim3(nb, P), 256, 0, c->stream>>>(M, R, dd, st, 0, pd);
   CQ_LAUNCHED(c, K_OTHER);
-  ns_setup_kernel<<<P, 256, 0, c->stream>>>(st, pd, nb, 0, g.prior_rel, isd, g.margin, d, use_shift, c->n_lift_init);
+  ns_setup_kernel<<<P, 256, 0, c->stream>>>(st, pd, nb, 0, g.prior_rel, isd, g.margin, d, use_shift, c->tc.e1_tau, c->n_lift_init);
   CQ_LAUNCHED(c, K_OTHER);
   if (g.prior_rel > 0.f) {
     sumsq_kernel<<<dim3(nb, P), 256, 0, c->stream>>>(M, R, dd, st, 1, pd);
     CQ_LAUNCHED(c, K_OTHER);
   }
-  ns_setup_kernel<<<P, 256, 0, c->stream>>>(st, pd, nb, 1, g.prior_rel, isd, g.margin, d, use_shift, c->n_lift_init);
+  ns_setup_kernel<<<P, 256, 0, c->stream>>>(st, pd, nb, 1, g.prior_rel, isd, g.margin, d, use_shift, c->tc.e1_tau, c->n_lift_init);
   CQ_LAUNCHED(c, K_OTHER);
   if (g.simt_ns) {
     ns_x0_kernel<<<dim3(ew_blocks(dd), P), 256, 0, c->stream>>>(M, R, c->at<float>(c->L.Xa), dd, st);

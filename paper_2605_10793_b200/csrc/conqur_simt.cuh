@@ -781,7 +781,7 @@ __device__ __forceinline__ void ns_adapt_lift_plan(DevState* s, int n_endgame, i
 // phase 0: lam = prior_rel * ||M_raw||_F / sqrt(d)      (reads partials of sumsq over M)
 // phase 1: scale = ||M_raw + lam R||_F ; arms the iteration
 static __global__ void ns_setup_kernel(DevState* st, const double* __restrict__ partials, int nblocks, int phase,
-                                float prior_rel, float inv_sqrt_d, float margin, int d, int use_shift,
+                                float prior_rel, float inv_sqrt_d, float margin, int d, int use_shift, float e1_tau,
                                 int n_lift_init) {
   const int p = blockIdx.x;
   __shared__ double red[8];
@@ -804,7 +804,7 @@ static __global__ void ns_setup_kernel(DevState* st, const double* __restrict__ 
       s->seg_x = 2;
       // ||X_0||_F = 1/(1+margin): mean sigma^2 of the first iterate (the tensor-core mode shifts by it)
       s->tau = use_shift ? 1.0f / ((1.0f + margin) * (1.0f + margin) * (float)d) : 1.0f;
-      s->seg_e = use_shift ? 1 : 3;
+      s->seg_e = (use_shift && !(e1_tau > 0.f && s->tau >= e1_tau)) ? 1 : 3;
     }
   }
 }
@@ -968,7 +968,8 @@ static __global__ void ns_control_kernel(DevState* st, const float* __restrict__
 
 // tau of the next residual product = mean sigma^2 of the new iterate = ||X||_F^2 / d (tensor-core mode), and how
 // many passes that product takes: three over the bf16 pair when it may accept the rotation, i.e. once the last endgame
-// entry has been applied or no step is left; one over the fp16 copy otherwise (see tc_ns_residual).  One pass leaves about
+// entry has been applied or no step is left; one over the fp16 copy otherwise (see tc_ns_residual), except that a caller's
+// threshold (e1_tau > 0) asks for three wherever tau has reached it.  One pass leaves about
 // 0.8 2^-12 / sqrt(d) in an entry of G and the last endgame step hands that on to X^T X - I, so that step's G takes three
 // passes as well where the largest of d^2 such entries (4.5 times as much) would come near the tolerance (d <= 1240 at 1e-4:
 // at d = 512 every update spent a step more).
@@ -985,7 +986,7 @@ static __global__ void ns_tau_kernel(DevState* st, const double* __restrict__ pa
     const float left = 4.5f * 0.8f / 4096.f * rsqrtf((float)d);
     const int first_full = left <= 0.25f * tol ? n_sched : n_sched - 1;
     const bool may_accept = s->ns_idx >= first_full || s->ns_steps_used >= max_steps;
-    s->seg_e = (may_accept && s->tau >= e1_tau) ? 3 : 1;
+    s->seg_e = (may_accept || (e1_tau > 0.f && s->tau >= e1_tau)) ? 3 : 1;
   }
 }
 

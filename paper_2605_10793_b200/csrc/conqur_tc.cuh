@@ -1011,7 +1011,7 @@ struct TcHost {
   int d, P, quant_bits, num_sms;
   int device;                                // CUDA device the context was created on
   int pair_clusters;                         // CTA pairs that can be co-resident (0: single-CTA kernels only)
-  float e1_tau;                              // residual product runs one pass while mean sigma^2 of the iterate is below this, see ns_tau_kernel
+  float e1_tau;                              // > 0: residual products take three passes once mean sigma^2 of the iterate has reached this, see ns_tau_kernel
   int64_t n_max;
   char* ws;
   TcLayout L;
@@ -1284,7 +1284,7 @@ inline int tc_init(TcHost* h, char* ws, const TcLayout& L, int d, int P, int64_t
   h->num_sms = f.sms;
   h->device = dev;
   h->pair_clusters = single_cta ? 0 : f.pair_clusters;
-  h->e1_tau = gram_single_pass_tau > 0.f ? gram_single_pass_tau : 2e-3f;
+  h->e1_tau = gram_single_pass_tau;
   const uint64_t D = (uint64_t)d;
   int rc = 0;
   if (P > 1) {

@@ -321,3 +321,27 @@ def test_lifting_count_comes_down_again_after_a_hard_update():
     assert peak >= low + 3, (low, peak)
     plans = [run(easy)[0] for _ in range(24)]
     assert plans[-1] <= peak - 3 and all(b <= a for a, b in zip(plans, plans[1:])), (low, peak, plans)
+
+
+@pytest.mark.parametrize("d", [256, 2048])
+def test_gram_threshold_never_keeps_an_update_from_being_accepted(d):
+    """ns_gram_single_pass_tau from "three passes everywhere" to above any iterate's mean squared singular value (1)."""
+    from paper_2605_10793_b200 import binding as B
+    torch = _torch()
+    rng = np.random.default_rng(d)
+    m = rng.standard_normal((d, d)).astype(np.float32)
+    dev = torch.from_numpy(m).cuda()
+    u, _, vt = torch.linalg.svd(dev.double())
+    ref, rots = u @ vt, []
+    for tau in (0.0, 1e-30, 2e-3, 0.5, 1.5, 1e30):
+        ctx = B.Context(d=d, n_max=128, in_dtype="bf16", mode="tc", ns_gram_single_pass_tau=tau)
+        for _ in range(2):
+            ctx.set_M(dev, 1.0, d)
+            ctx.update()
+            st = ctx.get_stats()
+            assert st.status == 0 and st.orth_err <= T["orth"], (tau, st.status, st.ns_steps_used)
+        rots.append(ctx.get_R())
+        # a Gaussian matrix' smallest singular value is about 1/d of its largest: fp16 operands move R by a few 1e-3
+        assert float((rots[-1].double() - ref).norm() / ref.norm()) <= 2e-2, tau
+    assert torch.equal(rots[0], rots[-1])            # 0: no threshold
+    assert not torch.equal(rots[0], rots[1])         # ... and a small one is heeded
