@@ -427,7 +427,7 @@ int update_step(conqur_ctx* c, int k, int cur, bool last) {
     CQ_LAUNCHED(c, K_NS_NEXT);
     return CONQUR_OK;
   }
-  return tc_ns_poly_next(c->tc, c->stream, cur, c->n_sched, g.ns_max_steps, g.orth_tol);
+  return tc_ns_poly_next(c->tc, c->stream, cur, c->n_sched, g.ns_max_steps);
 }
 
 int update_epilogue(conqur_ctx* c) {

@@ -967,14 +967,13 @@ static __global__ void ns_control_kernel(DevState* st, const float* __restrict__
 }
 
 // tau of the next residual product = mean sigma^2 of the new iterate = ||X||_F^2 / d (tensor-core mode), and how
-// many passes that product takes: three over the bf16 pair when it may accept the rotation, i.e. once the last endgame
-// entry has been applied or no step is left; one over the fp16 copy otherwise (see tc_ns_residual), except that a caller's
-// threshold (e1_tau > 0) asks for three wherever tau has reached it.  One pass leaves about
-// 0.8 2^-12 / sqrt(d) in an entry of G and the last endgame step hands that on to X^T X - I, so that step's G takes three
-// passes as well where the largest of d^2 such entries (4.5 times as much) would come near the tolerance (d <= 1240 at 1e-4:
-// at d = 512 every update spent a step more).
+// many passes that product takes.  Three over the bf16 pair when it may accept the rotation, i.e. once the last endgame
+// entry has been applied or no step is left, and for the step that applies that entry: it hands the rounding of its G on
+// to X^T X - I.  One over the fp16 copy otherwise (see tc_ns_residual), except that a caller's threshold (e1_tau > 0) asks
+// for three wherever tau has reached it.  (max|X^T X - I| of accepted rotations, d = 1280 .. 4096: 4e-5 .. 9e-5 with one
+// pass in that last step, 6e-6 .. 1e-5 with three; at d = 512 one pass cost every update a step more.)
 static __global__ void ns_tau_kernel(DevState* st, const double* __restrict__ part_x2, int nparts, int d, float e1_tau,
-                                     int n_sched, int max_steps, float tol) {
+                                     int n_sched, int max_steps) {
   DevState* s = st + blockIdx.x;
   if (s->ns_done) return;
   __shared__ double redd[8];
@@ -983,10 +982,8 @@ static __global__ void ns_tau_kernel(DevState* st, const double* __restrict__ pa
   const double tot = block_sum_d<256>(v, redd);
   if (threadIdx.x == 0) {
     s->tau = (float)(tot / (double)d);
-    const float left = 4.5f * 0.8f / 4096.f * rsqrtf((float)d);
-    const int first_full = left <= 0.25f * tol ? n_sched : n_sched - 1;
-    const bool may_accept = s->ns_idx >= first_full || s->ns_steps_used >= max_steps;
-    s->seg_e = (may_accept || (e1_tau > 0.f && s->tau >= e1_tau)) ? 3 : 1;
+    const bool full = s->ns_idx >= n_sched - 1 || s->ns_steps_used >= max_steps;
+    s->seg_e = (full || (e1_tau > 0.f && s->tau >= e1_tau)) ? 3 : 1;
   }
 }
 

@@ -1452,7 +1452,7 @@ inline int tc_ns_residual(TcHost& h, cudaStream_t s, int buf) {
 // B = beta2 E E + beta1 E - kappa I (one fp16 pass, symmetric tiles only) ;  X_next = X B + (gamma + kappa) X.  The iterate
 // enters the last product as the bf16 pair hi + lo while small singular values are still being lifted (B is then stored in
 // bf16, as an instruction's operands have one type), after that as its fp16 copy in one pass (B in scaled fp16).
-inline int tc_ns_poly_next(TcHost& h, cudaStream_t s, int cur, int n_sched, int max_steps, float tol) {
+inline int tc_ns_poly_next(TcHost& h, cudaStream_t s, int cur, int n_sched, int max_steps) {
   const int d = h.d;
   const long long dd = (long long)d * d;
   TcGemmArgs g = tc_args(h, d, d, d);
@@ -1470,7 +1470,7 @@ inline int tc_ns_poly_next(TcHost& h, cudaStream_t s, int cur, int n_sched, int 
   x.part_t = h.part_d + tc_ns_parts(h);
   rc = tc_launch_n<false, true, TC_EPI_NEXT>(h, s, h.tmXh_k[cur], h.tmBh_mn, x);
   if (rc) return rc;
-  ns_tau_kernel<<<1, 256, 0, s>>>(h.st, h.part_d + tc_ns_parts(h), tc_ns_next_parts(h), d, h.e1_tau, n_sched, max_steps, tol);
+  ns_tau_kernel<<<1, 256, 0, s>>>(h.st, h.part_d + tc_ns_parts(h), tc_ns_next_parts(h), d, h.e1_tau, n_sched, max_steps);
   if (h.prof) h.prof->count(K_OTHER);
   return cudaGetLastError() == cudaSuccess ? CONQUR_OK : CONQUR_ERR_CUDA;
 }

@@ -345,3 +345,31 @@ def test_gram_threshold_never_keeps_an_update_from_being_accepted(d):
         assert float((rots[-1].double() - ref).norm() / ref.norm()) <= 2e-2, tau
     assert torch.equal(rots[0], rots[-1])            # 0: no threshold
     assert not torch.equal(rots[0], rots[1])         # ... and a small one is heeded
+
+
+@pytest.mark.parametrize("d", [512, 1280, 2048, 3072])
+@pytest.mark.parametrize("spectrum", ["lin", "log1e4", "spiky1e8"])
+def test_accepted_rotations_are_orthogonal_to_the_precision_of_the_bf16_pair(d, spectrum):
+    """Widths on both sides of those where one pass would do for the tolerance, tails down to 1e-8 of the largest."""
+    from paper_2605_10793_b200 import binding as B
+    torch = _torch()
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d)
+    u, v = (torch.linalg.qr(torch.randn(d, d, generator=g, device="cuda", dtype=torch.float64))[0] for _ in range(2))
+    s = {"lin": np.linspace(1.0, 0.3, d), "log1e4": np.logspace(0, -4, d),
+         "spiky1e8": np.concatenate([np.ones(8), np.logspace(-3, -8, d - 8)])}[spectrum]
+    m = ((u * torch.from_numpy(s).cuda()) @ v.T).float()
+    ctx = B.Context(d=d, n_max=128, in_dtype="bf16", mode="tc")
+    errs = []
+    for _ in range(3):
+        ctx.set_M(m, 1.0, d)
+        ctx.update()
+        st = ctx.get_stats()
+        r = ctx.get_R().double()
+        errs.append(float((r.T @ r - torch.eye(d, device="cuda")).abs().max()))
+        assert st.status == 0 and errs[-1] <= T["orth"], (st.status, errs, st.ns_steps_used)
+        assert 1.0 - float((r * m.double()).sum()) / s.sum() <= T["gap"], errs
+    # Three passes leave lo * lo out of the last step's G, and the new iterate is rounded to its pair: 2^-18 of columns of
+    # norm 1 each, the scaled fp16 operands (E is below 0.01 there) less; 2.5e-5 is 6.5 x 2^-18.  An update may also stop a
+    # step early, just below the tolerance, which is its right: the middle one of three is looked at.
+    assert sorted(errs)[1] <= 2.5e-5, errs
