@@ -730,13 +730,19 @@ extern "C" int conqur_set_R(conqur_ctx* c, const float* R_dev) {
   CQ_LAUNCHED(c, K_OTHER);
   bool decided = false;
   const bool aligned = (reinterpret_cast<uintptr_t>(R_dev) & 15) == 0;
-  if (g.mode == CONQUR_TC_BF16 && aligned && (g.P > 1 || g.d >= 512)) {
-    // The decision max|R^T R - I| <= 1e-3 on the tensor cores first: the three-pass product of R's bf16 pair, whose
-    // entries are off by at most 2 2^-17 (the split) + (3 d / 16) 2^-23 (the accumulation) times the columns' norms, which
-    // are 1 within 1e-3 wherever a decision is close.  Only a result within that bound of the limit, or one that is not
-    // finite, goes on to the fp32 product below, so what is accepted and what is refused does not change
-    // (whole call at d = 4096: 1650 -> 213 us, 3072: 865 -> 154, 1024: 111 -> 66; at 256 the extra launches cost 7 us).
-    const double bound = 2.0e-5 + 2.5e-8 * g.d;
+  // The decision max|R^T R - I| <= 1e-3 on the tensor cores first, by the three-pass product of R's bf16 pair.  How far an
+  // entry of it can lie from the fp32 product's below, for columns of norm 1 within 1e-3 (wherever a decision is close):
+  //   the split       2 2^-17  (lo * lo and what the pair leaves out: 3 2^-18)
+  //   tensor cores    3 d / 16 instructions, each of which drops up to 2^-25 of each of its 16 products (they are aligned to
+  //                   the sum and cut two bits below it, as a sum of one large and many small terms shows) and 2^-23 of
+  //                   the sum: 5 2^-23
+  //   fp32 product    d roundings of 2^-24
+  // Only a result within that bound of the limit, or one that is not finite, goes on to the fp32 product, so what is accepted
+  // and what is refused does not change.  Widths whose bound leaves no room for what an update returns (1e-4) go there
+  // straight away (whole call at d = 4096: 1650 -> 213 us, 3072: 865 -> 154, 1024: 111 -> 66; at 256 the extra launches
+  // cost 7 us).
+  const double bound = 2.0e-5 + 1.72e-7 * g.d;
+  if (g.mode == CONQUR_TC_BF16 && aligned && (g.P > 1 || g.d >= 512) && bound <= 8.5e-4) {
     float* pf = c->at<float>(c->L.part_f);
     double* pd = c->at<double>(c->L.part_d);
     int rc;

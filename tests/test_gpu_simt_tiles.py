@@ -232,3 +232,31 @@ def test_set_R_refuses_nan(mode, d, P):
             c.set_R(r[0] if P == 1 else r)
         assert e.value.status == -3
         assert torch.equal(c.get_R(), q[0] if P == 1 else q)
+
+
+@pytest.mark.parametrize("d", [512, 1024, 2048, 4096, 8192])
+def test_set_R_decides_alike_where_every_term_is_rounded_the_same_way(d):
+    """One column of a large entry and small ones whose squares lie just above half a unit of its sum in fp32: the fp32
+    product adds a whole unit for each, the tensor cores half of one."""
+    tc = B.Context(d, 8, mode="tc")
+    ex = B.Context(d, 8, in_dtype="f32", mode="exact")
+    eps = 2.0 ** -12 * (1.0 + 2.0 ** -10)
+    r = torch.eye(d, device="cuda")
+    r[1:, 0] = eps
+    fp32 = (d - 1) * 2.0 ** -23
+    seen = set()
+    for delta in np.linspace(0.0, 1.1e-3, 45):
+        r[0, 0] = (1.0 + delta) ** 0.5
+        got = []
+        for c in (tc, ex):
+            try:
+                c.set_R(r)
+                got.append(True)
+            except B.ConqurError as e:
+                assert e.status == -3
+                got.append(False)
+        assert got[0] == got[1], (delta, got)
+        if abs(delta + fp32 - 1e-3) > 1e-6:              # (the entry's own rounding)
+            assert got[1] == (delta + fp32 < 1e-3), delta
+        seen.add(got[0])
+    assert seen == {True, False}
