@@ -841,8 +841,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 // MMA will see) and a bf16 copy of the row in the workspace; skipped rows are written as zeros so that they
 // cannot reach the accumulators.  A warp's share of a row (up to 4096 elements) sits in its registers as packed bf16, all
 // 16-byte loads in flight at once, so a row is read from memory once: bound by memory (4093 x 8192 bf16: 65 -> 28 us
-// against two passes over rows longer than 4096).  Rows that do not start on 16-byte boundaries take two passes of
-// narrow loads.
+// against two passes over rows longer than 4096).  Rows that do not start on 16-byte boundaries take two passes, four
+// elements a lane (one 8-byte load where a bf16 row starts on such a boundary) and 8-byte stores.
 template <typename TIn, int W>
 __global__ void __launch_bounds__(256) rownorm_stage_kernel(const TIn* __restrict__ X, int64_t n, int d, int64_t ld,
                                                             float* __restrict__ rnorm,
@@ -856,7 +856,16 @@ __global__ void __launch_bounds__(256) rownorm_stage_kernel(const TIn* __restric
   const int k0 = (warp % W) * slice, k1 = min(d, k0 + slice);           // this warp's columns
   const TIn* x = X + (live ? row : 0) * ld;
   __nv_bfloat16* dst = Xs + row * (int64_t)d;
-  const bool vec = (reinterpret_cast<uintptr_t>(x) & 15) == 0;          // (d and the slices are multiples of 8)
+  const bool vec = (reinterpret_cast<uintptr_t>(x) & 15) == 0;          // (d and the slices are multiples of 128)
+  const bool vec4 = (reinterpret_cast<uintptr_t>(x) & (sizeof(TIn) * 4 - 1)) == 0;
+  auto load4 = [&](const TIn* src, float (&v)[4]) {
+    if (vec4) {
+      ld4_as_float(src, v);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] = ld_as_float(src + j);
+    }
+  };
   uint4 buf[16];
   float ss = 0.f;
   if (live && vec) {
@@ -885,9 +894,11 @@ __global__ void __launch_bounds__(256) rownorm_stage_kernel(const TIn* __restric
     }
     ss = (s4[0] + s4[1]) + (s4[2] + s4[3]);
   } else if (live) {
-    for (int k = k0 + lane; k < k1; k += 32) {
-      const float v = bf16_round(ld_as_float(x + k));                   // (bf16 values are exact already)
-      ss = fmaf(v, v, ss);
+    for (int k = k0 + lane * 4; k < k1; k += 128) {
+      float v[4];
+      load4(x + k, v);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) { const float t = bf16_round(v[j]); ss = fmaf(t, t, ss); }      // (bf16 values are exact already)
     }
   }
   ss = warp_sum(ss);
@@ -907,7 +918,11 @@ __global__ void __launch_bounds__(256) rownorm_stage_kernel(const TIn* __restric
       if (k < k1) *reinterpret_cast<uint4*>(dst + k) = good ? buf[c] : make_uint4(0u, 0u, 0u, 0u);
     }
   } else {
-    for (int k = k0 + lane; k < k1; k += 32) dst[k] = __float2bfloat16(good ? ld_as_float(x + k) : 0.f);
+    for (int k = k0 + lane * 4; k < k1; k += 128) {
+      float v[4] = {0.f, 0.f, 0.f, 0.f};
+      if (good) load4(x + k, v);
+      *reinterpret_cast<uint2*>(dst + k) = make_uint2(bf16x2_pack(v[0], v[1]), bf16x2_pack(v[2], v[3]));
+    }
   }
   if (lane == 0 && warp % W == 0) {
     if (!good) {

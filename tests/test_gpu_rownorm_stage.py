@@ -42,3 +42,28 @@ def test_rows_that_take_no_part_and_alignment(d, dtype, offset):
     assert ((m - ref).abs() <= (2.0 ** -8 + n * 2.0 ** -23) * slack + 1e-9).all()
     jr = float((xb.abs().sum(dim=1) * rn).sum()) / d ** 0.5
     assert abs(j - jr) <= 1e-5 * jr                    # fp32 sums of squares and of d magnitudes
+
+
+@pytest.mark.parametrize("d", [128, 2176, 4224, 8192])
+@pytest.mark.parametrize("dtype,offset,pad", [("bf16", 0, 4), ("bf16", 4, 8), ("bf16", 2, 8), ("bf16", 1, 1), ("f32", 1, 4), ("f32", 2, 3)])
+def test_rows_off_16_byte_boundaries_match_the_same_rows_on_them(d, dtype, offset, pad):
+    """Some rows on 16-byte boundaries and some not (odd paddings), all of them or none: copied and normed alike."""
+    n = 37
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d + 10 * offset + pad)
+    tt = torch.float32 if dtype == "f32" else torch.bfloat16
+    wide = torch.randn(n, d + pad, generator=g, device="cuda").to(tt)
+    x = torch.as_strided(wide, (n, d), (d + pad, 1), min(offset, pad))
+    x[5] = 0.0
+    out = []
+    for rows in (x, x.contiguous()):
+        c = B.Context(d, n, in_dtype=dtype, mode="tc", prior_rel=0.01)
+        c.step(rows)
+        out.append((c.get_M().double(), c.get_objective(), c.debug_get_signs(n)))
+    (ma, (ja, na), sa), (mb, (jb, nb), sb) = out
+    assert na == nb == n - 1 and torch.equal(sa, sb)
+    xd = x.to(torch.bfloat16).double()
+    rn = torch.where(xd.abs().sum(dim=1) > 0, 1.0 / xd.norm(dim=1).clamp_min(1e-30), torch.zeros((), dtype=torch.float64, device="cuda"))
+    # sums of squares in another order: a scale may round to the next bf16 (2^-7 at most)
+    assert ((ma - mb).abs() <= 2.0 ** -7 * (xd.abs().T @ (rn[:, None] * (xd != 0).double())) / d ** 0.5 + 1e-9).all()
+    assert abs(ja - jb) <= 1e-6 * jb
