@@ -424,11 +424,11 @@ int conqur_fold_weight(const float* W_dev, int64_t ldw, int32_t rows, int32_t co
  * Enqueued on the stream; not synchronised.  Invalid arguments return CONQUR_ERR_INVALID_ARG and do nothing.
  * Arithmetic: fp32 throughout, error per element <= log2(d) 2^-24 ||x||_2 (plus the rounding of a bf16 output).
  *   - bf16 rows lying back to back (ldx == ldy == d, 16-byte aligned pointers, n*d a multiple of 128), or of d >= 128
- *     elements that start on 16-byte boundaries on both sides: H_d is
+ *     elements with bf16 results that start on 16-byte boundaries on both sides: H_d is
  *     taken as H_{d/128} (x) H_128; the 128-point transforms of all 128-element chunks run as one tensor-core
  *     product per tile with exact operands (the bf16 input and a +-1 matrix, fp32 accumulation), the remaining
  *     log2(d/128) butterfly levels in registers.  No d x d matrix is formed.
- *   - every other layout (fp32 input, unaligned or short strided rows): log2(d) butterfly levels on the CUDA cores; rows
+ *   - every other layout (fp32 input, unaligned or short strided rows, strided rows with fp32 results): log2(d) butterfly levels on the CUDA cores; rows
  *     that start on 16-byte boundaries are staged through shared memory by bulk asynchronous copies, others by
  *     plain loads.
  *

@@ -245,13 +245,15 @@ inline int hadamard_make_tmap(CUtensorMap* tm, const void* X, uint64_t chunks, u
   return CONQUR_OK;
 }
 
-// Whether the tensor-core kernel takes these rows.  Back to back, 16-byte aligned, n d a multiple of 128; or d >= 128 and
-// rows that start on 16-byte boundaries on both sides (32768 x 4096 bf16 with 8 elements between rows: 168 us on the CUDA
-// cores, 126 here; 8192-element rows to fp32 199 -> 169; d = 128 184 -> 181).
+// Whether the tensor-core kernel takes these rows.  Back to back, 16-byte aligned, n d a multiple of 128; or d >= 128, bf16
+// results and rows that start on 16-byte boundaries on both sides (32768 x 4096 bf16 with 8 elements between rows: 168 us on
+// the CUDA cores, 126 here; d = 128 184 -> 181).  There the rounding of the results covers what the tensor cores' sums
+// drop (the error against 64 bits is the same to ten digits); fp32 results would be up to a fifth further off (d = 256:
+// 0.99e-8 on the CUDA cores, 1.18e-8 here), so strided rows with fp32 results stay on the CUDA cores.
 inline bool hadamard_tc_takes(const void* X, int64_t ldx, const void* Y, int64_t ldy, size_t out_size, int64_t n, int d) {
   if ((reinterpret_cast<uintptr_t>(X) & 15) || (reinterpret_cast<uintptr_t>(Y) & 15)) return false;
   if (ldx == d && ldy == d) return (n * d) % 128 == 0;
-  return d >= 128 && (ldx * 2) % 16 == 0 && ((size_t)ldy * out_size) % 16 == 0 && ldx < (1ll << 38) && n <= 0x7fffffffll;
+  return d >= 128 && out_size == 2 && (ldx * 2) % 16 == 0 && (ldy * 2) % 16 == 0 && ldx < (1ll << 38) && n <= 0x7fffffffll;
 }
 
 template <typename TOut>
@@ -261,12 +263,15 @@ inline int hadamard_tc_launch(const __nv_bfloat16* X, int64_t ldx, TOut* Y, int6
   TcDevFacts f;
   if (tc_device_facts(dev, &f) != CONQUR_OK) return CONQUR_ERR_CUDA;
   if (f.major != 10) return CONQUR_ERR_UNSUPPORTED;
+  constexpr bool STRIDED = sizeof(TOut) == 2;                   // see hadamard_tc_takes
   static std::atomic<unsigned long long> attr_dev_mask{0};      // the attributes are per device
   const unsigned long long dev_bit = 1ull << (dev & 63);
   if (!(attr_dev_mask.load(std::memory_order_acquire) & dev_bit)) {
-    if (cudaFuncSetAttribute(hadamard_tc_kernel<TOut, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, HTC_SMEM_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(hadamard_tc_kernel<TOut, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, HTC_SMEM_BYTES) != cudaSuccess)
+    if (cudaFuncSetAttribute(hadamard_tc_kernel<TOut, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, HTC_SMEM_BYTES) != cudaSuccess)
       return CONQUR_ERR_CUDA;
+    if constexpr (STRIDED)
+      if (cudaFuncSetAttribute(hadamard_tc_kernel<TOut, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, HTC_SMEM_BYTES) != cudaSuccess)
+        return CONQUR_ERR_CUDA;
     attr_dev_mask.fetch_or(dev_bit, std::memory_order_release);
   }
   const long long NC = (long long)n * (1ll << logd) / 128;
@@ -280,8 +285,14 @@ inline int hadamard_tc_launch(const __nv_bfloat16* X, int64_t ldx, TOut* Y, int6
   const long long tiles = (NC + HTC_N - 1) / HTC_N;
   const int grid = (int)(tiles < f.sms ? tiles : f.sms);
   const float scale = (float)(1.0 / sqrt((double)(1 << logd)));
-  if (flat) hadamard_tc_kernel<TOut, true><<<grid, HTC_THREADS, HTC_SMEM_BYTES, s>>>(tm, Y, NC, logd, scale, lr, (long long)ldy);
-  else hadamard_tc_kernel<TOut, false><<<grid, HTC_THREADS, HTC_SMEM_BYTES, s>>>(tm, Y, NC, logd, scale, lr, (long long)ldy);
+  if constexpr (STRIDED) {
+    if (!flat) {
+      hadamard_tc_kernel<TOut, false><<<grid, HTC_THREADS, HTC_SMEM_BYTES, s>>>(tm, Y, NC, logd, scale, lr, (long long)ldy);
+      return cudaGetLastError() == cudaSuccess ? CONQUR_OK : CONQUR_ERR_CUDA;
+    }
+  }
+  if (!flat) return CONQUR_ERR_UNSUPPORTED;
+  hadamard_tc_kernel<TOut, true><<<grid, HTC_THREADS, HTC_SMEM_BYTES, s>>>(tm, Y, NC, logd, scale, lr, (long long)ldy);
   return cudaGetLastError() == cudaSuccess ? CONQUR_OK : CONQUR_ERR_CUDA;
 }
 

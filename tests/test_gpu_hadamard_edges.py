@@ -53,3 +53,16 @@ def test_strided_rows_agree_with_the_cuda_core_kernel(d, n, padx, pady, out):
         y[:, :d] = x
         B.conqur_hadamard_rows(y[:, :d], out=y[:, :d])
         assert torch.equal(y[:, :d], bufs[0][:, :d]) and (y[:, d:] == 7.0).all()
+
+
+@pytest.mark.parametrize("d,n", [(128, 300), (256, 129), (1024, 65), (8192, 20)])
+def test_strided_fp32_results_keep_the_cuda_cores_rounding(d, n):
+    """fp32 results show what the tensor cores' sums drop: rows inside wider buffers have theirs from fp32 additions."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d + n)
+    x = torch.randn(n, d + 8, generator=g, device="cuda").to(torch.bfloat16)[:, :d]
+    a, b = (torch.full((n, d + 8), 7.0, device="cuda") for _ in range(2))
+    B.conqur_hadamard_rows(x, out=a[:, :d])
+    B.conqur_hadamard_rows(x, out=b[:, :d], cuda_cores_only=True)
+    assert B.conqur_hadamard_status() == 0
+    assert torch.equal(a, b)
