@@ -445,8 +445,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const CUtensorMap* const mapA = one16 ? &tmF : &tmA;
   const CUtensorMap* const mapB = (one16 && EPI == TC_EPI_RESID) ? &tmF : &tmB;
   // operand tiles the passes in use need; the shared memory holds as many stages of them as fit
+  // (known when the kernel is compiled where there is one of each: the steps' two products)
   int na = 1, nb = 1;
-  if (PAIR) {
+  if (PAIR && NA * NB > 1) {
     for (int sg = 0; sg < nseg; ++sg) { na = max(na, g.a_tile[sg] + 1); nb = max(nb, g.b_tile[sg] + 1); }
     na = min(na, NA); nb = min(nb, NB);
   }
