@@ -246,8 +246,8 @@ inline int hadamard_make_tmap(CUtensorMap* tm, const void* X, uint64_t chunks, u
 }
 
 // Whether the tensor-core kernel takes these rows.  Back to back, 16-byte aligned, n d a multiple of 128; or d >= 128, bf16
-// results and rows that start on 16-byte boundaries on both sides (32768 x 4096 bf16 with 8 elements between rows: 168 us on
-// the CUDA cores, 126 here; d = 128 184 -> 181).  There the rounding of the results covers what the tensor cores' sums
+// results and rows that start on 16-byte boundaries on both sides (32768 x 4096 bf16 with 8 elements between rows: 177 us on
+// the CUDA cores, 102 here; d = 128 194 -> 148).  There the rounding of the results covers what the tensor cores' sums
 // drop (the error against 64 bits is the same to ten digits); fp32 results would be up to a fifth further off (d = 256:
 // 0.99e-8 on the CUDA cores, 1.18e-8 here), so strided rows with fp32 results stay on the CUDA cores.
 inline bool hadamard_tc_takes(const void* X, int64_t ldx, const void* Y, int64_t ldy, size_t out_size, int64_t n, int d) {
