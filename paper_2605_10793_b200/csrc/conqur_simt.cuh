@@ -179,7 +179,8 @@ using SgSmall = SgTile<32, 32, 4, 4, 32, 8>;
 enum { SG_LARGE = 0, SG_HALF = 1, SG_SMALL = 2 };
 // Rounds of tiles per SM times the tile's time (its area over the rate the tile reaches when the chip is full: 1, 0.98 and
 // 0.65 of the large tile's, measured).  max_tiles: most tiles the caller's per-tile partials have room for.  sym: only
-// the tiles that touch the upper triangle of the (square) output are computed.
+// the tiles that touch the upper triangle of the (square) output are computed.  sms: a B200's, the only part the library is
+// built for; no result depends on the choice.
 inline int sg_pick(int64_t M, int64_t N, int64_t problems, int64_t max_tiles = INT64_MAX, bool sym = false, int sms = 148) {
   auto cdv = [](int64_t a, int64_t b) { return (a + b - 1) / b; };
   const int64_t nl = cdv(M, 128) * cdv(N, 128), nh = cdv(M, 64) * cdv(N, 128), ns = cdv(M, 32) * cdv(N, 32);

@@ -1,9 +1,10 @@
-// Tensor-core mode for many small problems (the per-head case, d = 128): one fused kernel per streamed batch.
+// Tensor-core mode for many small problems (the per-head case, d = 128): one fused kernel per streamed batch,
+// tcb_step_kernel with fake-quantisation and tcb_step_plain_kernel (further down) without, and one per update.
 //
-// A CTA owns one problem at a time and walks its tokens in tiles of 128 rows.  Per tile
+// tcb_step_kernel: a CTA owns one problem at a time and walks its tokens in tiles of 128 rows.  Per tile
 //   TMA            X tile (128 tokens x 128, bf16)              -> shared memory (read ONCE from HBM)
 //   tcgen05.mma    Y = X_tile R                                 -> TMEM          (R: bf16, resident in shared memory)
-//   epilogue       the rows' scales from a pass over Y (||x R~||, see the kernel), sign / fake-quant of Y,
+//   epilogue       the rows' scales and ranges from a pass over Y (||x R~||, see the kernel), fake-quantised Y,
 //                  C' = sgn(.) * scale as bf16                   -> shared memory
 //   tcgen05.mma    M += X_tile^T C'                              -> TMEM accumulator that lives for the whole problem
 // and after the last tile the accumulator is added to the problem's fp32 M in global memory.  The X tile in
@@ -16,11 +17,12 @@
 // product.  The two products have their own issuing threads and Y has three TMEM buffers, so the first product runs
 // up to three tiles ahead of the epilogue.  Shared-memory bandwidth sets the floor of a tile: both products read
 // both operands from it (4 x 32 KB), TMA writes 32 KB and the targets 32 KB.  Every wait is bounded.
+// At the end of a problem the accumulator leaves through the copy engine (tensor reduce-add into M), handed over by
+// one of the epilogue groups while the other goes on with the next problem.
 //
 // Objective without fake-quantisation: sum_i ||y_i||_1 rnorm_i = <R, X_tilde^T S> = <R, M> while R is fixed (Section
-// 3.2 with Eq. 2), so this kernel does not sum it: the update kernel forms it from M, and so does a read in between.
-// At the end of a problem the accumulator leaves through the copy engine (tensor reduce-add into M), handed over by
-// the epilogue group that owned the last tile while the other group goes on with the next problem.
+// 3.2 with Eq. 2), so tcb_step_plain_kernel does not sum it: the update kernel forms it from M, and so does a read in
+// between.
 #pragma once
 #include <type_traits>
 
@@ -67,11 +69,11 @@ struct TcbStepArgs {
   int p0;                     // its index in the context (row block of the rotation map)
   int xp_outer_tokens;        // 1: the input map's dimensions are (column, problem, token) -- head-interleaved rows --
                               //    instead of (column, token, problem)
-  QuantSpec qs;               // bits == 0: corner target of the rotated row; else per-token fake-quantisation first
+  QuantSpec qs;               // tcb_step_kernel: the per-token fake-quantisation
   float* M;                   // P x 128 x 128 fp32 (without the 1/sqrt(d))
   int S;                      // token splits per problem: work item i = (problem i / S, tiles [T (i % S) / S, T (i % S + 1) / S))
   float* Mpart;               // S > 1: P * S partial cross-covariances (item order), summed into M by tcb_finish_kernel
-  double* part_d;             // fake-quantisation only: P * S * TCB_PARTS objective partials (one per epilogue warp), item order
+  double* part_d;             // tcb_step_kernel: P * S * TCB_PARTS objective partials (one per epilogue warp), item order
   DevState* st;               // P
   long long* trace;           // measurement hook: when set, CTA 0 records SM-clock timestamps of its first TCB_TRACE_TILES tiles
   int8_t* signs;              // test hook: when set, the sign decisions (-1/0/+1) of this call, (P * n) x 128 row-major
@@ -315,7 +317,7 @@ tcb_step_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         // product uses.  It differs from ||x|| by at most ||R~ R~^T - I||_2 / 2 (about 1e-4 for a typical row at
         // d = 128), an order below the rounding of the scale itself to bf16 in the target tile, and costs no pass
         // over the input tile in shared memory, whose bandwidth bounds this kernel.  Every warp reads the whole
-        // row (both warps of a row pair get the same sum); with fake-quantisation the same pass finds the row's range.
+        // row (both warps of a row pair get the same sum); the same pass finds the row's range.
         if (tr_epi) TCB_TR(it, TCB_EV_NORM_BEGIN);
         float ss;
         float vmax = -3.0e38f, vmin = 3.0e38f;
@@ -330,10 +332,8 @@ tcb_step_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
               s0 = fmaf(v[i], v[i], s0); s1 = fmaf(v[i + 1], v[i + 1], s1);
               s2 = fmaf(v[i + 2], v[i + 2], s2); s3 = fmaf(v[i + 3], v[i + 3], s3);
             }
-            if (g.qs.bits > 0) {
 #pragma unroll
-              for (int i = 0; i < 32; ++i) { vmax = fmaxf(vmax, v[i]); vmin = fminf(vmin, v[i]); }
-            }
+            for (int i = 0; i < 32; ++i) { vmax = fmaxf(vmax, v[i]); vmin = fminf(vmin, v[i]); }
           }
           ss = (s0 + s1) + (s2 + s3);
         }
@@ -351,12 +351,11 @@ tcb_step_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         const float rn = good ? 1.0f / sqrtf(ss) : 0.f;
         const uint32_t rn_bits = bf16_bits(rn);
         if (tr_epi) TCB_TR(it, TCB_EV_EPI_NORMS);
-        RowQuant rq{0.f, 0.f, 0.f, 0.f};
-        if (g.qs.bits > 0) rq = row_quant(g.qs, vmax, vmin, good);
+        const RowQuant rq = row_quant(g.qs, vmax, vmin, good);
         // the target buffer is needed only now (the second product of the tile two back has read it)
         if (!tc_wait(&aux->cfree[cb], par2 ^ 1u, abort_flag)) { ok = false; timeout_site = 31; break; }
         if (tr_epi) TCB_TR(it, TCB_EV_EPI_CFREE);
-        const bool live = (g.qs.bits == 0) ? good : (rq.inv > 0.f);
+        const bool live = rq.inv > 0.f;
         float acc_t = 0.f;
 #pragma unroll 1
         for (int cc = 0; cc < 2; ++cc) {
@@ -365,27 +364,14 @@ tcb_step_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
           ptx::tmem_ld32(t_addr + (uint32_t)(c * 32), v);
           if (tr_epi) TCB_TR(it, cc == 0 ? TCB_EV_EPI_LD0 : TCB_EV_EPI_LD1);
           uint32_t w[16];
-          if (g.qs.bits > 0) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const float a = fminf(fmaxf(rintf(v[2 * i] * rq.inv), rq.klo), rq.khi);
-              const float b = fminf(fmaxf(rintf(v[2 * i + 1] * rq.inv), rq.klo), rq.khi);
-              acc_t += fabsf(a) + fabsf(b);
-              const uint32_t lo = (a == 0.f) ? 0u : (rn_bits | ((__float_as_uint(a) >> 16) & 0x8000u));
-              const uint32_t hi = (b == 0.f) ? 0u : (rn_bits | ((__float_as_uint(b) >> 16) & 0x8000u));
-              w[i] = live ? (lo | (hi << 16)) : 0u;
-            }
-          } else {
-            // two elements per instruction: the sign bits and a non-zero mask (0xffff per half that is not +-0) of the
-            // packed bf16 pair; the objective comes from the accumulator at the end of the problem
-            const uint32_t rn2 = live ? (rn_bits | (rn_bits << 16)) : 0u;
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const uint32_t pk = bf16x2_pack(v[2 * i], v[2 * i + 1]);
-              uint32_t nz;
-              asm("set.neu.u32.bf16x2 %0, %1, %2;" : "=r"(nz) : "r"(pk), "r"(0u));
-              w[i] = (rn2 | (pk & 0x80008000u)) & nz;
-            }
+          for (int i = 0; i < 16; ++i) {
+            const float a = fminf(fmaxf(rintf(v[2 * i] * rq.inv), rq.klo), rq.khi);
+            const float b = fminf(fmaxf(rintf(v[2 * i + 1] * rq.inv), rq.klo), rq.khi);
+            acc_t += fabsf(a) + fabsf(b);
+            const uint32_t lo = (a == 0.f) ? 0u : (rn_bits | ((__float_as_uint(a) >> 16) & 0x8000u));
+            const uint32_t hi = (b == 0.f) ? 0u : (rn_bits | ((__float_as_uint(b) >> 16) & 0x8000u));
+            w[i] = live ? (lo | (hi << 16)) : 0u;
           }
 #pragma unroll
           for (int k = 0; k < 4; ++k)
@@ -411,7 +397,7 @@ tcb_step_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
           }
           if (tr_epi && cc == 0) TCB_TR(it, TCB_EV_EPI_ST0);
         }
-        if (live && g.qs.bits > 0) acc += (double)(rn * rq.delta) * (double)acc_t;
+        if (live) acc += (double)(rn * rq.delta) * (double)acc_t;
         // hand the tile to the second product: shared-memory writes must be visible to the tensor-core proxy
         ptx::tc_fence_before();
         ptx::fence_proxy_async();
@@ -460,12 +446,9 @@ tcb_step_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         if (!tc_wait(&aux->pdone[grp], wo_count & 1u, abort_flag)) { ok = false; timeout_site = 36; break; }
         ++wo_count;
       }
-      // With fake-quantisation every warp leaves its objective partial of the problem (summed in a fixed order by the
-      // kernel that follows); without, the objective is <R, M> / sqrt(d) and is formed from M when it is read.
-      if (g.qs.bits > 0) {
-        const double wsum = warp_sum_d(acc);
-        if (lane == 0) g.part_d[(long long)item * TCB_PARTS + grp * 8 + ew] = wsum;
-      }
+      // every warp leaves its objective partial of the problem (summed in a fixed order by the kernel that follows)
+      const double wsum = warp_sum_d(acc);
+      if (lane == 0) g.part_d[(long long)item * TCB_PARTS + grp * 8 + ew] = wsum;
     }
   }
 
@@ -494,7 +477,7 @@ tcb_step_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
 // TMEM: Y^T 256 columns, C'^T 2 x 64, M^T 128: all 512.
 // What bounds it: power.  Streaming the input and the two products draw the board's 1000 W limit between them (a plain copy
 // of the same bytes does, too), so the SM clock settles at 1.38-1.5 GHz and fewer bytes moved inside the SM count, not
-// fewer cycles: 1024 problems x 4096 rows in 341 us sustained, 282-330 us in bursts of 20-150 ms; tcb_step_kernel 371 and
+// fewer cycles: 1024 problems x 4096 rows in 341 us sustained, 282-330 us in bursts of 20-150 ms; tcb_step_kernel with this target 371 and
 // 312-366 us, single tiles with a second R and five stages 345 and 293-335 us.
 // With fake-quantisation the row's range is needed as well, and tcb_step_kernel, where a thread owns a token, stays.
 constexpr int TCBT_STAGES = 3;                                  // input stages of two tiles
