@@ -275,7 +275,7 @@ def run_batched(args, g, w):
     peaks = _peaks()
     step_bytes = 2.0 * P * n * d
     ach = step_bytes / (step_ms * 1e-3) / 1e9
-    heads_traffic, heads_src = ncu_traffic("c4b.tcb_step")
+    heads_traffic, heads_src = ncu_traffic("c4b.tcb_step_plain")
     if not g.is_main:
         D.finish(g)
         return 0
@@ -291,7 +291,7 @@ def run_batched(args, g, w):
                 "d2h_bytes_per_step": 16 * P, "ms_per_step": ms_e2e},
         "gpu_launches": int(launches),
         "roofline": {"bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": ach / peaks["hbm_gbs"],
-                     "traffic": (heads_traffic * (P * n) / (592 * 2048)) if heads_traffic else None, "kernel": "tcb_step_kernel",
+                     "traffic": (heads_traffic * (P * n) / (592 * 2048)) if heads_traffic else None, "kernel": "tcb_step_plain_kernel",
                      "avg_launch_ms": step_ms,
                      "traffic_note": (f"dram read+write of an ncu capture at 592 problems x 2048 tokens ({heads_src}), scaled by the "
                                       "tokens processed: the kernel streams its input once") if heads_src else "no capture",
@@ -702,7 +702,7 @@ def main():
         "data": "synthetic",
         "config": {"workload": _workload_desc(w), "tokens_per_step": cyc * w.n, "mode": "tc (bf16 operands, fp32 accumulate; "
                    "the two step products run once per cycle over its 8 queued batches; Newton-Schulz: residual product "
-                   "in one fp16 pass (the accepting check as 3-term bf16 split) and polynomial product in one fp16 pass on "
+                   "in one fp16 pass (the last endgame step's and the accepting check as 3-term bf16 split) and polynomial product in one fp16 pass on "
                    "symmetric tiles, iterate product 2 bf16 terms then one fp16 pass)", "l2": f"inputs larger than L2: {resident_bytes / 1e6:.0f} MB "
                    f"of distinct batches resident, each read once per cycle", "replicas": g.world,
                    "input_gen_s": round(t_gen, 1)},

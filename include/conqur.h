@@ -273,8 +273,8 @@ int conqur_set_M(conqur_ctx* ctx, const float* M_dev, const double* J_sum, const
  * see conqur_debug_capture_signs.  Synchronises. */
 int conqur_debug_get_signs(conqur_ctx* ctx, int8_t* S_out_dev, int64_t capacity_rows);
 
-/* The same read-out for tensor-core contexts with batch > 1, whose fused per-head kernel keeps the targets in shared
- * memory only (Section 3.4, a Procrustes problem per head): after this call every conqur_step_batched(_range) also
+/* The same read-out for tensor-core contexts with batch > 1, whose fused per-head kernels keep the targets on the
+ * chip only (Section 3.4, a Procrustes problem per head): after this call every conqur_step_batched(_range) also
  * writes the decisions it takes to S_dev, laid out as above with q counted from the call's first problem; a call with
  * problems * n > capacity_rows then returns CONQUR_ERR_INVALID_ARG and enqueues nothing.  S_dev: device, 16-byte
  * aligned, owned by the caller, valid until replaced; NULL switches the capture off.  Synchronises. */

@@ -1452,8 +1452,8 @@ inline int tc_ns_next_parts(const TcHost& h) { return tc_part_slots(h, tc_varian
 
 // G = X^T X (symmetric tiles only), stored as E = G - tau I in (scaled) fp16, and the statistics of G - I.  Between the
 // steps G only has to be about as good as its rounding (2^-12): one pass over the iterate's fp16 copy does.  The check
-// that may accept the rotation takes three passes over the bf16 pair in Xh[buf]: hi hi, hi lo, lo hi.
-// (d = 4096: 60 us against 150; with a one-pass product of the bf16 hi part instead, early steps lost the directions
+// that may accept the rotation, and the last endgame step in front of it, take three passes over the bf16 pair in Xh[buf]: hi
+// hi, hi lo, lo hi (d = 4096: 71 us against 152; with a one-pass product of the bf16 hi part instead, early steps lost the directions
 // below 1e-4 of the largest and endgame steps had to be repeated.)
 inline int tc_ns_residual(TcHost& h, cudaStream_t s, int buf) {
   const int d = h.d;
