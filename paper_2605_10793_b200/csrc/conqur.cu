@@ -739,8 +739,8 @@ extern "C" int conqur_set_R(conqur_ctx* c, const float* R_dev) {
   //   fp32 product    d roundings of 2^-24
   // Only a result within that bound of the limit, or one that is not finite, goes on to the fp32 product, so what is accepted
   // and what is refused does not change.  Widths whose bound leaves no room for what an update returns (1e-4) go there
-  // straight away (whole call at d = 4096: 1650 -> 213 us, 3072: 865 -> 154, 1024: 111 -> 66; at 256 the extra launches
-  // cost 7 us).
+  // straight away (whole call, fp32 product alone -> with this: d = 4096 1650 -> 211 us, 3072 865 -> 150, 1024 111 -> 62; at
+  // 256 the extra launches cost 7 us; 8192 stays at 11.9 ms).
   const double bound = 2.0e-5 + 1.72e-7 * g.d;
   if (g.mode == CONQUR_TC_BF16 && aligned && (g.P > 1 || g.d >= 512) && bound <= 8.5e-4) {
     float* pf = c->at<float>(c->L.part_f);

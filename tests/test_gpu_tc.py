@@ -370,6 +370,6 @@ def test_accepted_rotations_are_orthogonal_to_the_precision_of_the_bf16_pair(d, 
         assert st.status == 0 and errs[-1] <= T["orth"], (st.status, errs, st.ns_steps_used)
         assert 1.0 - float((r * m.double()).sum()) / s.sum() <= T["gap"], errs
     # The check's three-pass sums are cut, never rounded up: columns come out longer by what they lose, 5.8e-9 d (measured up
-    # to d = 8192).  lo * lo, left out of the last step's G, and the pair's rounding add 2^-18 each: 2.55e-5 at d = 3072.  An update may also stop a step early, just below the tolerance, which is its right: the middle one
-    # of three is looked at.
+    # to d = 8192).  lo * lo, left out of the last step's G, and the pair's rounding add 2^-18 each: 2.55e-5 at d = 3072.
+    # An update may also stop a step early, just below the tolerance, which is its right: the middle one of three is looked at.
     assert sorted(errs)[1] <= 2.6e-5, errs
