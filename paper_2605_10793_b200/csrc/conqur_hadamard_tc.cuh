@@ -54,7 +54,7 @@ hadamard_tc_kernel(const __grid_constant__ CUtensorMap tmX, TOut* Y, long long N
   uint8_t* sStg = sX + HTC_STAGES * HTC_X_BYTES;
   HtcAux* aux = reinterpret_cast<HtcAux*>(sStg + HTC_EPI_WARPS * HTC_STG_BYTES);
   volatile int* abort_flag = &aux->abort_flag;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const long long tiles = (NC + HTC_N - 1) / HTC_N;
 
   if (threadIdx.x == 0) {
@@ -120,7 +120,8 @@ hadamard_tc_kernel(const __grid_constant__ CUtensorMap tmX, TOut* Y, long long N
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
+      const uint32_t leader = ptx::elect_one();
       // bf16 x bf16 -> fp32, both operands K-major, M = 128, N = 256
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(HTC_N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
       const uint32_t sA_a = ptx::smem_u32(sA), sX_a = ptx::smem_u32(sX);
@@ -128,16 +129,16 @@ hadamard_tc_kernel(const __grid_constant__ CUtensorMap tmX, TOut* Y, long long N
       int it = 0;
       for (long long t = blockIdx.x; t < tiles; t += gridDim.x, ++it) {
         const int buf = it & 1;
-        if (!tc_wait(&aux->xfull[s], ph, abort_flag)) { timeout_site = 2; break; }
-        if (!tc_wait(&aux->dempty[buf], (((uint32_t)it >> 1) & 1u) ^ 1u, abort_flag)) { timeout_site = 3; break; }
+        if (!tc_wait_warp(&aux->xfull[s], ph, abort_flag)) { timeout_site = 2; break; }
+        if (!tc_wait_warp(&aux->dempty[buf], (((uint32_t)it >> 1) & 1u) ^ 1u, abort_flag)) { timeout_site = 3; break; }
         ptx::tc_fence_after();
         const uint32_t xb = sX_a + s * HTC_X_BYTES;
 #pragma unroll
         for (int j = 0; j < 8; ++j)                // 16 e per instruction: chunk j / 4, 32 bytes per step inside the swizzled row
-          ptx::umma_bf16(tmem_base + (uint32_t)(buf * HTC_N), tc_smem_desc(sA_a + (j >> 2) * 16384 + (j & 3) * 32, 16, 1024),
+          ptx::umma_bf16_by<false>(leader, tmem_base + (uint32_t)(buf * HTC_N), tc_smem_desc(sA_a + (j >> 2) * 16384 + (j & 3) * 32, 16, 1024),
                          tc_smem_desc(xb + (j >> 2) * (HTC_X_BYTES / 2) + (j & 3) * 32, 16, 1024), idesc, j > 0 ? 1u : 0u);
-        ptx::umma_commit(&aux->xempty[s]);
-        ptx::umma_commit(&aux->dfull[buf]);
+        ptx::umma_commit_by<false>(leader, ptx::smem_u32(&aux->xempty[s]));
+        ptx::umma_commit_by<false>(leader, ptx::smem_u32(&aux->dfull[buf]));
         if (++s == HTC_STAGES) { s = 0; ph ^= 1u; }
       }
     }

@@ -102,21 +102,6 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// D(tmem) (+)= A(smem desc) * B(smem desc); accumulate == 0 overwrites D.
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                          uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// Arrives on the mbarrier once every previously issued MMA of this thread has completed.
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
-}
 // 32 lanes x 32 consecutive fp32 columns: thread t of the warp receives row (lane base + t).
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
   uint32_t r[32];
@@ -172,24 +157,57 @@ __device__ __forceinline__ void tmem_relinquish_pair() {
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
-__device__ __forceinline__ void umma_bf16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                               uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
+// ---- D(tmem) (+)= A(smem desc) * B(smem desc); accumulate == 0 overwrites D.  The forms an issuing WARP uses: every lane executes
+// them and the one with leader != 0 issues.  The loop around them then stays uniform, so that descriptors and barrier addresses are
+// worked out in uniform registers, which is where the instruction takes them from.  With the loop inside `if (lane == 0)` each
+// instruction waited for its operands to be moved over: 148 SM cycles from one to the next, more than a 256 x 256 x 16 product
+// takes (128).  d = 4096, one pass: residual 68 -> 58 us, polynomial 67 -> 55, next iterate 132 -> 112 (two passes 195 -> 173);
+// steps' products of 2048 rows 63 -> 55 and 65 -> 59.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(r));
+  return r;
 }
-// Arrives on the barrier at this shared-memory offset in both CTAs of the pair once the MMAs issued so far retire.
-__device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
+template <bool PAIR>
+__device__ __forceinline__ void umma_bf16_by(uint32_t leader, uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                             uint32_t accumulate) {
+  if (PAIR)
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(leader)
+        : "memory");
+  else
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(leader)
+        : "memory");
+}
+// Arrives on the barrier (at this shared-memory offset in both CTAs of a pair) once the MMAs issued so far retire.
+template <bool PAIR>
+__device__ __forceinline__ void umma_commit_by(uint32_t leader, uint32_t bar) {
   const uint16_t mask = 3;
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-               ::"r"(smem_u32(bar)), "h"(mask)
-               : "memory");
+  if (PAIR)
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t"
+        "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}"
+        ::"r"(bar), "h"(mask), "r"(leader)
+        : "memory");
+  else
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+        ::"r"(bar), "r"(leader)
+        : "memory");
 }
 
 }  // namespace ptx
+
+// The warp's number, as a value that is the same for all its lanes (roles branched on it stay uniform).
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
 
 // ------------------------------------------------------------------ kernel configuration
 constexpr int TC_BM = 128;
@@ -297,6 +315,11 @@ __device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, volatile
     }
   }
   return true;
+}
+
+// The same for a whole warp: every lane waits, and all of them agree on the outcome.
+__device__ __forceinline__ bool tc_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  return __all_sync(0xffffffffu, tc_wait(bar, parity, abort_flag));
 }
 
 __device__ __forceinline__ uint64_t tc_smem_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
@@ -421,7 +444,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   TcAux* aux = reinterpret_cast<TcAux*>(smem + Cfg::STAGES * Cfg::STAGE_BYTES);
   volatile int* abort_flag = &aux->abort_flag;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = PAIR ? ptx::cluster_ctarank() : 0u;        // 0: the CTA that issues the pair's MMAs
   const int worker = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
   const int n_workers = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
@@ -565,55 +588,50 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer (CTA 0 of a pair issues for both)
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
+      const uint32_t leader = ptx::elect_one();
       const uint32_t types = f16 ? 0u : ((1u << 7) | (1u << 10));          // fp16 or bf16 operands
       const uint32_t idesc = (1u << 4) | types | ((A_MN ? 1u : 0u) << 15) | ((B_MN ? 1u : 0u) << 16) |
                              ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+      const uint32_t idesc_half = (idesc & ~(0x3fu << 17)) | ((uint32_t)((BN / 2) >> 3) << 17);   // N = BN / 2
+      // K-major: 16 k = 32 bytes inside the swizzled 128-byte row; 8-row groups 1024 bytes apart.
+      // MN-major: 16 k = two 8-row groups of 1024 bytes; 64-wide m|n chunks 8192 bytes apart.
+      // For a pair the descriptors name this CTA's tiles; the peer's halves sit at the same offsets in its memory.
+      // (addresses in units of 16 bytes: the low word of a descriptor)
+      const uint64_t a0 = tc_smem_desc(ptx::smem_u32(smem), A_MN ? 8192 : 16, 1024), b0 = tc_smem_desc(ptx::smem_u32(smem), B_MN ? 8192 : 16, 1024);
+      constexpr uint32_t A_STEP = A_MN ? 2048 / 16 : 32 / 16, B_STEP = B_MN ? 2048 / 16 : 32 / 16;
+      const uint32_t full0 = ptx::smem_u32(&aux->full[0]);
+      const uint32_t empty0 = full0 + (uint32_t)(offsetof(TcAux, empty) - offsetof(TcAux, full));
+      const uint32_t tfull0 = full0 + (uint32_t)(offsetof(TcAux, tfull) - offsetof(TcAux, full));
       int stage = 0;
       uint32_t phase = 0;
       int local = 0;
       bool ok = true;
-      const uint32_t idesc_half = (idesc & ~(0x3fu << 17)) | ((uint32_t)((BN / 2) >> 3) << 17);   // N = BN / 2
       for (int tile = worker; tile < num_items && ok; tile += n_workers, ++local) {
         const int buf = local & 1;
         const uint32_t idesc_t = (tile >= full_tiles) ? idesc_half : idesc;
-        if (!tc_wait(&aux->tempty[buf], ((uint32_t)(local >> 1) & 1u) ^ 1u, abort_flag)) { ok = false; timeout_site = 2; break; }
+        if (!tc_wait_warp(&aux->tempty[buf], ((uint32_t)(local >> 1) & 1u) ^ 1u, abort_flag)) { ok = false; timeout_site = 2; break; }
         ptx::tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
         for (int it = 0; it < k_iters; ++it) {
-          if (!tc_wait(&aux->full[stage], phase, abort_flag)) { ok = false; timeout_site = 3; break; }
+          if (!tc_wait_warp(&aux->full[stage], phase, abort_flag)) { ok = false; timeout_site = 3; break; }
           ptx::tc_fence_after();
-          const uint32_t sa = ptx::smem_u32(smem + stage * stage_bytes);
-          // K-major: 16 k = 32 bytes inside the swizzled 128-byte row; 8-row groups 1024 bytes apart.
-          // MN-major: 16 k = two 8-row groups of 1024 bytes; 64-wide m|n chunks 8192 bytes apart.
-          // For a pair the descriptors name this CTA's tiles; the peer's halves sit at the same offsets in its memory.
-          if (PAIR) {
-            for (int sg = 0; sg < nseg; ++sg) {
-              const uint32_t ta = sa + (uint32_t)(g.a_tile[sg] * Cfg::A_BYTES);
-              const uint32_t tb = sa + (uint32_t)(na * Cfg::A_BYTES + g.b_tile[sg] * Cfg::B_BYTES);
-#pragma unroll
-              for (int j = 0; j < TC_BK / 16; ++j) {
-                const uint64_t ad = A_MN ? tc_smem_desc(ta + j * 2048, 8192, 1024) : tc_smem_desc(ta + j * 32, 16, 1024);
-                const uint64_t bd = B_MN ? tc_smem_desc(tb + j * 2048, 8192, 1024) : tc_smem_desc(tb + j * 32, 16, 1024);
-                ptx::umma_bf16_pair(d_tmem, ad, bd, idesc_t, (it > 0 || sg > 0 || j > 0) ? 1u : 0u);
-              }
+          const uint32_t at = (uint32_t)(stage * stage_bytes) >> 4;
+          for (int sg = 0; sg < (PAIR ? nseg : 1); ++sg) {
+            uint64_t ad = a0 + at, bd = b0 + at + Cfg::A_BYTES / 16;
+            if (PAIR && NA * NB > 1) {
+              ad = a0 + at + (uint32_t)(g.a_tile[sg] * (Cfg::A_BYTES / 16));
+              bd = b0 + at + (uint32_t)(na * (Cfg::A_BYTES / 16) + g.b_tile[sg] * (Cfg::B_BYTES / 16));
             }
-          } else {
-            const uint32_t sb = sa + Cfg::A_BYTES;
 #pragma unroll
-            for (int j = 0; j < TC_BK / 16; ++j) {
-              const uint64_t ad = A_MN ? tc_smem_desc(sa + j * 2048, 8192, 1024) : tc_smem_desc(sa + j * 32, 16, 1024);
-              const uint64_t bd = B_MN ? tc_smem_desc(sb + j * 2048, 8192, 1024) : tc_smem_desc(sb + j * 32, 16, 1024);
-              ptx::umma_bf16(d_tmem, ad, bd, idesc, (it > 0 || j > 0) ? 1u : 0u);
-            }
+            for (int j = 0; j < TC_BK / 16; ++j)
+              ptx::umma_bf16_by<PAIR>(leader, d_tmem, ad + j * A_STEP, bd + j * B_STEP, idesc_t, (it > 0 || sg > 0 || j > 0) ? 1u : 0u);
           }
           // frees the shared-memory stage (in both CTAs of a pair) once these MMAs retire
-          if (PAIR) ptx::umma_commit_pair(&aux->empty[stage]); else ptx::umma_commit(&aux->empty[stage]);
+          ptx::umma_commit_by<PAIR>(leader, empty0 + (uint32_t)stage * 8u);
           if (++stage == n_stages) { stage = 0; phase ^= 1u; }
         }
-        if (ok) {                                         // accumulator complete
-          if (PAIR) ptx::umma_commit_pair(&aux->tfull[buf]); else ptx::umma_commit(&aux->tfull[buf]);
-        }
+        if (ok) ptx::umma_commit_by<PAIR>(leader, tfull0 + (uint32_t)buf * 8u);            // accumulator complete
       }
     }
   } else {

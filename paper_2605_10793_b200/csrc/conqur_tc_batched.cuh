@@ -158,7 +158,7 @@ tcb_step_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   uint8_t* sC = smem + TCB_TILE_BYTES * (1 + TCB_XSTAGES);
   TcbAux* aux = reinterpret_cast<TcbAux*>(smem + TCB_TILE_BYTES * (1 + TCB_XSTAGES + 2));
   volatile int* abort_flag = &aux->abort_flag;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int T = (g.n + 127) / 128;                 // token tiles per problem
 
   if (threadIdx.x == 0) {
@@ -222,7 +222,8 @@ tcb_step_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- first product: Y = X_tile R
-    if (lane == 0) {
+    {
+      const uint32_t leader = ptx::elect_one();
       // instruction descriptor: bf16 x bf16 -> fp32, M = N = 128; A K-major, B MN-major
       const uint32_t idesc1 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24) | (1u << 16);
       const uint32_t sR_a = ptx::smem_u32(sR), sX_a = ptx::smem_u32(sX);
@@ -233,27 +234,28 @@ tcb_step_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         int p_item, tb_item, te_item;
         tcb_item(item, T, g.S, p_item, tb_item, te_item);
         const int T_item = te_item - tb_item;
-        if (!tc_wait(&aux->rfull, (uint32_t)lp & 1u, abort_flag)) { ok = false; timeout_site = 20; break; }
+        if (!tc_wait_warp(&aux->rfull, (uint32_t)lp & 1u, abort_flag)) { ok = false; timeout_site = 20; break; }
         for (int t = 0; t < T_item && ok; ++t, ++it) {
           const int yb = it % TCB_YBUF;
-          if (!tc_wait(&aux->xfull[xs], xph, abort_flag)) { ok = false; timeout_site = 22; break; }
-          if (!tc_wait(&aux->yempty[yb], (((uint32_t)(it / TCB_YBUF)) & 1u) ^ 1u, abort_flag)) { ok = false; timeout_site = 24; break; }
+          if (!tc_wait_warp(&aux->xfull[xs], xph, abort_flag)) { ok = false; timeout_site = 22; break; }
+          if (!tc_wait_warp(&aux->yempty[yb], (((uint32_t)(it / TCB_YBUF)) & 1u) ^ 1u, abort_flag)) { ok = false; timeout_site = 24; break; }
           ptx::tc_fence_after();
-          TCB_TR(it, TCB_EV_MMA1);
+          if (leader) TCB_TR(it, TCB_EV_MMA1);
           const uint32_t xa = sX_a + xs * TCB_TILE_BYTES;
 #pragma unroll
           for (int j = 0; j < 8; ++j)        // 16 features per instruction: chunk j/4, 32 bytes per step inside the swizzled row
-            ptx::umma_bf16(tmem_base + yb * 128, tc_smem_desc(xa + (j >> 2) * 16384 + (j & 3) * 32, 16, 1024),
+            ptx::umma_bf16_by<false>(leader, tmem_base + yb * 128, tc_smem_desc(xa + (j >> 2) * 16384 + (j & 3) * 32, 16, 1024),
                            tc_smem_desc(sR_a + j * 2048, 16384, 1024), idesc1, j > 0 ? 1u : 0u);
-          ptx::umma_commit(&aux->yfull[yb]);
-          if (t == T_item - 1) ptx::umma_commit(&aux->rempty);     // R may be replaced once every first product has run
+          ptx::umma_commit_by<false>(leader, ptx::smem_u32(&aux->yfull[yb]));
+          if (t == T_item - 1) ptx::umma_commit_by<false>(leader, ptx::smem_u32(&aux->rempty));     // R may be replaced once every first product has run
           if (++xs == TCB_XSTAGES) { xs = 0; xph ^= 1u; }
         }
       }
     }
   } else if (warp == TCB_MMA2_WARP) {
     // ---------------------------------------------------------------- second product: M += X_tile^T C'
-    if (lane == 0) {
+    {
+      const uint32_t leader = ptx::elect_one();
       // both operands MN-major (contraction over the tokens, the slow dimension of both tiles)
       const uint32_t idesc2 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24) |
                               (1u << 15) | (1u << 16);
@@ -267,23 +269,23 @@ tcb_step_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         const int T_item = te_item - tb_item;
         // the accumulator of the previous problem has been read out
         const int mb = lp % TCB_MBUF;
-        if (!tc_wait(&aux->mempty[mb], (((uint32_t)(lp / TCB_MBUF)) & 1u) ^ 1u, abort_flag)) { ok = false; timeout_site = 21; break; }
+        if (!tc_wait_warp(&aux->mempty[mb], (((uint32_t)(lp / TCB_MBUF)) & 1u) ^ 1u, abort_flag)) { ok = false; timeout_site = 21; break; }
         for (int t = 0; t < T_item && ok; ++t, ++it) {
           const int cb = it & 1;
-          if (!tc_wait(&aux->xfull[xs], xph, abort_flag)) { ok = false; timeout_site = 25; break; }
-          if (!tc_wait(&aux->cready[cb], ((uint32_t)it >> 1) & 1u, abort_flag)) { ok = false; timeout_site = 23; break; }
+          if (!tc_wait_warp(&aux->xfull[xs], xph, abort_flag)) { ok = false; timeout_site = 25; break; }
+          if (!tc_wait_warp(&aux->cready[cb], ((uint32_t)it >> 1) & 1u, abort_flag)) { ok = false; timeout_site = 23; break; }
           ptx::tc_fence_after();
-          TCB_TR(it, TCB_EV_MMA2);
+          if (leader) TCB_TR(it, TCB_EV_MMA2);
           const uint32_t xa = sX_a + xs * TCB_TILE_BYTES, ca = sC_a + cb * TCB_TILE_BYTES;
 #pragma unroll
           for (int j = 0; j < 8; ++j)          // 16 tokens per instruction: two 8-row groups, 2048 bytes per step
-            ptx::umma_bf16(tmem_base + TM_M + mb * 128, tc_smem_desc(xa + j * 2048, 16384, 1024), tc_smem_desc(ca + j * 2048, 16384, 1024),
+            ptx::umma_bf16_by<false>(leader, tmem_base + TM_M + mb * 128, tc_smem_desc(xa + j * 2048, 16384, 1024), tc_smem_desc(ca + j * 2048, 16384, 1024),
                            idesc2, (t > 0 || j > 0) ? 1u : 0u);
-          ptx::umma_commit(&aux->xempty[xs]);
-          ptx::umma_commit(&aux->cfree[cb]);
+          ptx::umma_commit_by<false>(leader, ptx::smem_u32(&aux->xempty[xs]));
+          ptx::umma_commit_by<false>(leader, ptx::smem_u32(&aux->cfree[cb]));
           if (++xs == TCB_XSTAGES) { xs = 0; xph ^= 1u; }
         }
-        if (ok) ptx::umma_commit(&aux->mfull[mb]);
+        if (ok) ptx::umma_commit_by<false>(leader, ptx::smem_u32(&aux->mfull[mb]));
       }
     }
   } else {
@@ -501,12 +503,13 @@ static_assert(TCBT_SMEM_BYTES <= 232448, "227 KB of dynamic shared memory per CT
 
 namespace ptx {
 // D(tmem) (+)= A(tmem: lane = row, two consecutive 16-bit k per column) * B(smem desc)
-__device__ __forceinline__ void umma_bf16_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+__device__ __forceinline__ void umma_bf16_ta_by(uint32_t leader, uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc,
+                                                uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(tmem_d), "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      ::"r"(tmem_d), "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(leader)
       : "memory");
 }
 // 32 lanes x 16 consecutive columns: thread t of the warp writes row (lane base + t); complete after tmem_st_wait.
@@ -520,10 +523,6 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&w)[16
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 }  // namespace ptx
 
-// A wait of a whole warp: every lane waits (bounded), and all of them agree on the outcome.
-__device__ __forceinline__ bool tc_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-  return __all_sync(0xffffffffu, tc_wait(bar, parity, abort_flag) ? 1 : 0) != 0;
-}
 // Byte offset of the 16-byte piece `c16` (0..15) of row `r` (0..255) inside a stage.
 __device__ __forceinline__ uint32_t tcbt_piece(int r, int c16) {
   return (uint32_t)((c16 >> 3) * TCBT_CHUNK_BYTES + r * 128 + (((c16 & 7) ^ (r & 7)) << 4));
@@ -537,7 +536,7 @@ tcb_step_plain_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
   uint8_t* sX = smem + TCB_TILE_BYTES;
   TcbtAux* aux = reinterpret_cast<TcbtAux*>(sX + TCBT_STAGES * TCBT_STAGE_BYTES);
   volatile int* abort_flag = &aux->abort_flag;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int T = (g.n + 255) / 256;                 // double tiles per problem
 
   if (threadIdx.x == 0) {
@@ -596,7 +595,8 @@ tcb_step_plain_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- first product: Y^T = R^T X^T
-    if (lane == 0) {
+    {
+      const uint32_t leader = ptx::elect_one();
       const uint32_t idesc1 = idesc0 | (1u << 15) | ((uint32_t)(256 >> 3) << 17);    // A (R, read transposed) MN-major, B (X) K-major
       int xs = 0; uint32_t xph = 0;
       int it = 0, lp = 0;
@@ -605,23 +605,25 @@ tcb_step_plain_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         int p, t_begin, t_end;
         tcb_item(item, T, g.S, p, t_begin, t_end);
         // the rotation: this thread's own products are the only readers of its buffer
-        if (!tc_wait(&aux->rempty, ((uint32_t)lp & 1u) ^ 1u, abort_flag)) { ok = false; timeout_site = 11; break; }
-        ptx::mbar_expect_tx(&aux->rfull, TCB_TILE_BYTES);
-        ptx::tma_load_2d(sR, &tmR, &aux->rfull, 0, (g.p0 + p) * TCB_D);
-        ptx::tma_load_2d(sR + 16384, &tmR, &aux->rfull, 64, (g.p0 + p) * TCB_D);
-        if (!tc_wait(&aux->rfull, (uint32_t)lp & 1u, abort_flag)) { ok = false; timeout_site = 20; break; }
+        if (!tc_wait_warp(&aux->rempty, ((uint32_t)lp & 1u) ^ 1u, abort_flag)) { ok = false; timeout_site = 11; break; }
+        if (leader) {
+          ptx::mbar_expect_tx(&aux->rfull, TCB_TILE_BYTES);
+          ptx::tma_load_2d(sR, &tmR, &aux->rfull, 0, (g.p0 + p) * TCB_D);
+          ptx::tma_load_2d(sR + 16384, &tmR, &aux->rfull, 64, (g.p0 + p) * TCB_D);
+        }
+        if (!tc_wait_warp(&aux->rfull, (uint32_t)lp & 1u, abort_flag)) { ok = false; timeout_site = 20; break; }
         for (int t = t_begin; t < t_end && ok; ++t, ++it) {
-          if (!tc_wait(&aux->xfull[xs], xph, abort_flag)) { ok = false; timeout_site = 22; break; }
-          if (!tc_wait(&aux->yempty, ((uint32_t)it & 1u) ^ 1u, abort_flag)) { ok = false; timeout_site = 24; break; }
+          if (!tc_wait_warp(&aux->xfull[xs], xph, abort_flag)) { ok = false; timeout_site = 22; break; }
+          if (!tc_wait_warp(&aux->yempty, ((uint32_t)it & 1u) ^ 1u, abort_flag)) { ok = false; timeout_site = 24; break; }
           ptx::tc_fence_after();
-          TCB_TR(2 * it, TCB_EV_MMA1); TCB_TR(2 * it + 1, TCB_EV_MMA1);
+          if (leader) { TCB_TR(2 * it, TCB_EV_MMA1); TCB_TR(2 * it + 1, TCB_EV_MMA1); }
           const uint32_t xa = sX_a + xs * TCBT_STAGE_BYTES;
 #pragma unroll
           for (int j = 0; j < 8; ++j)              // 16 features per instruction
-            ptx::umma_bf16(tmem_base, tc_smem_desc(sR_a + j * 2048, 16384, 1024),
+            ptx::umma_bf16_by<false>(leader, tmem_base, tc_smem_desc(sR_a + j * 2048, 16384, 1024),
                            tc_smem_desc(xa + (j >> 2) * TCBT_CHUNK_BYTES + (j & 3) * 32, 16, 1024), idesc1, j > 0 ? 1u : 0u);
-          ptx::umma_commit(&aux->yfull);
-          if (t == t_end - 1) ptx::umma_commit(&aux->rempty);
+          ptx::umma_commit_by<false>(leader, ptx::smem_u32(&aux->yfull));
+          if (t == t_end - 1) ptx::umma_commit_by<false>(leader, ptx::smem_u32(&aux->rempty));
           if (++xs == TCBT_STAGES) { xs = 0; xph ^= 1u; }
         }
       }
@@ -632,7 +634,8 @@ tcb_step_plain_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     }
   } else if (warp == 2) {
     // ---------------------------------------------------------------- second product: M^T += C'^T X
-    if (lane == 0) {
+    {
+      const uint32_t leader = ptx::elect_one();
       const uint32_t idesc2 = idesc0 | (1u << 16) | ((uint32_t)(128 >> 3) << 17);    // A from TMEM, B (X, contraction over the tokens) MN-major
       int xs = 0; uint32_t xph = 0;
       int it = 0, lp = 0;
@@ -640,26 +643,26 @@ tcb_step_plain_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
       for (int item = blockIdx.x; item < g.P * g.S && ok; item += gridDim.x, ++lp) {
         int p, t_begin, t_end;
         tcb_item(item, T, g.S, p, t_begin, t_end);
-        if (!tc_wait(&aux->mempty, ((uint32_t)lp & 1u) ^ 1u, abort_flag)) { ok = false; timeout_site = 21; break; }
+        if (!tc_wait_warp(&aux->mempty, ((uint32_t)lp & 1u) ^ 1u, abort_flag)) { ok = false; timeout_site = 21; break; }
         for (int t = t_begin; t < t_end && ok; ++t, ++it) {
-          if (!tc_wait(&aux->xfull[xs], xph, abort_flag)) { ok = false; timeout_site = 25; break; }
+          if (!tc_wait_warp(&aux->xfull[xs], xph, abort_flag)) { ok = false; timeout_site = 25; break; }
           const uint32_t xa = sX_a + xs * TCBT_STAGE_BYTES;
           for (int h = 0; h < 2; ++h) {
-            if (!tc_wait(&aux->cready[h], (uint32_t)it & 1u, abort_flag)) { ok = false; timeout_site = 23; break; }
+            if (!tc_wait_warp(&aux->cready[h], (uint32_t)it & 1u, abort_flag)) { ok = false; timeout_site = 23; break; }
             ptx::tc_fence_after();
-            TCB_TR(2 * it + h, TCB_EV_MMA2);
+            if (leader) TCB_TR(2 * it + h, TCB_EV_MMA2);
 #pragma unroll
             for (int j = 0; j < 8; ++j)            // 16 tokens per instruction, 8 columns of C'^T
-              ptx::umma_bf16_ta(tmem_base + TCBT_M_COL, tmem_base + TCBT_C_COL + h * 64 + j * 8,
+              ptx::umma_bf16_ta_by(leader, tmem_base + TCBT_M_COL, tmem_base + TCBT_C_COL + h * 64 + j * 8,
                                 tc_smem_desc(xa + h * 16384 + j * 2048, TCBT_CHUNK_BYTES, 1024), idesc2,
                                 (t > t_begin || h > 0 || j > 0) ? 1u : 0u);
-            ptx::umma_commit(&aux->cfree[h]);
+            ptx::umma_commit_by<false>(leader, ptx::smem_u32(&aux->cfree[h]));
           }
           if (!ok) break;
-          ptx::umma_commit(&aux->xempty[xs]);
+          ptx::umma_commit_by<false>(leader, ptx::smem_u32(&aux->xempty[xs]));
           if (++xs == TCBT_STAGES) { xs = 0; xph ^= 1u; }
         }
-        if (ok) ptx::umma_commit(&aux->mfull);
+        if (ok) ptx::umma_commit_by<false>(leader, ptx::smem_u32(&aux->mfull));
       }
     }
   } else if (warp < TCBT_EPI_WARP0) {
@@ -1037,7 +1040,7 @@ __global__ void __launch_bounds__(TCBU_THREADS, 2) tcb_update_kernel(const TcbUp
   uint8_t* sEB = smem + 2 * TCB_TILE_BYTES;
   TcbUpdAux* aux = reinterpret_cast<TcbUpdAux*>(smem + 3 * TCB_TILE_BYTES);
   volatile int* abort_flag = &aux->abort_flag;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int r = threadIdx.x & 127;                 // the row this thread works on everywhere
   const int half = threadIdx.x >> 7;               // ... and which 64 of its 128 columns
   const int c_diag = r >> 5;                       // the 32-column chunk holding the row's diagonal element (one per warp)
@@ -1060,6 +1063,7 @@ __global__ void __launch_bounds__(TCBU_THREADS, 2) tcb_update_kernel(const TcbUp
   const uint32_t idesc_base = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
   const uint32_t idesc_mm = idesc_base | (1u << 15) | (1u << 16);       // both operands read "transposed" (MN-major)
   const uint32_t idesc_km = idesc_base | (1u << 16);                    // A as stored (K-major), B MN-major
+  const uint32_t mbar_a = ptx::smem_u32(&aux->mbar);
   uint32_t mph = 0;
   bool timed_out = false;
   const float isd = rsqrtf((float)TCB_D);
@@ -1067,17 +1071,19 @@ __global__ void __launch_bounds__(TCBU_THREADS, 2) tcb_update_kernel(const TcbUp
   // descriptor of k-step j (16 of the 128 contraction indices) of a 128 x 128 tile held as two swizzled 64-column chunks
   auto desc_k = [](uint32_t base, int j) { return tc_smem_desc(base + (j >> 2) * 16384 + (j & 3) * 32, 16, 1024); };   // contraction along columns
   auto desc_mn = [](uint32_t base, int j) { return tc_smem_desc(base + j * 2048, 16384, 1024); };                        // contraction along rows
-  // all threads: make shared-memory writes visible to the tensor cores, then thread 0 issues `issue`; the block barrier
+  // all threads: make shared-memory writes visible to the tensor cores, then warp 0 issues `issue`; the block barrier
   // inside also publishes whatever the threads wrote to the control block before the call.  wait_products: everyone
   // waits for the products issued last.  Work placed between the two overlaps the products.
   auto issue_products = [&](auto issue) {
     ptx::fence_proxy_async();
     ptx::tc_fence_before();
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (warp == 0) {
+      const uint32_t leader = ptx::elect_one();
       ptx::tc_fence_after();
-      issue();
-      ptx::umma_commit(&aux->mbar);
+      issue(leader);
+      ptx::umma_commit_by<false>(leader, mbar_a);
+      __syncwarp();
     }
   };
   auto wait_products = [&]() -> bool {
@@ -1086,13 +1092,13 @@ __global__ void __launch_bounds__(TCBU_THREADS, 2) tcb_update_kernel(const TcbUp
     ptx::tc_fence_after();
     return okw;
   };
-  auto issue_gram = [&] {                          // G = X^T X (hi hi + hi lo + lo hi)
+  auto issue_gram = [&](uint32_t leader) {                          // G = X^T X (hi hi + hi lo + lo hi)
     const uint32_t aa[3] = {aXh, aXh, aXl}, bb[3] = {aXh, aXl, aXh};
 #pragma unroll
     for (int seg = 0; seg < 3; ++seg)
 #pragma unroll
       for (int j = 0; j < 8; ++j)
-        ptx::umma_bf16(tmem_base, desc_mn(aa[seg], j), desc_mn(bb[seg], j), idesc_mm, (seg > 0 || j > 0) ? 1u : 0u);
+        ptx::umma_bf16_by<false>(leader, tmem_base, desc_mn(aa[seg], j), desc_mn(bb[seg], j), idesc_mm, (seg > 0 || j > 0) ? 1u : 0u);
   };
 
   NsCtl ctl{};                                     // thread 0 only
@@ -1199,10 +1205,10 @@ __global__ void __launch_bounds__(TCBU_THREADS, 2) tcb_update_kernel(const TcbUp
         }
         // ---- E E, which does not depend on the control decision: issued first, the decision is taken while it runs
         // (a step that turns out to be the last one throws the product away)
-        issue_products([&] {
+        issue_products([&](uint32_t leader) {
 #pragma unroll
           for (int j = 0; j < 8; ++j)
-            ptx::umma_bf16(tmem_base + 128, desc_k(aEB, j), desc_mn(aEB, j), idesc_km, j > 0 ? 1u : 0u);
+            ptx::umma_bf16_by<false>(leader, tmem_base + 128, desc_k(aEB, j), desc_mn(aEB, j), idesc_km, j > 0 ? 1u : 0u);
         });
         if (threadIdx.x == 0) {
           double tsq = 0.0, ttr = 0.0;
@@ -1245,12 +1251,12 @@ __global__ void __launch_bounds__(TCBU_THREADS, 2) tcb_update_kernel(const TcbUp
           if (c == c_diag) poly_chunk(c, std::true_type{}); else poly_chunk(c, std::false_type{});
         }
         // ---- X B
-        issue_products([&] {
+        issue_products([&](uint32_t leader) {
 #pragma unroll
-          for (int j = 0; j < 8; ++j) ptx::umma_bf16(tmem_base, desc_k(aXh, j), desc_mn(aEB, j), idesc_km, j > 0 ? 1u : 0u);
+          for (int j = 0; j < 8; ++j) ptx::umma_bf16_by<false>(leader, tmem_base, desc_k(aXh, j), desc_mn(aEB, j), idesc_km, j > 0 ? 1u : 0u);
           if (seg_x > 1) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) ptx::umma_bf16(tmem_base, desc_k(aXl, j), desc_mn(aEB, j), idesc_km, 1u);
+            for (int j = 0; j < 8; ++j) ptx::umma_bf16_by<false>(leader, tmem_base, desc_k(aXl, j), desc_mn(aEB, j), idesc_km, 1u);
           }
         });
         if (!wait_products()) { timed_out = true; break; }
@@ -1366,7 +1372,7 @@ __global__ void __launch_bounds__(TCBU_THREADS, 3) tcb_check_kernel(const float*
   uint8_t* sXh = smem;
   uint8_t* sXl = smem + TCB_TILE_BYTES;
   TcbCheckAux* aux = reinterpret_cast<TcbCheckAux*>(smem + 2 * TCB_TILE_BYTES);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int r = threadIdx.x & 127, half = threadIdx.x >> 7;        // row, and which 64 of its columns
   if (threadIdx.x == 0) {
     ptx::mbar_init(&aux->mbar, 1);
@@ -1398,16 +1404,18 @@ __global__ void __launch_bounds__(TCBU_THREADS, 3) tcb_check_kernel(const float*
     ptx::fence_proxy_async();
     ptx::tc_fence_before();
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (warp == 0) {
+      const uint32_t leader = ptx::elect_one();
       ptx::tc_fence_after();
       const uint32_t aa[3] = {aXh, aXh, aXl}, bb[3] = {aXh, aXl, aXh};
 #pragma unroll
       for (int seg = 0; seg < 3; ++seg)
 #pragma unroll
         for (int j = 0; j < 8; ++j)
-          ptx::umma_bf16(tmem_base, tc_smem_desc(aa[seg] + j * 2048, 16384, 1024), tc_smem_desc(bb[seg] + j * 2048, 16384, 1024), idesc,
+          ptx::umma_bf16_by<false>(leader, tmem_base, tc_smem_desc(aa[seg] + j * 2048, 16384, 1024), tc_smem_desc(bb[seg] + j * 2048, 16384, 1024), idesc,
                          (seg > 0 || j > 0) ? 1u : 0u);
-      ptx::umma_commit(&aux->mbar);
+      ptx::umma_commit_by<false>(leader, ptx::smem_u32(&aux->mbar));
+      __syncwarp();
     }
     if (!__syncthreads_and(tc_wait(&aux->mbar, ph, &aux->abort_flag) ? 1 : 0)) { ok = false; break; }
     ph ^= 1u;
