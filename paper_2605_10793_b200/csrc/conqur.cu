@@ -18,6 +18,7 @@
 #include "conqur_simt.cuh"
 #include "conqur_tc.cuh"
 #include "conqur_tc_batched.cuh"
+#include "conqur_split_tc.cuh"
 #include "conqur_aux.cuh"
 #include "conqur_hadamard_tc.cuh"
 #include "ns_schedule.h"
@@ -36,6 +37,7 @@ struct Layout {
   size_t Xa, Xb, E, B;      // Newton-Schulz fp32 matrices (P x d x d each)
   size_t splitk;            // exact accumulate split-K partials
   TcLayout tc;              // tensor-core mode buffers
+  SpLayout sp;              // exact mode: bf16 pieces of the rows, targets and R (ldp == 0: none)
   size_t total;
   int64_t max_partials;
   int acc_splits;
@@ -105,6 +107,8 @@ bool make_layout(int d, const conqur_config* c, Layout* L) {
   mp = std::max<int64_t>(mp, cdiv(n, 8));
   mp = std::max<int64_t>(mp, 2 * (int64_t)cdiv(d, 128) * cdiv(d, 128) + 64);   // two partial arrays per Newton-Schulz product
   mp = std::max<int64_t>(mp, 1024);
+  const bool pieces = c->mode == CONQUR_EXACT_F32 && sp_layout_wanted(d, (int)P);
+  if (pieces) mp = std::max<int64_t>(mp, 16 * (int64_t)cdiv(n, 256) * cdiv(d, 128));   // sixteen per tile of at least 256 x 128
   L->max_partials = mp;
   L->part_d = take(sizeof(double) * mp * P);
   L->part_f = take(sizeof(float) * mp * P);
@@ -113,6 +117,7 @@ bool make_layout(int d, const conqur_config* c, Layout* L) {
   L->obj_out = take(16 * P);                         // J (double) and N (int64) of every problem, for the asynchronous read
   L->acc_splits = 1;
   L->C = L->splitk = 0;
+  L->sp = SpLayout{};
   // the four Newton-Schulz matrices form ONE region: a token-split per-head step borrows all of it as scratch
   const size_t ns_one = align_up(sizeof(float) * dd * P);
   L->Xa = take(4 * ns_one);
@@ -123,6 +128,7 @@ bool make_layout(int d, const conqur_config* c, Layout* L) {
     L->C = take(sizeof(float) * (size_t)n * d * P);
     L->acc_splits = pick_acc_splits(d, (int)P, n);
     if (L->acc_splits > 1) L->splitk = take(sizeof(float) * dd * P * L->acc_splits);
+    if (pieces) sp_make_layout(d, n, c->in_dtype, &L->sp, take);
   } else {
     if ((c->quant_bits || c->diagnostics) && P == 1) L->C = take(sizeof(float) * (size_t)n * d);
     tc_make_layout(d, (int)P, n, c->quant_bits, c->in_dtype, &L->tc, take);
@@ -142,6 +148,8 @@ struct conqur_ctx {
   std::vector<int64_t> tokens_at_update;   // ... as they stood when the last update was enqueued (restored if it is rejected)
   int64_t last_n;            // rows per problem of the last step (for debug_get_signs)
   int last_np;               // problems the last step call covered
+  bool last_pieces = false;  // the last step left its targets as bf16 pieces (exact mode)
+  int device = 0, sp_pairs = 0;   // exact contexts with pieces: CTA pairs that can be co-resident (0: CUDA cores only)
   int64_t pending_rows = 0;  // deferring context: rows staged but not yet run through the two products
   int pending_batches = 0;
   int8_t* sign_capture = nullptr;   // conqur_debug_capture_signs: where the fused per-head kernel writes its decisions
@@ -248,12 +256,81 @@ int sync_status(conqur_ctx* c) {
 int ew_blocks(int64_t count) { return (int)std::min<int64_t>(148 * 8, (count + 255) / 256); }
 
 // ---------------------------------------------------------------- exact-mode step
+__nv_bfloat16* sp_ptr(const conqur_ctx* c, size_t off) { return c->at<__nv_bfloat16>(off); }
+
+// The pieces of R^T follow R.
+int sp_refresh_R(conqur_ctx* c) {
+  if (c->sp_pairs == 0) return CONQUR_OK;
+  const int d = c->cfg.d, t = cdiv(d, 32);
+  const SpLayout& L = c->L.sp;
+  sp_split_rt_kernel<<<dim3(t, t), 256, 0, c->stream>>>(c->at<float>(c->L.R), d, sp_ptr(c, L.Rp), L.ldp, d * L.ldp);
+  CQ_LAUNCHED(c, K_OTHER);
+  return CONQUR_OK;
+}
+
+// One problem's step with both products on the tensor cores (see conqur_split_tc.cuh).
+template <typename TIn>
+int step_pieces(conqur_ctx* c, const TIn* X, int64_t n, int64_t ld) {
+  const Cfg& g = c->cfg;
+  const SpLayout& L = c->L.sp;
+  const int d = g.d;
+  float* rnorm = c->at<float>(c->L.rnorm);
+  float* rs = c->at<float>(L.rs);
+  double* part = c->at<double>(c->L.part_d);
+  const int64_t xpiece = n * L.ldp;                       // the pieces of this step's rows lie one behind another
+  sp_stage_kernel<TIn><<<(unsigned)n, 128, 0, c->stream>>>(X, n, d, ld, rnorm, rs, sp_ptr(c, L.Xp), L.ldp, xpiece, c->state());
+  CQ_LAUNCHED(c, K_ROWNORM);
+  const int bn = sp_pick_bn(n, d, c->sp_pairs, false), bm = sp_pick_bn(d, d, c->sp_pairs, true);
+  CUtensorMap xk, rk, xm, sm;
+  int rc = sp_make_tmap(&xk, sp_ptr(c, L.Xp), n, d, L.ldp, L.px, xpiece, TC_BM);
+  rc |= sp_make_tmap(&rk, sp_ptr(c, L.Rp), d, d, L.ldp, 3, d * L.ldp, bn / 2);
+  rc |= sp_make_tmap(&xm, sp_ptr(c, L.Xp), n, d, L.ldp, L.px, xpiece, TC_BK);
+  rc |= sp_make_tmap(&sm, sp_ptr(c, L.Sp), n, d, L.ldp, L.pc, xpiece, TC_BK);
+  if (rc) return CONQUR_ERR_CUDA;
+  SpArgs a{};
+  a.M = (int)n; a.N = d; a.K = d; a.pa = L.px; a.pb = 3;
+  a.rs = rs; a.part_d = part; a.st = c->state();
+  a.outS = sp_ptr(c, L.Sp); a.lds = L.ldp; a.s_piece = xpiece; a.pc = L.pc;
+  double* pdiag = g.diagnostics ? c->at<double>(c->L.part_diag) : nullptr;
+  int per_problem;
+  if (g.quant_bits == 0 && !g.diagnostics) {
+    rc = sp_launch<SP_EPI_ROTATE>(bn, c->device, c->sp_pairs, c->stream, xk, rk, a);
+    if (rc) return rc;
+    c->prof.count(K_ROTATE);
+    per_problem = (int)(16 * sp_tiles(n, d, bn));
+  } else {
+    a.rowmax = c->at<unsigned>(c->L.rowmax); a.rowmin = a.rowmax + g.n_max;
+    a.outF = c->at<float>(c->L.C); a.ldo = d;
+    CQ_CUDA(cudaMemsetAsync(a.rowmax, 0, sizeof(unsigned) * n, c->stream));
+    CQ_CUDA(cudaMemsetAsync(a.rowmin, 0xff, sizeof(unsigned) * n, c->stream));
+    rc = sp_launch<SP_EPI_ROTATE_Q>(bn, c->device, c->sp_pairs, c->stream, xk, rk, a);
+    if (rc) return rc;
+    c->prof.count(K_ROTATE);
+    sp_quant_target_kernel<<<cdiv(n, 8), 256, 0, c->stream>>>(a.outF, n, d, rnorm, rs, a.rowmax, a.rowmin, g.qs, part, a.outS,
+                                                              L.ldp, xpiece, L.pc, pdiag);
+    CQ_LAUNCHED(c, K_OTHER);
+    per_problem = cdiv(n, 8);
+  }
+  finalize_step_kernel<<<1, 256, 0, c->stream>>>(c->state(), part, per_problem, n, 1.0 / std::sqrt((double)d), pdiag,
+                                                 pdiag ? cdiv(n, 8) : 0);
+  CQ_LAUNCHED(c, K_OTHER);
+  SpArgs m{};
+  m.M = d; m.N = d; m.K = (int)n; m.pa = L.px; m.pb = L.pc; m.st = c->state();
+  m.outF = c->at<float>(c->L.M); m.ldo = d;
+  rc = sp_launch<SP_EPI_ACCUM>(bm, c->device, c->sp_pairs, c->stream, xm, sm, m);
+  if (rc) return rc;
+  c->prof.count(K_ACCUM);
+  return CONQUR_OK;
+}
+
 template <typename TIn>
 int step_exact(conqur_ctx* c, const TIn* X, int64_t n, int64_t ld, int64_t pstride, int p0, int np) {
   // problems [p0, p0 + np): state, R and M are theirs; the per-step scratch (row norms, targets, partials) is used
   // from its start
   const Cfg& g = c->cfg;
   const int d = g.d, P = np;
+  c->last_pieces = c->sp_pairs > 0 && sp_takes(n, d, g.in_dtype == CONQUR_F32);
+  if (c->last_pieces) return step_pieces(c, X, n, ld);
   const int64_t pdd = (int64_t)p0 * d * d;
   DevState* st = c->state() + p0;
   float* rnorm = c->at<float>(c->L.rnorm);
@@ -438,6 +515,8 @@ int update_epilogue(conqur_ctx* c) {
     ns_commit_kernel<<<dim3(ew_blocks(dd), g.P), 256, 0, c->stream>>>(st, c->at<float>(c->L.Xa), c->at<float>(c->L.Xb),
                                                                      c->at<float>(c->L.R), c->at<float>(c->L.M), dd);
     CQ_LAUNCHED(c, K_OTHER);
+    int rc = sp_refresh_R(c);
+    if (rc) return rc;
   } else {
     int rc = tc_ns_commit(c->tc, c->stream);
     if (rc) return rc;
@@ -696,6 +775,13 @@ extern "C" int conqur_init(conqur_ctx** out, int32_t d, const conqur_config* cfg
     rc = tc_refresh_R(c->tc, c->stream, 0);
     if (rc) return fail(rc);
   }
+  if (L.sp.ldp) {
+    TcDevFacts f;
+    if (cudaGetDevice(&c->device) != cudaSuccess || tc_device_facts(c->device, &f) != CONQUR_OK) return fail(CONQUR_ERR_CUDA);
+    c->sp_pairs = (g.debug_flags & CONQUR_DEBUG_SINGLE_CTA) ? 0 : f.pair_clusters;
+    const int rc = sp_refresh_R(c);
+    if (rc) return fail(rc);
+  }
   if (cudaStreamSynchronize(c->stream) != cudaSuccess) return fail(CONQUR_ERR_CUDA);   // coef is a local
   *out = c;
   return CONQUR_OK;
@@ -775,7 +861,7 @@ extern "C" int conqur_set_R(conqur_ctx* c, const float* R_dev) {
   if (g.mode == CONQUR_TC_BF16 && aligned) return tc_take_R(c->tc, c->stream, R_dev);
   CQ_CUDA(cudaMemcpyAsync(c->at<float>(c->L.R), R_dev, sizeof(float) * dd * g.P, cudaMemcpyDeviceToDevice, c->stream));
   if (g.mode == CONQUR_TC_BF16) return tc_refresh_R(c->tc, c->stream, 0);
-  return CONQUR_OK;
+  return sp_refresh_R(c);
 }
 
 static int step_common(conqur_ctx* c, const void* X, int64_t n, int64_t ld, int64_t pstride, int p0, int np) {
@@ -947,10 +1033,13 @@ extern "C" int conqur_debug_get_signs(conqur_ctx* c, int8_t* S_out_dev, int64_t 
   const int64_t total = c->last_n * g.d;
   const dim3 grid(ew_blocks(total), c->last_np);
   if (g.mode == CONQUR_EXACT_F32) {
-    signs_from_c_kernel<<<grid, 256, 0, c->stream>>>(c->at<float>(c->L.C), nullptr, c->last_n, g.d, (int64_t)g.n_max * g.d,
-                                                     S_out_dev);
+    if (c->last_pieces)                                  // (the first piece has the target's sign)
+      signs_from_c_kernel<<<grid, 256, 0, c->stream>>>(nullptr, sp_ptr(c, c->L.sp.Sp), c->last_n, g.d, c->L.sp.ldp, 0, S_out_dev);
+    else
+      signs_from_c_kernel<<<grid, 256, 0, c->stream>>>(c->at<float>(c->L.C), nullptr, c->last_n, g.d, g.d, (int64_t)g.n_max * g.d,
+                                                       S_out_dev);
   } else {
-    signs_from_c_kernel<<<grid, 256, 0, c->stream>>>(nullptr, tc_cp_ptr(c->tc), c->last_n, g.d, 0, S_out_dev);
+    signs_from_c_kernel<<<grid, 256, 0, c->stream>>>(nullptr, tc_cp_ptr(c->tc), c->last_n, g.d, g.d, 0, S_out_dev);
   }
   CQ_LAUNCHED(c, K_OTHER);
   return sync_status(c);

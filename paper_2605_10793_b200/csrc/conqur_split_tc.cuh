@@ -1,0 +1,585 @@
+// The fp32 step's two products on the tensor cores, at no less than fp32's precision.
+//
+// An fp32 number is the sum of three bf16 numbers (8 bits each, exactly: x = p0 + p1 + p2), so an fp32 product is six bf16
+// products, p0 q0 + (p0 q1 + p1 q0) + (p0 q2 + p1 q1 + p2 q0); what is left out lies 2^-26 below a term.  bf16 rows and sign
+// targets are one piece, which leaves three products.  The tensor cores cut what they add (2^-23 of the sum, once per
+// instruction of 16 terms), so a long sum kept in TMEM loses more than an fp32 chain does.  Here an accumulator holds 64 terms
+// only, small pieces first; the epilogue warps then add it to running sums in their registers, in fp32, round to nearest.
+// Error of a rotated row, in 2^-24 of its norm, fp32 chain of fused multiply-adds / this (rows of the calibration recipe):
+// K = 64 2.9 / 2.4, 128 3.7 / 1.4, 512 6.8 / 2.1, 1024 9.8 / 2.5, 3072 19.6 / 3.1; all terms in one accumulator: 77 at 3072.
+//
+// What bounds it: the tensor cores and, with them busy, the board's power (128 cycles per 256 x 256 x 16 instruction of a CTA pair, 24
+// of them per k block of 64 with six products), where the CUDA cores' product is bound by its shared-memory reads.  1000 x 3072
+// fp32 rows: rotate 504 -> 95 us (116 Gflop of bf16 products: 1.2 PFLOP/s on 64 of 74 pairs), accumulate 409 -> 57, staging
+// 8 -> 8; the whole step 889 -> 165.  Operand pieces arrive at 32 B/clk per SM and the sums leave TMEM at 43 B/clk, both below
+// what one-product kernels take.  (Releasing a stage piece by piece instead of whole: 97 -> 110; 128 terms an accumulator would
+// halve the sums' traffic and cost accuracy: 4.0 instead of 3.1 at K = 3072.)
+#pragma once
+#include "conqur_simt.cuh"
+#include "conqur_tc.cuh"
+
+namespace conqur {
+
+enum { SP_EPI_ROTATE = 0, SP_EPI_ROTATE_Q = 1, SP_EPI_ACCUM = 2 };
+
+constexpr int SP_STAGES_MAX = 6;
+constexpr int SP_THREADS = 384;                          // a warpgroup that loads and issues, two that add up
+constexpr int SP_REGS_ISSUE = 56, SP_REGS_EPI = 208;     // registers a thread (launched with 168: 56 + 2 x 208 <= 3 x 168)
+constexpr int SP_RING_BYTES = 196608;                    // operand tiles: two stages of 3 + 3 pieces
+constexpr int SP_SMEM_BYTES = SP_RING_BYTES + 1024 + 8 * 4096 + 1024;   // ring, barriers, transposition buffers, alignment slack
+
+struct SpArgs {
+  int M, N, K;
+  int pa, pb;                                            // pieces of A and of B: 1 or 3
+  int n_stages, stage_bytes;
+  float* outF; long long ldo;                            // Y (quantised targets) or M
+  __nv_bfloat16* outS; long long lds, s_piece; int pc;   // targets: pc pieces, s_piece elements apart
+  const float* rs;                                       // the targets' row scale (and the objective's)
+  unsigned *rowmax, *rowmin;
+  double* part_d;                                        // objective partials: sixteen per tile (a warp's of either CTA)
+  DevState* st;
+};
+
+struct SpAux {
+  uint64_t full[SP_STAGES_MAX], empty[SP_STAGES_MAX], tfull[2], tempty[2];
+  uint32_t tmem_base;
+  int abort_flag;
+};
+static_assert(sizeof(SpAux) <= 1024, "reserved behind the ring");
+
+namespace ptx {
+// box of a 3-D map (column, row, piece) into this CTA's shared memory, its bytes counted on a barrier of the pair
+__device__ __forceinline__ void tma_load_3d_pair(void* smem_dst, const CUtensorMap* tmap, uint32_t bar_cluster_addr, int x, int y,
+                                                 int z) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+      ::"r"(smem_u32(smem_dst)), "l"(tmap), "r"(bar_cluster_addr), "r"(x), "r"(y), "r"(z)
+      : "memory");
+}
+template <int N> __device__ __forceinline__ void regs_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N> __device__ __forceinline__ void regs_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+// 32 lanes x 32 consecutive fp32 columns.  The wait is tied to r, so that no use of it can move in front.
+__device__ __forceinline__ void tmem_ld32_tied(uint32_t taddr, uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr)
+      : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]),
+                 "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]),
+                 "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]),
+                 "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
+               :
+               : "memory");
+}
+// ... 16 columns
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]),
+                 "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :
+               : "memory");
+}
+}  // namespace ptx
+
+// Three bf16 pieces of v (+ rest, a remainder below v's last bit).
+__device__ __forceinline__ void sp_split(float v, float rest, uint32_t& p0, uint32_t& p1, uint32_t& p2) {
+  p0 = bf16_bits(v);
+  const float r1 = v - __uint_as_float(p0 << 16);
+  p1 = bf16_bits(r1);
+  p2 = bf16_bits((r1 - __uint_as_float(p1 << 16)) + rest);
+}
+
+// Two numbers at a time: packed pieces, the first number in the low half.  e0, e1: remainders below their last bits.
+__device__ __forceinline__ void sp_split2(float a, float b, float e0, float e1, uint32_t& w0, uint32_t& w1, uint32_t& w2) {
+  w0 = bf16x2_pack(a, b);
+  const float ra = a - __uint_as_float(w0 << 16), rb = b - __uint_as_float(w0 & 0xffff0000u);
+  w1 = bf16x2_pack(ra, rb);
+  w2 = bf16x2_pack((ra - __uint_as_float(w1 << 16)) + e0, (rb - __uint_as_float(w1 & 0xffff0000u)) + e1);
+}
+__device__ __forceinline__ void sp_split2(float a, float b, uint32_t& w0, uint32_t& w1, uint32_t& w2) {
+  w0 = bf16x2_pack(a, b);
+  const float ra = a - __uint_as_float(w0 << 16), rb = b - __uint_as_float(w0 & 0xffff0000u);
+  w1 = bf16x2_pack(ra, rb);
+  w2 = bf16x2_pack(ra - __uint_as_float(w1 << 16), rb - __uint_as_float(w1 & 0xffff0000u));
+}
+
+// A 32 x 32 fp32 block (lane = row) through the warp's transposition buffer to `out`: stored, or added with reductions at the
+// L2.  Rows and columns past rows_ok / cols_ok are left out; 16-byte pieces where the block is whole and its rows aligned.
+template <bool ADD>
+__device__ __forceinline__ void sp_put_block(uint8_t* stg, int lane, const float (&v)[32], float* out, long long ld, int rows_ok,
+                                             int cols_ok) {
+  if (cols_ok >= 32 && (ld & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
+    if (ADD) tc_red_block_f32(stg, lane, v, out, ld, rows_ok); else tc_store_block_f32(stg, lane, v, out, ld, rows_ok);
+    return;
+  }
+#pragma unroll
+  for (int p = 0; p < 8; ++p)
+    *reinterpret_cast<float4*>(stg + lane * 128 + ((p ^ (lane & 7)) << 4)) = make_float4(v[4 * p], v[4 * p + 1], v[4 * p + 2], v[4 * p + 3]);
+  __syncwarp();
+  if (lane < cols_ok)
+    for (int r = 0; r < rows_ok; ++r) {
+      const float t = *reinterpret_cast<const float*>(stg + r * 128 + (((lane >> 2) ^ (r & 7)) << 4) + (lane & 3) * 4);
+      if (ADD) atomicAdd(out + (long long)r * ld + lane, t); else out[(long long)r * ld + lane] = t;
+    }
+  __syncwarp();
+}
+
+// D[m][n] = sum_k A(m, k) B(n, k) on 256 x BN tiles of CTA pairs, operands as stacks of bf16 pieces (3-D maps: column, row,
+// piece).  Warp 0 loads, warp 1 issues (CTA 0 for both), warps 2-9 add up the accumulators and write the tile.
+//   ROTATE    A = X (K-major), B = R^T (K-major): targets sgn(y) * rs as pc bf16 pieces, objective partials sum |y| rs
+//   ROTATE_Q  the same products, stored as fp32 Y with the row's range
+//   ACCUM     A = X, B = targets (both MN-major, contraction over rows): added to M, once per element and launch
+template <int BN, int EPI>
+__global__ void __launch_bounds__(SP_THREADS, 1)
+sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const SpArgs g) {
+  constexpr bool MN = EPI == SP_EPI_ACCUM;               // orientation of both operands
+  static_assert(!MN || BN % 128 == 0, "MN-major tiles are 64 columns wide in each CTA of the pair");
+  constexpr int A_BYTES = TC_BM * TC_BK * 2, B_ROWS = BN / 2, B_BYTES = B_ROWS * TC_BK * 2;
+  constexpr int HALF = BN / 2, BLOCKS = HALF / 32;       // columns of the tile a warp adds up
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  SpAux* aux = reinterpret_cast<SpAux*>(smem + SP_RING_BYTES);
+  volatile int* abort_flag = &aux->abort_flag;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
+  const uint32_t rank = ptx::cluster_ctarank();
+  const int worker = (int)(blockIdx.x >> 1), n_workers = (int)(gridDim.x >> 1);
+  const int tiles_m = (g.M + 255) / 256, tiles_n = (g.N + BN - 1) / BN, num_tiles = tiles_m * tiles_n;
+  const int num_kb = (g.K + TC_BK - 1) / TC_BK;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < g.n_stages; ++s) { ptx::mbar_init(&aux->full[s], 1); ptx::mbar_init(&aux->empty[s], 1); }
+    for (int b = 0; b < 2; ++b) { ptx::mbar_init(&aux->tfull[b], 1); ptx::mbar_init(&aux->tempty[b], 16); }   // a warp's one arrival, both CTAs
+    aux->abort_flag = 0;
+    ptx::fence_barrier_init();
+    ptx::fence_proxy_async();
+    ptx::prefetch_tmap(&tmA);
+    ptx::prefetch_tmap(&tmB);
+  }
+  if (warp == 1) { ptx::tmem_alloc_pair(&aux->tmem_base, 512); ptx::tmem_relinquish_pair(); }
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::cluster_sync_all();
+  ptx::tc_fence_after();
+  const uint32_t tmem_base = aux->tmem_base;
+  int timeout_site = 0;
+
+  if (warp < 4) {
+    ptx::regs_dec<SP_REGS_ISSUE>();
+    if (warp == 0 && lane == 0) {
+      int stage = 0;
+      uint32_t phase = 0;
+      bool ok = true;
+      for (int tile = worker; tile < num_tiles && ok; tile += n_workers) {
+        int tm, tn;
+        tc_tile_coords<1>(tile, tiles_m, tiles_n, 0, tm, tn);
+        const int m0 = tm * 256 + (int)rank * TC_BM, n0 = tn * BN + (int)rank * B_ROWS;
+        for (int kb = 0; kb < num_kb; ++kb) {
+          if (!tc_wait(&aux->empty[stage], phase ^ 1u, abort_flag)) { ok = false; timeout_site = 1; break; }
+          uint8_t* sa = smem + stage * g.stage_bytes;
+          uint8_t* sb = sa + g.pa * A_BYTES;
+          const uint32_t bar = ptx::mapa_u32(ptx::smem_u32(&aux->full[stage]), 0);
+          if (rank == 0) ptx::mbar_expect_tx(&aux->full[stage], 2 * (g.pa * A_BYTES + g.pb * B_BYTES));
+          const int k0 = kb * TC_BK;
+          for (int p = 0; p < g.pa; ++p) {
+            if (MN) {
+#pragma unroll
+              for (int h = 0; h < TC_BM / 64; ++h) ptx::tma_load_3d_pair(sa + p * A_BYTES + h * 8192, &tmA, bar, m0 + 64 * h, k0, p);
+            } else {
+              ptx::tma_load_3d_pair(sa + p * A_BYTES, &tmA, bar, k0, m0, p);
+            }
+          }
+          for (int p = 0; p < g.pb; ++p) {
+            if (MN) {
+#pragma unroll
+              for (int h = 0; h < B_ROWS / 64; ++h) ptx::tma_load_3d_pair(sb + p * B_BYTES + h * 8192, &tmB, bar, n0 + 64 * h, k0, p);
+            } else {
+              ptx::tma_load_3d_pair(sb + p * B_BYTES, &tmB, bar, k0, n0, p);
+            }
+          }
+          if (++stage == g.n_stages) { stage = 0; phase ^= 1u; }
+        }
+      }
+      if (!ok) {                                         // copies in flight are counted in the other CTA: give them a fixed time
+        const long long t0 = clock64();
+        while (clock64() - t0 < 4000000ll) {}
+      }
+    } else if (warp == 1 && rank == 0) {
+      const uint32_t leader = ptx::elect_one();
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((MN ? 1u : 0u) << 15) | ((MN ? 1u : 0u) << 16) |
+                             ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
+      const uint64_t ab0 = tc_smem_desc(ptx::smem_u32(smem), MN ? 8192 : 16, 1024);      // (addresses in units of 16 bytes)
+      constexpr uint32_t STEP = MN ? 2048 / 16 : 32 / 16;
+      const uint32_t full0 = ptx::smem_u32(&aux->full[0]);
+      const uint32_t empty0 = full0 + (uint32_t)(offsetof(SpAux, empty) - offsetof(SpAux, full));
+      const uint32_t tfull0 = full0 + (uint32_t)(offsetof(SpAux, tfull) - offsetof(SpAux, full));
+      int stage = 0;
+      uint32_t phase = 0, n_acc = 0;
+      bool ok = true;
+      for (int tile = worker; tile < num_tiles && ok; tile += n_workers) {
+        for (int kb = 0; kb < num_kb; ++kb, ++n_acc) {
+          const uint32_t buf = n_acc & 1u;
+          if (!tc_wait_warp(&aux->tempty[buf], ((n_acc >> 1) & 1u) ^ 1u, abort_flag)) { ok = false; timeout_site = 2; break; }
+          if (!tc_wait_warp(&aux->full[stage], phase, abort_flag)) { ok = false; timeout_site = 3; break; }
+          ptx::tc_fence_after();
+          const uint64_t sa = ab0 + ((uint32_t)(stage * g.stage_bytes) >> 4), sb = sa + (uint32_t)(g.pa * (A_BYTES / 16));
+          const uint32_t d_tmem = tmem_base + buf * 256u;
+          uint32_t acc = 0;
+          for (int sum = min(2, g.pa + g.pb - 2); sum >= 0; --sum)          // piece numbers add up to 2, 1, 0: small products first
+            for (int i = max(0, sum - (g.pb - 1)); i <= min(sum, g.pa - 1); ++i) {
+              const uint64_t ad = sa + (uint32_t)(i * (A_BYTES / 16)), bd = sb + (uint32_t)((sum - i) * (B_BYTES / 16));
+#pragma unroll
+              for (int j = 0; j < TC_BK / 16; ++j) {
+                ptx::umma_bf16_by<true>(leader, d_tmem, ad + j * STEP, bd + j * STEP, idesc, acc);
+                acc = 1u;
+              }
+            }
+          ptx::umma_commit_by<true>(leader, empty0 + (uint32_t)stage * 8u);
+          ptx::umma_commit_by<true>(leader, tfull0 + buf * 8u);
+          if (++stage == g.n_stages) { stage = 0; phase ^= 1u; }
+        }
+      }
+    }
+  } else {
+    ptx::regs_inc<SP_REGS_EPI>();
+    const int q = warp & 3, half = (warp >> 2) - 1, ew = warp - 4;
+    uint8_t* stg = smem + SP_RING_BYTES + 1024 + ew * 4096;
+    const uint32_t tempty0 = ptx::mapa_u32(ptx::smem_u32(&aux->tempty[0]), 0);
+    const uint32_t t_lane = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * HALF);
+    uint32_t n_acc = 0;
+    bool ok = true;
+    for (int tile = worker; tile < num_tiles && ok; tile += n_workers) {
+      int tm, tn;
+      tc_tile_coords<1>(tile, tiles_m, tiles_n, 0, tm, tn);
+      float acc[HALF];
+#pragma unroll
+      for (int i = 0; i < HALF; ++i) acc[i] = 0.f;
+      for (int kb = 0; kb < num_kb; ++kb, ++n_acc) {
+        const uint32_t buf = n_acc & 1u;
+        if (!tc_wait(&aux->tfull[buf], (n_acc >> 1) & 1u, abort_flag)) { ok = false; timeout_site = 4; break; }
+        ptx::tc_fence_after();
+#pragma unroll
+        for (int c = 0; c < BLOCKS; ++c) {
+          uint32_t r[32];
+          ptx::tmem_ld32_tied(t_lane + buf * 256u + (uint32_t)(c * 32), r);
+#pragma unroll
+          for (int i = 0; i < 32; ++i) acc[c * 32 + i] += __uint_as_float(r[i]);
+        }
+        ptx::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive_cluster(tempty0 + buf * (uint32_t)sizeof(uint64_t));
+      }
+      if (!ok) break;
+      const int wrow0 = tm * 256 + (int)rank * TC_BM + q * 32, row = wrow0 + lane;
+      const int rows_ok = min(32, max(0, g.M - wrow0));
+      const bool row_ok = row < g.M;
+      float rs = 0.f;
+      uint32_t p0 = 0, p1 = 0, p2 = 0;
+      if (EPI != SP_EPI_ACCUM) {
+        rs = row_ok ? g.rs[row] : 0.f;
+        sp_split(rs, 0.f, p0, p1, p2);
+      }
+      double sum = 0.0;
+      float vmax = -3.0e38f, vmin = 3.0e38f;
+#pragma unroll
+      for (int c = 0; c < BLOCKS; ++c) {
+        const int col0 = tn * BN + half * HALF + c * 32;
+        if (rows_ok == 0 || col0 >= g.N) continue;       // uniform over the warp
+        const int cols_ok = min(32, g.N - col0);
+        float v[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[i] = row_ok ? acc[c * 32 + i] : 0.f;
+        if (EPI == SP_EPI_ROTATE) {
+#pragma unroll
+          for (int h = 0; h < 4; ++h) {                  // eight terms in fp32, then in double
+            float a = 0.f;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) a += fabsf(v[h * 8 + i]);
+            sum += (double)a;
+          }
+          const uint32_t bits[3] = {p0, p1, p2};
+#pragma unroll
+          for (int p = 0; p < 3; ++p) {
+            if (p >= g.pc) break;
+            uint32_t w[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              const float a = v[2 * i], b = v[2 * i + 1];
+              const uint32_t lo = (a == 0.f) ? 0u : (bits[p] ^ ((__float_as_uint(a) >> 16) & 0x8000u));
+              const uint32_t hi = (b == 0.f) ? 0u : (bits[p] ^ ((__float_as_uint(b) >> 16) & 0x8000u));
+              w[i] = lo | (hi << 16);
+            }
+            // (the targets' rows are padded to 64 columns; columns past N hold the zero operand's zeros)
+            tc_store_block_bf16(stg, lane, w, g.outS + p * g.s_piece + (long long)wrow0 * g.lds + col0, g.lds, rows_ok);
+          }
+        } else if (EPI == SP_EPI_ROTATE_Q) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            if (i < cols_ok) { vmax = fmaxf(vmax, v[i]); vmin = fminf(vmin, v[i]); }
+          sp_put_block<false>(stg, lane, v, g.outF + (long long)wrow0 * g.ldo + col0, g.ldo, rows_ok, cols_ok);
+        } else {
+          sp_put_block<true>(stg, lane, v, g.outF + (long long)wrow0 * g.ldo + col0, g.ldo, rows_ok, cols_ok);
+        }
+      }
+      if (EPI == SP_EPI_ROTATE_Q) {
+        if (rs > 0.f) { atomicMax(g.rowmax + row, f2ord(vmax)); atomicMin(g.rowmin + row, f2ord(vmin)); }
+      }
+      if (EPI == SP_EPI_ROTATE) {
+        const double t = warp_sum_d(sum * (double)rs);
+        if (lane == 0) g.part_d[(2 * tile + (int)rank) * 8 + ew] = t;
+      }
+    }
+  }
+
+  if (timeout_site != 0) {
+    atomicOr(&g.st->status_flags, STATUS_FLAG_TIMEOUT);
+    g.st->timeout_site = timeout_site;
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::cluster_sync_all();
+  if (warp == 1) {
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc_pair(tmem_base, 512);
+  }
+}
+
+// a1: row norms in fp32, and the rows as bf16 pieces; skipped rows are zeros.  bf16 rows are their own single piece (targets then
+// carry 1/||x||, rs = rnorm); fp32 rows are normalised first, the product x * rnorm split with its rounding error (rs = 1).
+// Four warps a row, whose pieces of it stay in the L1 between the two passes (1000 x 3072 fp32 rows: one warp a row 14.1 us).
+template <typename TIn>
+__global__ void __launch_bounds__(128) sp_stage_kernel(const TIn* __restrict__ X, int64_t n, int d, int64_t ld, float* __restrict__ rnorm,
+                                                       float* __restrict__ rs, __nv_bfloat16* __restrict__ Xp, int64_t ldp,
+                                                       int64_t piece, DevState* st) {
+  __shared__ float part[4];
+  const int64_t row = blockIdx.x;
+  const int lane = threadIdx.x & 31;
+  const TIn* x = X + row * ld;
+  const bool vec = ((d & 3) == 0) && ((reinterpret_cast<uintptr_t>(x) & (sizeof(TIn) * 4 - 1)) == 0);
+  auto load = [&](int k, float (&v)[4]) {
+    if (vec) {
+      ld4_as_float(x + k, v);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] = k + j < d ? ld_as_float(x + k + j) : 0.f;
+    }
+  };
+  float ss = 0.f;
+#pragma unroll 2
+  for (int k = (int)threadIdx.x * 4; k < d; k += 512) {
+    float v[4];
+    load(k, v);
+    ss = fmaf(v[0], v[0], ss); ss = fmaf(v[1], v[1], ss); ss = fmaf(v[2], v[2], ss); ss = fmaf(v[3], v[3], ss);
+  }
+  ss = warp_sum(ss);
+  if (lane == 0) part[threadIdx.x >> 5] = ss;
+  __syncthreads();
+  ss = (part[0] + part[1]) + (part[2] + part[3]);
+  const bool good = ss > 0.f && ss <= 3.0e38f;
+  const float r = good ? 1.0f / sqrtf(ss) : 0.f;
+  __nv_bfloat16* dst = Xp + row * ldp;
+#pragma unroll 2
+  for (int k = (int)threadIdx.x * 4; k < d; k += 512) {  // (rows of Xp are padded to 64 elements)
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+    if (good) load(k, v);
+    if (sizeof(TIn) == 2) {
+      *reinterpret_cast<uint2*>(dst + k) = make_uint2(bf16x2_pack(v[0], v[1]), bf16x2_pack(v[2], v[3]));
+    } else {
+      uint2 p[3];
+      float t[4], e[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) { t[j] = v[j] * r; e[j] = fmaf(v[j], r, -t[j]); }
+      sp_split2(t[0], t[1], e[0], e[1], p[0].x, p[1].x, p[2].x);
+      sp_split2(t[2], t[3], e[2], e[3], p[0].y, p[1].y, p[2].y);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) *reinterpret_cast<uint2*>(dst + i * piece + k) = p[i];
+    }
+  }
+  if (threadIdx.x == 0) {
+    if (!good) {
+      atomicAdd(reinterpret_cast<unsigned long long*>(&st->step_skipped), 1ull);
+      if (!(ss == 0.f)) atomicOr(&st->status_flags, STATUS_FLAG_NONFINITE);
+    }
+    rnorm[row] = r;
+    rs[row] = sizeof(TIn) == 2 ? r : (good ? 1.f : 0.f);
+  }
+}
+
+// R^T as three pieces (row n, column k), rows ldp elements long: the rotate product then reads both operands along k.
+static __global__ void __launch_bounds__(256) sp_split_rt_kernel(const float* __restrict__ R, int d, __nv_bfloat16* __restrict__ Rp,
+                                                                 int64_t ldp, int64_t piece) {
+  __shared__ float t[32][33];
+  const int k0 = blockIdx.y * 32, n0 = blockIdx.x * 32, x = threadIdx.x & 31, y = threadIdx.x >> 5;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int k = k0 + y + 8 * i, n = n0 + x;
+    t[y + 8 * i][x] = (k < d && n < d) ? R[(int64_t)k * d + n] : 0.f;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int n = n0 + y + 8 * i, k = k0 + x;
+    if (n >= d || k >= d) continue;
+    uint32_t p[3];
+    sp_split(t[x][y + 8 * i], 0.f, p[0], p[1], p[2]);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) reinterpret_cast<unsigned short*>(Rp)[j * piece + (int64_t)n * ldp + k] = (unsigned short)p[j];
+  }
+}
+
+// Second pass of the two-pass step (see quant_target_kernel): Y -> target pieces, objective partials, diagnostics partials.
+static __global__ void __launch_bounds__(256) sp_quant_target_kernel(const float* __restrict__ Y, int64_t n, int d,
+                                                                     const float* __restrict__ rnorm, const float* __restrict__ rs,
+                                                                     const unsigned* __restrict__ rowmax_ord,
+                                                                     const unsigned* __restrict__ rowmin_ord, QuantSpec qs,
+                                                                     double* __restrict__ partials, __nv_bfloat16* __restrict__ S,
+                                                                     int64_t lds, int64_t piece, int pc, double* __restrict__ part_diag) {
+  const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  const bool diag = part_diag != nullptr;
+  double contrib = 0.0, dterm[4] = {0.0, 0.0, 0.0, 0.0};
+  if (row < n) {
+    const float r = rs[row];
+    RowQuant rq{0.f, 1.f, 0.f, 0.f};
+    if (qs.bits) rq = row_quant(qs, ord2f(rowmax_ord[row]), ord2f(rowmin_ord[row]), r > 0.f);
+    const bool live = qs.bits ? (rq.inv > 0.f) : (r > 0.f);
+    const float* y = Y + row * (int64_t)d;
+    unsigned short* s = reinterpret_cast<unsigned short*>(S) + row * lds;
+    uint32_t p[3];
+    sp_split(r, 0.f, p[0], p[1], p[2]);
+    float qsum = 0.f;
+    RowDiag dg{0.f, 0.f, 0.f, 0.f};
+    for (int j = lane; j < d; j += 32) {
+      const float sg = second_pass_elem(y[j], r, qs, rq, qsum, diag && live, dg);
+      const uint32_t neg = sg < 0.f ? 0x8000u : 0u;
+      const bool zero = !live || sg == 0.f;
+      for (int i = 0; i < pc; ++i) s[i * piece + j] = (unsigned short)(zero ? 0u : (p[i] ^ neg));
+    }
+    qsum = warp_sum(qsum);
+    if (live) contrib = (double)(r * rq.delta) * (double)qsum;
+    if (diag) row_diag_terms(dg, rnorm[row], d, live, dterm);
+  }
+  __shared__ double red[8][5];
+  if (lane == 0) {
+    red[threadIdx.x >> 5][0] = contrib;
+    for (int k = 0; k < 4; ++k) red[threadIdx.x >> 5][1 + k] = dterm[k];
+  }
+  __syncthreads();
+  if (threadIdx.x < 5) {
+    double t = 0.0;
+    for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x];
+    if (threadIdx.x == 0) partials[blockIdx.x] = t;
+    else if (diag) part_diag[(int64_t)(threadIdx.x - 1) * gridDim.x + blockIdx.x] = t;
+  }
+}
+
+// ------------------------------------------------------------------ host side
+// Contexts that lay the pieces out, and their steps that take them.  Whole step, CUDA cores -> this, us (one B200):
+//   fp32 rows, d = 384  n = 1000 49 -> 49, 2048 68 -> 66;  512  256 37 -> 41, 512 47 -> 45, 1000 70 -> 54;  640  256 45 -> 43;
+//              1024  64 49 -> 49, 128 55 -> 51, 1000 147 -> 68;  2048  16 72 -> 78, 64 82 -> 78;  3072  1000 889 -> 165, 2048 1668 -> 288
+//   bf16 rows, d = 320  2048 69 -> 66;  384  16 31 -> 33, 64 37 -> 33, 2048 82 -> 66;  1024  16 56 -> 43, 1000 178 -> 60;
+//              3072  2048 1833 -> 244
+// (below: too few 256-row tiles to fill the chip, and six products for one)
+constexpr int SP_MIN_D = 384;
+inline bool sp_takes(int64_t n, int d, bool f32) {
+  if (!f32) return d >= SP_MIN_D && n >= 64;
+  return n * d >= (d >= 1024 ? (int64_t)1 << 17 : (int64_t)1 << 18) && d >= 512;
+}
+struct SpLayout {
+  int64_t ldp;                                           // row length of all pieces: d rounded up to 64
+  int px, pc;                                            // pieces of the rows and of the targets
+  size_t Xp, Sp, Rp, rs;
+};
+inline bool sp_layout_wanted(int d, int P) { return P == 1 && d >= SP_MIN_D; }
+
+template <typename Take>
+inline void sp_make_layout(int d, int64_t n, int in_dtype, SpLayout* L, Take&& take) {
+  L->ldp = ((int64_t)d + 63) / 64 * 64;
+  L->px = in_dtype == CONQUR_F32 ? 3 : 1;
+  L->pc = in_dtype == CONQUR_F32 ? 1 : 3;
+  L->Xp = take((size_t)(2 * L->px * n * L->ldp));
+  L->Sp = take((size_t)(2 * L->pc * n * L->ldp));
+  L->Rp = take((size_t)(2 * 3 * d * L->ldp));
+  L->rs = take(sizeof(float) * (size_t)n);
+}
+
+// (column, row, piece) map over `pieces` bf16 matrices of rows x cols, `piece` elements apart; box 64 columns x box_rows.
+inline int sp_make_tmap(CUtensorMap* tm, const void* ptr, uint64_t rows, uint64_t cols, uint64_t ld, uint64_t pieces, uint64_t piece,
+                        uint32_t box_rows) {
+  PFN_encodeTiled fn = tc_encode_fn();
+  if (!fn) return CONQUR_ERR_CUDA;
+  const cuuint64_t dims[3] = {cols, rows, pieces};
+  const cuuint64_t strides[2] = {ld * 2, piece * 2};
+  const cuuint32_t box[3] = {64, box_rows, 1};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  const CUresult r = fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) {
+    std::fprintf(stderr, "conqur: cuTensorMapEncodeTiled (pieces) failed (%d)\n", (int)r);
+    return CONQUR_ERR_CUDA;
+  }
+  return CONQUR_OK;
+}
+
+// Tile width of a product of M x N outputs on `pairs` CTA pairs: the one with the least rounds x width.
+inline int sp_pick_bn(int64_t M, int64_t N, int pairs, bool mn) {
+  int best = 256;
+  double cost = 1e300;
+  for (int bn : {256, 192, 128}) {
+    if (mn && bn == 192) continue;                       // (MN-major tiles come 64 columns wide per CTA)
+    const int64_t tiles = ((M + 255) / 256) * ((N + bn - 1) / bn);
+    const double c = (double)((tiles + pairs - 1) / pairs) * (bn + 16);
+    if (c < cost) { cost = c; best = bn; }
+  }
+  return best;
+}
+inline int64_t sp_tiles(int64_t M, int64_t N, int bn) { return ((M + 255) / 256) * ((N + bn - 1) / bn); }
+
+template <int BN, int EPI>
+inline int sp_launch_bn(int device, int pairs, cudaStream_t s, const CUtensorMap& a, const CUtensorMap& b, SpArgs g) {
+  auto kern = sp_gemm_kernel<BN, EPI>;
+  static std::atomic<unsigned long long> attr_dev_mask{0};
+  const unsigned long long dev_bit = 1ull << (device & 63);
+  if (!(attr_dev_mask.load(std::memory_order_acquire) & dev_bit)) {
+    // the warpgroups' shares of registers come out of what the block is launched with: less, and they would wait for more forever
+    cudaFuncAttributes fa;
+    if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess || fa.numRegs * 3 < SP_REGS_ISSUE + 2 * SP_REGS_EPI) return CONQUR_ERR_CUDA;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SP_SMEM_BYTES) != cudaSuccess) return CONQUR_ERR_CUDA;
+    attr_dev_mask.fetch_or(dev_bit, std::memory_order_release);
+  }
+  g.stage_bytes = g.pa * (TC_BM * TC_BK * 2) + g.pb * (BN / 2 * TC_BK * 2);
+  g.n_stages = SP_RING_BYTES / g.stage_bytes < SP_STAGES_MAX ? SP_RING_BYTES / g.stage_bytes : SP_STAGES_MAX;
+  const int64_t tiles = sp_tiles(g.M, g.N, BN);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * (unsigned)(tiles < pairs ? tiles : pairs)); cfg.blockDim = dim3(SP_THREADS);
+  cfg.dynamicSmemBytes = SP_SMEM_BYTES; cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, a, b, g) == cudaSuccess ? CONQUR_OK : CONQUR_ERR_CUDA;
+}
+template <int EPI>
+inline int sp_launch(int bn, int device, int pairs, cudaStream_t s, const CUtensorMap& a, const CUtensorMap& b, const SpArgs& g) {
+  if (bn == 256) return sp_launch_bn<256, EPI>(device, pairs, s, a, b, g);
+  if constexpr (EPI != SP_EPI_ACCUM) {
+    if (bn == 192) return sp_launch_bn<192, EPI>(device, pairs, s, a, b, g);
+  }
+  return sp_launch_bn<128, EPI>(device, pairs, s, a, b, g);
+}
+
+}  // namespace conqur
