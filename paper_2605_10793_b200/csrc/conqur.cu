@@ -19,6 +19,7 @@
 #include "conqur_tc.cuh"
 #include "conqur_tc_batched.cuh"
 #include "conqur_split_tc.cuh"
+#include "conqur_ns_cluster.cuh"
 #include "conqur_aux.cuh"
 #include "conqur_hadamard_tc.cuh"
 #include "ns_schedule.h"
@@ -149,6 +150,7 @@ struct conqur_ctx {
   int64_t last_n;            // rows per problem of the last step (for debug_get_signs)
   int last_np;               // problems the last step call covered
   bool last_pieces = false;  // the last step left its targets as bf16 pieces (exact mode)
+  bool one_cluster = false;  // exact mode, one narrow problem: its update is one kernel (conqur_ns_cluster.cuh)
   int device = 0, sp_pairs = 0;   // exact contexts with pieces: CTA pairs that can be co-resident (0: CUDA cores only)
   int64_t pending_rows = 0;  // deferring context: rows staged but not yet run through the two products
   int pending_batches = 0;
@@ -536,6 +538,20 @@ int update_impl(conqur_ctx* c) {
                               g.orth_tol, g.fro_tol, g.margin, g.lo_budget, 1.0 / (double)g.d, 0, 1.f / 256.f};
     return tcb_update(c->tc, c->stream, ncp, g.prior_rel, g.margin);
   }
+  if (c->one_cluster) {
+    NcArgs a{};
+    a.M = c->at<float>(c->L.M); a.R = c->at<float>(c->L.R); a.Xa = c->at<float>(c->L.Xa); a.Xb = c->at<float>(c->L.Xb);
+    a.E = c->at<float>(c->L.E); a.B = c->at<float>(c->L.B);
+    a.st = c->state();
+    a.c = NsControlParams{c->at<SchedEntry>(c->L.sched), c->n_sched, c->n_lift_init, g.ns_max_steps, g.d, 0, g.orth_tol,
+                          g.fro_tol, g.margin, g.lo_budget, 1.0 / (double)g.d, 0, 1.f / 2048.f};
+    a.d = g.d; a.n_endgame = c->n_sched - 1;
+    a.prior_rel = g.prior_rel; a.inv_sqrt_d = (float)(1.0 / std::sqrt((double)g.d)); a.margin = g.margin;
+    const int rc = nc_launch(a, c->stream);
+    if (rc) return rc;
+    c->prof.count(K_NS_NEXT);
+    return CONQUR_OK;
+  }
   int rc = update_prologue(c);
   if (rc) return rc;
   for (int k = 0; k <= g.ns_max_steps; ++k) {
@@ -645,7 +661,7 @@ bool build_looped_update_graph(conqur_ctx* c) {
 // took longer than the work (exact mode, d = 128: 704 -> 340 us for set_R, step, update and get_R).  (Many tensor-core problems: one kernel.)
 int update_enqueue(conqur_ctx* c) {
   const bool no_graph = (c->cfg.debug_flags & CONQUR_DEBUG_NO_GRAPH) != 0;
-  const bool eligible = !no_graph && (c->cfg.mode == CONQUR_EXACT_F32 || c->cfg.P == 1) && !c->prof.enabled;
+  const bool eligible = !no_graph && !c->one_cluster && (c->cfg.mode == CONQUR_EXACT_F32 || c->cfg.P == 1) && !c->prof.enabled;
   cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
   if (eligible && cudaStreamIsCapturing(c->stream, &capturing) != cudaSuccess) { cudaGetLastError(); capturing = cudaStreamCaptureStatusNone; }
   // (a caller that captures the stream gets the launches themselves: an instantiated graph cannot be captured)
@@ -775,9 +791,11 @@ extern "C" int conqur_init(conqur_ctx** out, int32_t d, const conqur_config* cfg
     rc = tc_refresh_R(c->tc, c->stream, 0);
     if (rc) return fail(rc);
   }
+  if (g.mode == CONQUR_EXACT_F32 && cudaGetDevice(&c->device) != cudaSuccess) return fail(CONQUR_ERR_CUDA);
+  c->one_cluster = g.mode == CONQUR_EXACT_F32 && g.P == 1 && d <= NC_MAX_D && !(g.debug_flags & CONQUR_DEBUG_NO_GRAPH) && nc_available(c->device);
   if (L.sp.ldp) {
     TcDevFacts f;
-    if (cudaGetDevice(&c->device) != cudaSuccess || tc_device_facts(c->device, &f) != CONQUR_OK) return fail(CONQUR_ERR_CUDA);
+    if (tc_device_facts(c->device, &f) != CONQUR_OK) return fail(CONQUR_ERR_CUDA);
     c->sp_pairs = (g.debug_flags & CONQUR_DEBUG_SINGLE_CTA) ? 0 : f.pair_clusters;
     const int rc = sp_refresh_R(c);
     if (rc) return fail(rc);

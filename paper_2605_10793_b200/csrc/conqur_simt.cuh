@@ -1000,9 +1000,8 @@ static __global__ void ns_commit_kernel(DevState* st, const float* __restrict__ 
     M[p * dd + i] = 0.f;
   }
 }
-static __global__ void ns_commit_state_kernel(DevState* st, int n_endgame) {
-  DevState* s = st + blockIdx.x;
-  if (threadIdx.x != 0) return;
+// The problem's state after an update (one thread).
+__device__ __forceinline__ void ns_commit_state(DevState* s, int n_endgame) {
   ns_adapt_lift_plan(s, n_endgame, s->ns_done == NS_DONE_CONVERGED);
   if (s->ns_done == NS_DONE_CONVERGED) {
     s->last_J = s->J;
@@ -1016,6 +1015,9 @@ static __global__ void ns_commit_state_kernel(DevState* st, int n_endgame) {
   } else {
     atomicOr(&s->status_flags, STATUS_FLAG_NS_FAILED);
   }
+}
+static __global__ void ns_commit_state_kernel(DevState* st, int n_endgame) {
+  if (threadIdx.x == 0) ns_commit_state(st + blockIdx.x, n_endgame);
 }
 
 // ------------------------------------------------------------------ misc element-wise

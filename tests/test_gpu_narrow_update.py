@@ -1,0 +1,75 @@
+"""The one-kernel exact update of narrow problems against the polar factor in float64 and against the launches it replaces."""
+import pytest
+import torch
+
+from paper_2605_10793_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+
+
+def _rand(seed, *shape):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    return torch.randn(*shape, generator=g, device="cuda")
+
+
+# edges of the 32-wide tiles, widths whose rows are not whole 16-byte pieces, one tile to twenty-five, the first wider ones
+WIDTHS = [2, 3, 31, 32, 33, 64, 97, 127, 128, 130, 159, 160, 161]
+
+
+def _spectrum(d, kind):
+    u = torch.linalg.qr(_rand(d, d, d).double())[0]
+    v = torch.linalg.qr(_rand(d + 1, d, d).double())[0]
+    if kind == "flat":
+        s = torch.linspace(1.0, 0.3, d, dtype=torch.float64, device="cuda")
+    else:
+        s = torch.logspace(0, -4, d, dtype=torch.float64, device="cuda")
+    return ((u * s) @ v.T).float().contiguous()
+
+
+@pytest.mark.parametrize("d", WIDTHS)
+@pytest.mark.parametrize("kind,prior", [("flat", 0.0), ("steep", 0.0), ("steep", 0.05)])
+def test_update_is_the_polar_factor(d, kind, prior):
+    m = _spectrum(d, kind)
+    r0 = torch.linalg.qr(_rand(5, d, d).double())[0].float().contiguous()
+    got = []
+    for flags in (0, B.CONQUR_DEBUG_NO_GRAPH):
+        c = B.Context(d, 4096, in_dtype="f32", mode="exact", prior_rel=prior, debug_flags=flags)
+        for _ in range(2):                               # (the second with the lifting count learnt)
+            c.set_R(r0)
+            c.set_M(m, 1.0, 4096)
+            c.update()
+        st = c.get_stats()
+        assert st.status == 0 and st.updates == 2
+        assert c.get_objective() == (0.0, 0) and float(c.get_M().abs().max()) == 0.0
+        got.append((c.get_R().double(), st.ns_steps_used, st.ns_lift_plan))
+    r = got[0][0]
+    me = m.double() + (prior * m.double().norm() / d ** 0.5 * r0.double() if prior else 0.0)
+    u, s, vt = torch.linalg.svd(me)
+    assert 1.0 - float((r * me).sum() / s.sum()) <= 2e-5
+    assert float((r.T @ r - torch.eye(d, device="cuda", dtype=torch.float64)).abs().max()) <= 1e-4
+    assert got[0][1:] == got[1][1:]                      # steps taken and count learnt
+    # a direction whose sigma is s turns by the iteration's rounding, about sqrt(d) 2^-22 of the largest sigma, over s
+    turn = d ** 0.5 * 2.0 ** -22 * float((1.0 / s.clamp_min(1e-30)).square().sum().sqrt()) * float(s[0])
+    assert float((r - got[1][0]).norm()) <= turn + 1e-4
+
+
+def test_rejected_updates_keep_the_rotation():
+    d = 100
+    c = B.Context(d, 128, in_dtype="f32", mode="exact")
+    r0 = torch.linalg.qr(_rand(5, d, d).double())[0].float().contiguous()
+    c.set_R(r0)
+    m = _spectrum(d, "flat")
+    for bad in (float("nan"), float("inf")):
+        w = m.clone()
+        w[3, 7] = bad
+        c.set_M(w, 1.0, 128)
+        c.update()
+        assert c.get_stats().status == -6
+        assert torch.equal(c.get_R(), r0)
+    c.set_M(torch.zeros_like(m), 1.0, 128)
+    c.update()
+    assert c.get_stats().status == -6
+    c.set_M(m, 1.0, 128)
+    c.update()
+    assert c.get_stats().status == 0 and not torch.equal(c.get_R(), r0)
