@@ -111,13 +111,13 @@ def load() -> C.CDLL:
     lib.conqur_get_R.restype = C.c_int
     lib.conqur_get_R.argtypes = [vp, vp]
     lib.conqur_get_objective.restype = C.c_int
-    lib.conqur_get_objective.argtypes = [vp, C.POINTER(C.c_double), C.POINTER(i64)]
+    lib.conqur_get_objective.argtypes = [vp, vp, vp]
     lib.conqur_get_objective_async.restype = C.c_int
     lib.conqur_get_objective_async.argtypes = [vp, vp, vp]
     lib.conqur_get_M.restype = C.c_int
     lib.conqur_get_M.argtypes = [vp, vp]
     lib.conqur_set_M.restype = C.c_int
-    lib.conqur_set_M.argtypes = [vp, vp, C.POINTER(C.c_double), C.POINTER(i64)]
+    lib.conqur_set_M.argtypes = [vp, vp, vp, vp]
     lib.conqur_debug_get_signs.restype = C.c_int
     lib.conqur_debug_get_signs.argtypes = [vp, vp, i64]
     lib.conqur_debug_capture_signs.restype = C.c_int
@@ -169,6 +169,11 @@ def make_config(*, in_dtype=CONQUR_BF16, mode=CONQUR_TC_BF16, quant_bits=0, ns_s
                          defer_batches, ns_gram_single_pass_tau, ns_lo_gap_budget, debug_flags)
 
 
+def _stream(torch) -> int:
+    """Handle of the current stream of the current device."""
+    return torch.cuda.current_stream().cuda_stream
+
+
 # ---- the C calls, one to one -------------------------------------------------------------------
 
 def conqur_workspace_bytes(d: int, cfg: conqur_config) -> int:
@@ -212,10 +217,9 @@ def conqur_get_R(h: int, out_ptr: int) -> int:
 
 
 def conqur_get_objective(h: int, batch: int) -> Tuple[int, np.ndarray, np.ndarray]:
-    j = (C.c_double * batch)()
-    n = (C.c_int64 * batch)()
-    rc = load().conqur_get_objective(h, j, n)
-    return rc, np.array(j[:], dtype=np.float64), np.array(n[:], dtype=np.int64)
+    j, n = np.zeros(batch), np.zeros(batch, dtype=np.int64)
+    rc = load().conqur_get_objective(h, j.ctypes.data, n.ctypes.data)
+    return rc, j, n
 
 
 def conqur_get_M(h: int, out_ptr: int) -> int:
@@ -223,11 +227,9 @@ def conqur_get_M(h: int, out_ptr: int) -> int:
 
 
 def conqur_set_M(h: int, m_ptr: int, j_sum, n_tokens) -> int:
-    j_sum = np.atleast_1d(np.asarray(j_sum, dtype=np.float64))
-    n_tokens = np.atleast_1d(np.asarray(n_tokens, dtype=np.int64))
-    j = (C.c_double * j_sum.size)(*j_sum.tolist())
-    n = (C.c_int64 * n_tokens.size)(*n_tokens.tolist())
-    return load().conqur_set_M(h, m_ptr, j, n)
+    j = np.ascontiguousarray(j_sum, dtype=np.float64)
+    n = np.ascontiguousarray(n_tokens, dtype=np.int64)
+    return load().conqur_set_M(h, m_ptr, j.ctypes.data, n.ctypes.data)
 
 
 def conqur_debug_get_signs(h: int, out_ptr: int, capacity_rows: int) -> int:
@@ -317,18 +319,26 @@ def conqur_fold_weight(w, r, side: str, mode: str = "tc"):
     return out
 
 
+_hadamard_codes = None                            # torch dtype -> C code (torch is imported on first use)
+
+
 def conqur_hadamard_rows(x, out_dtype=None, out=None, cuda_cores_only=False):
     """y = x H_d / sqrt(d) for every row of a 2-D fp32 / bf16 CUDA tensor (see include/conqur.h)."""
+    global _hadamard_codes
     import torch
-    code = {torch.float32: CONQUR_F32, torch.bfloat16: CONQUR_BF16}
-    assert x.is_cuda and x.dim() == 2 and x.stride(1) == 1 and x.dtype in code
+    if _hadamard_codes is None:
+        _hadamard_codes = {torch.float32: CONQUR_F32, torch.bfloat16: CONQUR_BF16}
+    in_code = _hadamard_codes.get(x.dtype)
+    assert x.is_cuda and x.dim() == 2 and in_code is not None
+    (n, d), (ldx, unit) = x.shape, x.stride()
     if out is None:
-        out = torch.empty(x.shape, dtype=out_dtype or x.dtype, device="cuda")
-    assert out.is_cuda and out.shape == x.shape and out.stride(1) == 1 and out.dtype in code
-    rc = load().conqur_hadamard_rows(x.data_ptr(), code[x.dtype], x.shape[0], x.shape[1], x.stride(0), out.data_ptr(),
-                                     code[out.dtype], out.stride(0),
-                                     CONQUR_HADAMARD_CUDA_CORES_ONLY if cuda_cores_only else 0,
-                                     torch.cuda.current_stream().cuda_stream)
+        out = torch.empty((n, d), dtype=out_dtype or x.dtype, device="cuda")
+    out_code = _hadamard_codes.get(out.dtype)
+    assert unit == 1 and out.is_cuda and out.shape == x.shape and out_code is not None
+    ldy, unit = out.stride()
+    assert unit == 1
+    rc = (_lib or load()).conqur_hadamard_rows(x.data_ptr(), in_code, n, d, ldx, out.data_ptr(), out_code, ldy,
+                                               CONQUR_HADAMARD_CUDA_CORES_ONLY if cuda_cores_only else 0, _stream(torch))
     if rc != 0:
         raise ConqurError(rc, "conqur_hadamard_rows")
     return out

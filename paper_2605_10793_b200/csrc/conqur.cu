@@ -11,6 +11,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -138,6 +139,41 @@ bool make_layout(int d, const conqur_config* c, Layout* L) {
   return true;
 }
 
+// Page-locked host memory that a context's synchronising calls exchange small results through: kernels write (or read) it
+// directly, where a copy through pageable memory costs a node of its own and about 8 us more.  Slots go back to a small pool
+// (allocating and freeing one takes ~0.1 ms and may wait for the device); at most MAIL_KEPT idle ones are held.
+constexpr size_t MAIL_BYTES = 32768;
+constexpr size_t MAIL_KEPT = 8;
+struct RelaxedCapture {                                 // (a stream that another thread captures is not disturbed by the allocation)
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+struct MailPool {
+  std::mutex mu;
+  std::vector<void*> idle;
+  void* take() {
+    {
+      std::lock_guard<std::mutex> lock(mu);
+      if (!idle.empty()) { void* p = idle.back(); idle.pop_back(); return p; }
+    }
+    RelaxedCapture relaxed;
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, MAIL_BYTES, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    return p;
+  }
+  void give(void* p) {
+    if (!p) return;
+    {
+      std::lock_guard<std::mutex> lock(mu);
+      if (idle.size() < MAIL_KEPT) { idle.push_back(p); return; }
+    }
+    RelaxedCapture relaxed;
+    cudaFreeHost(p);
+  }
+};
+MailPool& mail_pool() { static MailPool* pool = new MailPool; return *pool; }   // (never destroyed: contexts may outlive statics)
+
 }  // namespace
 
 struct conqur_ctx {
@@ -145,6 +181,7 @@ struct conqur_ctx {
   Layout L;
   char* ws;
   cudaStream_t stream;
+  unsigned char* mail = nullptr;   // MAIL_BYTES of page-locked memory, used between a call's launch and its synchronise only
   std::vector<int64_t> tokens;   // per problem: rows enqueued since the last update
   std::vector<int64_t> tokens_at_update;   // ... as they stood when the last update was enqueued (restored if it is rejected)
   int64_t last_n;            // rows per problem of the last step (for debug_get_signs)
@@ -232,10 +269,36 @@ __global__ void check_reduce_kernel(const DevState* st, const float* pmax, const
 __global__ void export_sums_kernel(const DevState* st, double* J, long long* N, int P) {
   for (int i = threadIdx.x; i < P; i += blockDim.x) { J[i] = st[i].J; N[i] = st[i].N; }
 }
-__global__ void set_sums_kernel(DevState* st, const double* J, const long long* N, int P) {
-  for (int i = threadIdx.x; i < P; i += blockDim.x) { st[i].J = J[i]; st[i].N = N[i]; }
+// dst = src * f; block 0 besides takes the sums over (J given; set_M) or reads the latched status of all problems out (agg
+// given; get_M, get_R), which the copies of the other blocks hide.
+__global__ void __launch_bounds__(256) scale_copy_kernel(const float* __restrict__ src, float* __restrict__ dst, int64_t count, float f,
+                                                         DevState* st, int P, int* agg, const double* J, const long long* N) {
+  __shared__ int all;
+  if (blockIdx.x == 0) {
+    if (threadIdx.x == 0) all = 0;
+    __syncthreads();
+    int fl = 0;
+    for (int i = threadIdx.x; i < P; i += blockDim.x) {
+      if (J) { st[i].J = J[i]; st[i].N = N[i]; } else { fl |= st[i].status_flags; }
+    }
+    if (agg) {
+      fl = __reduce_or_sync(0xffffffffu, fl);
+      if ((threadIdx.x & 31) == 0 && fl) atomicOr(&all, fl);
+      __syncthreads();
+      if (threadIdx.x == 0) *agg = all;
+    }
+  }
+  const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+  if ((count & 3) == 0 && ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0) {
+    for (int64_t i = first; i < count / 4; i += step) {
+      float4 v = __ldcs(reinterpret_cast<const float4*>(src) + i);
+      v.x *= f; v.y *= f; v.z *= f; v.w *= f;
+      reinterpret_cast<float4*>(dst)[i] = v;
+    }
+  } else {
+    for (int64_t i = first; i < count; i += step) dst[i] = src[i] * f;
+  }
 }
-__global__ void set_sum_kernel(DevState* st, double J, long long N) { st->J = J; st->N = N; }
 
 int flags_to_status(int f) {
   if (f & STATUS_FLAG_TIMEOUT) return CONQUR_ERR_TIMEOUT;
@@ -244,18 +307,39 @@ int flags_to_status(int f) {
   return CONQUR_OK;
 }
 
+int ew_blocks(int64_t count) { return (int)std::min<int64_t>(148 * 8, (count + 255) / 256); }
+
+// Where the kernels of a synchronising call leave `bytes` of results: the mailbox, or `dev` where they do not fit it.
+template <typename T> T* result_area(conqur_ctx* c, size_t bytes, T* dev) {
+  return c->mail && bytes <= MAIL_BYTES ? reinterpret_cast<T*>(c->mail) : dev;
+}
+// Synchronise and take them over.
+int take_results(conqur_ctx* c, const void* area, void* host, size_t bytes) {
+  if (area != c->mail) CQ_CUDA(cudaMemcpyAsync(host, area, bytes, cudaMemcpyDeviceToHost, c->stream));
+  CQ_CUDA(cudaStreamSynchronize(c->stream));
+  if (area == c->mail) std::memcpy(host, area, bytes);
+  return CONQUR_OK;
+}
+
 // Synchronise and return the latched device status (not cleared).
 int sync_status(conqur_ctx* c) {
-  int* agg = c->at<int>(c->L.flags_agg);
+  int* agg = result_area(c, sizeof(int), c->at<int>(c->L.flags_agg));
   read_out_kernel<<<1, c->cfg.P > 32 ? 256 : 32, 0, c->stream>>>(c->state(), c->cfg.P, agg, nullptr, nullptr);
   CQ_LAUNCHED(c, K_OTHER);
   int f = 0;
-  CQ_CUDA(cudaMemcpyAsync(&f, agg, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  CQ_CUDA(cudaStreamSynchronize(c->stream));
-  return flags_to_status(f);
+  const int rc = take_results(c, agg, &f, sizeof(int));
+  return rc ? rc : flags_to_status(f);
 }
-
-int ew_blocks(int64_t count) { return (int)std::min<int64_t>(148 * 8, (count + 255) / 256); }
+// dst = src * f over all problems' matrices, then synchronise and return the latched device status.
+int copy_out(conqur_ctx* c, const float* src, float* dst, float f) {
+  const int64_t count = (int64_t)c->cfg.d * c->cfg.d * c->cfg.P;
+  int* agg = result_area(c, sizeof(int), c->at<int>(c->L.flags_agg));
+  scale_copy_kernel<<<ew_blocks((count + 3) / 4), 256, 0, c->stream>>>(src, dst, count, f, c->state(), c->cfg.P, agg, nullptr, nullptr);
+  CQ_LAUNCHED(c, K_OTHER);
+  int flags = 0;
+  const int rc = take_results(c, agg, &flags, sizeof(int));
+  return rc ? rc : flags_to_status(flags);
+}
 
 // ---------------------------------------------------------------- exact-mode step
 __nv_bfloat16* sp_ptr(const conqur_ctx* c, size_t off) { return c->at<__nv_bfloat16>(off); }
@@ -801,6 +885,7 @@ extern "C" int conqur_init(conqur_ctx** out, int32_t d, const conqur_config* cfg
     if (rc) return fail(rc);
   }
   if (cudaStreamSynchronize(c->stream) != cudaSuccess) return fail(CONQUR_ERR_CUDA);   // coef is a local
+  c->mail = static_cast<unsigned char*>(mail_pool().take());   // (none: results are copied)
   *out = c;
   return CONQUR_OK;
 }
@@ -810,6 +895,7 @@ extern "C" int conqur_destroy(conqur_ctx* ctx) {
   cudaStreamSynchronize(ctx->stream);
   if (ctx->upd_graph) cudaGraphExecDestroy(ctx->upd_graph);
   if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
+  mail_pool().give(ctx->mail);
   delete ctx;
   return CONQUR_OK;
 }
@@ -817,12 +903,10 @@ extern "C" int conqur_destroy(conqur_ctx* ctx) {
 // What a residual product left in `n` partials, on the host: h[0] = max|G - I| without NaN, h[1] = sum (G - I)^2 (NaN where
 // any entry is; infinite where the tensor-core product of state `st` gave up).
 static int check_read(conqur_ctx* c, const DevState* st, int n, double (&h)[2]) {
-  double* out = c->at<double>(c->L.obj_out);
+  double* out = result_area(c, sizeof(h), c->at<double>(c->L.obj_out));
   check_reduce_kernel<<<1, 256, 0, c->stream>>>(st, c->at<float>(c->L.part_f), c->at<double>(c->L.part_d), n, out);
   CQ_LAUNCHED(c, K_OTHER);
-  CQ_CUDA(cudaMemcpyAsync(h, out, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
-  CQ_CUDA(cudaStreamSynchronize(c->stream));
-  return CONQUR_OK;
+  return take_results(c, out, h, sizeof(h));
 }
 
 extern "C" int conqur_set_R(conqur_ctx* c, const float* R_dev) {
@@ -948,9 +1032,7 @@ extern "C" int conqur_update(conqur_ctx* c) {
 extern "C" int conqur_get_R(conqur_ctx* c, float* R_out_dev) {
   if (!c || !R_out_dev) return CONQUR_ERR_INVALID_ARG;
   { const int frc = flush_pending(c); if (frc) return frc; }
-  const size_t bytes = sizeof(float) * (size_t)c->cfg.d * c->cfg.d * c->cfg.P;
-  CQ_CUDA(cudaMemcpyAsync(R_out_dev, c->at<float>(c->L.R), bytes, cudaMemcpyDeviceToDevice, c->stream));
-  return sync_status(c);
+  return copy_out(c, c->at<float>(c->L.R), R_out_dev, 1.0f);
 }
 
 extern "C" int conqur_get_objective(conqur_ctx* c, double* J_sum, int64_t* n_tokens) {
@@ -958,15 +1040,16 @@ extern "C" int conqur_get_objective(conqur_ctx* c, double* J_sum, int64_t* n_tok
   { const int frc = flush_pending(c); if (frc) return frc; }
   const int P = c->cfg.P;
   if (c->cfg.mode == CONQUR_TC_BF16) { const int orc = tcb_refresh_objective(c->tc, c->stream); if (orc) return orc; }
-  // J, N and the status leave together through the (idle) partials: one launch and one copy of 16 bytes a problem
-  double* dJ = c->at<double>(c->L.part_d);
+  // J, N and the status leave together, 16 bytes a problem (through the idle partials where the mailbox is too small)
+  const size_t bytes = 16 * (size_t)P + sizeof(int);
+  double* dJ = result_area(c, bytes, c->at<double>(c->L.part_d));
   long long* dN = reinterpret_cast<long long*>(dJ + P);
   int* df = reinterpret_cast<int*>(dN + P);
   read_out_kernel<<<1, P > 32 ? 256 : 32, 0, c->stream>>>(c->state(), P, df, dJ, dN);
   CQ_LAUNCHED(c, K_OTHER);
-  std::vector<unsigned char> h(16 * (size_t)P + sizeof(int));
-  CQ_CUDA(cudaMemcpyAsync(h.data(), dJ, h.size(), cudaMemcpyDeviceToHost, c->stream));
-  CQ_CUDA(cudaStreamSynchronize(c->stream));
+  std::vector<unsigned char> h(bytes);
+  const int rc = take_results(c, dJ, h.data(), bytes);
+  if (rc) return rc;
   std::memcpy(J_sum, h.data(), 8 * (size_t)P);
   std::memcpy(n_tokens, h.data() + 8 * (size_t)P, 8 * (size_t)P);
   int f;
@@ -1007,11 +1090,7 @@ extern "C" int conqur_get_diagnostics(conqur_ctx* c, conqur_diagnostics* out) {
 extern "C" int conqur_get_M(conqur_ctx* c, float* M_out_dev) {
   if (!c || !M_out_dev) return CONQUR_ERR_INVALID_ARG;
   { const int frc = flush_pending(c); if (frc) return frc; }
-  const int64_t count = (int64_t)c->cfg.d * c->cfg.d * c->cfg.P;
-  scale_copy_kernel<<<ew_blocks(count), 256, 0, c->stream>>>(c->at<float>(c->L.M), M_out_dev, count,
-                                                             (float)(1.0 / std::sqrt((double)c->cfg.d)));
-  CQ_LAUNCHED(c, K_OTHER);
-  return sync_status(c);
+  return copy_out(c, c->at<float>(c->L.M), M_out_dev, (float)(1.0 / std::sqrt((double)c->cfg.d)));
 }
 
 extern "C" int conqur_set_M(conqur_ctx* c, const float* M_dev, const double* J_sum, const int64_t* n_tokens) {
@@ -1019,23 +1098,18 @@ extern "C" int conqur_set_M(conqur_ctx* c, const float* M_dev, const double* J_s
   { const int frc = flush_pending(c); if (frc) return frc; }
   const int P = c->cfg.P;
   const int64_t count = (int64_t)c->cfg.d * c->cfg.d * P;
-  scale_copy_kernel<<<ew_blocks(count), 256, 0, c->stream>>>(M_dev, c->at<float>(c->L.M), count,
-                                                             (float)std::sqrt((double)c->cfg.d));
-  CQ_LAUNCHED(c, K_OTHER);
+  // the sums go in beside the copy: the kernel reads them from the mailbox, or from the idle partials where they do not fit it
+  const size_t bytes = 16 * (size_t)P;
   std::vector<unsigned char> h;                       // (outlives the copy: the stream is synchronised below)
-  if (P == 1) {
-    set_sum_kernel<<<1, 1, 0, c->stream>>>(c->state(), J_sum[0], (long long)n_tokens[0]);
-    CQ_LAUNCHED(c, K_OTHER);
-  } else {
-    // stage the sums through the partials buffer, in one copy
-    double* dJ = c->at<double>(c->L.part_d);
-    h.resize(16 * (size_t)P);
-    std::memcpy(h.data(), J_sum, 8 * (size_t)P);
-    std::memcpy(h.data() + 8 * (size_t)P, n_tokens, 8 * (size_t)P);
-    CQ_CUDA(cudaMemcpyAsync(dJ, h.data(), h.size(), cudaMemcpyHostToDevice, c->stream));
-    set_sums_kernel<<<1, 256, 0, c->stream>>>(c->state(), dJ, reinterpret_cast<const long long*>(dJ + P), P);
-    CQ_LAUNCHED(c, K_OTHER);
-  }
+  double* dJ = result_area(c, bytes, c->at<double>(c->L.part_d));
+  unsigned char* to = c->mail;
+  if (reinterpret_cast<unsigned char*>(dJ) != c->mail) { h.resize(bytes); to = h.data(); }
+  std::memcpy(to, J_sum, 8 * (size_t)P);
+  std::memcpy(to + 8 * (size_t)P, n_tokens, 8 * (size_t)P);
+  if (to != c->mail) CQ_CUDA(cudaMemcpyAsync(dJ, to, bytes, cudaMemcpyHostToDevice, c->stream));
+  scale_copy_kernel<<<ew_blocks((count + 3) / 4), 256, 0, c->stream>>>(M_dev, c->at<float>(c->L.M), count, (float)std::sqrt((double)c->cfg.d),
+                                                                       c->state(), P, nullptr, dJ, reinterpret_cast<const long long*>(dJ + P));
+  CQ_LAUNCHED(c, K_OTHER);
   CQ_CUDA(cudaStreamSynchronize(c->stream));
   for (int p = 0; p < P; ++p) c->tokens[p] = n_tokens[p];
   return CONQUR_OK;

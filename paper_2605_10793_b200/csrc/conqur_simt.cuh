@@ -1021,10 +1021,6 @@ static __global__ void ns_commit_state_kernel(DevState* st, int n_endgame) {
 }
 
 // ------------------------------------------------------------------ misc element-wise
-static __global__ void scale_copy_kernel(const float* __restrict__ src, float* __restrict__ dst, int64_t count, float f) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
-    dst[i] = src[i] * f;
-}
 static __global__ void set_identity_kernel(float* __restrict__ R, int d, int P) {
   const int64_t dd = (int64_t)d * d;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < dd * P; i += (int64_t)gridDim.x * blockDim.x) {

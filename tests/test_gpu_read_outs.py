@@ -1,0 +1,45 @@
+"""Read-outs and set_M: small results go through page-locked memory, those of many problems by a copy."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2605_10793_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+
+
+# 16 bytes a problem and the status: 2047 problems fill the 32 KB they go through, 2048 do not; odd widths leave the 16-byte pieces
+@pytest.mark.parametrize("batch,d", [(1, 3), (1, 640), (2, 5), (2047, 2), (2048, 2), (2500, 3)])
+def test_statistics_round_trip(batch, d):
+    g = torch.Generator(device="cuda").manual_seed(batch + d)
+    contexts = [B.Context(d, 4, in_dtype="f32", mode="exact", batch=batch) for _ in range(3)]      # (more than one at a time)
+    kept = []
+    for i, c in enumerate(contexts):
+        m = torch.randn(batch, d, d, generator=g, device="cuda")
+        j, n = np.arange(batch) * 0.5 + i, np.arange(batch) + 7 * i
+        c.set_M(m if batch > 1 else m[0], j, n)
+        kept.append((m, j, n))
+    for c, (m, j, n) in zip(contexts, kept):
+        got_j, got_n = c.get_objective()
+        assert np.array_equal(np.atleast_1d(got_j), j) and np.array_equal(np.atleast_1d(got_n), n)
+        # scaled by sqrt(d) and back, each factor and product rounded to fp32
+        assert torch.allclose(c.get_M().view(batch, d, d), m, rtol=4 * 2.0 ** -24, atol=0.0)
+        eye = torch.eye(d, device="cuda").expand(batch, d, d)
+        assert torch.equal(c.get_R().view(batch, d, d), eye)
+    contexts[0].close()
+    again = B.Context(d, 4, in_dtype="f32", mode="exact", batch=batch)                             # (takes the freed slot)
+    assert np.array_equal(np.atleast_1d(again.get_objective()[0]), np.zeros(batch))
+    assert np.array_equal(np.atleast_1d(contexts[1].get_objective()[0]), kept[1][1])
+
+
+def test_status_of_any_problem_is_reported():
+    c = B.Context(2, 4, in_dtype="f32", mode="exact", batch=300)
+    x = torch.randn(300, 4, 2, device="cuda")
+    x[299, 1, 0] = float("nan")
+    c.step_batched(x, 4, 2, 8)
+    for call in (c.get_R, c.get_M, c.get_objective):
+        with pytest.raises(B.ConqurError) as e:
+            call()
+        assert e.value.status == -7
+    assert c.get_stats().status == -7
+    c.get_R()
