@@ -21,6 +21,7 @@
 #include "conqur_tc_batched.cuh"
 #include "conqur_split_tc.cuh"
 #include "conqur_ns_cluster.cuh"
+#include "conqur_fold_tc.cuh"
 #include "conqur_aux.cuh"
 #include "conqur_hadamard_tc.cuh"
 #include "ns_schedule.h"
@@ -1338,6 +1339,21 @@ extern "C" int conqur_fold_weight(const float* W_dev, int64_t ldw, int32_t rows,
     CQ_CUDA(cudaMemcpyAsync(&h, st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
     CQ_CUDA(cudaStreamSynchronize(s));
     return flags_to_status(h.status_flags);
+  }
+  int dev = 0;
+  TcDevFacts facts;
+  if (fold_blocks_takes(rows, cols, block, side) && cudaGetDevice(&dev) == cudaSuccess && tc_device_facts(dev, &facts) == CONQUR_OK &&
+      facts.major == 10) {
+    if (int* status = static_cast<int*>(mail_pool().take())) {
+      *status = 0;
+      const int rc = fold_blocks_launch(W_dev, ldw, rows, cols, R_dev, block, side, out_dev, ldo, status, dev, facts.sms, s);
+      const cudaError_t e = cudaStreamSynchronize(s);
+      const int f = *status;
+      mail_pool().give(status);
+      if (rc) return rc;
+      CQ_CUDA(e);
+      return flags_to_status(f);
+    }
   }
   const int64_t fm = side == CONQUR_FOLD_INPUT ? rows : block, fn = side == CONQUR_FOLD_INPUT ? block : cols;
   sg_with_tile(sg_pick(fm, fn, nblk), [&](auto tile) {

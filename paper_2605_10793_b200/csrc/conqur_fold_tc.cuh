@@ -1,0 +1,359 @@
+// Block-diagonal weight folds on the tensor cores, at no less than fp32's precision (see conqur_split_tc.cuh for the pieces).
+//
+//   SIDE 0:  out[:, b] = W[:, b] R_b        SIDE 1:  out[b, :] = R_b^T W[b, :]        blocks of 64 or 128
+//
+// Both are R^T times W (SIDE 0 of W transposed): the product's first operand is 128 x 128 of blockdiag(R)^T (two 64-blocks and
+// zeros), whose three bf16 pieces a CTA keeps in TMEM while it walks 128 x 128 tiles of W.  A tile arrives through the copy engine
+// half a k at a time (three 32 KB buffers); eight warps split it into pieces in the swizzled operand layout, one half while the
+// products read the other; one warp issues the six products of each half into an accumulator of its own (64 terms, small pieces
+// first); eight warps add the two halves in fp32 and write the tile (on SIDE 0 a TMEM lane is a column of the output, so a warp's
+// stores are whole lines as they are).  W is read once and out written once: bound by that (128 KB a tile, 5.7 k cycles of an SM's
+// share of the HBM rate; the products take 3.1 k).  32 blocks of 128, W 4096 x 4096: 90 -> 42 us, of which half is each CTA's
+// rotation (4 k cycles, once or twice) and the pipeline's fill; 4096 x 14336 4.4 TB/s.
+// Error against 64 bits, in 2^-24 of the result's norm, fp32 chain / this: 128-blocks 3.4 / 1.4, 64-blocks 2.4 / 1.3.
+//
+// A tile with values that pieces cannot hold (not finite; or below 2^-100, whose low pieces would underflow) is computed with
+// fp32 multiply-adds by the warps that write it.
+#pragma once
+#include "conqur_split_tc.cuh"
+#include "conqur_tc_batched.cuh"
+
+namespace conqur {
+
+namespace ptx {
+// 32 lanes x 8 consecutive columns: thread t of the warp writes row (lane base + t); complete after tmem_st_wait.
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&w)[8]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+               ::"r"(taddr), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+               : "memory");
+}
+}  // namespace ptx
+
+constexpr int FB_CONV = 256;                             // splitting threads: two warpgroups; then loading and issuing, then two that write
+constexpr int FB_THREADS = FB_CONV + 128 + 256;
+constexpr int FB_REGS_CONV = 96, FB_REGS_ISSUE = 40, FB_REGS_EPI = 120;   // (launched with 96: 40 + 2 x 120 <= 3 x 96)
+static_assert(FB_REGS_ISSUE + 2 * FB_REGS_EPI <= 3 * FB_REGS_CONV, "registers the block is launched with");
+constexpr int FB_PIECE = 128 * 128 * 2;
+constexpr int FB_HALF = 128 * 64 * 4, FB_RAW = 3;        // half a tile in fp32, and how many of them
+constexpr int FB_TM_A = 256;                             // TMEM: two accumulators, then three pieces of 64 columns
+constexpr int FB_SMEM_BYTES = 3 * FB_PIECE + FB_RAW * FB_HALF + 1024 + 8 * 4096 + 1024;
+static_assert(FB_SMEM_BYTES <= 232448, "227 KB of dynamic shared memory per CTA");
+
+struct FbArgs {
+  const float *W, *R;
+  float* out;
+  int64_t ldw, ldo;
+  int logdb, rows, cols;            // blocks of 1 << logdb
+  int n_super, tiles;               // 128-wide groups of blocks; W tiles along the other dimension
+  int copied;                       // 1: W's rows suit the copy engine (16-byte aligned)
+  int* status;                      // page-locked host memory, cleared by the caller
+};
+struct FbAux {
+  uint64_t raw_full[FB_RAW], raw_free[FB_RAW], full[2], free_[2], tfull, tempty;
+  uint32_t tmem_base;
+  int abort_flag;
+  int bad[4][2][8];                 // per tile (ring), half and splitting warp: values that pieces cannot hold
+};
+static_assert(sizeof(FbAux) <= 1024, "reserved behind the operands");
+
+// Largest and smallest nonzero magnitude of what it is shown, as integers: pieces hold values from 2^-100 to below 2^128 - 2^119.
+struct FbRange {
+  uint32_t hi = 0u, lo = 0xffffffffu;
+  __device__ __forceinline__ void see(float v) {
+    const uint32_t m = __float_as_uint(v) << 1;
+    hi = max(hi, m);
+    lo = min(lo, m - 1u);                                // (zero wraps to the largest number)
+  }
+  __device__ __forceinline__ bool unfit() const { return hi >= (0x7f7f8000u << 1) || lo < (0x0d800000u << 1) - 1u; }
+};
+
+template <int SIDE>
+__global__ void __launch_bounds__(FB_THREADS, 1) fold_blocks_kernel(const __grid_constant__ CUtensorMap tmW, const FbArgs g) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* sW = smem;                                    // pieces: two 64-column chunks of 128 rows x 128 bytes each, swizzled by the row
+  uint8_t* sRaw = smem + 3 * FB_PIECE;
+  FbAux* aux = reinterpret_cast<FbAux*>(sRaw + FB_RAW * FB_HALF);
+  volatile int* abort_flag = &aux->abort_flag;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
+  const int total = g.n_super * g.tiles;
+  const int t0 = (int)((int64_t)total * blockIdx.x / gridDim.x), t1 = (int)((int64_t)total * (blockIdx.x + 1) / gridDim.x);
+  const int folded = SIDE == 0 ? g.cols : g.rows;       // length of the folded dimension
+  const int db = 1 << g.logdb;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < FB_RAW; ++s) { ptx::mbar_init(&aux->raw_full[s], 1); ptx::mbar_init(&aux->raw_free[s], FB_CONV / 32); }
+    for (int b = 0; b < 2; ++b) { ptx::mbar_init(&aux->full[b], FB_CONV / 32); ptx::mbar_init(&aux->free_[b], 1); }
+    ptx::mbar_init(&aux->tfull, 1);
+    ptx::mbar_init(&aux->tempty, 8);
+    aux->abort_flag = 0;
+    ptx::fence_barrier_init();
+    ptx::fence_proxy_async();
+    if (g.copied) ptx::prefetch_tmap(&tmW);
+  }
+  if (warp == FB_CONV / 32 + 1) { ptx::tmem_alloc(&aux->tmem_base, 512); ptx::tmem_relinquish(); }
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem_base = aux->tmem_base;
+  int timeout_site = 0;
+
+  if (warp < FB_CONV / 32) {
+    // ---- splitting, one half of k after the other (64 rows of the tile on SIDE 1, 64 columns on SIDE 0): 4 elements eight times a thread
+    int cur_sb = -1;
+    bool r_bad = false;
+    uint32_t n = 0, it = 0;
+    bool ok = true;
+    for (int t = t0; t < t1 && ok; ++t, ++n) {
+      const int sb = t / g.tiles, j = t - sb * g.tiles;
+      const uint32_t ph = (n & 1u) ^ 1u;
+      if (sb != cur_sb) {
+        // R^T into TMEM: lane = its row, two consecutive k per column.  (The products of the tile before read the old one last.)
+        if (!tc_wait_warp(&aux->free_[0], ph, abort_flag) || !tc_wait_warp(&aux->free_[1], ph, abort_flag)) { timeout_site = 1; break; }
+        ptx::tc_fence_after();
+        cur_sb = sb;
+        FbRange rr;
+        const int a = (warp & 3) * 32 + lane, ag = sb * 128 + a;
+        const uint32_t ta = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + FB_TM_A;
+#pragma unroll 1
+        for (int c = 0; c < 4; ++c) {                    // 16 k, 8 columns of each piece
+          const int k0 = (warp >> 2) * 64 + c * 16;
+          float v[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            const int k = k0 + i, kg = sb * 128 + k;
+            // (two or more blocks side by side: element (k, a) lies in one of them where their block numbers agree)
+            v[i] = (kg < folded && ag < folded && (k >> g.logdb) == (a >> g.logdb))
+                       ? __ldg(g.R + ((int64_t)kg << g.logdb) + (a & (db - 1))) : 0.f;
+          }
+          uint32_t w[3][8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            rr.see(v[2 * i]); rr.see(v[2 * i + 1]);
+            sp_split2(v[2 * i], v[2 * i + 1], w[0][i], w[1][i], w[2][i]);
+          }
+#pragma unroll
+          for (int p = 0; p < 3; ++p) ptx::tmem_st8(ta + (uint32_t)(p * 64 + k0 / 2), w[p]);
+        }
+        r_bad = rr.unfit();
+        ptx::tmem_st_wait();
+        ptx::tc_fence_before();
+      }
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h, ++it) {
+        const uint32_t slot = it % FB_RAW;
+        if (g.copied && !tc_wait_warp(&aux->raw_full[slot], (it / FB_RAW) & 1u, abort_flag)) { ok = false; timeout_site = 2; break; }
+        if (!tc_wait_warp(&aux->free_[h], ph, abort_flag)) { ok = false; timeout_site = 1; break; }
+        FbRange rr;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int e = threadIdx.x + 256 * i;
+          const int row = SIDE == 0 ? e >> 4 : e >> 5, c4 = SIDE == 0 ? e & 15 : e & 31;
+          const int r = SIDE == 0 ? row : 64 * h + row, u = SIDE == 0 ? 8 * h + (c4 >> 1) : c4 >> 1;
+          float4 v;
+          if (g.copied) {
+            v = *reinterpret_cast<const float4*>(sRaw + slot * FB_HALF + (SIDE == 0 ? row * 256 : row * 512) + c4 * 16);
+          } else {
+            const int gr = (SIDE == 0 ? j * 128 + row : sb * 128 + 64 * h + row), gc = (SIDE == 0 ? sb * 128 + 64 * h : j * 128) + c4 * 4;
+            const float* p = g.W + (int64_t)gr * g.ldw + gc;
+            const bool in = gr < g.rows;
+            v.x = in && gc < g.cols ? p[0] : 0.f; v.y = in && gc + 1 < g.cols ? p[1] : 0.f;
+            v.z = in && gc + 2 < g.cols ? p[2] : 0.f; v.w = in && gc + 3 < g.cols ? p[3] : 0.f;
+          }
+          rr.see(v.x); rr.see(v.y); rr.see(v.z); rr.see(v.w);
+          uint2 w[3];
+          sp_split2(v.x, v.y, w[0].x, w[1].x, w[2].x);
+          sp_split2(v.z, v.w, w[0].y, w[1].y, w[2].y);
+          uint8_t* q = sW + (u >> 3) * 16384 + r * 128 + (((u & 7) ^ (r & 7)) << 4) + (c4 & 1) * 8;
+#pragma unroll
+          for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2*>(q + p * FB_PIECE) = w[p];
+        }
+        const bool any = __any_sync(0xffffffffu, r_bad || rr.unfit());
+        ptx::fence_proxy_async();
+        if (lane == 0) aux->bad[n & 3u][h][warp] = any ? 1 : 0;
+        __syncwarp();
+        if (lane == 0) {
+          if (g.copied) ptx::mbar_arrive(&aux->raw_free[slot]);
+          ptx::mbar_arrive(&aux->full[h]);
+        }
+      }
+    }
+  } else if (warp < FB_CONV / 32 + 4) {
+    ptx::regs_dec<FB_REGS_ISSUE>();
+    if (warp == FB_CONV / 32 && lane == 0 && g.copied) {
+      // ---- copies of W, half a k of a tile at a time
+      uint32_t it = 0;
+      bool ok = true;
+      for (int t = t0; t < t1 && ok; ++t) {
+        const int sb = t / g.tiles, j = t - sb * g.tiles;
+        for (int h = 0; h < 2; ++h, ++it) {
+          const uint32_t slot = it % FB_RAW;
+          if (!tc_wait(&aux->raw_free[slot], ((it / FB_RAW) & 1u) ^ 1u, abort_flag)) { ok = false; timeout_site = 3; break; }
+          ptx::mbar_expect_tx(&aux->raw_full[slot], FB_HALF);
+          if (SIDE == 0) ptx::tma_load_2d(sRaw + slot * FB_HALF, &tmW, &aux->raw_full[slot], sb * 128 + 64 * h, j * 128);
+          else ptx::tma_load_2d(sRaw + slot * FB_HALF, &tmW, &aux->raw_full[slot], j * 128, sb * 128 + 64 * h);
+        }
+      }
+      if (!ok) {                                         // let the copies in flight land before the CTA's shared memory goes
+        const long long c0 = clock64();
+        while (clock64() - c0 < 4000000ll) {}
+      }
+    } else if (warp == FB_CONV / 32 + 1) {
+      const uint32_t leader = ptx::elect_one();
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((SIDE == 1 ? 1u : 0u) << 16) | ((uint32_t)(128 >> 3) << 17) |
+                             ((uint32_t)(128 >> 4) << 24);
+      const uint64_t dW = tc_smem_desc(ptx::smem_u32(sW), SIDE == 1 ? 16384 : 16, 1024);
+      uint32_t n = 0;
+      bool ok = true;
+      for (int t = t0; t < t1 && ok; ++t, ++n) {
+        if (!tc_wait_warp(&aux->tempty, (n & 1u) ^ 1u, abort_flag)) { timeout_site = 4; break; }
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {                    // halves of k, an accumulator each
+          if (!tc_wait_warp(&aux->full[h], n & 1u, abort_flag)) { ok = false; timeout_site = 5; break; }
+          ptx::tc_fence_after();
+          uint32_t acc = 0;
+#pragma unroll
+          for (int sum = 2; sum >= 0; --sum)
+#pragma unroll
+            for (int i = 0; i <= sum; ++i)               // piece i of R, piece sum - i of W
+#pragma unroll
+              for (int jj = 0; jj < 4; ++jj) {
+                ptx::umma_bf16_ta_by(leader, tmem_base + (uint32_t)(h * 128), tmem_base + (uint32_t)(FB_TM_A + i * 64 + (h * 4 + jj) * 8),
+                                     dW + (uint32_t)(((sum - i) * FB_PIECE + (SIDE == 1 ? (h * 4 + jj) * 2048 : h * 16384 + jj * 32)) >> 4),
+                                     idesc, acc);
+                acc = 1u;
+              }
+          ptx::umma_commit_by<false>(leader, ptx::smem_u32(&aux->free_[h]));
+        }
+        if (ok) ptx::umma_commit_by<false>(leader, ptx::smem_u32(&aux->tfull));
+      }
+    }
+  } else {
+    ptx::regs_inc<FB_REGS_EPI>();
+    // ---- writing: a warp takes 32 TMEM lanes and one half of the columns
+    const int ew = warp - (FB_CONV / 32 + 4), q = warp & 3, half = ew >> 2;
+    uint8_t* stg = smem + 3 * FB_PIECE + FB_RAW * FB_HALF + 1024 + ew * 4096;
+    uint32_t n = 0;
+    for (int t = t0; t < t1; ++t, ++n) {
+      if (!tc_wait_warp(&aux->tfull, n & 1u, abort_flag)) { timeout_site = 6; break; }
+      ptx::tc_fence_after();
+      bool bad = false;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) bad |= (aux->bad[n & 3u][0][i] | aux->bad[n & 3u][1][i]) != 0;
+      const uint32_t ta = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * 64);
+      float v[64];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        uint32_t a[16], b[16];
+        ptx::tmem_ld16(ta + (uint32_t)(c * 16), a);
+        ptx::tmem_ld16(ta + 128u + (uint32_t)(c * 16), b);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[c * 16 + i] = __uint_as_float(a[i]) + __uint_as_float(b[i]);
+      }
+      ptx::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(&aux->tempty);
+      const int sb = t / g.tiles, j = t - sb * g.tiles;
+      // lane: row of the rotation's transpose, i.e. of out (SIDE 1) or column of it (SIDE 0); v: the other coordinate
+      const int f = sb * 128 + q * 32 + lane, o0 = j * 128 + half * 64;
+      const int other = SIDE == 0 ? g.rows : g.cols;
+      if (bad && f < folded) {
+        const int first = f & ~(db - 1);                 // of the block
+        const float* rb = g.R + ((int64_t)first << g.logdb) + (f - first);
+#pragma unroll
+        for (int i = 0; i < 64; ++i) {
+          if (o0 + i >= other) continue;
+          const float* w = SIDE == 0 ? g.W + (int64_t)(o0 + i) * g.ldw + first : g.W + (int64_t)first * g.ldw + o0 + i;
+          float s = 0.f;
+#pragma unroll 1
+          for (int k = 0; k < db; ++k) s = fmaf(rb[(int64_t)k << g.logdb], SIDE == 0 ? w[k] : w[(int64_t)k * g.ldw], s);
+          v[i] = s;
+        }
+      }
+      __syncwarp();
+      if (SIDE == 0) {
+        if (f < folded) {
+          float* p = g.out + (int64_t)o0 * g.ldo + f;
+#pragma unroll
+          for (int i = 0; i < 64; ++i)
+            if (o0 + i < other) __stcs(p + (int64_t)i * g.ldo, v[i]);
+        }
+      } else {
+        const int m0 = sb * 128 + q * 32, rows_ok = min(32, max(0, g.rows - m0));
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          float b[32];
+#pragma unroll
+          for (int i = 0; i < 32; ++i) b[i] = v[c * 32 + i];
+          const int cols_ok = min(32, max(0, g.cols - (o0 + c * 32)));
+          if (cols_ok > 0) sp_put_block<false>(stg, lane, b, g.out + (int64_t)m0 * g.ldo + o0 + c * 32, g.ldo, rows_ok, cols_ok);
+        }
+      }
+    }
+  }
+  if (timeout_site != 0) *reinterpret_cast<volatile int*>(g.status) = STATUS_FLAG_TIMEOUT;
+  ptx::tc_fence_before();
+  __syncthreads();
+  if (warp == FB_CONV / 32 + 1) {
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc(tmem_base, 512);
+  }
+}
+
+// 2-D fp32 tensor (rows x cols, row stride ld elements); box of box_cols x box_rows, out-of-range elements read as zero.
+inline int tc_make_tmap_f32(CUtensorMap* tm, const void* ptr, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_cols, uint32_t box_rows) {
+  PFN_encodeTiled fn = tc_encode_fn();
+  if (!fn) return CONQUR_ERR_CUDA;
+  const cuuint64_t dims[2] = {cols, rows};
+  const cuuint64_t strides[1] = {ld * 4};
+  const cuuint32_t box[2] = {box_cols, box_rows};
+  const cuuint32_t estr[2] = {1, 1};
+  const CUresult r = fn(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(ptr), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) {
+    std::fprintf(stderr, "conqur: cuTensorMapEncodeTiled (fp32) failed (%d)\n", (int)r);
+    return CONQUR_ERR_CUDA;
+  }
+  return CONQUR_OK;
+}
+
+// Folds that take this kernel: several blocks of 64 or 128, and enough tiles.  Whole call (as timed in a row), fp32 CUDA cores ->
+// this, us:  blocks of 128: 2 tiles 28 -> 33, 8 29 -> 34, 64 37 -> 35, 128 39 -> 35, 160 46 -> 39, 1024 111 -> 64, 3584 319 -> 128;
+// of 64 (half the multiply-adds): 4 tiles 27 -> 34, 80 33 -> 35, 320 43 -> 41, 1792 105 -> 84 (SIDE 0 148 -> 93).
+inline bool fold_blocks_takes(int64_t rows, int64_t cols, int block, int side) {
+  const int64_t folded = side == CONQUR_FOLD_INPUT ? cols : rows, other = side == CONQUR_FOLD_INPUT ? rows : cols;
+  if ((block != 64 && block != 128) || folded < 2 * (int64_t)block) return false;
+  const int64_t tiles = ((folded + 127) / 128) * ((other + 127) / 128);
+  return tiles >= (block == 128 ? 64 : 256) && tiles < (int64_t)1 << 30;
+}
+inline int fold_blocks_launch(const float* W, int64_t ldw, int rows, int cols, const float* R, int block, int side, float* out,
+                              int64_t ldo, int* status, int dev, int sms, cudaStream_t s) {
+  static std::atomic<unsigned long long> attr_dev_mask{0};
+  const unsigned long long dev_bit = 1ull << (dev & 63);
+  if (!(attr_dev_mask.load(std::memory_order_acquire) & dev_bit)) {
+    for (auto kern : {fold_blocks_kernel<0>, fold_blocks_kernel<1>}) {
+      // (the warpgroups' shares of registers come out of what the block is launched with)
+      cudaFuncAttributes fa;
+      if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess || fa.numRegs < FB_REGS_CONV) return CONQUR_ERR_CUDA;
+      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, FB_SMEM_BYTES) != cudaSuccess) return CONQUR_ERR_CUDA;
+    }
+    attr_dev_mask.fetch_or(dev_bit, std::memory_order_release);
+  }
+  FbArgs g{W, R, out, ldw, ldo, block == 64 ? 6 : 7, rows, cols, 0, 0, 0, status};
+  const bool in = side == CONQUR_FOLD_INPUT;
+  g.n_super = ((in ? cols : rows) + 127) / 128;
+  g.tiles = ((in ? rows : cols) + 127) / 128;
+  CUtensorMap tm = {};
+  if ((ldw & 3) == 0 && (reinterpret_cast<uintptr_t>(W) & 15) == 0) {
+    if (tc_make_tmap_f32(&tm, W, (uint64_t)rows, (uint64_t)cols, (uint64_t)ldw, in ? 64 : 128, in ? 128 : 64) != CONQUR_OK) return CONQUR_ERR_CUDA;
+    g.copied = 1;
+  }
+  const int64_t total = (int64_t)g.n_super * g.tiles;
+  const unsigned grid = (unsigned)(total < sms ? total : sms);
+  if (in) fold_blocks_kernel<0><<<grid, FB_THREADS, FB_SMEM_BYTES, s>>>(tm, g);
+  else fold_blocks_kernel<1><<<grid, FB_THREADS, FB_SMEM_BYTES, s>>>(tm, g);
+  return cudaGetLastError() == cudaSuccess ? CONQUR_OK : CONQUR_ERR_CUDA;
+}
+
+}  // namespace conqur

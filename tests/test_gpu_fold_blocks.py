@@ -1,0 +1,69 @@
+"""Block-diagonal weight folds over bf16 pieces on the tensor cores against float64, and the values that pieces cannot hold."""
+import pytest
+import torch
+
+from paper_2605_10793_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+
+
+def _rand(seed, *shape):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    return torch.randn(*shape, generator=g, device="cuda")
+
+
+def _reference(w, r, side):
+    k, b = r.shape[0], r.shape[1]
+    w, r = w.double(), r.double()
+    if side == "input":
+        return torch.einsum("akb,kbc->akc", w.view(-1, k, b), r).reshape(w.shape)
+    return torch.einsum("kba,kbc->kac", r, w.view(k, b, -1)).reshape(w.shape)
+
+
+# (blocks, block, other side): odd numbers of 64-blocks, fewest tiles and more than one a block of threads, remainders of a tile
+# and of 16-byte pieces; the first two stay on the CUDA cores
+SHAPES = [(2, 64, 32), (3, 128, 127), (65, 64, 993), (2, 128, 4065), (3, 128, 2690), (32, 128, 1003), (127, 64, 640), (4, 128, 9000)]
+
+
+@pytest.mark.parametrize("k,b,other", SHAPES)
+@pytest.mark.parametrize("side", ["input", "output"])
+@pytest.mark.parametrize("mode", ["exact", "tc"])
+def test_fold_of_several_blocks(k, b, other, side, mode):
+    shape = (other, k * b) if side == "input" else (k * b, other)
+    r = _rand(k + b, k, b, b) / b ** 0.5
+    wide = _rand(other, shape[0], shape[1] + 3) * torch.exp(3.0 * _rand(other + 1, shape[0], 1))
+    for w in (wide[:, : shape[1]].contiguous(), wide[:, 1: shape[1] + 1]):           # (the second off 16-byte boundaries)
+        got = B.conqur_fold_weight(w, r, side, mode).double()
+        ref, size = _reference(w.contiguous(), r, side), _reference(w.abs().contiguous(), r.abs(), side)
+        # two sums of 64 terms: per sum 4 instructions' cuts of 16 2^-25 + 2^-23, the smaller pieces' twenty at 2^-7 of that,
+        # the pieces' remainder 2^-25; one fp32 addition
+        assert ((got - ref).abs() <= (4 * 10 + 4 + 2) * 2.0 ** -24 * size).all()
+        assert float((got - ref).norm() / ref.norm()) <= 4.0 * 2.0 ** -24           # an fp32 chain of 64 leaves 2.4 .. 2.9, of 128 3.4 .. 3.7
+
+
+@pytest.mark.parametrize("side", ["input", "output"])
+@pytest.mark.parametrize("b", [64, 128])
+def test_values_that_pieces_cannot_hold(side, b):
+    """Infinities, NaN, the largest and tiny values give what a fold of the one block by itself gives."""
+    k, other = 4, 16500
+    r = _rand(1, k, b, b) / b ** 0.5
+    w = _rand(2, *((other, k * b) if side == "input" else (k * b, other)))
+    v = w if side == "input" else w.T                   # (other, folded)
+    v[3, b + 5] = float("inf")
+    v[4, 5] = float("nan")
+    v[140, 2 * b + 1] = 3.4e38
+    v[290, : k * b] *= 1e-36
+    r[3, 2, 2] = float("-inf")
+    got = B.conqur_fold_weight(w, r, side, "exact")
+    for i in range(k):
+        part = w[:, i * b:(i + 1) * b] if side == "input" else w[i * b:(i + 1) * b]
+        ref = B.conqur_fold_weight(part, r[i], side, "exact")
+        out = got[:, i * b:(i + 1) * b] if side == "input" else got[i * b:(i + 1) * b]
+        assert torch.equal(torch.isnan(out), torch.isnan(ref))
+        assert torch.equal(torch.isinf(out), torch.isinf(ref))
+        assert torch.equal(out[torch.isinf(out)], ref[torch.isinf(ref)])
+        fine = torch.isfinite(ref)
+        p, q = out.double(), ref.double()
+        sz = _reference(torch.nan_to_num(part, 0.0, 0.0, 0.0).abs(), torch.nan_to_num(r[i:i + 1], 0.0, 0.0, 0.0).abs(), side)
+        assert ((p - q).abs()[fine] <= (b + 46) * 2.0 ** -24 * sz[fine]).all()
