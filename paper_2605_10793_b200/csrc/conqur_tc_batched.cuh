@@ -520,6 +520,10 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&w)[16
         "r"(w[9]), "r"(w[10]), "r"(w[11]), "r"(w[12]), "r"(w[13]), "r"(w[14]), "r"(w[15])
       : "memory");
 }
+// Brings `bytes` (a multiple of 16, from a 16-byte boundary) of global memory into the L2; nothing waits for it.
+__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 }  // namespace ptx
 
@@ -1164,6 +1168,13 @@ __global__ void __launch_bounds__(TCBU_THREADS, 2) tcb_update_kernel(const TcbUp
         *reinterpret_cast<uint2*>(sXl + off) = make_uint2(l0, l1);
       }
       issue_products(issue_gram);
+      // the next problem's matrices come into the L2 while this one is iterated (read from memory when they were needed, they took
+      // 19 k of a problem's 187 k SM cycles: all blocks ask for theirs at about the same time)
+      const int pn = p + (int)gridDim.x;
+      if (threadIdx.x == 64 && pn < g.P) {
+        ptx::prefetch_l2(g.M + (long long)pn * TCB_D * TCB_D, TCB_D * TCB_D * 4);
+        if (need_r) ptx::prefetch_l2(g.R + (long long)pn * TCB_D * TCB_D, TCB_D * TCB_D * 4);
+      }
       bool gram_in_flight = true;
       for (int k = 0; k <= ncp.max_steps; ++k) {
         // ---- G = X^T X (issued before the loop / at the end of the previous step)
