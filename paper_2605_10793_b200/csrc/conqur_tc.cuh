@@ -1155,14 +1155,20 @@ inline int tc_epi_class(int epi) {
   }
 }
 
-// Which kernel variant a product of output width N runs with.
+// Which kernel variant a product of M x N outputs runs with.
 //   pair : CTA pairs on 256 x 256 tiles (needs N % 256 == 0 and a device that can co-schedule the pairs)
 //   else : single CTAs on 128 x 256 (N % 256 == 0) or 128 x 128 tiles
+// Steps of few rows at small widths take 128 x 128 tiles throughout: more SMs work, and the last epilogue, which nothing hides
+// there, is a quarter.  Whole step, us: 64 x 256 24.8 -> 22.7, 512 x 512 28.9 -> 24.7, 64 x 1024 28.8 -> 24.8, 512 x 1024 30.9 -> 28.9;
+// beyond, a tile's operands take longer: 4096 x 512 45.3 -> 46.0, 64 x 4096 53 -> 56 (and the Newton-Schulz products, whose split
+// operands a pair fetches once for all passes: a step at d = 1024 67 -> 70, 1536 80 -> 89).
 struct TcVariant { bool pair; int tile_m, tile_n; };
-inline TcVariant tc_variant(const TcHost& h, int N) {
-  if (N % 256 == 0) return h.pair_clusters > 0 ? TcVariant{true, 256, 256} : TcVariant{false, 128, 256};
+inline TcVariant tc_variant(const TcHost& h, int N, bool small = false) {
+  if (N % 256 == 0 && !small) return h.pair_clusters > 0 ? TcVariant{true, 256, 256} : TcVariant{false, 128, 256};
   return TcVariant{false, 128, 128};
 }
+// (M x N outputs of a step's product over K)
+inline bool tc_small_step(int64_t M, int64_t N, int64_t K) { return ((M + 127) / 128) * ((N + 127) / 128) <= 64 && K <= 1024; }
 // tiles the kernel computes
 inline int tc_tiles(const TcVariant& v, int M, int N, int sym) {
   const int tn = (N + v.tile_n - 1) / v.tile_n, tm = (M + v.tile_m - 1) / v.tile_m;
@@ -1251,7 +1257,8 @@ inline int tc_launch(TcHost& h, cudaStream_t s, const CUtensorMap& a, const CUte
 // dispatch on the kernel variant (see tc_variant)
 template <bool A_MN, bool B_MN, int EPI>
 inline int tc_launch_n(TcHost& h, cudaStream_t s, const CUtensorMap& a, const CUtensorMap& b, const TcGemmArgs& g) {
-  const TcVariant v = tc_variant(h, g.N);
+  constexpr bool step = EPI == TC_EPI_ROTATE || EPI == TC_EPI_ROTATE_Q || EPI == TC_EPI_ACCUM;
+  const TcVariant v = tc_variant(h, g.N, step && tc_small_step(g.M, g.N, g.K));
   if (v.pair) {
     TcGemmArgs gg = g;
     tc_fuse_passes(&gg);
@@ -1414,7 +1421,7 @@ inline int tc_process(TcHost& h, cudaStream_t s, int64_t n) {
     g.outH = Cp; g.ldh = d;
     rc = tc_launch_n<false, true, TC_EPI_ROTATE>(h, s, tmXs_k, h.tmRb_mn, g);
     if (rc) return rc;
-    per_problem = tc_part_slots(h, tc_variant(h, d), (int)n, d, 0);
+    per_problem = tc_part_slots(h, tc_variant(h, d, tc_small_step(n, d, d)), (int)n, d, 0);
   } else {
     unsigned* rowmin = h.rowmax + h.n_max;
     if (cudaMemsetAsync(h.rowmax, 0, sizeof(unsigned) * n, s) != cudaSuccess) return CONQUR_ERR_CUDA;
