@@ -108,7 +108,7 @@ bool make_layout(int d, const conqur_config* c, Layout* L) {
   L->rowmax = take(sizeof(unsigned) * 2 * n * P);   // per row: ordered max, then ordered min (quant modes)
   int64_t mp = std::max<int64_t>((int64_t)cdiv(n, 128) * cdiv(d, 128), (int64_t)cdiv(d, 128) * cdiv(d, 128));
   mp = std::max<int64_t>(mp, cdiv(n, 8));
-  mp = std::max<int64_t>(mp, 2 * (int64_t)cdiv(d, 128) * cdiv(d, 128) + 64);   // two partial arrays per Newton-Schulz product
+  mp = std::max<int64_t>(mp, 3 * (int64_t)cdiv(d, 128) * cdiv(d, 128) + 64);   // three partial arrays of a Newton-Schulz step
   mp = std::max<int64_t>(mp, 1024);
   const bool pieces = c->mode == CONQUR_EXACT_F32 && sp_layout_wanted(d, (int)P);
   if (pieces) mp = std::max<int64_t>(mp, 16 * (int64_t)cdiv(n, 256) * cdiv(d, 128));   // sixteen per tile of at least 256 x 128
@@ -608,7 +608,6 @@ int update_epilogue(conqur_ctx* c) {
     int rc = tc_ns_commit(c->tc, c->stream);
     if (rc) return rc;
   }
-  if (g.mode == CONQUR_TC_BF16) { int rc = tc_refresh_R(c->tc, c->stream, /*only_if_converged=*/1); if (rc) return rc; }
   ns_commit_state_kernel<<<g.P, 32, 0, c->stream>>>(st, c->n_sched - 1);
   CQ_LAUNCHED(c, K_OTHER);
   c->tc.ns_k = -1;

@@ -939,6 +939,15 @@ __device__ __forceinline__ unsigned char ns_control_decide(NsCtl* s, float tmx, 
   return log_entry;
 }
 
+// Whether the next residual product takes three passes over the bf16 pair: when it may accept the rotation, i.e. once the last
+// endgame entry has been applied or no step is left, and for the step that applies that entry: it hands the rounding of its G on
+// to X^T X - I.  One over the fp16 copy otherwise (see tc_ns_residual), except that a caller's threshold (e1_tau > 0, ns_tau_kernel)
+// asks for three wherever tau has reached it.  (max|X^T X - I| of accepted rotations, d = 1280 .. 4096: 4e-5 .. 9e-5 with one
+// pass in that last step, 6e-6 .. 1e-5 with three; at d = 512 one pass cost every update a step more.)
+__device__ __forceinline__ bool ns_full_residual(const DevState* s, int n_sched, int max_steps) {
+  return s->ns_idx >= n_sched - 1 || s->ns_steps_used >= max_steps;
+}
+
 static __global__ void ns_control_kernel(DevState* st, const float* __restrict__ part_max,
                                   const double* __restrict__ part_sq, const double* __restrict__ part_tr,
                                   int nparts, int k, int cur_buf, const NsControlParams c) {
@@ -964,15 +973,12 @@ static __global__ void ns_control_kernel(DevState* st, const float* __restrict__
     const unsigned char log_entry = ns_control_decide(&t, tmx, tsq, ttr, k, cur_buf, c);
     ns_ctl_store(t, s);
     if (log_entry && k < 128) s->seg_log[k] = log_entry;
+    if (log_entry && c.full_check) s->seg_e = ns_full_residual(s, c.n_sched, c.max_steps) ? 3 : 1;
   }
 }
 
-// tau of the next residual product = mean sigma^2 of the new iterate = ||X||_F^2 / d (tensor-core mode), and how
-// many passes that product takes.  Three over the bf16 pair when it may accept the rotation, i.e. once the last endgame
-// entry has been applied or no step is left, and for the step that applies that entry: it hands the rounding of its G on
-// to X^T X - I.  One over the fp16 copy otherwise (see tc_ns_residual), except that a caller's threshold (e1_tau > 0) asks
-// for three wherever tau has reached it.  (max|X^T X - I| of accepted rotations, d = 1280 .. 4096: 4e-5 .. 9e-5 with one
-// pass in that last step, 6e-6 .. 1e-5 with three; at d = 512 one pass cost every update a step more.)
+// tau of the next residual product, where a threshold on it decides the passes that product takes (e1_tau > 0): mean sigma^2 of
+// the new iterate = ||X||_F^2 / d.  (Otherwise the product's own epilogue forms it.)
 static __global__ void ns_tau_kernel(DevState* st, const double* __restrict__ part_x2, int nparts, int d, float e1_tau,
                                      int n_sched, int max_steps) {
   DevState* s = st + blockIdx.x;
@@ -983,7 +989,7 @@ static __global__ void ns_tau_kernel(DevState* st, const double* __restrict__ pa
   const double tot = block_sum_d<256>(v, redd);
   if (threadIdx.x == 0) {
     s->tau = (float)(tot / (double)d);
-    const bool full = s->ns_idx >= n_sched - 1 || s->ns_steps_used >= max_steps;
+    const bool full = ns_full_residual(s, n_sched, max_steps);
     s->seg_e = (full || (e1_tau > 0.f && s->tau >= e1_tau)) ? 3 : 1;
   }
 }

@@ -260,6 +260,7 @@ struct TcGemmArgs {
   unsigned* rowmax; unsigned* rowmin;   // per-row ordered max / min of the raw products (quant modes)
   double* part_d; float* part_f;
   double* part_t;               // per-tile trace (residual) or sum of squares (next iterate)
+  const double* x2_part; int n_x2;   // residual: the sums of squares the last next-iterate product left (n_x2 == 0: tau is in the state)
   DevState* st;
   int check_done;
 };
@@ -650,7 +651,17 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       c_b1 *= 1.f / TC_F16_SCALE;
     }
     const bool b16 = EPI == TC_EPI_POLY && g.st->seg_x == 1;       // B goes into a product on fp16 operands
-    if (EPI == TC_EPI_RESID) c_tau = g.st->tau;
+    if (EPI == TC_EPI_RESID) {
+      // tau = mean sigma^2 of the iterate = ||X||_F^2 / d; every warp adds the parts up in the same order while the first tile's
+      // products run (a launch of its own took 4.5 us a step)
+      c_tau = g.st->tau;
+      if (g.n_x2 > 0 && g.st->ns_steps_used > 0) {
+        double x2 = 0.0;
+        for (int i = lane; i < g.n_x2; i += 32) x2 += g.x2_part[i];
+        c_tau = (float)(warp_sum_d(x2) / (double)g.N);
+        if (worker == 0 && rank == 0 && ew == 0 && lane == 0) g.st->tau = c_tau;      // (for the decision that follows this launch)
+      }
+    }
     int local = 0;
     bool ok = true;
     const uint32_t tempty_addr0 = PAIR ? ptx::mapa_u32(ptx::smem_u32(&aux->tempty[0]), 0) : 0u;
@@ -1471,7 +1482,7 @@ inline int tc_ns_begin(TcHost& h, cudaStream_t s) {
 }
 
 
-// Partials of the Newton-Schulz epilogues: [0, parts) sums of squares, [parts, 2 parts) traces / iterate norms.
+// Partials of the Newton-Schulz epilogues: [0, parts) sums of squares, [parts, 2 parts) traces, then the iterate's norms.
 inline int tc_ns_parts(const TcHost& h) { return tc_part_slots(h, tc_variant(h, h.d), h.d, h.d, 1); }
 inline int tc_ns_next_parts(const TcHost& h) { return tc_part_slots(h, tc_variant(h, h.d), h.d, h.d, 0); }
 
@@ -1486,6 +1497,8 @@ inline int tc_ns_residual(TcHost& h, cudaStream_t s, int buf) {
   g.nseg = 3; g.nseg_from_state = 2; g.a_off[2] = d; g.b_off[1] = d; g.check_done = 1; g.sym = 1;
   g.outH = reinterpret_cast<__nv_bfloat16*>(h.ws + h.L.Eh); g.ldh = d;
   g.part_t = h.part_d + tc_ns_parts(h);
+  g.x2_part = h.part_d + 2 * tc_ns_parts(h);
+  g.n_x2 = h.e1_tau > 0.f ? 0 : tc_ns_next_parts(h);
   h.f16_map = &h.tmX16_mn[buf];
   return tc_launch_n<true, true, TC_EPI_RESID>(h, s, h.tmXh_mn[buf], h.tmXh_mn[buf], g);
 }
@@ -1508,17 +1521,19 @@ inline int tc_ns_poly_next(TcHost& h, cudaStream_t s, int cur, int n_sched, int 
   x.outH = reinterpret_cast<__nv_bfloat16*>(h.ws + h.L.Xh[1 - cur]); x.ldh = d; x.lo_elems = dd;
   x.out16 = reinterpret_cast<uint16_t*>(cur ? h.Xa : h.Xb);
   h.f16_map = &h.tmX16_k[cur];
-  x.part_t = h.part_d + tc_ns_parts(h);
+  x.part_t = h.part_d + 2 * tc_ns_parts(h);
   rc = tc_launch_n<false, true, TC_EPI_NEXT>(h, s, h.tmXh_k[cur], h.tmBh_mn, x);
   if (rc) return rc;
-  ns_tau_kernel<<<1, 256, 0, s>>>(h.st, h.part_d + tc_ns_parts(h), tc_ns_next_parts(h), d, h.e1_tau, n_sched, max_steps);
-  if (h.prof) h.prof->count(K_OTHER);
+  if (h.e1_tau > 0.f) {                                     // the threshold on tau decides how many passes the next residual takes
+    ns_tau_kernel<<<1, 256, 0, s>>>(h.st, x.part_t, tc_ns_next_parts(h), d, h.e1_tau, n_sched, max_steps);
+    if (h.prof) h.prof->count(K_OTHER);
+  }
   return cudaGetLastError() == cudaSuccess ? CONQUR_OK : CONQUR_ERR_CUDA;
 }
 
-// Accept the update in tensor-core mode: R <- hi + lo of the final iterate, M <- 0.
+// Accept the update in tensor-core mode: R <- hi + lo of the final iterate, with the bf16 copy the products read; M <- 0.
 static __global__ void tc_commit_kernel(DevState* st, const __nv_bfloat16* __restrict__ X0, const __nv_bfloat16* __restrict__ X1,
-                                        float* __restrict__ R, float* __restrict__ M, int64_t dd) {
+                                        float* __restrict__ R, float* __restrict__ M, __nv_bfloat16* __restrict__ Rb, int64_t dd) {
   if (st->ns_done != NS_DONE_CONVERGED) return;
   const __nv_bfloat16* X = st->ns_final_buf ? X1 : X0;
   for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 2; i < dd; i += (int64_t)gridDim.x * blockDim.x * 2) {
@@ -1527,13 +1542,15 @@ static __global__ void tc_commit_kernel(DevState* st, const __nv_bfloat16* __res
     o.x = __uint_as_float(hb << 16) + __uint_as_float(lb << 16);
     o.y = __uint_as_float(hb & 0xffff0000u) + __uint_as_float(lb & 0xffff0000u);
     *reinterpret_cast<float2*>(R + i) = o;
+    *reinterpret_cast<uint32_t*>(Rb + i) = bf16x2_pack(o.x, o.y);
     *reinterpret_cast<float2*>(M + i) = make_float2(0.f, 0.f);
   }
 }
 inline int tc_ns_commit(TcHost& h, cudaStream_t s) {
   const int64_t dd = (int64_t)h.d * h.d;
   tc_commit_kernel<<<tc_ew_blocks(dd / 2), 256, 0, s>>>(h.st, reinterpret_cast<const __nv_bfloat16*>(h.ws + h.L.Xh[0]),
-                                                       reinterpret_cast<const __nv_bfloat16*>(h.ws + h.L.Xh[1]), h.R, h.M, dd);
+                                                       reinterpret_cast<const __nv_bfloat16*>(h.ws + h.L.Xh[1]), h.R, h.M,
+                                                       reinterpret_cast<__nv_bfloat16*>(h.ws + h.L.Rb), dd);
   if (h.prof) h.prof->count(K_OTHER);
   return cudaGetLastError() == cudaSuccess ? CONQUR_OK : CONQUR_ERR_CUDA;
 }
