@@ -54,7 +54,9 @@ enum { CONQUR_EXACT_F32 = 0, CONQUR_TC_BF16 = 1 };   /* arithmetic mode */
 enum { CONQUR_QUANT_SYMMETRIC = 0, CONQUR_QUANT_ZEROPOINT = 1 };   /* fake-quantiser applied when quant_bits > 0 */
 
 /*
- * mode CONQUR_EXACT_F32: fp32 CUDA-core contractions throughout (parity anchor).
+ * mode CONQUR_EXACT_F32: fp32 contractions throughout (parity anchor): on the CUDA cores, or for steps of one wide
+ *                        problem on the tensor cores over exact three-term bf16 splits whose sums are carried in
+ *                        fp32 (no less precise; the workspace then holds the split rows, targets and rotation).
  * mode CONQUR_TC_BF16:   bf16 operands, fp32 accumulation on the tcgen05 tensor
  *                        cores; fp32 X is rounded to bf16 on the way in; the
  *                        Newton-Schulz iterate is held as a two-term bf16 split hi + lo
@@ -396,13 +398,14 @@ int conqur_objective_noalloc(const void* X_dev, int32_t in_dtype, int64_t n, int
  * block.
  *   W_dev / out_dev   device fp32, rows x cols, row strides ldw / ldo elements (>= cols); out_dev must not
  *                     overlap W_dev
- *   mode              CONQUR_EXACT_F32: fp32 CUDA-core product.
+ *   mode              CONQUR_EXACT_F32: fp32 product.
  *                     CONQUR_TC_BF16: for one full rotation (block == folded dimension, a multiple of 128;
  *                     rows % 8 == 0 for INPUT, cols % 32 == 0 for OUTPUT; ldw, ldo multiples of 4; 16-byte
  *                     aligned pointers) both operands are split into bf16 hi + lo and the product is taken
  *                     in three tensor-core passes (hi hi, hi lo, lo hi) with fp32 accumulation, relative
  *                     error about 2^-16; shapes outside these limits return CONQUR_ERR_UNSUPPORTED.
- *                     Block-diagonal folds (block < folded dimension) use the fp32 product in either mode.
+ *                     Block-diagonal folds (block < folded dimension) use the fp32 product in either mode: on the
+ *                     CUDA cores, or for enough blocks of 64 or 128 on the tensor cores over three-term splits.
  *   scratch_dev       device memory, 256-byte aligned, >= conqur_fold_scratch_bytes(...) bytes (returns -1 for
  *                     invalid arguments); owned by the caller, free to reuse after the call returns
  * Synchronises the stream and returns the status (CONQUR_ERR_TIMEOUT if a bounded device wait expired).
