@@ -1344,14 +1344,14 @@ extern "C" int conqur_fold_weight(const float* W_dev, int64_t ldw, int32_t rows,
   if (fold_blocks_takes(rows, cols, block, side) && cudaGetDevice(&dev) == cudaSuccess && tc_device_facts(dev, &facts) == CONQUR_OK &&
       facts.major == 10) {
     if (int* status = static_cast<int*>(mail_pool().take())) {
-      *status = 0;
+      status[0] = status[1] = 0;
       const int rc = fold_blocks_launch(W_dev, ldw, rows, cols, R_dev, block, side, out_dev, ldo, status, dev, facts.sms, s);
       const cudaError_t e = cudaStreamSynchronize(s);
-      const int f = *status;
+      const int f = status[0], unfit = status[1];
       mail_pool().give(status);
       if (rc) return rc;
       CQ_CUDA(e);
-      return flags_to_status(f);
+      if (f || !unfit) return flags_to_status(f);     // (values that pieces cannot hold: all of it on the CUDA cores)
     }
   }
   const int64_t fm = side == CONQUR_FOLD_INPUT ? rows : block, fn = side == CONQUR_FOLD_INPUT ? block : cols;

@@ -12,8 +12,9 @@
 // rotation (4 k cycles, once or twice) and the pipeline's fill; 4096 x 14336 4.4 TB/s.
 // Error against 64 bits, in 2^-24 of the result's norm, fp32 chain / this: 128-blocks 3.4 / 1.4, 64-blocks 2.4 / 1.3.
 //
-// A tile with values that pieces cannot hold (not finite; or below 2^-100, whose low pieces would underflow) is computed with
-// fp32 multiply-adds by the warps that write it.
+// Both operands are split after a multiplication by 2^32, so that no piece of any fp32 number is subnormal (its last bit is worth
+// 2^-149 at least), and the sums come back by 2^-64: powers of two, which change no bit.  What is left are values that are not
+// finite or so large that scaled sums could overflow; a fold that meets one says so, and the caller runs the CUDA-core kernel instead.
 #pragma once
 #include "conqur_split_tc.cuh"
 #include "conqur_tc_batched.cuh"
@@ -46,25 +47,22 @@ struct FbArgs {
   int logdb, rows, cols;            // blocks of 1 << logdb
   int n_super, tiles;               // 128-wide groups of blocks; W tiles along the other dimension
   int copied;                       // 1: W's rows suit the copy engine (16-byte aligned)
-  int* status;                      // page-locked host memory, cleared by the caller
+  int* status;                      // page-locked host memory, two words cleared by the caller: flags, and whether a value was unfit
 };
 struct FbAux {
   uint64_t raw_full[FB_RAW], raw_free[FB_RAW], full[2], free_[2], tfull, tempty;
   uint32_t tmem_base;
   int abort_flag;
-  int bad[4][2][8];                 // per tile (ring), half and splitting warp: values that pieces cannot hold
 };
 static_assert(sizeof(FbAux) <= 1024, "reserved behind the operands");
 
-// Largest and smallest nonzero magnitude of what it is shown, as integers: pieces hold values from 2^-100 to below 2^128 - 2^119.
+constexpr float FB_UP = 4294967296.f, FB_DOWN = 1.f / FB_UP / FB_UP;     // 2^32, and back (128 products: 2^39 2^16 2^64 2^7 < 2^128)
+constexpr float FB_W_LIMIT = 549755813888.f, FB_R_LIMIT = 65536.f;       // 2^39, 2^16
+// Largest magnitude of what it is shown; NaN stays.
 struct FbRange {
-  uint32_t hi = 0u, lo = 0xffffffffu;
-  __device__ __forceinline__ void see(float v) {
-    const uint32_t m = __float_as_uint(v) << 1;
-    hi = max(hi, m);
-    lo = min(lo, m - 1u);                                // (zero wraps to the largest number)
-  }
-  __device__ __forceinline__ bool unfit() const { return hi >= (0x7f7f8000u << 1) || lo < (0x0d800000u << 1) - 1u; }
+  float hi = 0.f;
+  __device__ __forceinline__ void see(float v) { asm("max.NaN.f32 %0, %0, %1;" : "+f"(hi) : "f"(fabsf(v))); }
+  __device__ __forceinline__ bool within(float limit) const { return hi < limit; }
 };
 
 template <int SIDE>
@@ -101,7 +99,7 @@ __global__ void __launch_bounds__(FB_THREADS, 1) fold_blocks_kernel(const __grid
   if (warp < FB_CONV / 32) {
     // ---- splitting, one half of k after the other (64 rows of the tile on SIDE 1, 64 columns on SIDE 0): 4 elements eight times a thread
     int cur_sb = -1;
-    bool r_bad = false;
+    bool bad = false;
     uint32_t n = 0, it = 0;
     bool ok = true;
     for (int t = t0; t < t1 && ok; ++t, ++n) {
@@ -130,12 +128,12 @@ __global__ void __launch_bounds__(FB_THREADS, 1) fold_blocks_kernel(const __grid
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             rr.see(v[2 * i]); rr.see(v[2 * i + 1]);
-            sp_split2(v[2 * i], v[2 * i + 1], w[0][i], w[1][i], w[2][i]);
+            sp_split2(v[2 * i] * FB_UP, v[2 * i + 1] * FB_UP, w[0][i], w[1][i], w[2][i]);
           }
 #pragma unroll
           for (int p = 0; p < 3; ++p) ptx::tmem_st8(ta + (uint32_t)(p * 64 + k0 / 2), w[p]);
         }
-        r_bad = rr.unfit();
+        bad |= !rr.within(FB_R_LIMIT);
         ptx::tmem_st_wait();
         ptx::tc_fence_before();
       }
@@ -145,32 +143,37 @@ __global__ void __launch_bounds__(FB_THREADS, 1) fold_blocks_kernel(const __grid
         if (g.copied && !tc_wait_warp(&aux->raw_full[slot], (it / FB_RAW) & 1u, abort_flag)) { ok = false; timeout_site = 2; break; }
         if (!tc_wait_warp(&aux->free_[h], ph, abort_flag)) { ok = false; timeout_site = 1; break; }
         FbRange rr;
+        const int row0 = threadIdx.x >> (SIDE == 0 ? 4 : 5), c4 = threadIdx.x & (SIDE == 0 ? 15 : 31);
+        constexpr int ROWS = SIDE == 0 ? 16 : 8;         // from one of a thread's eight pieces to the next
+        float4 v[8];                                     // (all on their way before the first is split)
+        if (g.copied) {
+          const uint8_t* src = sRaw + slot * FB_HALF + row0 * (SIDE == 0 ? 256 : 512) + c4 * 16;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int e = threadIdx.x + 256 * i;
-          const int row = SIDE == 0 ? e >> 4 : e >> 5, c4 = SIDE == 0 ? e & 15 : e & 31;
-          const int r = SIDE == 0 ? row : 64 * h + row, u = SIDE == 0 ? 8 * h + (c4 >> 1) : c4 >> 1;
-          float4 v;
-          if (g.copied) {
-            v = *reinterpret_cast<const float4*>(sRaw + slot * FB_HALF + (SIDE == 0 ? row * 256 : row * 512) + c4 * 16);
-          } else {
+          for (int i = 0; i < 8; ++i) v[i] = *reinterpret_cast<const float4*>(src + i * ROWS * (SIDE == 0 ? 256 : 512));
+        } else {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const int row = row0 + i * ROWS;
             const int gr = (SIDE == 0 ? j * 128 + row : sb * 128 + 64 * h + row), gc = (SIDE == 0 ? sb * 128 + 64 * h : j * 128) + c4 * 4;
             const float* p = g.W + (int64_t)gr * g.ldw + gc;
             const bool in = gr < g.rows;
-            v.x = in && gc < g.cols ? p[0] : 0.f; v.y = in && gc + 1 < g.cols ? p[1] : 0.f;
-            v.z = in && gc + 2 < g.cols ? p[2] : 0.f; v.w = in && gc + 3 < g.cols ? p[3] : 0.f;
+            v[i].x = in && gc < g.cols ? p[0] : 0.f; v[i].y = in && gc + 1 < g.cols ? p[1] : 0.f;
+            v[i].z = in && gc + 2 < g.cols ? p[2] : 0.f; v[i].w = in && gc + 3 < g.cols ? p[3] : 0.f;
           }
-          rr.see(v.x); rr.see(v.y); rr.see(v.z); rr.see(v.w);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int row = row0 + i * ROWS, r = SIDE == 0 ? row : 64 * h + row, u = SIDE == 0 ? 8 * h + (c4 >> 1) : c4 >> 1;
+          rr.see(v[i].x); rr.see(v[i].y); rr.see(v[i].z); rr.see(v[i].w);
           uint2 w[3];
-          sp_split2(v.x, v.y, w[0].x, w[1].x, w[2].x);
-          sp_split2(v.z, v.w, w[0].y, w[1].y, w[2].y);
+          sp_split2(v[i].x * FB_UP, v[i].y * FB_UP, w[0].x, w[1].x, w[2].x);
+          sp_split2(v[i].z * FB_UP, v[i].w * FB_UP, w[0].y, w[1].y, w[2].y);
           uint8_t* q = sW + (u >> 3) * 16384 + r * 128 + (((u & 7) ^ (r & 7)) << 4) + (c4 & 1) * 8;
 #pragma unroll
           for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2*>(q + p * FB_PIECE) = w[p];
         }
-        const bool any = __any_sync(0xffffffffu, r_bad || rr.unfit());
+        bad |= !rr.within(FB_W_LIMIT);
         ptx::fence_proxy_async();
-        if (lane == 0) aux->bad[n & 3u][h][warp] = any ? 1 : 0;
         __syncwarp();
         if (lane == 0) {
           if (g.copied) ptx::mbar_arrive(&aux->raw_free[slot]);
@@ -178,6 +181,7 @@ __global__ void __launch_bounds__(FB_THREADS, 1) fold_blocks_kernel(const __grid
         }
       }
     }
+    if (bad) reinterpret_cast<volatile int*>(g.status)[1] = 1;
   } else if (warp < FB_CONV / 32 + 4) {
     ptx::regs_dec<FB_REGS_ISSUE>();
     if (warp == FB_CONV / 32 && lane == 0 && g.copied) {
@@ -237,9 +241,6 @@ __global__ void __launch_bounds__(FB_THREADS, 1) fold_blocks_kernel(const __grid
     for (int t = t0; t < t1; ++t, ++n) {
       if (!tc_wait_warp(&aux->tfull, n & 1u, abort_flag)) { timeout_site = 6; break; }
       ptx::tc_fence_after();
-      bool bad = false;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) bad |= (aux->bad[n & 3u][0][i] | aux->bad[n & 3u][1][i]) != 0;
       const uint32_t ta = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * 64);
       float v[64];
 #pragma unroll
@@ -257,26 +258,12 @@ __global__ void __launch_bounds__(FB_THREADS, 1) fold_blocks_kernel(const __grid
       // lane: row of the rotation's transpose, i.e. of out (SIDE 1) or column of it (SIDE 0); v: the other coordinate
       const int f = sb * 128 + q * 32 + lane, o0 = j * 128 + half * 64;
       const int other = SIDE == 0 ? g.rows : g.cols;
-      if (bad && f < folded) {
-        const int first = f & ~(db - 1);                 // of the block
-        const float* rb = g.R + ((int64_t)first << g.logdb) + (f - first);
-#pragma unroll
-        for (int i = 0; i < 64; ++i) {
-          if (o0 + i >= other) continue;
-          const float* w = SIDE == 0 ? g.W + (int64_t)(o0 + i) * g.ldw + first : g.W + (int64_t)first * g.ldw + o0 + i;
-          float s = 0.f;
-#pragma unroll 1
-          for (int k = 0; k < db; ++k) s = fmaf(rb[(int64_t)k << g.logdb], SIDE == 0 ? w[k] : w[(int64_t)k * g.ldw], s);
-          v[i] = s;
-        }
-      }
-      __syncwarp();
       if (SIDE == 0) {
         if (f < folded) {
           float* p = g.out + (int64_t)o0 * g.ldo + f;
 #pragma unroll
           for (int i = 0; i < 64; ++i)
-            if (o0 + i < other) __stcs(p + (int64_t)i * g.ldo, v[i]);
+            if (o0 + i < other) __stcs(p + (int64_t)i * g.ldo, v[i] * FB_DOWN);
         }
       } else {
         const int m0 = sb * 128 + q * 32, rows_ok = min(32, max(0, g.rows - m0));
@@ -284,7 +271,7 @@ __global__ void __launch_bounds__(FB_THREADS, 1) fold_blocks_kernel(const __grid
         for (int c = 0; c < 2; ++c) {
           float b[32];
 #pragma unroll
-          for (int i = 0; i < 32; ++i) b[i] = v[c * 32 + i];
+          for (int i = 0; i < 32; ++i) b[i] = v[c * 32 + i] * FB_DOWN;
           const int cols_ok = min(32, max(0, g.cols - (o0 + c * 32)));
           if (cols_ok > 0) sp_put_block<false>(stg, lane, b, g.out + (int64_t)m0 * g.ldo + o0 + c * 32, g.ldo, rows_ok, cols_ok);
         }

@@ -67,3 +67,73 @@ def test_values_that_pieces_cannot_hold(side, b):
         p, q = out.double(), ref.double()
         sz = _reference(torch.nan_to_num(part, 0.0, 0.0, 0.0).abs(), torch.nan_to_num(r[i:i + 1], 0.0, 0.0, 0.0).abs(), side)
         assert ((p - q).abs()[fine] <= (b + 46) * 2.0 ** -24 * sz[fine]).all()
+
+
+def _median_us(call, n=21):
+    for _ in range(3):
+        call()
+    times = []
+    for _ in range(n):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        call()
+        b.record()
+        torch.cuda.synchronize()
+        times.append(a.elapsed_time(b) * 1e3)
+    return sorted(times)[n // 2]
+
+
+# (blocks, block, other side): whole tiles and remainders, an odd number of 64-blocks; W off 16-byte boundaries in the last two
+@pytest.mark.parametrize("k,b,other,pad", [(32, 128, 2048, 0), (65, 64, 4100, 1), (5, 128, 2690, 1)])
+@pytest.mark.parametrize("side", ["input", "output"])
+@pytest.mark.parametrize("where", ["one a tile", "every row", "rotation", "all"])
+def test_tiny_values_change_no_other_element_and_cost_nothing(k, b, other, pad, side, where):
+    """Values whose low pieces would be subnormal, and subnormal ones: held exactly, at the speed of any others."""
+    r = _rand(k, k, b, b) / b ** 0.5
+    w = _rand(other, *((other, k * b + pad) if side == "input" else (k * b, other + pad)))
+    w = w[:, : w.shape[1] - pad]
+    v, q = w.clone(), r.clone()
+    if pad:
+        v = torch.nn.functional.pad(v, (0, 1))[:, :-1]
+    vo = v if side == "input" else v.T                                   # (other, folded)
+    touched = torch.zeros(other, k, b, dtype=torch.bool, device="cuda")  # element (o, block, column of its rotation)
+    if where == "one a tile":
+        vo[5::128, 7::128] = 1e-35
+        touched[5::128, 0::(128 // b)] = True
+    elif where == "every row":
+        vo[:, 3::b] = 3e-39
+        touched[:] = True
+    elif where == "rotation":
+        q[:, 3, 9::32] = -2e-41
+        touched[:, :, 9::32] = True
+    else:
+        vo *= 1e-33
+        q *= 1e-3
+        touched[:] = True
+    clean, got = (B.conqur_fold_weight(a, c, side, "exact") for a, c in ((w, r), (v, q)))
+    back = lambda t: (t if side == "input" else t.T).reshape(other, k, b)
+    assert torch.equal(back(got)[~touched], back(clean)[~touched])
+    ref = torch.einsum("okb,kbc->okc", vo.double().reshape(other, k, b), q.double())
+    size = torch.einsum("okb,kbc->okc", vo.double().abs().reshape(other, k, b), q.double().abs())
+    # (the bound of the first test; a subnormal result is rounded to a multiple of 2^-149)
+    assert ((back(got) - ref).abs() <= (4 * 10 + 4 + 2) * 2.0 ** -24 * size + 2.0 ** -150).all()
+    t = [_median_us(lambda a=a, c=c: B.conqur_fold_weight(a, c, side, "exact")) for a, c in ((w, r), (v, q))]
+    assert t[1] <= 2.0 * t[0] + 20.0, t                                  # (element by element it took 5 .. 11 ms for 70 us)
+
+
+@pytest.mark.parametrize("side", ["input", "output"])
+def test_large_values_cost_one_more_fold(side):
+    """Infinities, NaN and values whose scaled sums could overflow: the fold is done again on the CUDA cores, and once is enough."""
+    k, b, other = 32, 128, 2048
+    r = _rand(1, k, b, b) / b ** 0.5
+    w = _rand(2, *((other, k * b) if side == "input" else (k * b, other)))
+    clean = _median_us(lambda: B.conqur_fold_weight(w, r, side, "exact"))
+    for bad in (float("nan"), float("inf"), 6e11):
+        v = w.clone()
+        v[7::128, 5::128] = bad
+        assert _median_us(lambda: B.conqur_fold_weight(v, r, side, "exact")) <= 6.0 * clean + 100.0
+    # the limits themselves: |W| < 2^39 and |R| < 2^16 stay on the pieces, beyond them a chain of fp32 multiply-adds gives the same
+    for scale_w, scale_r in ((2.0 ** 36, 2.0 ** 14), (2.0 ** 60, 2.0 ** 40)):
+        got = B.conqur_fold_weight(w * scale_w, r * scale_r, side, "exact").double() / (scale_w * scale_r)
+        ref, size = _reference(w, r, side), _reference(w.abs(), r.abs(), side)
+        assert ((got - ref).abs() <= (b + 2) * 2.0 ** -24 * size).all()
