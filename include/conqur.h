@@ -405,7 +405,12 @@ int conqur_objective_noalloc(const void* X_dev, int32_t in_dtype, int64_t n, int
  *                     in three tensor-core passes (hi hi, hi lo, lo hi) with fp32 accumulation, relative
  *                     error about 2^-16; shapes outside these limits return CONQUR_ERR_UNSUPPORTED.
  *                     Block-diagonal folds (block < folded dimension) use the fp32 product in either mode: on the
- *                     CUDA cores, or for enough blocks of 64 or 128 on the tensor cores over three-term splits.
+ *                     CUDA cores, or for large weights and several blocks of 64 or 128 on the tensor cores over exact
+ *                     three-term splits.  Both are as precise as fp32 or better, but not the same bits: a weight
+ *                     folded in shards may differ in the last bits from the whole where a shard is too small for the
+ *                     tensor cores (fewer than 96 rows or columns beside the folded dimension or 60 x 128 x 128
+ *                     elements; for blocks of 64, INPUT / OUTPUT, 256 / 512 and 240 / 480 x 128 x 128), and one that
+ *                     holds values not finite or from 2^39 on (2^16 in R) is folded on the CUDA cores.
  *   scratch_dev       device memory, 256-byte aligned, >= conqur_fold_scratch_bytes(...) bytes (returns -1 for
  *                     invalid arguments); owned by the caller, free to reuse after the call returns
  * Synchronises the stream and returns the status (CONQUR_ERR_TIMEOUT if a bounded device wait expired).

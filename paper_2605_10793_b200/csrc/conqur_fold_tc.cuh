@@ -14,7 +14,8 @@
 //
 // Both operands are split after a multiplication by 2^32, so that no piece of any fp32 number is subnormal (its last bit is worth
 // 2^-149 at least), and the sums come back by 2^-64: powers of two, which change no bit.  What is left are values that are not
-// finite or so large that scaled sums could overflow; a fold that meets one says so, and the caller runs the CUDA-core kernel instead.
+// finite or so large that scaled sums could overflow; a fold that meets one says so, and the caller runs the CUDA-core kernel instead
+// (32 blocks of 128, W 4096 x 4096 with a NaN: 64 -> 157 us; tiny values anywhere: 64).
 #pragma once
 #include "conqur_split_tc.cuh"
 #include "conqur_tc_batched.cuh"
@@ -305,14 +306,20 @@ inline int tc_make_tmap_f32(CUtensorMap* tm, const void* ptr, uint64_t rows, uin
   return CONQUR_OK;
 }
 
-// Folds that take this kernel: several blocks of 64 or 128, and enough tiles.  Whole call (as timed in a row), fp32 CUDA cores ->
-// this, us:  blocks of 128: 2 tiles 28 -> 33, 8 29 -> 34, 64 37 -> 35, 128 39 -> 35, 160 46 -> 39, 1024 111 -> 64, 3584 319 -> 128;
-// of 64 (half the multiply-adds): 4 tiles 27 -> 34, 80 33 -> 35, 320 43 -> 41, 1792 105 -> 84 (SIDE 0 148 -> 93).
+// Folds that take this kernel: several blocks of 64 or 128, enough of W, and tiles that are not mostly empty (each group of blocks
+// costs its rotation's splitting, however short the other side is).  Whole call (as timed in a row), fp32 CUDA cores -> this, us,
+// blocks x other side:
+//   of 128         8 x 1024 35 -> 34, 64 x 96 35 -> 34, 64 x 512 52 -> 42, 64 x 2048 118 -> 67, 256 x 128 52 -> 42, 1024 x 96 116 -> 93;
+//                  not 32 x 160 31.5 -> 34, 64 x 64 30 -> 33, 128 x 32 30 -> 33, 512 x 64 53 -> 55, 1024 x 1 57 -> 82, 1024 x 64 75 -> 91
+//   of 64, INPUT   64 x 1024 42 -> 42, 512 x 256 61 -> 53, 1024 x 256 97 -> 84;  not 512 x 160 48 -> 52, 1024 x 1 33 -> 54
+//   of 64, OUTPUT  64 x 2048 48 -> 47, 512 x 512 71 -> 69, 256 x 2048 114 -> 91; not 64 x 1024 38 -> 40, 1024 x 256 71 -> 77
+// (the CUDA cores give an element the same bits in a call of any shape; this kernel gives it its own)
 inline bool fold_blocks_takes(int64_t rows, int64_t cols, int block, int side) {
-  const int64_t folded = side == CONQUR_FOLD_INPUT ? cols : rows, other = side == CONQUR_FOLD_INPUT ? rows : cols;
+  const bool in = side == CONQUR_FOLD_INPUT;
+  const int64_t folded = in ? cols : rows, other = in ? rows : cols;
   if ((block != 64 && block != 128) || folded < 2 * (int64_t)block) return false;
-  const int64_t tiles = ((folded + 127) / 128) * ((other + 127) / 128);
-  return tiles >= (block == 128 ? 64 : 256) && tiles < (int64_t)1 << 30;
+  const int64_t least = block == 128 ? 96 : in ? 256 : 512, whole = block == 128 ? 60 : in ? 240 : 480;
+  return other >= least && rows * cols >= whole * (128 * 128) && ((folded + 127) / 128) * ((other + 127) / 128) < (int64_t)1 << 30;
 }
 inline int fold_blocks_launch(const float* W, int64_t ldw, int rows, int cols, const float* R, int block, int side, float* out,
                               int64_t ldo, int* status, int dev, int sms, cudaStream_t s) {
@@ -332,7 +339,7 @@ inline int fold_blocks_launch(const float* W, int64_t ldw, int rows, int cols, c
   g.n_super = ((in ? cols : rows) + 127) / 128;
   g.tiles = ((in ? rows : cols) + 127) / 128;
   CUtensorMap tm = {};
-  if ((ldw & 3) == 0 && (reinterpret_cast<uintptr_t>(W) & 15) == 0) {
+  if ((ldw & 3) == 0 && ldw < (int64_t)1 << 38 && (reinterpret_cast<uintptr_t>(W) & 15) == 0) {    // (a map's strides end at 2^40 bytes)
     if (tc_make_tmap_f32(&tm, W, (uint64_t)rows, (uint64_t)cols, (uint64_t)ldw, in ? 64 : 128, in ? 128 : 64) != CONQUR_OK) return CONQUR_ERR_CUDA;
     g.copied = 1;
   }

@@ -22,8 +22,9 @@ def _reference(w, r, side):
 
 
 # (blocks, block, other side): odd numbers of 64-blocks, fewest tiles and more than one a block of threads, remainders of a tile
-# and of 16-byte pieces; the first two stay on the CUDA cores
-SHAPES = [(2, 64, 32), (3, 128, 127), (65, 64, 993), (2, 128, 4065), (3, 128, 2690), (32, 128, 1003), (127, 64, 640), (4, 128, 9000)]
+# and of 16-byte pieces; the first two and some of the next three stay on the CUDA cores, the last four are the smallest that do not
+SHAPES = [(2, 64, 32), (3, 128, 127), (65, 64, 993), (2, 128, 4065), (3, 128, 2690), (32, 128, 1003), (127, 64, 640), (4, 128, 9000),
+          (3, 128, 2560), (80, 128, 96), (241, 64, 512), (129, 64, 1030)]
 
 
 @pytest.mark.parametrize("k,b,other", SHAPES)
@@ -121,10 +122,10 @@ def test_tiny_values_change_no_other_element_and_cost_nothing(k, b, other, pad, 
     assert t[1] <= 2.0 * t[0] + 20.0, t                                  # (element by element it took 5 .. 11 ms for 70 us)
 
 
+@pytest.mark.parametrize("k,b,other", [(32, 128, 2048), (65, 64, 4100)])
 @pytest.mark.parametrize("side", ["input", "output"])
-def test_large_values_cost_one_more_fold(side):
+def test_large_values_cost_one_more_fold(side, k, b, other):
     """Infinities, NaN and values whose scaled sums could overflow: the fold is done again on the CUDA cores, and once is enough."""
-    k, b, other = 32, 128, 2048
     r = _rand(1, k, b, b) / b ** 0.5
     w = _rand(2, *((other, k * b) if side == "input" else (k * b, other)))
     clean = _median_us(lambda: B.conqur_fold_weight(w, r, side, "exact"))
@@ -137,3 +138,17 @@ def test_large_values_cost_one_more_fold(side):
         got = B.conqur_fold_weight(w * scale_w, r * scale_r, side, "exact").double() / (scale_w * scale_r)
         ref, size = _reference(w, r, side), _reference(w.abs(), r.abs(), side)
         assert ((got - ref).abs() <= (b + 2) * 2.0 ** -24 * size).all()
+
+
+# many blocks and a short other side, and just below each size from which the pieces are taken
+@pytest.mark.parametrize("k,b,other,side", [(1024, 64, 1, "input"), (512, 64, 32, "output"), (1024, 128, 17, "input"), (130, 128, 95, "output"),
+                                            (2, 128, 3839, "input"), (2, 128, 3839, "output"), (257, 64, 255, "input"),
+                                            (64, 64, 959, "input"), (257, 64, 511, "output"), (64, 64, 1919, "output")])
+def test_short_and_small_folds_stay_on_the_cuda_cores(k, b, other, side):
+    """Their tiles would be mostly empty: the same bits as block by block (one block is always folded there)."""
+    r = _rand(k, k, b, b) / b ** 0.5
+    w = _rand(other, *((other, k * b) if side == "input" else (k * b, other)))
+    got = B.conqur_fold_weight(w, r, side, "exact")
+    for i in range(0, k, max(1, k // 16)):
+        cut = (slice(None), slice(i * b, (i + 1) * b)) if side == "input" else (slice(i * b, (i + 1) * b), slice(None))
+        assert torch.equal(got[cut], B.conqur_fold_weight(w[cut], r[i], side, "exact"))
