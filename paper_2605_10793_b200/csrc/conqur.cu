@@ -110,7 +110,7 @@ bool make_layout(int d, const conqur_config* c, Layout* L) {
   mp = std::max<int64_t>(mp, cdiv(n, 8));
   mp = std::max<int64_t>(mp, 3 * (int64_t)cdiv(d, 128) * cdiv(d, 128) + 64);   // three partial arrays of a Newton-Schulz step
   mp = std::max<int64_t>(mp, 1024);
-  const bool pieces = c->mode == CONQUR_EXACT_F32 && sp_layout_wanted(d, (int)P);
+  const bool pieces = c->mode == CONQUR_EXACT_F32 && sp_layout_wanted(d, (int)P, n, c->in_dtype == CONQUR_F32);
   if (pieces) mp = std::max<int64_t>(mp, 16 * (int64_t)cdiv(n, 256) * cdiv(d, 128));   // sixteen per tile of at least 256 x 128
   L->max_partials = mp;
   L->part_d = take(sizeof(double) * mp * P);
@@ -345,7 +345,8 @@ int copy_out(conqur_ctx* c, const float* src, float* dst, float f) {
 // ---------------------------------------------------------------- exact-mode step
 __nv_bfloat16* sp_ptr(const conqur_ctx* c, size_t off) { return c->at<__nv_bfloat16>(off); }
 
-// The pieces of R^T follow R.
+// The pieces of R^T follow R at once, not with the next step that reads them: a step that a caller captured is replayed after updates
+// that the host did not see.
 int sp_refresh_R(conqur_ctx* c) {
   if (c->sp_pairs == 0) return CONQUR_OK;
   const int d = c->cfg.d, t = cdiv(d, 32);

@@ -487,7 +487,7 @@ static __global__ void __launch_bounds__(256) sp_quant_target_kernel(const float
 }
 
 // ------------------------------------------------------------------ host side
-// Contexts that lay the pieces out, and their steps that take them.  Whole step, CUDA cores -> this, us (one B200):
+// Steps that take the pieces.  Whole step, CUDA cores -> this, us (one B200):
 //   fp32 rows, d = 384  n = 1000 49 -> 49, 2048 68 -> 66;  512  256 37 -> 41, 512 47 -> 45, 1000 70 -> 54;  640  256 45 -> 43;
 //              1024  64 49 -> 49, 128 55 -> 51, 1000 147 -> 68;  2048  16 72 -> 78, 64 82 -> 78;  3072  1000 889 -> 165, 2048 1668 -> 288
 //   bf16 rows, d = 320  2048 69 -> 66;  384  16 31 -> 33, 64 37 -> 33, 2048 82 -> 66;  1024  16 56 -> 43, 1000 178 -> 60;
@@ -503,7 +503,8 @@ struct SpLayout {
   int px, pc;                                            // pieces of the rows and of the targets
   size_t Xp, Sp, Rp, rs;
 };
-inline bool sp_layout_wanted(int d, int P) { return P == 1 && d >= SP_MIN_D; }
+// Contexts that lay them out: those whose longest step takes them (a shorter one may not, a longer one always does).
+inline bool sp_layout_wanted(int d, int P, int64_t n_max, bool f32) { return P == 1 && sp_takes(n_max, d, f32); }
 
 template <typename Take>
 inline void sp_make_layout(int d, int64_t n, int in_dtype, SpLayout* L, Take&& take) {

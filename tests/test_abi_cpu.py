@@ -126,3 +126,15 @@ def test_lifting_polynomial_is_the_minimax_quintic(B):
     assert abs(p[-1] - top) < 1e-6 * top
     interior_min = p[(x > 0.4) & (x < 0.95)].min()
     assert abs((1 - interior_min / top) - err[0]) < 1e-6
+
+
+def test_exact_contexts_hold_pieces_only_where_a_step_takes_them(B):
+    """The rotation's three bf16 pieces (6 d^2 bytes) and the rows' and targets' belong to contexts whose longest step runs over them."""
+    def ws(d, n, f32):
+        return B.conqur_workspace_bytes(d, B.make_config(in_dtype=B.CONQUR_F32 if f32 else B.CONQUR_BF16, mode=B.CONQUR_EXACT_F32, n_max=n))
+    # (longest step that stays on the CUDA cores, one row more); fp32 rows take the pieces from d = 512 on, bf16 rows from 384
+    for d, n, f32 in ((512, 511, True), (1000, 262, True), (2048, 63, True), (384, 63, False), (2048, 63, False)):
+        assert ws(d, n + 1, f32) - ws(d, n, f32) >= 6 * d * d
+    for d, f32 in ((383, False), (384, True), (448, True), (511, True)):
+        # a row costs its fp32 target, its norm and its range, and its share of the partials
+        assert ws(d, 32768, f32) - ws(d, 16384, f32) <= 16384 * (4 * d + 128)
