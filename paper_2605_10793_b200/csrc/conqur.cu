@@ -121,17 +121,18 @@ bool make_layout(int d, const conqur_config* c, Layout* L) {
   L->acc_splits = 1;
   L->C = L->splitk = 0;
   L->sp = SpLayout{};
-  // the four Newton-Schulz matrices form ONE region: a token-split per-head step borrows all of it as scratch
+  // the four Newton-Schulz matrices form ONE region: a token-split per-head step borrows all of it as scratch, an exact step its
+  // rows' pieces
   const size_t ns_one = align_up(sizeof(float) * dd * P);
   L->Xa = take(4 * ns_one);
   L->Xb = L->Xa + ns_one;
   L->E = L->Xb + ns_one;
   L->B = L->E + ns_one;
   if (c->mode == CONQUR_EXACT_F32) {
-    L->C = take(sizeof(float) * (size_t)n * d * P);
+    if (pieces) sp_make_layout(d, n, c->in_dtype, c->quant_bits || c->diagnostics, L->Xa, 4 * ns_one, &L->C, &L->sp, take);
+    else L->C = take(sizeof(float) * (size_t)n * d * P);
     L->acc_splits = pick_acc_splits(d, (int)P, n);
     if (L->acc_splits > 1) L->splitk = take(sizeof(float) * dd * P * L->acc_splits);
-    if (pieces) sp_make_layout(d, n, c->in_dtype, &L->sp, take);
   } else {
     if ((c->quant_bits || c->diagnostics) && P == 1) L->C = take(sizeof(float) * (size_t)n * d);
     tc_make_layout(d, (int)P, n, c->quant_bits, c->in_dtype, &L->tc, take);

@@ -506,13 +506,23 @@ struct SpLayout {
 // Contexts that lay them out: those whose longest step takes them (a shorter one may not, a longer one always does).
 inline bool sp_layout_wanted(int d, int P, int64_t n_max, bool f32) { return P == 1 && sp_takes(n_max, d, f32); }
 
+// The rows' pieces borrow `scratch` (the update's matrices: no update runs during a step) where they fit it.  The fp32 target matrix C
+// of a step on the CUDA cores shares its place with what a step over pieces writes instead, except where such a step goes through it
+// too (fake-quantisation, diagnostics).  A row element costs 4 bytes as without pieces for fp32 rows up to 2.7 d of them, else 8; 6 or 8
+// for bf16 rows.
 template <typename Take>
-inline void sp_make_layout(int d, int64_t n, int in_dtype, SpLayout* L, Take&& take) {
+inline void sp_make_layout(int d, int64_t n, int in_dtype, bool through_c, size_t scratch, size_t scratch_bytes, size_t* C, SpLayout* L,
+                           Take&& take) {
   L->ldp = ((int64_t)d + 63) / 64 * 64;
   L->px = in_dtype == CONQUR_F32 ? 3 : 1;
   L->pc = in_dtype == CONQUR_F32 ? 1 : 3;
-  L->Xp = take((size_t)(2 * L->px * n * L->ldp));
-  L->Sp = take((size_t)(2 * L->pc * n * L->ldp));
+  const size_t rows = (size_t)(2 * L->px * n * L->ldp), targets = ((size_t)(2 * L->pc * n * L->ldp) + 255) / 256 * 256;
+  const size_t c_bytes = sizeof(float) * (size_t)n * d;
+  const bool borrow = rows <= scratch_bytes;
+  const size_t mine = targets + (borrow ? 0 : rows);
+  *C = take(through_c || c_bytes > mine ? c_bytes : mine);
+  L->Sp = through_c ? take(mine) : *C;
+  L->Xp = borrow ? scratch : L->Sp + targets;
   L->Rp = take((size_t)(2 * 3 * d * L->ldp));
   L->rs = take(sizeof(float) * (size_t)n);
 }

@@ -138,3 +138,18 @@ def test_exact_contexts_hold_pieces_only_where_a_step_takes_them(B):
     for d, f32 in ((383, False), (384, True), (448, True), (511, True)):
         # a row costs its fp32 target, its norm and its range, and its share of the partials
         assert ws(d, 32768, f32) - ws(d, 16384, f32) <= 16384 * (4 * d + 128)
+
+
+def test_exact_workspace_grows_with_rows_as_little_as_the_pieces_allow(B):
+    """The rows' pieces share the update's matrices, the targets' pieces the CUDA cores' target matrix."""
+    def row(d, n1, n2, f32, **kw):                       # bytes a row costs, without those of its norm, range, scale and partials
+        ws = [B.conqur_workspace_bytes(d, B.make_config(in_dtype=B.CONQUR_F32 if f32 else B.CONQUR_BF16, mode=B.CONQUR_EXACT_F32,
+                                                        n_max=n, **kw)) for n in (n1, n2)]
+        return (ws[1] - ws[0]) / (n2 - n1) - 128
+    for d in (1024, 4096, 8192):
+        assert row(d, d // 2, 2 * d, True) <= 4 * d      # what a row took before there were pieces
+        assert row(d, 4 * d, 8 * d, True) <= 8 * d
+        assert row(d, 2 * d, 7 * d, False) <= 6 * d
+        assert row(d, 10 * d, 20 * d, False) <= 8 * d
+        assert row(d, d // 2, 2 * d, True, quant_bits=4) <= 6 * d
+        assert row(d, 4 * d, 8 * d, True, quant_bits=4) <= 12 * d
