@@ -269,7 +269,8 @@ sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       for (int i = 0; i < HALF; ++i) acc[i] = 0.f;
       for (int kb = 0; kb < num_kb; ++kb, ++n_acc) {
         const uint32_t buf = n_acc & 1u;
-        if (!tc_wait(&aux->tfull[buf], (n_acc >> 1) & 1u, abort_flag)) { ok = false; timeout_site = 4; break; }
+        // (a lane that gives up takes part in the warp's loads all the same; the vote below ends the loop for all lanes at once)
+        if (!tc_wait(&aux->tfull[buf], (n_acc >> 1) & 1u, abort_flag)) { ok = false; timeout_site = 4; }
         ptx::tc_fence_after();
 #pragma unroll
         for (int c = 0; c < BLOCKS; ++c) {
@@ -279,8 +280,9 @@ sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           for (int i = 0; i < 32; ++i) acc[c * 32 + i] += __uint_as_float(r[i]);
         }
         ptx::tc_fence_before();
-        __syncwarp();
+        ok = __all_sync(0xffffffffu, ok);
         if (lane == 0) ptx::mbar_arrive_cluster(tempty0 + buf * (uint32_t)sizeof(uint64_t));
+        if (!ok) break;
       }
       if (!ok) break;
       const int wrow0 = tm * 256 + (int)rank * TC_BM + q * 32, row = wrow0 + lane;
