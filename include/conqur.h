@@ -213,7 +213,8 @@ int conqur_step_batched_range(conqur_ctx* ctx, const void* X_dev, int64_t n, int
  */
 int conqur_update(conqur_ctx* ctx);
 
-/* Copy out the current rotation(s): device fp32 batch x d x d.  Synchronises. */
+/* Copy out the current rotation(s): device fp32 batch x d x d (of another GPU too; conqur_get_M and conqur_set_M
+ * need memory that this GPU's kernels can reach).  Synchronises. */
 int conqur_get_R(conqur_ctx* ctx, float* R_out_dev);
 
 /*

@@ -190,7 +190,8 @@ struct conqur_ctx {
   int last_np;               // problems the last step call covered
   bool last_pieces = false;  // the last step left its targets as bf16 pieces (exact mode)
   bool one_cluster = false;  // exact mode, one narrow problem: its update is one kernel (conqur_ns_cluster.cuh)
-  int device = 0, sp_pairs = 0;   // exact contexts with pieces: CTA pairs that can be co-resident (0: CUDA cores only)
+  int device = 0;
+  int sp_pairs = 0;          // exact contexts with pieces: CTA pairs that can be co-resident (0: CUDA cores only)
   int64_t pending_rows = 0;  // deferring context: rows staged but not yet run through the two products
   int pending_batches = 0;
   int8_t* sign_capture = nullptr;   // conqur_debug_capture_signs: where the fused per-head kernel writes its decisions
@@ -877,7 +878,7 @@ extern "C" int conqur_init(conqur_ctx** out, int32_t d, const conqur_config* cfg
     rc = tc_refresh_R(c->tc, c->stream, 0);
     if (rc) return fail(rc);
   }
-  if (g.mode == CONQUR_EXACT_F32 && cudaGetDevice(&c->device) != cudaSuccess) return fail(CONQUR_ERR_CUDA);
+  if (cudaGetDevice(&c->device) != cudaSuccess) return fail(CONQUR_ERR_CUDA);
   c->one_cluster = g.mode == CONQUR_EXACT_F32 && g.P == 1 && d <= NC_MAX_D && !(g.debug_flags & CONQUR_DEBUG_NO_GRAPH) && nc_available(c->device);
   if (L.sp.ldp) {
     TcDevFacts f;
@@ -1034,7 +1035,14 @@ extern "C" int conqur_update(conqur_ctx* c) {
 extern "C" int conqur_get_R(conqur_ctx* c, float* R_out_dev) {
   if (!c || !R_out_dev) return CONQUR_ERR_INVALID_ARG;
   { const int frc = flush_pending(c); if (frc) return frc; }
-  return copy_out(c, c->at<float>(c->L.R), R_out_dev, 1.0f);
+  // A kernel writes this GPU's memory.  Whatever else the caller gives (another GPU's memory, with or without peer access, or the
+  // host's) is the copy's to reach or to refuse.
+  cudaPointerAttributes to;
+  CQ_CUDA(cudaPointerGetAttributes(&to, R_out_dev));
+  if (to.type == cudaMemoryTypeDevice && to.device == c->device) return copy_out(c, c->at<float>(c->L.R), R_out_dev, 1.0f);
+  CQ_CUDA(cudaMemcpyAsync(R_out_dev, c->at<float>(c->L.R), sizeof(float) * (size_t)c->cfg.d * c->cfg.d * c->cfg.P,
+                          cudaMemcpyDeviceToDevice, c->stream));
+  return sync_status(c);
 }
 
 extern "C" int conqur_get_objective(conqur_ctx* c, double* J_sum, int64_t* n_tokens) {

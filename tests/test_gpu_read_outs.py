@@ -43,3 +43,17 @@ def test_status_of_any_problem_is_reported():
         assert e.value.status == -7
     assert c.get_stats().status == -7
     c.get_R()
+
+
+@pytest.mark.parametrize("mode,d,batch", [("exact", 33, 1), ("tc", 256, 1), ("tc", 128, 3)])
+def test_rotation_into_memory_that_is_not_this_gpus(mode, d, batch):
+    """conqur_get_R into page-locked host memory and at an odd device address: what a device-to-device copy reaches."""
+    c = B.Context(d, 64, in_dtype="bf16", mode=mode, batch=batch)
+    r = torch.linalg.qr(torch.randn(batch, d, d, device="cuda", dtype=torch.float64))[0].float().contiguous()
+    c.set_R(r if batch > 1 else r[0])
+    host = torch.zeros(batch, d, d, dtype=torch.float32).pin_memory()
+    assert B.conqur_get_R(c.h, host.data_ptr()) == 0
+    assert torch.equal(host, r.cpu())
+    odd = torch.zeros(batch * d * d + 1, device="cuda")
+    assert B.conqur_get_R(c.h, odd.data_ptr() + 4) == 0
+    assert torch.equal(odd[1:].view(batch, d, d), r)
