@@ -207,6 +207,26 @@ def test_single_cta_kernels_on_a_device_that_would_use_pairs():
         assert rep["orth"] <= TOL["tc"]["orth"] and rep["gap"] <= TOL["tc"]["gap"], rep
 
 
+# d = 512: both products on 128 x 128 tiles; the accumulate product beyond (K = 1025); rotate at its last 64 tiles and beyond (68)
+@pytest.mark.parametrize("n", [1024, 1025, 2048, 2049])
+@pytest.mark.parametrize("single", [False, True])
+@pytest.mark.parametrize("bits", [0, 4])
+def test_tile_choice_of_small_steps(n, single, bits):
+    """Either side of the rule that gives small steps 128 x 128 tiles, with CTA pairs and with the 128 x 256 single-CTA kernels."""
+    from paper_2605_10793_b200 import binding as B
+    d = 512
+    w = I.scaled(I.WORKLOADS["c4a" if bits else "c2"], d=d, n=n, n_outlier=2)
+    r0 = I.initial_rotation(w)
+    x = I.batch(w, 0)
+    ctx = B.Context(d=d, n_max=n, in_dtype="bf16", mode="tc", quant_bits=bits, debug_flags=B.CONQUR_DEBUG_SINGLE_CTA if single else 0)
+    ctx.set_R(_dev(r0, "f32"))
+    ctx.step(_dev(x))
+    j, nn = ctx.get_objective()
+    m = ctx.get_M().cpu().numpy().astype(np.float64)
+    s = ctx.debug_get_signs(n).cpu().numpy()
+    assert_step(step_parity(x.astype(np.float64), r0.astype(np.float64), s, m, j, nn, "tc", bits), "tc", 2e-2)
+
+
 SHARD_WORKER = textwrap.dedent("""
     import sys
     sys.path.insert(0, %r)

@@ -127,3 +127,29 @@ def test_rows_accumulate_and_rotation_follows():
     ref = float((xt @ r1.double()).abs().sum()) / math.sqrt(d)
     j, n = c.get_objective()
     assert n == 700 and abs(j - ref) <= 2e-6 * ref
+
+
+# the smallest steps that take the pieces, by row type and width: one row of tiles of which the second CTA's half is empty or nearly so
+@pytest.mark.parametrize("d,n,dtype", [(384, 64, torch.bfloat16), (385, 65, torch.bfloat16), (511, 100, torch.bfloat16),
+                                       (2050, 64, torch.bfloat16), (512, 129, torch.bfloat16), (1024, 128, torch.float32),
+                                       (1030, 130, torch.float32), (2050, 64, torch.float32)])
+def test_smallest_steps_over_pieces(d, n, dtype):
+    test_signs_statistics_and_objective(d, n, dtype)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_a_feature_of_tiny_values(dtype):
+    """Low pieces of values below 2^-110 or so are subnormal: a feature that small everywhere loses up to 2^-126 a row, absolutely."""
+    d, n = 520, 1000
+    x = _rand(1, n, d)
+    x[:, 7] *= 1e-36
+    x = x.to(dtype)
+    r = torch.linalg.qr(_rand(7, d, d).double())[0].float().contiguous()
+    c = B.Context(d, n, in_dtype="f32" if dtype == torch.float32 else "bf16", mode="exact")
+    c.set_R(r)
+    c.step(x)
+    m, s = c.get_M().double(), c.debug_get_signs(n).double()
+    xt = x.double() / x.double().norm(dim=1, keepdim=True)
+    err = (m - xt.T @ s / math.sqrt(d)).abs()
+    bound = (_unit(n) + (d / 32 + 9) * 2.0 ** -24) * (xt.abs().T @ s.abs()) / math.sqrt(d)
+    assert (err <= bound + n * 2.0 ** -126 / math.sqrt(d)).all() and float(m[7].abs().max()) > 0.0
