@@ -109,9 +109,10 @@ typedef struct {
 
 /* debug_flags bits.  CANARIES: every region of the workspace is followed by a 256-byte guard band with a fixed
  * pattern, checked by conqur_debug_check_canaries (a stand-in for a memory checker).  SINGLE_CTA: the tensor-core
- * products never use CTA pairs (exercises the single-CTA kernels on a device that would use pairs).  NO_GRAPH: the
- * update's launch sequence is enqueued directly every time instead of being replayed from a captured graph (so that a
- * profiler's launch list shows its kernels). */
+ * products never use CTA pairs (exercises the single-CTA kernels on a device that would use pairs); exact steps, whose
+ * tensor-core kernels are made of pairs, then run on the CUDA cores.  NO_GRAPH: the update's launch sequence is enqueued
+ * directly every time instead of being replayed from a captured graph (so that a profiler's launch list shows its
+ * kernels); the exact update of one narrow problem (d <= 160), otherwise one kernel, takes the launches too. */
 enum { CONQUR_DEBUG_CANARIES = 1, CONQUR_DEBUG_SINGLE_CTA = 2, CONQUR_DEBUG_NO_GRAPH = 4 };
 
 typedef struct {
@@ -310,7 +311,8 @@ int conqur_get_stats(conqur_ctx* ctx, conqur_stats* out);
  * CUDA events on the context's stream and conqur_update synchronises at its end (so enable it only
  * in a measurement pass); flops are those of the tiles a launch computes (2 * 128|256 * tile width * K per tile
  * and bf16 pass: a symmetric product counts its upper-triangle tiles only, a split product every pass it
- * takes), for launches that did not early-exit.
+ * takes), for launches that did not early-exit.  Updates in one kernel count as one launch and are not timed: of
+ * class 5 in exact mode with one problem of d <= 160, of class 3 in tensor-core mode with several problems.
  */
 #define CONQUR_KERNEL_CLASSES 8
 typedef struct {
@@ -367,7 +369,8 @@ int conqur_debug_wait_timeout(void* scratch_dev, int64_t limit_cycles, void* cud
  * running under a runtime that owns all device memory, or a plugin in a process whose device
  * memory is pre-assigned -- and therefore cannot provide the workspace conqur_init needs).
  *
- * Computes, in the exact fp32 arithmetic of conqur_step's exact mode and with R fixed,
+ * Computes, in fp32 on the CUDA cores (conqur_step's exact mode as it is for short or narrow steps; its wide ones take
+ * the tensor cores over exact splits and differ by rounding) and with R fixed,
  *   J = sum_i ||x_tilde_i R||_1 / sqrt(d)   and   N = rows with a finite, non-zero norm
  * (the quantities conqur_get_objective reports after one conqur_step on a fresh context).
  *   X_dev      device, n rows of d elements of in_dtype (CONQUR_F32 | CONQUR_BF16), row stride ld elements

@@ -3,11 +3,15 @@
 // At these widths a launch of the iteration costs more than its work: 128^3 multiply-adds are 0.1 us of the chip, a launch with
 // the load latency of its operands about 6 us, and a step takes three of them and the control decision.  Sixteen CTAs of one
 // cluster share the 32 x 32 tiles of every product instead, a cluster barrier stands between the products, and every CTA takes the
-// decision itself from the same sums.  Sums are added in the order of the launches' kernels: the same bits.
-// What a step takes now (d = 128, SM cycles, clock stamps): products 3 x 4.1 k (a warp's multiply-adds: two cycles each, 16 per k),
-// operands from the L2 6 k, barriers 6 k (the stores in front of them have to reach the L2), stores 2.7 k, norms and decision 1.8 k.
-// Whole update, graph of launches -> this, us (one B200): d = 16 124 -> 40, 64 151 -> 75, 128 196 -> 104, 160 221 -> 160;
-// 192 237 -> 291 (three tiles a CTA).
+// decision itself from the same sums.  An element of a product is the same chain of multiply-adds as in the launches' kernels, and
+// the coefficients of a step depend on its place in the plan alone: the same bits wherever the start scale rounds to the same number
+// and the decisions agree.  (The squares behind these are added in another grouping, sixteen CTAs' instead of a block's per 1024
+// elements or per tile: double sums rounded to fp32, so a last bit may differ.)
+// What a step takes (d = 128, SM cycles, clock stamps): products 3 x 4.1 k (a warp's multiply-adds: two cycles each, 16 per k),
+// operands from the L2 6 k, barriers 6 k (the stores in front of them have to reach the L2), stores 2.7 k, norms and decision 1.8 k;
+// an update of eight steps 116 us.  Whole update of the statistics of 16 d rows once its step count is learnt, from an idle stream,
+// graph of launches -> this, us (one B200): d = 16, 8 steps 139 -> 57;  64, 9 steps 194 -> 106;  128, 9 steps 223 -> 136;  160, 12
+// steps 258 -> 200;  192 (three tiles a CTA) would take 291 in a row of updates where the launches take 237.
 #pragma once
 #include <mutex>
 

@@ -73,3 +73,22 @@ def test_rejected_updates_keep_the_rotation():
     c.set_M(m, 1.0, 128)
     c.update()
     assert c.get_stats().status == 0 and not torch.equal(c.get_R(), r0)
+
+
+@pytest.mark.parametrize("d", WIDTHS[:-1])
+@pytest.mark.parametrize("kind", ["flat", "steep"])
+def test_same_steps_from_the_same_scale_give_the_same_bits(d, kind):
+    """The products' chains are those of the launches; only the sums of squares are grouped otherwise."""
+    m = _spectrum(d, kind)
+    got = []
+    for flags in (0, B.CONQUR_DEBUG_NO_GRAPH):
+        c = B.Context(d, 4096, in_dtype="f32", mode="exact", debug_flags=flags)
+        for _ in range(2):
+            c.set_M(m, 1.0, 4096)
+            c.update()
+            st = c.get_stats()
+            got.append((st.scale, (st.status, st.ns_steps_used, st.ns_lift_plan), c.get_R()))
+    for (s1, n1, r1), (s2, n2, r2) in zip(got[:2], got[2:]):
+        # sqrt of a sum of d^2 squares in double, whatever its grouping, then one rounding to fp32
+        assert abs(s1 - s2) <= 2.0 ** -23 * s2 and n1 == n2
+        assert s1 != s2 or torch.equal(r1, r2)
