@@ -875,7 +875,7 @@ extern "C" int conqur_init(conqur_ctx** out, int32_t d, const conqur_config* cfg
                      g.diagnostics, g.diagnostics ? c->at<double>(L.part_diag) : nullptr, &c->prof,
                      (g.debug_flags & CONQUR_DEBUG_SINGLE_CTA) != 0, cfg->ns_gram_single_pass_tau);
     if (rc) return fail(rc);
-    rc = tc_refresh_R(c->tc, c->stream, 0);
+    rc = tc_refresh_R(c->tc, c->stream);
     if (rc) return fail(rc);
   }
   if (cudaGetDevice(&c->device) != cudaSuccess) return fail(CONQUR_ERR_CUDA);
@@ -965,7 +965,7 @@ extern "C" int conqur_set_R(conqur_ctx* c, const float* R_dev) {
   }
   if (g.mode == CONQUR_TC_BF16 && aligned) return tc_take_R(c->tc, c->stream, R_dev);
   CQ_CUDA(cudaMemcpyAsync(c->at<float>(c->L.R), R_dev, sizeof(float) * dd * g.P, cudaMemcpyDeviceToDevice, c->stream));
-  if (g.mode == CONQUR_TC_BF16) return tc_refresh_R(c->tc, c->stream, 0);
+  if (g.mode == CONQUR_TC_BF16) return tc_refresh_R(c->tc, c->stream);
   return sp_refresh_R(c);
 }
 

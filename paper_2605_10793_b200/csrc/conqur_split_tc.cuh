@@ -95,7 +95,10 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
 }
 }  // namespace ptx
 
-// Three bf16 pieces of v (+ rest, a remainder below v's last bit).
+// Three bf16 pieces of v (+ rest, a remainder below v's last bit).  A piece below 2^-126 is subnormal, so of values below about 2^-110
+// the low pieces are cut off at 2^-133 and their products with the other side at 2^-126 or so.  A step needs no other path for them:
+// normalised rows and rotations have norm 1, so that much lies far below the rounding of any sum they enter, except that a feature
+// which is that small in every row gets its row of M to 2^-126 absolutely, not relatively (fp32 itself ends at 2^-149).
 __device__ __forceinline__ void sp_split(float v, float rest, uint32_t& p0, uint32_t& p1, uint32_t& p2) {
   p0 = bf16_bits(v);
   const float r1 = v - __uint_as_float(p0 << 16);
@@ -139,7 +142,9 @@ __device__ __forceinline__ void sp_put_block(uint8_t* stg, int lane, const float
 }
 
 // D[m][n] = sum_k A(m, k) B(n, k) on 256 x BN tiles of CTA pairs, operands as stacks of bf16 pieces (3-D maps: column, row,
-// piece).  Warp 0 loads, warp 1 issues (CTA 0 for both), warps 2-9 add up the accumulators and write the tile.
+// piece).  Warp 0 loads, warp 1 issues (CTA 0 for both), warps 4-11 add up the accumulators and write the tile (2 and 3 idle: the
+// registers go by warpgroups).  A warp's 128 running sums, a block on its way from TMEM and the write-out's addresses do not all fit 208
+// registers: the 256-wide variants spill up to 52 bytes a thread outside the accumulation loop, the others up to 12 or nothing.
 //   ROTATE    A = X (K-major), B = R^T (K-major): targets sgn(y) * rs as pc bf16 pieces, objective partials sum |y| rs
 //   ROTATE_Q  the same products, stored as fp32 Y with the row's range
 //   ACCUM     A = X, B = targets (both MN-major, contraction over rows): added to M, once per element and launch

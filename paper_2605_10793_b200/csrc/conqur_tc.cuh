@@ -1384,7 +1384,7 @@ inline int tc_ew_blocks(int64_t count4) {
   return (int)(b < 148 * 8 ? b : 148 * 8);
 }
 
-inline int tc_refresh_R(TcHost& h, cudaStream_t s, int) {
+inline int tc_refresh_R(TcHost& h, cudaStream_t s) {
   const int64_t dd = (int64_t)h.d * h.d * h.P;
   split_bf16_kernel<<<tc_ew_blocks(dd / 4), 256, 0, s>>>(h.R, reinterpret_cast<__nv_bfloat16*>(h.ws + h.L.Rb), dd, 0);
   if (h.prof) h.prof->count(K_OTHER);
