@@ -129,7 +129,7 @@ bool make_layout(int d, const conqur_config* c, Layout* L) {
   L->E = L->Xb + ns_one;
   L->B = L->E + ns_one;
   if (c->mode == CONQUR_EXACT_F32) {
-    if (pieces) sp_make_layout(d, n, c->in_dtype, c->quant_bits || c->diagnostics, L->Xa, 4 * ns_one, &L->C, &L->sp, take);
+    if (pieces) sp_make_layout(d, n, c->quant_bits || c->diagnostics, L->Xa, 4 * ns_one, &L->C, &L->sp, take);
     else L->C = take(sizeof(float) * (size_t)n * d * P);
     L->acc_splits = pick_acc_splits(d, (int)P, n);
     if (L->acc_splits > 1) L->splitk = take(sizeof(float) * dd * P * L->acc_splits);
@@ -353,7 +353,11 @@ int sp_refresh_R(conqur_ctx* c) {
   if (c->sp_pairs == 0) return CONQUR_OK;
   const int d = c->cfg.d, t = cdiv(d, 32);
   const SpLayout& L = c->L.sp;
-  sp_split_rt_kernel<<<dim3(t, t), 256, 0, c->stream>>>(c->at<float>(c->L.R), d, sp_ptr(c, L.Rp), L.ldp, d * L.ldp);
+  unsigned* colmax = c->at<unsigned>(L.colmax);
+  CQ_CUDA(cudaMemsetAsync(colmax, 0, sizeof(unsigned) * d, c->stream));
+  sp_colmax_kernel<<<dim3(t, 16), 256, 0, c->stream>>>(c->at<float>(c->L.R), d, colmax);
+  CQ_LAUNCHED(c, K_OTHER);
+  sp_split_rt_kernel<<<dim3(t, t), 256, 0, c->stream>>>(c->at<float>(c->L.R), d, colmax, sp_ptr(c, L.Rp), L.ldp, d * L.ldp);
   CQ_LAUNCHED(c, K_OTHER);
   return CONQUR_OK;
 }
@@ -368,36 +372,36 @@ int step_pieces(conqur_ctx* c, const TIn* X, int64_t n, int64_t ld) {
   float* rs = c->at<float>(L.rs);
   double* part = c->at<double>(c->L.part_d);
   const int64_t xpiece = n * L.ldp;                       // the pieces of this step's rows lie one behind another
-  sp_stage_kernel<TIn><<<(unsigned)n, 128, 0, c->stream>>>(X, n, d, ld, rnorm, rs, sp_ptr(c, L.Xp), L.ldp, xpiece, c->state());
+  sp_stage_kernel<TIn, true><<<(unsigned)n, 128, 0, c->stream>>>(X, n, d, ld, rnorm, rs, sp_ptr(c, L.Xp), L.ldp, xpiece, c->state());
   CQ_LAUNCHED(c, K_ROWNORM);
-  const int bn = sp_pick_bn(n, d, c->sp_pairs, false), bm = sp_pick_bn(d, d, c->sp_pairs, true);
+  const int bm = sp_pick_bn(d, d, c->sp_pairs);
   CUtensorMap xk, rk, xm, sm;
-  int rc = sp_make_tmap(&xk, sp_ptr(c, L.Xp), n, d, L.ldp, L.px, xpiece, TC_BM);
-  rc |= sp_make_tmap(&rk, sp_ptr(c, L.Rp), d, d, L.ldp, 3, d * L.ldp, bn / 2);
-  rc |= sp_make_tmap(&xm, sp_ptr(c, L.Xp), n, d, L.ldp, L.px, xpiece, TC_BK);
-  rc |= sp_make_tmap(&sm, sp_ptr(c, L.Sp), n, d, L.ldp, L.pc, xpiece, TC_BK);
+  int rc = sp_make_tmap(&xk, sp_ptr(c, L.Xp), n, d, L.ldp, 3, xpiece, TC_BM);
+  rc |= sp_make_tmap(&rk, sp_ptr(c, L.Rp), d, d, L.ldp, 3, d * L.ldp, SP_ROT_BN / 2);
+  rc |= sp_make_tmap(&xm, sp_ptr(c, L.Xp), n, d, L.ldp, 3, xpiece, TC_BK);
+  rc |= sp_make_tmap(&sm, sp_ptr(c, L.Sp), n, d, L.ldp, 1, xpiece, TC_BK);
   if (rc) return CONQUR_ERR_CUDA;
   SpArgs a{};
-  a.M = (int)n; a.N = d; a.K = d; a.pa = L.px; a.pb = 3;
+  a.M = (int)n; a.N = d; a.K = d;
   a.rs = rs; a.part_d = part; a.st = c->state();
-  a.outS = sp_ptr(c, L.Sp); a.lds = L.ldp; a.s_piece = xpiece; a.pc = L.pc;
+  a.outS = sp_ptr(c, L.Sp); a.lds = L.ldp;
   double* pdiag = g.diagnostics ? c->at<double>(c->L.part_diag) : nullptr;
   int per_problem;
   if (g.quant_bits == 0 && !g.diagnostics) {
-    rc = sp_launch<SP_EPI_ROTATE>(bn, c->device, c->sp_pairs, c->stream, xk, rk, a);
+    rc = sp_launch_bn<SP_ROT_BN, SP_EPI_ROTATE>(c->device, c->sp_pairs, c->stream, xk, rk, a);
     if (rc) return rc;
     c->prof.count(K_ROTATE);
-    per_problem = (int)(16 * sp_tiles(n, d, bn));
+    per_problem = (int)(16 * sp_tiles(n, d, SP_ROT_BN));
   } else {
     a.rowmax = c->at<unsigned>(c->L.rowmax); a.rowmin = a.rowmax + g.n_max;
     a.outF = c->at<float>(c->L.C); a.ldo = d;
     CQ_CUDA(cudaMemsetAsync(a.rowmax, 0, sizeof(unsigned) * n, c->stream));
     CQ_CUDA(cudaMemsetAsync(a.rowmin, 0xff, sizeof(unsigned) * n, c->stream));
-    rc = sp_launch<SP_EPI_ROTATE_Q>(bn, c->device, c->sp_pairs, c->stream, xk, rk, a);
+    rc = sp_launch_bn<SP_ROT_BN, SP_EPI_ROTATE_Q>(c->device, c->sp_pairs, c->stream, xk, rk, a);
     if (rc) return rc;
     c->prof.count(K_ROTATE);
     sp_quant_target_kernel<<<cdiv(n, 8), 256, 0, c->stream>>>(a.outF, n, d, rnorm, rs, a.rowmax, a.rowmin, g.qs, part, a.outS,
-                                                              L.ldp, xpiece, L.pc, pdiag);
+                                                              L.ldp, pdiag);
     CQ_LAUNCHED(c, K_OTHER);
     per_problem = cdiv(n, 8);
   }
@@ -405,9 +409,12 @@ int step_pieces(conqur_ctx* c, const TIn* X, int64_t n, int64_t ld) {
                                                  pdiag ? cdiv(n, 8) : 0);
   CQ_LAUNCHED(c, K_OTHER);
   SpArgs m{};
-  m.M = d; m.N = d; m.K = (int)n; m.pa = L.px; m.pb = L.pc; m.st = c->state();
+  m.M = d; m.N = d; m.K = (int)n; m.st = c->state();
   m.outF = c->at<float>(c->L.M); m.ldo = d;
-  rc = sp_launch<SP_EPI_ACCUM>(bm, c->device, c->sp_pairs, c->stream, xm, sm, m);
+  sp_stage_kernel<TIn, false><<<(unsigned)n, 128, 0, c->stream>>>(X, n, d, ld, rnorm, rs, sp_ptr(c, L.Xp), L.ldp, xpiece, c->state());
+  CQ_LAUNCHED(c, K_ROWNORM);
+  rc = bm == 256 ? sp_launch_bn<256, SP_EPI_ACCUM>(c->device, c->sp_pairs, c->stream, xm, sm, m)
+                 : sp_launch_bn<128, SP_EPI_ACCUM>(c->device, c->sp_pairs, c->stream, xm, sm, m);
   if (rc) return rc;
   c->prof.count(K_ACCUM);
   return CONQUR_OK;

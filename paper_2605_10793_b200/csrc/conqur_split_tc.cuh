@@ -1,19 +1,25 @@
 // The fp32 step's two products on the tensor cores, at no less than fp32's precision.
 //
-// An fp32 number is the sum of three bf16 numbers (8 bits each, exactly: x = p0 + p1 + p2), so an fp32 product is six bf16
-// products, p0 q0 + (p0 q1 + p1 q0) + (p0 q2 + p1 q1 + p2 q0); what is left out lies 2^-26 below a term.  bf16 rows and sign
-// targets are one piece, which leaves three products.  The tensor cores cut what they add (2^-23 of the sum, once per
-// instruction of 16 terms), so a long sum kept in TMEM loses more than an fp32 chain does.  Here an accumulator holds 64 terms
-// only, small pieces first; the epilogue warps then add it to running sums in their registers, in fp32, round to nearest.
-// Error of a rotated row, in 2^-24 of its norm, fp32 chain of fused multiply-adds / this (rows of the calibration recipe):
-// K = 64 2.9 / 2.4, 128 3.7 / 1.4, 512 6.8 / 2.1, 1024 9.8 / 2.5, 3072 19.6 / 3.1; all terms in one accumulator: 77 at 3072.
+// An fp32 number is the sum of three bf16 numbers of 8 bits each, and products of them are exact; but the tensor cores cut what they
+// add toward zero (2^-23 of the sum, once per instruction of 16 terms).  A long sum kept in TMEM loses more than an fp32 chain
+// does, and what is lost has the sum's sign, so that it does not average out over a matrix.
 //
-// What bounds it: the tensor cores and, with them busy, the board's power (128 cycles per 256 x 256 x 16 instruction of a CTA pair, 24
-// of them per k block of 64 with six products), where the CUDA cores' product is bound by its shared-memory reads.  1000 x 3072
-// fp32 rows: rotate 504 -> 95 us (116 Gflop of bf16 products: 1.2 PFLOP/s on 64 of 74 pairs), accumulate 409 -> 57, staging
-// 8 -> 8; the whole step 889 -> 165.  Operand pieces arrive at 32 B/clk per SM and the sums leave TMEM at 43 B/clk, both below
-// what one-product kernels take.  (Releasing a stage piece by piece instead of whole: 97 -> 110; 128 terms an accumulator would
-// halve the sums' traffic and cost accuracy: 4.0 instead of 3.1 at K = 3072.)
+// Rotate.  The first two pieces of a number are multiples of units that its row of X (its column of R) shares: 2^-6 and 2^-14 of its
+// largest number's power of two, at most 128 of them; the third is the rest, rounded.  Products of first pieces then add up exactly in
+// one accumulator over 512 terms (2^14 2^9 units), first with second pieces exactly in another, and a third one takes the second with
+// second pieces, first with third and second with third, whose sums are 2^-10 of the whole and less.  Eight products; the epilogue
+// warps add the three to running fp32 sums, to nearest, every 512 terms.  Objectives of 384 .. 4096 wide rows of the calibration
+// recipe lie 1e-10 .. 4e-8 from 64 bits on either side, as a chain of fp32 multiply-adds has them (pieces of each number's own leading bits,
+// 64 terms an accumulator: 6e-8 .. 1.2e-7, always below).
+//
+// Accumulate.  Pieces of each number's own leading bits (x = p0 + p1 + p2 exactly) times signs, three products; an accumulator holds 64 terms,
+// small pieces first, and is then added to running fp32 sums.  M lies 0.5e-7 .. 1.1e-7 from 64 bits where the chains have 0.8e-7 .. 6e-7
+// (from d = 768 on, at no size more than they).
+//
+// What bounds it: the tensor cores and, with them busy, the board's power, where the CUDA cores' product is bound by its
+// shared-memory reads.  1000 x 3072 fp32 rows: rotate 504 -> 149 us (96 tiles of 256 x 128 in two rounds on 74 pairs, 32 instructions of
+// 64 cycles a k block), accumulate 409 -> 51, staging 8 -> 8 + 7 (the second pieces take the first ones' place); the whole step 885 ->
+// 218.  (Six products of each number's own pieces, on tiles of 256 x 192: rotate 96, step 158.)
 #pragma once
 #include "conqur_simt.cuh"
 #include "conqur_tc.cuh"
@@ -30,11 +36,10 @@ constexpr int SP_SMEM_BYTES = SP_RING_BYTES + 1024 + 8 * 4096 + 1024;   // ring,
 
 struct SpArgs {
   int M, N, K;
-  int pa, pb;                                            // pieces of A and of B: 1 or 3
   int n_stages, stage_bytes;
   float* outF; long long ldo;                            // Y (quantised targets) or M
-  __nv_bfloat16* outS; long long lds, s_piece; int pc;   // targets: pc pieces, s_piece elements apart
-  const float* rs;                                       // the targets' row scale (and the objective's)
+  __nv_bfloat16* outS; long long lds;                    // targets
+  const float* rs;                                       // 1, or 0 for rows that are left out
   unsigned *rowmax, *rowmin;
   double* part_d;                                        // objective partials: sixteen per tile (a warp's of either CTA)
   DevState* st;
@@ -152,7 +157,11 @@ template <int BN, int EPI>
 __global__ void __launch_bounds__(SP_THREADS, 1)
 sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const SpArgs g) {
   constexpr bool MN = EPI == SP_EPI_ACCUM;               // orientation of both operands
+  constexpr int PA = 3, PB = MN ? 1 : 3;                 // pieces of either operand
+  constexpr int SUMS = MN ? 1 : 3, BUFS = MN ? 2 : 1;    // accumulators of a tile at a time, and sets of them
+  constexpr int CHUNK = MN ? 1 : 8;                      // k blocks an accumulator holds
   static_assert(!MN || BN % 128 == 0, "MN-major tiles are 64 columns wide in each CTA of the pair");
+  static_assert(SUMS * BUFS * BN <= 512, "TMEM columns");
   constexpr int A_BYTES = TC_BM * TC_BK * 2, B_ROWS = BN / 2, B_BYTES = B_ROWS * TC_BK * 2;
   constexpr int HALF = BN / 2, BLOCKS = HALF / 32;       // columns of the tile a warp adds up
   extern __shared__ uint8_t smem_raw[];
@@ -195,11 +204,11 @@ sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         for (int kb = 0; kb < num_kb; ++kb) {
           if (!tc_wait(&aux->empty[stage], phase ^ 1u, abort_flag)) { ok = false; timeout_site = 1; break; }
           uint8_t* sa = smem + stage * g.stage_bytes;
-          uint8_t* sb = sa + g.pa * A_BYTES;
+          uint8_t* sb = sa + PA * A_BYTES;
           const uint32_t bar = ptx::mapa_u32(ptx::smem_u32(&aux->full[stage]), 0);
-          if (rank == 0) ptx::mbar_expect_tx(&aux->full[stage], 2 * (g.pa * A_BYTES + g.pb * B_BYTES));
+          if (rank == 0) ptx::mbar_expect_tx(&aux->full[stage], 2 * (PA * A_BYTES + PB * B_BYTES));
           const int k0 = kb * TC_BK;
-          for (int p = 0; p < g.pa; ++p) {
+          for (int p = 0; p < PA; ++p) {
             if (MN) {
 #pragma unroll
               for (int h = 0; h < TC_BM / 64; ++h) ptx::tma_load_3d_pair(sa + p * A_BYTES + h * 8192, &tmA, bar, m0 + 64 * h, k0, p);
@@ -207,7 +216,7 @@ sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
               ptx::tma_load_3d_pair(sa + p * A_BYTES, &tmA, bar, k0, m0, p);
             }
           }
-          for (int p = 0; p < g.pb; ++p) {
+          for (int p = 0; p < PB; ++p) {
             if (MN) {
 #pragma unroll
               for (int h = 0; h < B_ROWS / 64; ++h) ptx::tma_load_3d_pair(sb + p * B_BYTES + h * 8192, &tmB, bar, n0 + 64 * h, k0, p);
@@ -235,25 +244,30 @@ sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       uint32_t phase = 0, n_acc = 0;
       bool ok = true;
       for (int tile = worker; tile < num_tiles && ok; tile += n_workers) {
-        for (int kb = 0; kb < num_kb; ++kb, ++n_acc) {
-          const uint32_t buf = n_acc & 1u;
-          if (!tc_wait_warp(&aux->tempty[buf], ((n_acc >> 1) & 1u) ^ 1u, abort_flag)) { ok = false; timeout_site = 2; break; }
+        for (int kb = 0; kb < num_kb; ++kb) {
+          const uint32_t buf = n_acc % BUFS;
+          const bool first = kb % CHUNK == 0;
+          if (first && !tc_wait_warp(&aux->tempty[buf], ((n_acc / BUFS) & 1u) ^ 1u, abort_flag)) { ok = false; timeout_site = 2; break; }
           if (!tc_wait_warp(&aux->full[stage], phase, abort_flag)) { ok = false; timeout_site = 3; break; }
           ptx::tc_fence_after();
-          const uint64_t sa = ab0 + ((uint32_t)(stage * g.stage_bytes) >> 4), sb = sa + (uint32_t)(g.pa * (A_BYTES / 16));
-          const uint32_t d_tmem = tmem_base + buf * 256u;
-          uint32_t acc = 0;
-          for (int sum = min(2, g.pa + g.pb - 2); sum >= 0; --sum)          // piece numbers add up to 2, 1, 0: small products first
-            for (int i = max(0, sum - (g.pb - 1)); i <= min(sum, g.pa - 1); ++i) {
-              const uint64_t ad = sa + (uint32_t)(i * (A_BYTES / 16)), bd = sb + (uint32_t)((sum - i) * (B_BYTES / 16));
+          const uint64_t sa = ab0 + ((uint32_t)(stage * g.stage_bytes) >> 4), sb = sa + (uint32_t)(PA * (A_BYTES / 16));
+          const uint32_t d_tmem = tmem_base + buf * (uint32_t)(SUMS * BN);
 #pragma unroll
-              for (int j = 0; j < TC_BK / 16; ++j) {
-                ptx::umma_bf16_by<true>(leader, d_tmem, ad + j * STEP, bd + j * STEP, idesc, acc);
-                acc = 1u;
-              }
+          for (int sum = MN ? 2 : 3; sum >= 0; --sum)    // what piece numbers add up to: small products first
+#pragma unroll
+            for (int i = sum > PB - 1 ? sum - (PB - 1) : 0; i <= (sum < PA - 1 ? sum : PA - 1); ++i) {
+              const uint64_t ad = sa + (uint32_t)(i * (A_BYTES / 16)), bd = sb + (uint32_t)((sum - i) * (B_BYTES / 16));
+              const bool starts = SUMS == 1 ? sum == 2 : sum == 3 ? i == 1 : sum < 2 && i == 0;
+#pragma unroll
+              for (int j = 0; j < TC_BK / 16; ++j)
+                ptx::umma_bf16_by<true>(leader, d_tmem + (uint32_t)(SUMS == 1 ? 0 : (sum < 2 ? sum : 2) * BN), ad + j * STEP, bd + j * STEP, idesc,
+                                        first && starts && j == 0 ? 0u : 1u);
             }
           ptx::umma_commit_by<true>(leader, empty0 + (uint32_t)stage * 8u);
-          ptx::umma_commit_by<true>(leader, tfull0 + buf * 8u);
+          if (kb % CHUNK == CHUNK - 1 || kb == num_kb - 1) {
+            ptx::umma_commit_by<true>(leader, tfull0 + buf * 8u);
+            ++n_acc;
+          }
           if (++stage == g.n_stages) { stage = 0; phase ^= 1u; }
         }
       }
@@ -272,17 +286,25 @@ sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       float acc[HALF];
 #pragma unroll
       for (int i = 0; i < HALF; ++i) acc[i] = 0.f;
-      for (int kb = 0; kb < num_kb; ++kb, ++n_acc) {
-        const uint32_t buf = n_acc & 1u;
+      for (int kb = 0; kb < num_kb; kb += CHUNK, ++n_acc) {
+        const uint32_t buf = n_acc % BUFS;
         // (a lane that gives up takes part in the warp's loads all the same; the vote below ends the loop for all lanes at once)
-        if (!tc_wait(&aux->tfull[buf], (n_acc >> 1) & 1u, abort_flag)) { ok = false; timeout_site = 4; }
+        if (!tc_wait(&aux->tfull[buf], (n_acc / BUFS) & 1u, abort_flag)) { ok = false; timeout_site = 4; }
         ptx::tc_fence_after();
 #pragma unroll
         for (int c = 0; c < BLOCKS; ++c) {
+          const uint32_t at = t_lane + buf * (uint32_t)(SUMS * BN) + (uint32_t)(c * 32);
           uint32_t r[32];
-          ptx::tmem_ld32_tied(t_lane + buf * 256u + (uint32_t)(c * 32), r);
+          ptx::tmem_ld32_tied(at, r);
 #pragma unroll
           for (int i = 0; i < 32; ++i) acc[c * 32 + i] += __uint_as_float(r[i]);
+          if (SUMS == 3) {
+            uint32_t m[32];
+            ptx::tmem_ld32_tied(at + (uint32_t)(SUMS == 3 ? BN : 0), r);
+            ptx::tmem_ld32_tied(at + (uint32_t)(SUMS == 3 ? 2 * BN : 0), m);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) acc[c * 32 + i] += __uint_as_float(r[i]) + __uint_as_float(m[i]);
+          }
         }
         ptx::tc_fence_before();
         ok = __all_sync(0xffffffffu, ok);
@@ -294,11 +316,8 @@ sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       const int rows_ok = min(32, max(0, g.M - wrow0));
       const bool row_ok = row < g.M;
       float rs = 0.f;
-      uint32_t p0 = 0, p1 = 0, p2 = 0;
-      if (EPI != SP_EPI_ACCUM) {
-        rs = row_ok ? g.rs[row] : 0.f;
-        sp_split(rs, 0.f, p0, p1, p2);
-      }
+      if (EPI != SP_EPI_ACCUM) rs = row_ok ? g.rs[row] : 0.f;
+      const uint32_t one = bf16_bits(rs);
       double sum = 0.0;
       float vmax = -3.0e38f, vmin = 3.0e38f;
 #pragma unroll
@@ -317,21 +336,16 @@ sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             for (int i = 0; i < 8; ++i) a += fabsf(v[h * 8 + i]);
             sum += (double)a;
           }
-          const uint32_t bits[3] = {p0, p1, p2};
+          uint32_t w[16];
 #pragma unroll
-          for (int p = 0; p < 3; ++p) {
-            if (p >= g.pc) break;
-            uint32_t w[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const float a = v[2 * i], b = v[2 * i + 1];
-              const uint32_t lo = (a == 0.f) ? 0u : (bits[p] ^ ((__float_as_uint(a) >> 16) & 0x8000u));
-              const uint32_t hi = (b == 0.f) ? 0u : (bits[p] ^ ((__float_as_uint(b) >> 16) & 0x8000u));
-              w[i] = lo | (hi << 16);
-            }
-            // (the targets' rows are padded to 64 columns; columns past N hold the zero operand's zeros)
-            tc_store_block_bf16(stg, lane, w, g.outS + p * g.s_piece + (long long)wrow0 * g.lds + col0, g.lds, rows_ok);
+          for (int i = 0; i < 16; ++i) {
+            const float a = v[2 * i], b = v[2 * i + 1];
+            const uint32_t lo = (a == 0.f) ? 0u : (one ^ ((__float_as_uint(a) >> 16) & 0x8000u));
+            const uint32_t hi = (b == 0.f) ? 0u : (one ^ ((__float_as_uint(b) >> 16) & 0x8000u));
+            w[i] = lo | (hi << 16);
           }
+          // (the targets' rows are padded to 64 columns; columns past N hold the zero operand's zeros)
+          tc_store_block_bf16(stg, lane, w, g.outS + (long long)wrow0 * g.lds + col0, g.lds, rows_ok);
         } else if (EPI == SP_EPI_ROTATE_Q) {
 #pragma unroll
           for (int i = 0; i < 32; ++i)
@@ -364,14 +378,26 @@ sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   }
 }
 
-// a1: row norms in fp32, and the rows as bf16 pieces; skipped rows are zeros.  bf16 rows are their own single piece (targets then
-// carry 1/||x||, rs = rnorm); fp32 rows are normalised first, the product x * rnorm split with its rounding error (rs = 1).
+// The power of two of max's leading bit; pieces on a grid are multiples of 2^-6 of it (at most 128 of them: 8 bits), then of 2^-14.
+__device__ __forceinline__ float sp_grid(float max) { return __uint_as_float(__float_as_uint(max) & 0x7f800000u); }
+// Two pieces on the grid and the rest rounded to bf16 (additions of 1.5 2^23 grid units round to whole units; all differences are exact).
+__device__ __forceinline__ void sp_split_grid(float v, float rest, float grid, float& p0, float& p1, float& p2) {
+  const float c0 = grid * 196608.f, c1 = grid * 768.f;
+  p0 = __fadd_rn(__fadd_rn(v, c0), -c0);
+  const float r = __fadd_rn(v, -p0);
+  p1 = __fadd_rn(__fadd_rn(r, c1), -c1);
+  p2 = __fadd_rn(__fadd_rn(r, -p1), rest);
+}
+
+// a1: row norms in fp32, and the normalised rows (the product x * rnorm with its rounding error) as pieces: on the row's grid for the
+// rotate product (GRID), which also leaves the norms, or each number's own leading bits for the accumulate product, into the same
+// place once the former has run.  Skipped rows are zeros.
 // Four warps a row, whose pieces of it stay in the L1 between the two passes (1000 x 3072 fp32 rows: one warp a row 14.1 us).
-template <typename TIn>
+template <typename TIn, bool GRID>
 __global__ void __launch_bounds__(128) sp_stage_kernel(const TIn* __restrict__ X, int64_t n, int d, int64_t ld, float* __restrict__ rnorm,
                                                        float* __restrict__ rs, __nv_bfloat16* __restrict__ Xp, int64_t ldp,
                                                        int64_t piece, DevState* st) {
-  __shared__ float part[4];
+  __shared__ float part[8];
   const int64_t row = blockIdx.x;
   const int lane = threadIdx.x & 31;
   const TIn* x = X + row * ld;
@@ -384,50 +410,82 @@ __global__ void __launch_bounds__(128) sp_stage_kernel(const TIn* __restrict__ X
       for (int j = 0; j < 4; ++j) v[j] = k + j < d ? ld_as_float(x + k + j) : 0.f;
     }
   };
-  float ss = 0.f;
+  float r, grid = 0.f;
+  if (GRID) {
+    float ss = 0.f, mx = 0.f;
 #pragma unroll 2
-  for (int k = (int)threadIdx.x * 4; k < d; k += 512) {
-    float v[4];
-    load(k, v);
-    ss = fmaf(v[0], v[0], ss); ss = fmaf(v[1], v[1], ss); ss = fmaf(v[2], v[2], ss); ss = fmaf(v[3], v[3], ss);
+    for (int k = (int)threadIdx.x * 4; k < d; k += 512) {
+      float v[4];
+      load(k, v);
+      ss = fmaf(v[0], v[0], ss); ss = fmaf(v[1], v[1], ss); ss = fmaf(v[2], v[2], ss); ss = fmaf(v[3], v[3], ss);
+      mx = fmaxf(fmaxf(mx, fmaxf(fabsf(v[0]), fabsf(v[1]))), fmaxf(fabsf(v[2]), fabsf(v[3])));
+    }
+    ss = warp_sum(ss);
+    mx = warp_max(mx);
+    if (lane == 0) { part[threadIdx.x >> 5] = ss; part[4 + (threadIdx.x >> 5)] = mx; }
+    __syncthreads();
+    ss = (part[0] + part[1]) + (part[2] + part[3]);
+    mx = fmaxf(fmaxf(part[4], part[5]), fmaxf(part[6], part[7]));
+    const bool good = ss > 0.f && ss <= 3.0e38f;
+    r = good ? 1.0f / sqrtf(ss) : 0.f;
+    grid = good ? sp_grid(mx * r) : 0.f;                 // (rounding keeps the order: no |x * rnorm| is larger)
+    if (threadIdx.x == 0) {
+      if (!good) {
+        atomicAdd(reinterpret_cast<unsigned long long*>(&st->step_skipped), 1ull);
+        if (!(ss == 0.f)) atomicOr(&st->status_flags, STATUS_FLAG_NONFINITE);
+      }
+      rnorm[row] = r;
+      rs[row] = good ? 1.f : 0.f;
+    }
+  } else {
+    r = rnorm[row];
   }
-  ss = warp_sum(ss);
-  if (lane == 0) part[threadIdx.x >> 5] = ss;
-  __syncthreads();
-  ss = (part[0] + part[1]) + (part[2] + part[3]);
-  const bool good = ss > 0.f && ss <= 3.0e38f;
-  const float r = good ? 1.0f / sqrtf(ss) : 0.f;
   __nv_bfloat16* dst = Xp + row * ldp;
 #pragma unroll 2
   for (int k = (int)threadIdx.x * 4; k < d; k += 512) {  // (rows of Xp are padded to 64 elements)
     float v[4] = {0.f, 0.f, 0.f, 0.f};
-    if (good) load(k, v);
-    if (sizeof(TIn) == 2) {
-      *reinterpret_cast<uint2*>(dst + k) = make_uint2(bf16x2_pack(v[0], v[1]), bf16x2_pack(v[2], v[3]));
-    } else {
-      uint2 p[3];
-      float t[4], e[4];
+    if (r > 0.f) load(k, v);
+    uint2 p[3];
+    float t[4], e[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) { t[j] = v[j] * r; e[j] = fmaf(v[j], r, -t[j]); }
+    for (int j = 0; j < 4; ++j) { t[j] = v[j] * r; e[j] = fmaf(v[j], r, -t[j]); }
+    if (GRID) {
+      float q[4][3];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) sp_split_grid(t[j], e[j], grid, q[j][0], q[j][1], q[j][2]);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) p[i] = make_uint2(bf16x2_pack(q[0][i], q[1][i]), bf16x2_pack(q[2][i], q[3][i]));
+    } else {
       sp_split2(t[0], t[1], e[0], e[1], p[0].x, p[1].x, p[2].x);
       sp_split2(t[2], t[3], e[2], e[3], p[0].y, p[1].y, p[2].y);
+    }
 #pragma unroll
-      for (int i = 0; i < 3; ++i) *reinterpret_cast<uint2*>(dst + i * piece + k) = p[i];
-    }
-  }
-  if (threadIdx.x == 0) {
-    if (!good) {
-      atomicAdd(reinterpret_cast<unsigned long long*>(&st->step_skipped), 1ull);
-      if (!(ss == 0.f)) atomicOr(&st->status_flags, STATUS_FLAG_NONFINITE);
-    }
-    rnorm[row] = r;
-    rs[row] = sizeof(TIn) == 2 ? r : (good ? 1.f : 0.f);
+    for (int i = 0; i < 3; ++i) *reinterpret_cast<uint2*>(dst + i * piece + k) = p[i];
   }
 }
 
-// R^T as three pieces (row n, column k), rows ldp elements long: the rotate product then reads both operands along k.
-static __global__ void __launch_bounds__(256) sp_split_rt_kernel(const float* __restrict__ R, int d, __nv_bfloat16* __restrict__ Rp,
-                                                                 int64_t ldp, int64_t piece) {
+// Largest magnitude of each column of R (cleared by the caller; the bits of numbers without sign are ordered like the numbers).
+static __global__ void __launch_bounds__(256) sp_colmax_kernel(const float* __restrict__ R, int d, unsigned* __restrict__ colmax) {
+  __shared__ float m[8][32];
+  const int n = blockIdx.x * 32 + (threadIdx.x & 31), y = threadIdx.x >> 5;
+  const int k0 = (int)((int64_t)d * blockIdx.y / gridDim.y), k1 = (int)((int64_t)d * (blockIdx.y + 1) / gridDim.y);
+  float v = 0.f;
+  if (n < d) {
+#pragma unroll 8
+    for (int k = k0 + y; k < k1; k += 8) v = fmaxf(v, fabsf(R[(int64_t)k * d + n]));
+  }
+  m[y][threadIdx.x & 31] = v;
+  __syncthreads();
+  if (y == 0 && n < d) {
+#pragma unroll
+    for (int i = 1; i < 8; ++i) v = fmaxf(v, m[i][threadIdx.x]);
+    atomicMax(colmax + n, __float_as_uint(v));
+  }
+}
+// R^T as three pieces (row n, column k), the first two on the grid of R's column n, rows ldp elements long: the rotate product then
+// reads both operands along k.
+static __global__ void __launch_bounds__(256) sp_split_rt_kernel(const float* __restrict__ R, int d, const unsigned* __restrict__ colmax,
+                                                                 __nv_bfloat16* __restrict__ Rp, int64_t ldp, int64_t piece) {
   __shared__ float t[32][33];
   const int k0 = blockIdx.y * 32, n0 = blockIdx.x * 32, x = threadIdx.x & 31, y = threadIdx.x >> 5;
 #pragma unroll
@@ -440,10 +498,10 @@ static __global__ void __launch_bounds__(256) sp_split_rt_kernel(const float* __
   for (int i = 0; i < 4; ++i) {
     const int n = n0 + y + 8 * i, k = k0 + x;
     if (n >= d || k >= d) continue;
-    uint32_t p[3];
-    sp_split(t[x][y + 8 * i], 0.f, p[0], p[1], p[2]);
+    float p[3];
+    sp_split_grid(t[x][y + 8 * i], 0.f, sp_grid(__uint_as_float(colmax[n])), p[0], p[1], p[2]);
 #pragma unroll
-    for (int j = 0; j < 3; ++j) reinterpret_cast<unsigned short*>(Rp)[j * piece + (int64_t)n * ldp + k] = (unsigned short)p[j];
+    for (int j = 0; j < 3; ++j) Rp[j * piece + (int64_t)n * ldp + k] = __float2bfloat16_rn(p[j]);
   }
 }
 
@@ -453,7 +511,7 @@ static __global__ void __launch_bounds__(256) sp_quant_target_kernel(const float
                                                                      const unsigned* __restrict__ rowmax_ord,
                                                                      const unsigned* __restrict__ rowmin_ord, QuantSpec qs,
                                                                      double* __restrict__ partials, __nv_bfloat16* __restrict__ S,
-                                                                     int64_t lds, int64_t piece, int pc, double* __restrict__ part_diag) {
+                                                                     int64_t lds, double* __restrict__ part_diag) {
   const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   const bool diag = part_diag != nullptr;
@@ -465,15 +523,13 @@ static __global__ void __launch_bounds__(256) sp_quant_target_kernel(const float
     const bool live = qs.bits ? (rq.inv > 0.f) : (r > 0.f);
     const float* y = Y + row * (int64_t)d;
     unsigned short* s = reinterpret_cast<unsigned short*>(S) + row * lds;
-    uint32_t p[3];
-    sp_split(r, 0.f, p[0], p[1], p[2]);
     float qsum = 0.f;
     RowDiag dg{0.f, 0.f, 0.f, 0.f};
     for (int j = lane; j < d; j += 32) {
       const float sg = second_pass_elem(y[j], r, qs, rq, qsum, diag && live, dg);
       const uint32_t neg = sg < 0.f ? 0x8000u : 0u;
       const bool zero = !live || sg == 0.f;
-      for (int i = 0; i < pc; ++i) s[i * piece + j] = (unsigned short)(zero ? 0u : (p[i] ^ neg));
+      s[j] = (unsigned short)(zero ? 0u : (0x3f80u ^ neg));                      // +-1
     }
     qsum = warp_sum(qsum);
     if (live) contrib = (double)(r * rq.delta) * (double)qsum;
@@ -495,35 +551,30 @@ static __global__ void __launch_bounds__(256) sp_quant_target_kernel(const float
 
 // ------------------------------------------------------------------ host side
 // Steps that take the pieces.  Whole step, CUDA cores -> this, us (one B200):
-//   fp32 rows, d = 384  n = 1000 49 -> 49, 2048 68 -> 66;  512  256 37 -> 41, 512 47 -> 45, 1000 70 -> 54;  640  256 45 -> 43;
-//              1024  64 49 -> 49, 128 55 -> 51, 1000 147 -> 68;  2048  16 72 -> 78, 64 82 -> 78;  3072  1000 889 -> 165, 2048 1668 -> 288
-//   bf16 rows, d = 320  2048 69 -> 66;  384  16 31 -> 33, 64 37 -> 33, 2048 82 -> 66;  1024  16 56 -> 43, 1000 178 -> 60;
-//              3072  2048 1833 -> 244
-// (below: too few 256-row tiles to fill the chip, and six products for one)
-constexpr int SP_MIN_D = 384;
+//   fp32 rows, d = 768  n = 512 71 -> 49, 2048 157 -> 79;  1024  128 55 -> 51, 256 68 -> 52, 1000 147 -> 64, 8192 806 -> 278;
+//              2048  64 82 -> 74, 2048 809 -> 170;  3072  1000 885 -> 218, 2048 1662 -> 336;  4096  32 214 -> 149, 2048 2747 -> 668
+//   bf16 rows, d = 768  n = 64 56 -> 44, 2048 177 -> 79;  1024  64 74 -> 49;  3072  2048 1835 -> 332
+// (below: too few 256-row tiles to fill the chip, and eight products for one.  Narrower ones would gain up to 1.4 times, but their M came
+// out further from 64 bits than the CUDA cores': 384 x 8192 rows 0.9e-7 -> 1.7e-7, 512 x 2048 0.8e-7 -> 1.0e-7; at 768 2.6e-7 -> 1.8e-7)
+constexpr int SP_MIN_D = 768;
 inline bool sp_takes(int64_t n, int d, bool f32) {
-  if (!f32) return d >= SP_MIN_D && n >= 64;
-  return n * d >= (d >= 1024 ? (int64_t)1 << 17 : (int64_t)1 << 18) && d >= 512;
+  return d >= SP_MIN_D && (f32 ? n * d >= (d >= 1024 ? (int64_t)1 << 17 : (int64_t)1 << 18) : n >= 64);
 }
 struct SpLayout {
   int64_t ldp;                                           // row length of all pieces: d rounded up to 64
-  int px, pc;                                            // pieces of the rows and of the targets
-  size_t Xp, Sp, Rp, rs;
+  size_t Xp, Sp, Rp, rs, colmax;
 };
 // Contexts that lay them out: those whose longest step takes them (a shorter one may not, a longer one always does).
 inline bool sp_layout_wanted(int d, int P, int64_t n_max, bool f32) { return P == 1 && sp_takes(n_max, d, f32); }
 
 // The rows' pieces borrow `scratch` (the update's matrices: no update runs during a step) where they fit it.  The fp32 target matrix C
 // of a step on the CUDA cores shares its place with what a step over pieces writes instead, except where such a step goes through it
-// too (fake-quantisation, diagnostics).  A row element costs 4 bytes as without pieces for fp32 rows up to 2.7 d of them, else 8; 6 or 8
-// for bf16 rows.
+// too (fake-quantisation, diagnostics).  A row element costs 4 bytes as without pieces for up to 2.7 d rows, else 8.
 template <typename Take>
-inline void sp_make_layout(int d, int64_t n, int in_dtype, bool through_c, size_t scratch, size_t scratch_bytes, size_t* C, SpLayout* L,
+inline void sp_make_layout(int d, int64_t n, bool through_c, size_t scratch, size_t scratch_bytes, size_t* C, SpLayout* L,
                            Take&& take) {
   L->ldp = ((int64_t)d + 63) / 64 * 64;
-  L->px = in_dtype == CONQUR_F32 ? 3 : 1;
-  L->pc = in_dtype == CONQUR_F32 ? 1 : 3;
-  const size_t rows = (size_t)(2 * L->px * n * L->ldp), targets = ((size_t)(2 * L->pc * n * L->ldp) + 255) / 256 * 256;
+  const size_t rows = (size_t)(2 * 3 * n * L->ldp), targets = ((size_t)(2 * n * L->ldp) + 255) / 256 * 256;
   const size_t c_bytes = sizeof(float) * (size_t)n * d;
   const bool borrow = rows <= scratch_bytes;
   const size_t mine = targets + (borrow ? 0 : rows);
@@ -532,6 +583,7 @@ inline void sp_make_layout(int d, int64_t n, int in_dtype, bool through_c, size_
   L->Xp = borrow ? scratch : L->Sp + targets;
   L->Rp = take((size_t)(2 * 3 * d * L->ldp));
   L->rs = take(sizeof(float) * (size_t)n);
+  L->colmax = take(sizeof(unsigned) * (size_t)d);
 }
 
 // (column, row, piece) map over `pieces` bf16 matrices of rows x cols, `piece` elements apart; box 64 columns x box_rows.
@@ -553,12 +605,13 @@ inline int sp_make_tmap(CUtensorMap* tm, const void* ptr, uint64_t rows, uint64_
   return CONQUR_OK;
 }
 
-// Tile width of a product of M x N outputs on `pairs` CTA pairs: the one with the least rounds x width.
-inline int sp_pick_bn(int64_t M, int64_t N, int pairs, bool mn) {
+// Tile width of the accumulate product of M x N outputs on `pairs` CTA pairs: the one with the least rounds x width.  (The rotate
+// product's three accumulators fill the TMEM at 128.)
+constexpr int SP_ROT_BN = 128;
+inline int sp_pick_bn(int64_t M, int64_t N, int pairs) {
   int best = 256;
   double cost = 1e300;
-  for (int bn : {256, 192, 128}) {
-    if (mn && bn == 192) continue;                       // (MN-major tiles come 64 columns wide per CTA)
+  for (int bn : {256, 128}) {
     const int64_t tiles = ((M + 255) / 256) * ((N + bn - 1) / bn);
     const double c = (double)((tiles + pairs - 1) / pairs) * (bn + 16);
     if (c < cost) { cost = c; best = bn; }
@@ -579,7 +632,7 @@ inline int sp_launch_bn(int device, int pairs, cudaStream_t s, const CUtensorMap
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SP_SMEM_BYTES) != cudaSuccess) return CONQUR_ERR_CUDA;
     attr_dev_mask.fetch_or(dev_bit, std::memory_order_release);
   }
-  g.stage_bytes = g.pa * (TC_BM * TC_BK * 2) + g.pb * (BN / 2 * TC_BK * 2);
+  g.stage_bytes = 3 * (TC_BM * TC_BK * 2) + (EPI == SP_EPI_ACCUM ? 1 : 3) * (BN / 2 * TC_BK * 2);
   g.n_stages = SP_RING_BYTES / g.stage_bytes < SP_STAGES_MAX ? SP_RING_BYTES / g.stage_bytes : SP_STAGES_MAX;
   const int64_t tiles = sp_tiles(g.M, g.N, BN);
   cudaLaunchConfig_t cfg = {};
@@ -591,13 +644,4 @@ inline int sp_launch_bn(int device, int pairs, cudaStream_t s, const CUtensorMap
   cfg.attrs = at; cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, a, b, g) == cudaSuccess ? CONQUR_OK : CONQUR_ERR_CUDA;
 }
-template <int EPI>
-inline int sp_launch(int bn, int device, int pairs, cudaStream_t s, const CUtensorMap& a, const CUtensorMap& b, const SpArgs& g) {
-  if (bn == 256) return sp_launch_bn<256, EPI>(device, pairs, s, a, b, g);
-  if constexpr (EPI != SP_EPI_ACCUM) {
-    if (bn == 192) return sp_launch_bn<192, EPI>(device, pairs, s, a, b, g);
-  }
-  return sp_launch_bn<128, EPI>(device, pairs, s, a, b, g);
-}
-
 }  // namespace conqur

@@ -132,10 +132,10 @@ def test_exact_contexts_hold_pieces_only_where_a_step_takes_them(B):
     """The rotation's three bf16 pieces (6 d^2 bytes) and the rows' and targets' belong to contexts whose longest step runs over them."""
     def ws(d, n, f32):
         return B.conqur_workspace_bytes(d, B.make_config(in_dtype=B.CONQUR_F32 if f32 else B.CONQUR_BF16, mode=B.CONQUR_EXACT_F32, n_max=n))
-    # (longest step that stays on the CUDA cores, one row more); fp32 rows take the pieces from d = 512 on, bf16 rows from 384
-    for d, n, f32 in ((512, 511, True), (1000, 262, True), (2048, 63, True), (384, 63, False), (2048, 63, False)):
+    # (longest step that stays on the CUDA cores, one row more)
+    for d, n, f32 in ((768, 341, True), (1000, 262, True), (2048, 63, True), (768, 63, False), (2048, 63, False)):
         assert ws(d, n + 1, f32) - ws(d, n, f32) >= 6 * d * d
-    for d, f32 in ((383, False), (384, True), (448, True), (511, True)):
+    for d, f32 in ((384, False), (767, False), (448, True), (767, True)):
         # a row costs its fp32 target, its norm and its range, and its share of the partials
         assert ws(d, 32768, f32) - ws(d, 16384, f32) <= 16384 * (4 * d + 128)
 
@@ -147,9 +147,8 @@ def test_exact_workspace_grows_with_rows_as_little_as_the_pieces_allow(B):
                                                         n_max=n, **kw)) for n in (n1, n2)]
         return (ws[1] - ws[0]) / (n2 - n1) - 128
     for d in (1024, 4096, 8192):
-        assert row(d, d // 2, 2 * d, True) <= 4 * d      # what a row took before there were pieces
-        assert row(d, 4 * d, 8 * d, True) <= 8 * d
-        assert row(d, 2 * d, 7 * d, False) <= 6 * d
-        assert row(d, 10 * d, 20 * d, False) <= 8 * d
-        assert row(d, d // 2, 2 * d, True, quant_bits=4) <= 6 * d
-        assert row(d, 4 * d, 8 * d, True, quant_bits=4) <= 12 * d
+        for f32 in (True, False):
+            assert row(d, d // 2, 2 * d, f32) <= 4 * d   # what a row takes without pieces
+            assert row(d, 4 * d, 8 * d, f32) <= 8 * d
+            assert row(d, d // 2, 2 * d, f32, quant_bits=4) <= 6 * d
+            assert row(d, 4 * d, 8 * d, f32, quant_bits=4) <= 12 * d

@@ -130,17 +130,44 @@ def test_rows_accumulate_and_rotation_follows():
 
 
 # the smallest steps that take the pieces, by row type and width: one row of tiles of which the second CTA's half is empty or nearly so
-@pytest.mark.parametrize("d,n,dtype", [(384, 64, torch.bfloat16), (385, 65, torch.bfloat16), (511, 100, torch.bfloat16),
-                                       (2050, 64, torch.bfloat16), (512, 129, torch.bfloat16), (1024, 128, torch.float32),
+@pytest.mark.parametrize("d,n,dtype", [(768, 64, torch.bfloat16), (769, 65, torch.bfloat16), (1023, 100, torch.bfloat16),
+                                       (2050, 64, torch.bfloat16), (768, 342, torch.float32), (1024, 128, torch.float32),
                                        (1030, 130, torch.float32), (2050, 64, torch.float32)])
 def test_smallest_steps_over_pieces(d, n, dtype):
     test_signs_statistics_and_objective(d, n, dtype)
 
 
+# one chunk of 512 terms and a part of another, whole chunks, one k block more; rows of one size and rows that one number rules
+@pytest.mark.parametrize("d,n", [(768, 700), (1024, 1024), (1088, 513), (2560, 300)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("massive", [False, True])
+def test_objective_is_not_biased(d, n, dtype, massive):
+    """What the tensor cores cut off has the sign of the sum: an objective of sums that lose any of it comes out below 64 bits."""
+    off = []
+    for seed in range(3):
+        x = _rand(d + seed, n, d)
+        if massive:
+            x[torch.arange(n, device="cuda"), torch.randint(0, d, (n,), generator=torch.Generator(device="cuda").manual_seed(n), device="cuda")] *= 300.0
+        x = x.to(dtype)
+        r = torch.linalg.qr(_rand(70 + seed, d, d).double())[0].float().contiguous()
+        c = B.Context(d, n, in_dtype="f32" if dtype == torch.float32 else "bf16", mode="exact")
+        c.set_R(r)
+        c.step(x)
+        xt = x.double() / x.double().norm(dim=1, keepdim=True)
+        y = xt @ r.double()
+        off.append((c.get_objective()[0] * math.sqrt(d) - float(y.abs().sum())) / float(y.abs().sum()))
+        s = c.debug_get_signs(n).double()
+        # a rotated number is off by a few 2^-24 of its row's norm over sqrt(d), whatever the number
+        assert (y.abs()[s != torch.sign(y)] <= 12.0 * 2.0 ** -24 / math.sqrt(768.0)).all()
+    # rows' norms in fp32: d squares in chains of d / 128 and three more sums, a root and a division, each to nearest, the same for a row's
+    # numbers and averaged over n rows; sums in one accumulator each of 64 terms left -6e-8 .. -1.2e-7 at any n
+    assert max(abs(o) for o in off) <= 2.5e-8, off
+
+
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 def test_a_feature_of_tiny_values(dtype):
     """Low pieces of values below 2^-110 or so are subnormal: a feature that small everywhere loses up to 2^-126 a row, absolutely."""
-    d, n = 520, 1000
+    d, n = 800, 1000
     x = _rand(1, n, d)
     x[:, 7] *= 1e-36
     x = x.to(dtype)
