@@ -4,13 +4,14 @@
 // add toward zero (2^-23 of the sum, once per instruction of 16 terms).  A long sum kept in TMEM loses more than an fp32 chain
 // does, and what is lost has the sum's sign, so that it does not average out over a matrix.
 //
-// Rotate.  The first two pieces of a number are multiples of units that its row of X (its column of R) shares: 2^-6 and 2^-14 of its
-// largest number's power of two, at most 128 of them; the third is the rest, rounded.  Products of first pieces then add up exactly in
-// one accumulator over 512 terms (2^14 2^9 units), first with second pieces exactly in another, and a third one takes the second with
+// Rotate.  The first two pieces of a number are multiples of units that its row of X (its column of R) shares: 2^-7 and 2^-16 of its
+// largest number's power of two, at most 256 of them; the third is the rest, rounded.  Products of first pieces then add up exactly in
+// one accumulator over 512 terms (at most 2^24 units, as neither side's norm exceeds 1 and its largest number is over 128 units; twice
+// that, for a last bit, only where a row is its column), first with second pieces in another, and a third one takes the second with
 // second pieces, first with third and second with third, whose sums are 2^-10 of the whole and less.  Eight products; the epilogue
-// warps add the three to running fp32 sums, to nearest, every 512 terms.  Objectives of 384 .. 4096 wide rows of the calibration
-// recipe lie 1e-10 .. 4e-8 from 64 bits on either side, as a chain of fp32 multiply-adds has them (pieces of each number's own leading bits,
-// 64 terms an accumulator: 6e-8 .. 1.2e-7, always below).
+// warps add the three to running fp32 sums, to nearest, every 512 terms.  Objectives of 768 .. 4096 wide rows of the calibration
+// recipe lie 2e-9 (at most 9e-9) from 64 bits on either side, chains of fp32 multiply-adds 6e-9 (2e-8), and signs fall the other way half
+// as often (pieces of each number's own leading bits, 64 terms an accumulator: fewer signs still, but 6e-8 .. 1.2e-7 low, always).
 //
 // Accumulate.  Pieces of each number's own leading bits (x = p0 + p1 + p2 exactly) times signs, three products; an accumulator holds 64 terms,
 // small pieces first, and is then added to running fp32 sums.  M lies 0.5e-7 .. 1.1e-7 from 64 bits where the chains have 0.8e-7 .. 6e-7
@@ -149,7 +150,7 @@ __device__ __forceinline__ void sp_put_block(uint8_t* stg, int lane, const float
 // D[m][n] = sum_k A(m, k) B(n, k) on 256 x BN tiles of CTA pairs, operands as stacks of bf16 pieces (3-D maps: column, row,
 // piece).  Warp 0 loads, warp 1 issues (CTA 0 for both), warps 4-11 add up the accumulators and write the tile (2 and 3 idle: the
 // registers go by warpgroups).  A warp's 128 running sums, a block on its way from TMEM and the write-out's addresses do not all fit 208
-// registers: the 256-wide variants spill up to 52 bytes a thread outside the accumulation loop, the others up to 12 or nothing.
+// registers: the variants with 128 sums spill up to 20 bytes a thread outside the accumulation loop, the others up to 16 or nothing.
 //   ROTATE    A = X (K-major), B = R^T (K-major): targets sgn(y) * rs as pc bf16 pieces, objective partials sum |y| rs
 //   ROTATE_Q  the same products, stored as fp32 Y with the row's range
 //   ACCUM     A = X, B = targets (both MN-major, contraction over rows): added to M, once per element and launch
@@ -378,11 +379,11 @@ sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   }
 }
 
-// The power of two of max's leading bit; pieces on a grid are multiples of 2^-6 of it (at most 128 of them: 8 bits), then of 2^-14.
+// The power of two of max's leading bit; pieces on a grid are multiples of 2^-7 of it (at most 256 of them: 8 bits), then of 2^-16.
 __device__ __forceinline__ float sp_grid(float max) { return __uint_as_float(__float_as_uint(max) & 0x7f800000u); }
 // Two pieces on the grid and the rest rounded to bf16 (additions of 1.5 2^23 grid units round to whole units; all differences are exact).
 __device__ __forceinline__ void sp_split_grid(float v, float rest, float grid, float& p0, float& p1, float& p2) {
-  const float c0 = grid * 196608.f, c1 = grid * 768.f;
+  const float c0 = grid * 98304.f, c1 = grid * 192.f;
   p0 = __fadd_rn(__fadd_rn(v, c0), -c0);
   const float r = __fadd_rn(v, -p0);
   p1 = __fadd_rn(__fadd_rn(r, c1), -c1);
