@@ -14,8 +14,8 @@
 // as often (pieces of each number's own leading bits, 64 terms an accumulator: fewer signs still, but 6e-8 .. 1.2e-7 low, always).
 //
 // Accumulate.  Pieces of each number's own leading bits (x = p0 + p1 + p2 exactly) times signs, three products; an accumulator holds 64 terms,
-// small pieces first, and is then added to running fp32 sums.  M lies 0.5e-7 .. 1.1e-7 from 64 bits where the chains have 0.8e-7 .. 6e-7
-// (from d = 768 on, at no size more than they).
+// small pieces first, and is then added to running fp32 sums.  M lies 0.5e-7 .. 1.8e-7 from 64 bits where the chains have 1.1e-7 ..
+// 1.3e-6 (from d = 768 on, at no size more than they).
 //
 // What bounds it: the tensor cores and, with them busy, the board's power, where the CUDA cores' product is bound by its
 // shared-memory reads.  1000 x 3072 fp32 rows: rotate 504 -> 149 us (96 tiles of 256 x 128 in two rounds on 74 pairs, 32 instructions of
@@ -101,18 +101,11 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
 }
 }  // namespace ptx
 
-// Three bf16 pieces of v (+ rest, a remainder below v's last bit).  A piece below 2^-126 is subnormal, so of values below about 2^-110
-// the low pieces are cut off at 2^-133 and their products with the other side at 2^-126 or so.  A step needs no other path for them:
-// normalised rows and rotations have norm 1, so that much lies far below the rounding of any sum they enter, except that a feature
-// which is that small in every row gets its row of M to 2^-126 absolutely, not relatively (fp32 itself ends at 2^-149).
-__device__ __forceinline__ void sp_split(float v, float rest, uint32_t& p0, uint32_t& p1, uint32_t& p2) {
-  p0 = bf16_bits(v);
-  const float r1 = v - __uint_as_float(p0 << 16);
-  p1 = bf16_bits(r1);
-  p2 = bf16_bits((r1 - __uint_as_float(p1 << 16)) + rest);
-}
-
-// Two numbers at a time: packed pieces, the first number in the low half.  e0, e1: remainders below their last bits.
+// Each number's own three bf16 pieces (+ e, a remainder below its last bit), two numbers at a time, packed with the first in the low half.
+// A piece below 2^-126 is subnormal, so of values below about 2^-110 the low pieces are cut off at 2^-133 and their products with the
+// other side at 2^-126 or so.  A step needs no other path for them: normalised rows have norm 1, so that much lies far below the rounding
+// of any sum they enter, except that a feature which is that small in every row gets its row of M to 2^-126 absolutely, not relatively
+// (fp32 itself ends at 2^-149).
 __device__ __forceinline__ void sp_split2(float a, float b, float e0, float e1, uint32_t& w0, uint32_t& w1, uint32_t& w2) {
   w0 = bf16x2_pack(a, b);
   const float ra = a - __uint_as_float(w0 << 16), rb = b - __uint_as_float(w0 & 0xffff0000u);
