@@ -372,7 +372,8 @@ int step_pieces(conqur_ctx* c, const TIn* X, int64_t n, int64_t ld) {
   float* rs = c->at<float>(L.rs);
   double* part = c->at<double>(c->L.part_d);
   const int64_t xpiece = n * L.ldp;                       // the pieces of this step's rows lie one behind another
-  sp_stage_kernel<TIn, true><<<(unsigned)n, 128, 0, c->stream>>>(X, n, d, ld, rnorm, rs, sp_ptr(c, L.Xp), L.ldp, xpiece, c->state());
+  sp_stage_kernel<TIn, true><<<(unsigned)n, 128, 0, c->stream>>>(X, n, d, ld, rnorm, rs, sp_ptr(c, L.Xp), L.ldp, xpiece, c->state(),
+                                                                 c->at<unsigned>(L.arrived));
   CQ_LAUNCHED(c, K_ROWNORM);
   const int bm = sp_pick_bn(d, d, c->sp_pairs);
   CUtensorMap xk, rk, xm, sm;
@@ -385,6 +386,10 @@ int step_pieces(conqur_ctx* c, const TIn* X, int64_t n, int64_t ld) {
   a.M = (int)n; a.N = d; a.K = d;
   a.rs = rs; a.part_d = part; a.st = c->state();
   a.outS = sp_ptr(c, L.Sp); a.lds = L.ldp;
+  const size_t used = align_up((size_t)(2 * 3 * xpiece));                  // behind this step's pieces in what they borrow
+  a.sums = c->at<float>(L.borrowed + used);
+  a.arrived = c->at<unsigned>(L.arrived);
+  a.share = sp_share_tail(sp_tiles(n, d, SP_ROT_BN), c->sp_pairs, d, L.borrowed_bytes > used ? L.borrowed_bytes - used : 0);
   double* pdiag = g.diagnostics ? c->at<double>(c->L.part_diag) : nullptr;
   int per_problem;
   if (g.quant_bits == 0 && !g.diagnostics) {
@@ -411,7 +416,8 @@ int step_pieces(conqur_ctx* c, const TIn* X, int64_t n, int64_t ld) {
   SpArgs m{};
   m.M = d; m.N = d; m.K = (int)n; m.st = c->state();
   m.outF = c->at<float>(c->L.M); m.ldo = d;
-  sp_stage_kernel<TIn, false><<<(unsigned)n, 128, 0, c->stream>>>(X, n, d, ld, rnorm, rs, sp_ptr(c, L.Xp), L.ldp, xpiece, c->state());
+  sp_stage_kernel<TIn, false><<<(unsigned)n, 128, 0, c->stream>>>(X, n, d, ld, rnorm, rs, sp_ptr(c, L.Xp), L.ldp, xpiece, c->state(),
+                                                                  nullptr);
   CQ_LAUNCHED(c, K_ROWNORM);
   rc = bm == 256 ? sp_launch_bn<256, SP_EPI_ACCUM>(c->device, c->sp_pairs, c->stream, xm, sm, m)
                  : sp_launch_bn<128, SP_EPI_ACCUM>(c->device, c->sp_pairs, c->stream, xm, sm, m);

@@ -18,9 +18,9 @@
 // 1.3e-6 (from d = 768 on, at no size more than they).
 //
 // What bounds it: the tensor cores and, with them busy, the board's power, where the CUDA cores' product is bound by its
-// shared-memory reads.  1000 x 3072 fp32 rows: rotate 504 -> 149 us (96 tiles of 256 x 128 in two rounds on 74 pairs, 32 instructions of
-// 64 cycles a k block), accumulate 409 -> 51, staging 8 -> 8 + 7 (the second pieces take the first ones' place); the whole step 885 ->
-// 218.  (Six products of each number's own pieces, on tiles of 256 x 192: rotate 96, step 158.)
+// shared-memory reads.  1000 x 3072 fp32 rows: rotate 504 -> 110 us (96 tiles of 256 x 128 on 74 pairs, 32 instructions of 64 cycles a k
+// block; 149 in two rounds of whole tiles), accumulate 409 -> 51, staging 8 -> 8 + 7 (the second pieces take the first ones' place); the
+// whole step 885 -> 181.  (Six products of each number's own pieces, on tiles of 256 x 192: rotate 96, step 158.)
 #pragma once
 #include "conqur_simt.cuh"
 #include "conqur_tc.cuh"
@@ -44,6 +44,10 @@ struct SpArgs {
   unsigned *rowmax, *rowmin;
   double* part_d;                                        // objective partials: sixteen per tile (a warp's of either CTA)
   DevState* st;
+  // rotate: tiles from `whole` on are shared out over k, `share` accumulators of them in a row to each pair (see sp_share_tail)
+  int whole, share;
+  float* sums;                                           // a shared part's running sums: HALF x 32 for each of its sixteen warps
+  unsigned* arrived;                                     // per shared tile and warp (zero before the launch): parts that have left theirs
 };
 
 struct SpAux {
@@ -147,7 +151,7 @@ __device__ __forceinline__ void sp_put_block(uint8_t* stg, int lane, const float
 //   ROTATE    A = X (K-major), B = R^T (K-major): targets sgn(y) * rs as pc bf16 pieces, objective partials sum |y| rs
 //   ROTATE_Q  the same products, stored as fp32 Y with the row's range
 //   ACCUM     A = X, B = targets (both MN-major, contraction over rows): added to M, once per element and launch
-template <int BN, int EPI>
+template <int BN, int EPI, bool SHARE>
 __global__ void __launch_bounds__(SP_THREADS, 1)
 sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const SpArgs g) {
   constexpr bool MN = EPI == SP_EPI_ACCUM;               // orientation of both operands
@@ -167,6 +171,25 @@ sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const int worker = (int)(blockIdx.x >> 1), n_workers = (int)(gridDim.x >> 1);
   const int tiles_m = (g.M + 255) / 256, tiles_n = (g.N + BN - 1) / BN, num_tiles = tiles_m * tiles_n;
   const int num_kb = (g.K + TC_BK - 1) / TC_BK;
+  const int whole = SHARE ? g.whole : num_tiles, share = SHARE ? g.share : 1;
+  const int chunks = (num_kb + CHUNK - 1) / CHUNK;       // accumulators of a tile
+  // This pair's pos-th work item: a whole tile, or what it has of a shared one (k blocks kb0 .. kb1, which begin where an accumulator
+  // does).
+  struct Item { int tile, kb0, kb1; };
+  auto get_item = [&](int pos, Item& w) -> bool {
+    w.kb0 = 0; w.kb1 = num_kb;
+    w.tile = worker + pos * n_workers;
+    if (w.tile < whole) return true;
+    if (!SHARE) return false;
+    const int i = pos - (whole > worker ? (whole - worker + n_workers - 1) / n_workers : 0);
+    const int units = (num_tiles - whole) * chunks, u0 = worker * share, u1 = min(units, u0 + share);
+    const int u = i == 0 ? u0 : (u0 / chunks + i) * chunks;
+    if (u >= u1) return false;
+    const int t = u / chunks, c0 = u - t * chunks, c1 = min(chunks, c0 + u1 - u);
+    w.tile = whole + t;
+    w.kb0 = c0 * CHUNK; w.kb1 = min(num_kb, c1 * CHUNK);
+    return true;
+  };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < g.n_stages; ++s) { ptx::mbar_init(&aux->full[s], 1); ptx::mbar_init(&aux->empty[s], 1); }
@@ -191,11 +214,12 @@ sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (int tile = worker; tile < num_tiles && ok; tile += n_workers) {
+      Item w;
+      for (int pos = 0; ok && get_item(pos, w); ++pos) {
         int tm, tn;
-        tc_tile_coords<1>(tile, tiles_m, tiles_n, 0, tm, tn);
+        tc_tile_coords<1>(w.tile, tiles_m, tiles_n, 0, tm, tn);
         const int m0 = tm * 256 + (int)rank * TC_BM, n0 = tn * BN + (int)rank * B_ROWS;
-        for (int kb = 0; kb < num_kb; ++kb) {
+        for (int kb = w.kb0; kb < w.kb1; ++kb) {
           if (!tc_wait(&aux->empty[stage], phase ^ 1u, abort_flag)) { ok = false; timeout_site = 1; break; }
           uint8_t* sa = smem + stage * g.stage_bytes;
           uint8_t* sb = sa + PA * A_BYTES;
@@ -237,8 +261,10 @@ sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       int stage = 0;
       uint32_t phase = 0, n_acc = 0;
       bool ok = true;
-      for (int tile = worker; tile < num_tiles && ok; tile += n_workers) {
-        for (int kb = 0; kb < num_kb; ++kb) {
+      Item w;
+      for (int pos = 0; ok && get_item(pos, w); ++pos) {
+        const int n_kb = SHARE ? w.kb1 - w.kb0 : num_kb;
+        for (int kb = 0; kb < n_kb; ++kb) {
           const uint32_t buf = n_acc % BUFS;
           const bool first = kb % CHUNK == 0;
           if (first && !tc_wait_warp(&aux->tempty[buf], ((n_acc / BUFS) & 1u) ^ 1u, abort_flag)) { ok = false; timeout_site = 2; break; }
@@ -258,7 +284,7 @@ sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                                         first && starts && j == 0 ? 0u : 1u);
             }
           ptx::umma_commit_by<true>(leader, empty0 + (uint32_t)stage * 8u);
-          if (kb % CHUNK == CHUNK - 1 || kb == num_kb - 1) {
+          if (kb % CHUNK == CHUNK - 1 || kb == n_kb - 1) {
             ptx::umma_commit_by<true>(leader, tfull0 + buf * 8u);
             ++n_acc;
           }
@@ -274,13 +300,14 @@ sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const uint32_t t_lane = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * HALF);
     uint32_t n_acc = 0;
     bool ok = true;
-    for (int tile = worker; tile < num_tiles && ok; tile += n_workers) {
+    Item w;
+    for (int pos = 0; ok && get_item(pos, w); ++pos) {
       int tm, tn;
-      tc_tile_coords<1>(tile, tiles_m, tiles_n, 0, tm, tn);
+      tc_tile_coords<1>(w.tile, tiles_m, tiles_n, 0, tm, tn);
       float acc[HALF];
 #pragma unroll
       for (int i = 0; i < HALF; ++i) acc[i] = 0.f;
-      for (int kb = 0; kb < num_kb; kb += CHUNK, ++n_acc) {
+      for (int kb = w.kb0; kb < w.kb1; kb += CHUNK, ++n_acc) {
         const uint32_t buf = n_acc % BUFS;
         // (a lane that gives up takes part in the warp's loads all the same; the vote below ends the loop for all lanes at once)
         if (!tc_wait(&aux->tfull[buf], (n_acc / BUFS) & 1u, abort_flag)) { ok = false; timeout_site = 4; }
@@ -306,6 +333,33 @@ sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (!ok) break;
       }
       if (!ok) break;
+      if (SHARE && w.kb1 - w.kb0 < num_kb) {
+        // A shared tile: every part leaves its sums, and whichever of them comes last adds them all up in the order of the parts (so the
+        // result does not depend on which that is) and goes on with the tile.  Warp by warp: nobody waits.
+        const int t = w.tile - whole, first = t * chunks / share, last = ((t + 1) * chunks - 1) / share;      // the pairs that share it
+        const int slots = chunks % share ? 2 : 1;        // (a pair has parts of at most two tiles)
+        auto sums_of = [&](int pair) {
+          const int slot = pair * slots + (pair * share / chunks == t ? 0 : 1);
+          return g.sums + ((int64_t)(slot * 2 + (int)rank) * 8 + ew) * (HALF * 32) + lane;
+        };
+        float* mine = sums_of(worker);
+#pragma unroll
+        for (int i = 0; i < HALF; ++i) __stcg(mine + i * 32, acc[i]);
+        __threadfence();
+        __syncwarp();
+        unsigned before = 0;
+        if (lane == 0) before = atomicAdd(g.arrived + (2 * t + (int)rank) * 8 + ew, 1u);
+        if (__shfl_sync(0xffffffffu, before, 0) != (unsigned)(last - first)) continue;
+        __threadfence();
+        const float* all = sums_of(first);
+#pragma unroll
+        for (int i = 0; i < HALF; ++i) acc[i] = __ldcg(all + i * 32);
+        for (int p = first + 1; p <= last; ++p) {
+          all = sums_of(p);
+#pragma unroll
+          for (int i = 0; i < HALF; ++i) acc[i] += __ldcg(all + i * 32);
+        }
+      }
       const int wrow0 = tm * 256 + (int)rank * TC_BM + q * 32, row = wrow0 + lane;
       const int rows_ok = min(32, max(0, g.M - wrow0));
       const bool row_ok = row < g.M;
@@ -330,16 +384,16 @@ sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             for (int i = 0; i < 8; ++i) a += fabsf(v[h * 8 + i]);
             sum += (double)a;
           }
-          uint32_t w[16];
+          uint32_t ws[16];
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             const float a = v[2 * i], b = v[2 * i + 1];
             const uint32_t lo = (a == 0.f) ? 0u : (one ^ ((__float_as_uint(a) >> 16) & 0x8000u));
             const uint32_t hi = (b == 0.f) ? 0u : (one ^ ((__float_as_uint(b) >> 16) & 0x8000u));
-            w[i] = lo | (hi << 16);
+            ws[i] = lo | (hi << 16);
           }
           // (the targets' rows are padded to 64 columns; columns past N hold the zero operand's zeros)
-          tc_store_block_bf16(stg, lane, w, g.outS + (long long)wrow0 * g.lds + col0, g.lds, rows_ok);
+          tc_store_block_bf16(stg, lane, ws, g.outS + (long long)wrow0 * g.lds + col0, g.lds, rows_ok);
         } else if (EPI == SP_EPI_ROTATE_Q) {
 #pragma unroll
           for (int i = 0; i < 32; ++i)
@@ -354,7 +408,7 @@ sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       }
       if (EPI == SP_EPI_ROTATE) {
         const double t = warp_sum_d(sum * (double)rs);
-        if (lane == 0) g.part_d[(2 * tile + (int)rank) * 8 + ew] = t;
+        if (lane == 0) g.part_d[(2 * w.tile + (int)rank) * 8 + ew] = t;
       }
     }
   }
@@ -383,6 +437,8 @@ __device__ __forceinline__ void sp_split_grid(float v, float rest, float grid, f
   p2 = __fadd_rn(__fadd_rn(r, -p1), rest);
 }
 
+constexpr int SP_ARRIVED = 2048;                         // counters: sixteen warps of at most 128 shared tiles
+
 // a1: row norms in fp32, and the normalised rows (the product x * rnorm with its rounding error) as pieces: on the row's grid for the
 // rotate product (GRID), which also leaves the norms, or each number's own leading bits for the accumulate product, into the same
 // place once the former has run.  Skipped rows are zeros.
@@ -390,7 +446,9 @@ __device__ __forceinline__ void sp_split_grid(float v, float rest, float grid, f
 template <typename TIn, bool GRID>
 __global__ void __launch_bounds__(128) sp_stage_kernel(const TIn* __restrict__ X, int64_t n, int d, int64_t ld, float* __restrict__ rnorm,
                                                        float* __restrict__ rs, __nv_bfloat16* __restrict__ Xp, int64_t ldp,
-                                                       int64_t piece, DevState* st) {
+                                                       int64_t piece, DevState* st, unsigned* arrived) {
+  if (GRID && blockIdx.x == 0)                           // (the rotate product that follows counts its shared tiles' parts there)
+    for (int i = threadIdx.x; i < SP_ARRIVED; i += 128) arrived[i] = 0u;
   __shared__ float part[8];
   const int64_t row = blockIdx.x;
   const int lane = threadIdx.x & 31;
@@ -545,9 +603,9 @@ static __global__ void __launch_bounds__(256) sp_quant_target_kernel(const float
 
 // ------------------------------------------------------------------ host side
 // Steps that take the pieces.  Whole step, CUDA cores -> this, us (one B200):
-//   fp32 rows, d = 768  n = 512 71 -> 49, 2048 157 -> 79;  1024  128 55 -> 51, 256 68 -> 52, 1000 147 -> 64, 8192 806 -> 278;
-//              2048  64 82 -> 74, 2048 809 -> 170;  3072  1000 885 -> 218, 2048 1662 -> 336;  4096  32 214 -> 149, 2048 2747 -> 668
-//   bf16 rows, d = 768  n = 64 56 -> 44, 2048 177 -> 79;  1024  64 74 -> 49;  3072  2048 1835 -> 332
+//   fp32 rows, d = 768  n = 512 71 -> 49, 2048 157 -> 79;  1024  128 55 -> 45, 256 68 -> 46, 1000 147 -> 59, 8192 806 -> 278;
+//              2048  64 82 -> 49, 2048 809 -> 164;  3072  1000 885 -> 181, 2048 1662 -> 321;  4096  32 214 -> 112, 2048 2747 -> 632
+//   bf16 rows, d = 768  n = 64 56 -> 43, 2048 177 -> 79;  1024  64 74 -> 43;  3072  2048 1835 -> 320
 // (below: too few 256-row tiles to fill the chip, and eight products for one.  Narrower ones would gain up to 1.4 times, but their M came
 // out further from 64 bits than the CUDA cores': 384 x 8192 rows 0.9e-7 -> 1.7e-7, 512 x 2048 0.8e-7 -> 1.0e-7; at 768 2.6e-7 -> 1.8e-7)
 constexpr int SP_MIN_D = 768;
@@ -556,7 +614,8 @@ inline bool sp_takes(int64_t n, int d, bool f32) {
 }
 struct SpLayout {
   int64_t ldp;                                           // row length of all pieces: d rounded up to 64
-  size_t Xp, Sp, Rp, rs, colmax;
+  size_t Xp, Sp, Rp, rs, colmax, arrived;
+  size_t borrowed, borrowed_bytes;                       // what the rows' pieces borrow, all of it (0 bytes: they do not)
 };
 // Contexts that lay them out: those whose longest step takes them (a shorter one may not, a longer one always does).
 inline bool sp_layout_wanted(int d, int P, int64_t n_max, bool f32) { return P == 1 && sp_takes(n_max, d, f32); }
@@ -578,6 +637,9 @@ inline void sp_make_layout(int d, int64_t n, bool through_c, size_t scratch, siz
   L->Rp = take((size_t)(2 * 3 * d * L->ldp));
   L->rs = take(sizeof(float) * (size_t)n);
   L->colmax = take(sizeof(unsigned) * (size_t)d);
+  L->arrived = take(sizeof(unsigned) * SP_ARRIVED);
+  L->borrowed = scratch;
+  L->borrowed_bytes = borrow ? scratch_bytes : 0;
 }
 
 // (column, row, piece) map over `pieces` bf16 matrices of rows x cols, `piece` elements apart; box 64 columns x box_rows.
@@ -614,9 +676,29 @@ inline int sp_pick_bn(int64_t M, int64_t N, int pairs) {
 }
 inline int64_t sp_tiles(int64_t M, int64_t N, int bn) { return ((M + 255) / 256) * ((N + bn - 1) / bn); }
 
-template <int BN, int EPI>
+// The rotate product's last, partial round of tiles is shared out over k: its accumulators (512 terms each), tile by tile, go to the
+// pairs in runs of equal length, so that a pair works on parts of at most two tiles.  96 tiles on 74 pairs at d = 3072 are one round of
+// six accumulators and 22 tiles in runs of two, 8 accumulator times instead of 12.  Whole step over whole tiles -> this, us, fp32 rows:
+//   d = 1024  n = 200 51.3 -> 45.4, 512 55.6 -> 49.5;  2048  64 73.9 -> 49.3, 2048 167 -> 164, 4096 314 -> 301;  3072  64 101 -> 71, 512 131 -> 117,
+//   1000 217 -> 181, 4096 660 -> 627;  4096  200 170 -> 132, 2048 668 -> 632
+// Returns the length of a run: the tile's own length, with nothing shared (and a kernel without the code for it: 0.7 us of 24), where the
+// longest run would be no shorter.  `room`: bytes for the parts' sums, which fewer and longer runs need less of.
+inline int sp_share_tail(int64_t tiles, int pairs, int K, size_t room) {
+  const int r = (int)(tiles % pairs), chunks = (K + 8 * TC_BK - 1) / (8 * TC_BK);
+  if (r == 0 || 16 * r > SP_ARRIVED) return chunks;
+  for (int share = (r * chunks + pairs - 1) / pairs; share < chunks; ++share) {
+    const size_t runs = (size_t)(r * chunks + share - 1) / share, slots = chunks % share ? 2 : 1;
+    if (runs * slots * 256 * SP_ROT_BN * sizeof(float) <= room) return share;
+  }
+  return chunks;
+}
+
+template <int BN, int EPI, bool SHARE = false>
 inline int sp_launch_bn(int device, int pairs, cudaStream_t s, const CUtensorMap& a, const CUtensorMap& b, SpArgs g) {
-  auto kern = sp_gemm_kernel<BN, EPI>;
+  if constexpr (EPI != SP_EPI_ACCUM && !SHARE) {
+    if (g.share < (g.K + 8 * TC_BK - 1) / (8 * TC_BK)) return sp_launch_bn<BN, EPI, true>(device, pairs, s, a, b, g);
+  }
+  auto kern = sp_gemm_kernel<BN, EPI, SHARE>;
   static std::atomic<unsigned long long> attr_dev_mask{0};
   const unsigned long long dev_bit = 1ull << (device & 63);
   if (!(attr_dev_mask.load(std::memory_order_acquire) & dev_bit)) {
@@ -629,8 +711,14 @@ inline int sp_launch_bn(int device, int pairs, cudaStream_t s, const CUtensorMap
   g.stage_bytes = 3 * (TC_BM * TC_BK * 2) + (EPI == SP_EPI_ACCUM ? 1 : 3) * (BN / 2 * TC_BK * 2);
   g.n_stages = SP_RING_BYTES / g.stage_bytes < SP_STAGES_MAX ? SP_RING_BYTES / g.stage_bytes : SP_STAGES_MAX;
   const int64_t tiles = sp_tiles(g.M, g.N, BN);
+  int64_t items = tiles;
+  if (SHARE) {
+    const int chunks = (g.K + 8 * TC_BK - 1) / (8 * TC_BK);
+    g.whole = (int)(tiles - tiles % pairs);
+    items = g.whole ? g.whole : (tiles * chunks + g.share - 1) / g.share;      // (runs are no more than pairs)
+  }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(2 * (unsigned)(tiles < pairs ? tiles : pairs)); cfg.blockDim = dim3(SP_THREADS);
+  cfg.gridDim = dim3(2 * (unsigned)(items < pairs ? items : pairs)); cfg.blockDim = dim3(SP_THREADS);
   cfg.dynamicSmemBytes = SP_SMEM_BYTES; cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;

@@ -180,3 +180,25 @@ def test_a_feature_of_tiny_values(dtype):
     err = (m - xt.T @ s / math.sqrt(d)).abs()
     bound = (_unit(n) + (d / 32 + 9) * 2.0 ** -24) * (xt.abs().T @ s.abs()) / math.sqrt(d)
     assert (err <= bound + n * 2.0 ** -126 / math.sqrt(d)).all() and float(m[7].abs().max()) > 0.0
+
+
+# tiles of the last round shared out over k: all of them (fewer tiles than pairs) in parts of one accumulator, and in runs that straddle two
+# tiles; those behind a round of whole tiles; odd widths; a row of tiles that is mostly past the end; quantised targets
+@pytest.mark.parametrize("d,n,bits", [(1024, 300, 0), (1100, 257, 0), (2560, 1100, 0), (3072, 512, 0), (3001, 900, 0), (3072, 1000, 4), (4096, 70, 4)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_tiles_shared_out_over_k(d, n, bits, dtype):
+    if bits == 0:
+        test_signs_statistics_and_objective(d, n, torch.float32 if dtype == "f32" else torch.bfloat16)
+    else:
+        test_quantised_targets_and_strided_rows(d, n, "sym", bits, 0.0, dtype)
+    # the parts are added in their order, whichever comes last
+    x = _rand(d + n, n, d).to(torch.float32 if dtype == "f32" else torch.bfloat16)
+    r = torch.linalg.qr(_rand(7, d, d).double())[0].float().contiguous()
+    c = B.Context(d, n, in_dtype=dtype, mode="exact", quant_bits=bits)
+    c.set_R(r)
+    runs = []
+    for _ in range(6):
+        c.set_M(torch.zeros(d, d, device="cuda"), 0.0, 0)
+        c.step(x)
+        runs.append((c.get_objective(), c.get_M()))
+    assert all(j == runs[0][0] and torch.equal(m, runs[0][1]) for j, m in runs[1:])
