@@ -640,8 +640,7 @@ int update_impl(conqur_ctx* c) {
   }
   if (c->one_cluster) {
     NcArgs a{};
-    a.M = c->at<float>(c->L.M); a.R = c->at<float>(c->L.R); a.Xa = c->at<float>(c->L.Xa); a.Xb = c->at<float>(c->L.Xb);
-    a.E = c->at<float>(c->L.E); a.B = c->at<float>(c->L.B);
+    a.M = c->at<float>(c->L.M); a.R = c->at<float>(c->L.R);
     a.st = c->state();
     a.c = NsControlParams{c->at<SchedEntry>(c->L.sched), c->n_sched, c->n_lift_init, g.ns_max_steps, g.d, 0, g.orth_tol,
                           g.fro_tol, g.margin, g.lo_budget, 1.0 / (double)g.d, 0, 1.f / 2048.f};

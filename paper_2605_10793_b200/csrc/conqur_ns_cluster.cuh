@@ -2,16 +2,18 @@
 //
 // At these widths a launch of the iteration costs more than its work: 128^3 multiply-adds are 0.1 us of the chip, a launch with
 // the load latency of its operands about 6 us, and a step takes three of them and the control decision.  Sixteen CTAs of one
-// cluster share the 32 x 32 tiles of every product instead, a cluster barrier stands between the products, and every CTA takes the
-// decision itself from the same sums.  An element of a product is the same chain of multiply-adds as in the launches' kernels, and
-// the coefficients of a step depend on its place in the plan alone: the same bits wherever the start scale rounds to the same number
-// and the decisions agree.  (The squares behind these are added in another grouping, sixteen CTAs' instead of a block's per 1024
-// elements or per tile: double sums rounded to fp32, so a last bit may differ.)
-// What a step takes (d = 128, SM cycles, clock stamps): products 3 x 4.1 k (a warp's multiply-adds: two cycles each, 16 per k),
-// operands from the L2 6 k, barriers 6 k (the stores in front of them have to reach the L2), stores 2.7 k, norms and decision 1.8 k;
-// an update of eight steps 116 us.  Whole update of the statistics of 16 d rows once its step count is learnt, from an idle stream,
-// graph of launches -> this, us (one B200): d = 16, 8 steps 139 -> 57;  64, 9 steps 194 -> 106;  128, 9 steps 223 -> 136;  160, 12
-// steps 258 -> 200;  192 (three tiles a CTA) would take 291 in a row of updates where the launches take 237.
+// cluster share the 32 x 32 tiles of every product instead, and every CTA takes the decision itself from the same sums.  The matrices
+// live in shared memory: a finished tile is written straight into that of the CTAs whose next products read it, so that between
+// two products stands one cluster barrier with no trip to the L2 in front of or behind it.  An element of a product is the same chain
+// of multiply-adds as in the launches' kernels, and the coefficients of a step depend on its place in the plan alone: the same bits
+// wherever the start scale rounds to the same number and the decisions agree.  (The squares behind these are added in another
+// grouping, sixteen CTAs' instead of a block's per 1024 elements or per tile: double sums rounded to fp32, so a last bit may differ.)
+// What a step takes (d = 128, SM cycles, clock stamps): products 3.3 k to 4.2 k each (a warp's packed multiply-adds, two cycles each, and
+// its 16-byte reads share their time unevenly: 16 would do per k, 26 to 32 are taken), sending 1.3 k (32 KB a CTA at 25 bytes a cycle) and
+// the barrier behind it 1.7 k to 2 k, norms 0.6 k; the decision runs beside the next product.  22 k in all; 29 k with the matrices in the
+// L2 between the products.  Whole update of given statistics once its step count is learnt, from an idle stream, matrices in the L2 -> this,
+// us (one B200): d = 16, 4 steps 36 -> 26;  64, 4 steps 49 -> 36;  128, 4 steps 70 -> 61;  160, 5 steps 121 -> 110 (as a graph of launches the
+// first took 139, with 8 steps, and 128 with 9 steps 223).  192 (three tiles a CTA) has no room for its matrices.
 #pragma once
 #include <mutex>
 
@@ -20,107 +22,121 @@
 
 namespace conqur {
 
-constexpr int NC_MAX_D = 160;                    // one or two tiles a CTA; the operand slabs (d x 32) stay in shared memory
+constexpr int NC_MAX_TILES = 5;                  // tiles of 32 along a side: one or two of a product's 25 a CTA
+constexpr int NC_MAX_D = 32 * NC_MAX_TILES;
 constexpr int NC_THREADS = 256;
 constexpr int NC_CTAS = 16;
-constexpr int NC_WORK = 64;                       // threads that multiply: a 4 x 4 piece of the tile each
-constexpr int NC_LD = 36;                        // slab rows: 32 columns and 4 floats against bank conflicts
+constexpr int NC_WORK = 64;                      // threads that multiply: a 4 x 4 piece of the tile each
+constexpr int NC_LD_TILE = 36;                   // rows of the tile on its way out: 32 columns and 4 floats against bank conflicts
 
 struct NcArgs {
-  float *M, *R, *Xa, *Xb, *E, *B;
+  float *M, *R;
   DevState* st;
   NsControlParams c;
   int d, n_endgame;
   float prior_rel, inv_sqrt_d, margin;
 };
 
-inline int nc_smem_bytes(int d) { return (d + 3) / 4 * 4 * 2 * NC_LD * (int)sizeof(float); }
+// A matrix in shared memory: 32 T rows of 32 T columns and 4 floats against bank conflicts, zeros past d.  Up to four tiles a side three
+// of them fit: the next iterate then takes the residual's place and never one that another CTA still reads.  With five tiles there are
+// two, written in place, and a barrier more in front of each write.
+__host__ __device__ inline int nc_ld(int tiles) { return 32 * tiles + 4; }
+__host__ __device__ inline int nc_matrix_floats(int tiles) { return 32 * tiles * nc_ld(tiles); }
+__host__ __device__ inline int nc_matrices(int tiles) { return tiles <= 4 ? 3 : 2; }
+inline int nc_smem_bytes(int d) {
+  const int tiles = (d + 31) / 32;
+  return (nc_matrices(tiles) * nc_matrix_floats(tiles) + 32 * NC_LD_TILE) * (int)sizeof(float);
+}
 
 __device__ __forceinline__ void nc_cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Four elements P[r][c .. c+3] of a d x d matrix, zeros outside.  Other CTAs of the cluster write these: read from the L2.
-__device__ __forceinline__ float4 nc_ld4(const float* P, int d, int r, int c, bool vec) {
-  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (r >= d || c >= d) return v;
-  const float* p = P + (size_t)r * d + c;
-  if (vec) return __ldcg(reinterpret_cast<const float4*>(p));        // d % 4 == 0: whole pieces
-  v.x = __ldcg(p);
-  if (c + 1 < d) v.y = __ldcg(p + 1);
-  if (c + 2 < d) v.z = __ldcg(p + 2);
-  if (c + 3 < d) v.w = __ldcg(p + 3);
-  return v;
-}
-
-// Tile (m0, n0) of sum_k A(m, k) B(k, n), each sum one chain in the order of k as sg_mainloop's: thread t < NC_WORK returns rows
-// 4 (t / 8) .. +3 and columns 4 (t % 8) .. +3, and the slabs stay in shared memory (row k: A(m0 .. +31, k), then B(k, n0 .. +31)).
-// A(m, k) = A[k][m], or A[m][k] with TRANS.  A 16-byte read takes the shared memory four cycles a warp whatever is equal in it,
-// so two warps with 4 x 4 pieces (16 cycles per k, 16 multiply-adds each) are faster than four with 2 x 4 (32).
+// Tile (m0, n0) of sum_k A(m, k) B(k, n), each sum one chain in the order of k as sg_mainloop's; k runs to kp, d rounded up to four.
+// A(m, k) = A[k][m]: thread t < NC_WORK returns rows 4 (t / 8) .. +3; A[m][k] with TRANS: rows t / 8 + 8 i (neighbouring rows of A lie
+// four banks apart).  Columns 4 (t % 8) .. +3 either way.  A 16-byte read takes the shared memory four cycles a warp whatever is equal
+// in it and a multiply-add the lanes two, packed or not: two warps with 4 x 4 pieces in packed pairs need 16 cycles of either per k.
 template <bool TRANS>
-__device__ __forceinline__ void nc_tile(const float* A, const float* B, int d, int m0, int n0, bool vec, float* smem, float (&out)[4][4]) {
-  const int t = threadIdx.x, kp = (d + 3) / 4 * 4;
-  float* sa = smem;
-  float* sb = sa + kp * NC_LD;
-  for (int e0 = 0; e0 < kp * 8; e0 += 4 * NC_THREADS) {            // four pieces of either slab in flight per thread
-    float4 va[4], vb[4];
+__device__ __forceinline__ void nc_tile(const float* A, const float* B, int ld, int kp, int m0, int n0, float (&out)[4][4]) {
+  const int ty = (int)threadIdx.x >> 3, tx = (int)threadIdx.x & 7;
+  const float* pb = B + n0 + 4 * tx;
+  const float* pa = TRANS ? A + (m0 + ty) * ld : A + m0 + 4 * ty;
+  unsigned long long acc[4][2] = {};
+  auto step = [&](const float (&a)[4], const float4& b) {
+    const unsigned long long b0 = f32x2_pack(b.x, b.y), b1 = f32x2_pack(b.z, b.w);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const int e = e0 + i * NC_THREADS + t;
-      va[i] = vb[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (e < kp * 8) {
-        vb[i] = nc_ld4(B, d, e >> 3, n0 + (e & 7) * 4, vec);
-        va[i] = TRANS ? nc_ld4(A, d, m0 + (e & 31), (e >> 5) * 4, vec) : nc_ld4(A, d, e >> 3, m0 + (e & 7) * 4, vec);
-      }
+      const unsigned long long a2 = f32x2_pack(a[i], a[i]);
+      f32x2_fma(acc[i][0], a2, b0);
+      f32x2_fma(acc[i][1], a2, b1);
     }
+  };
+  // (four k ahead in registers: a warp has nobody to hide its loads behind.  The last ones read past the matrix, into its row padding or
+  // what lies behind it, and go unused.)
+  float4 a[2][4], b[2][4];
+  auto fetch = [&](int k, float4 (&fa)[4], float4 (&fb)[4]) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const int e = e0 + i * NC_THREADS + t;
-      if (e >= kp * 8) continue;
-      *reinterpret_cast<float4*>(sb + (e >> 3) * NC_LD + (e & 7) * 4) = vb[i];
-      if (TRANS) {
-        float* q = sa + (e >> 5) * 4 * NC_LD + (e & 31);
-        q[0] = va[i].x; q[NC_LD] = va[i].y; q[2 * NC_LD] = va[i].z; q[3 * NC_LD] = va[i].w;
-      } else {
-        *reinterpret_cast<float4*>(sa + (e >> 3) * NC_LD + (e & 7) * 4) = va[i];
-      }
+      fa[i] = *reinterpret_cast<const float4*>(TRANS ? pa + 8 * i * ld + k : pa + (k + i) * ld);
+      fb[i] = *reinterpret_cast<const float4*>(pb + (k + i) * ld);
     }
-  }
-  __syncthreads();
-  if (t < NC_WORK) {
-    const float* pa = sa + 4 * (t >> 3);
-    const float* pb = sb + 4 * (t & 7);
+  };
+  auto multiply = [&](const float4 (&fa)[4], const float4 (&fb)[4]) {
+    const float m[4][4] = {{fa[0].x, fa[0].y, fa[0].z, fa[0].w}, {fa[1].x, fa[1].y, fa[1].z, fa[1].w},
+                           {fa[2].x, fa[2].y, fa[2].z, fa[2].w}, {fa[3].x, fa[3].y, fa[3].z, fa[3].w}};
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) out[i][j] = 0.f;
-#pragma unroll 8
-    for (int k = 0; k < kp; ++k) {
-      const float4 a = *reinterpret_cast<const float4*>(pa + k * NC_LD), b = *reinterpret_cast<const float4*>(pb + k * NC_LD);
-      const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) out[i][j] = fmaf(av[i], bv[j], out[i][j]);
+    for (int j = 0; j < 4; ++j) {
+      const float col[4] = {TRANS ? m[0][j] : m[j][0], TRANS ? m[1][j] : m[j][1], TRANS ? m[2][j] : m[j][2], TRANS ? m[3][j] : m[j][3]};
+      step(col, fb[j]);
     }
+  };
+  fetch(0, a[0], b[0]);
+  int k = 0;
+  for (; k + 8 <= kp; k += 8) {
+    fetch(k + 4, a[1], b[1]);
+    multiply(a[0], b[0]);
+    fetch(k + 8, a[0], b[0]);
+    multiply(a[1], b[1]);
   }
+  if (k < kp) multiply(a[0], b[0]);
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      out[i][2 * j] = __uint_as_float((uint32_t)acc[i][j]);
+      out[i][2 * j + 1] = __uint_as_float((uint32_t)(acc[i][j] >> 32));
+    }
 }
 
-__device__ __forceinline__ void nc_st4(float* P, int d, int r, int c, const float (&v)[4], bool vec, bool mirror) {
-  if (r >= d || c >= d) return;
-  float* p = P + (size_t)r * d + c;
-  if (vec) {
-    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+// This thread's piece of a tile into the tile's buffer (row r0 + step i).
+__device__ __forceinline__ void nc_put(float* tile, int r0, int step, const float (&v)[4][4]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    *reinterpret_cast<float4*>(tile + (r0 + step * i) * NC_LD_TILE + 4 * ((int)threadIdx.x & 7)) = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
+}
+
+__device__ __forceinline__ uint32_t nc_smem_u32(const void* p) {
+  uint32_t a;
+  asm("{ .reg .u64 t; cvta.to.shared.u64 t, %1; cvt.u32.u64 %0, t; }" : "=r"(a) : "l"(p));
+  return a;
+}
+// The tile (or its transpose) to place (r, c) of `matrix` in every CTA of the mask, 16 bytes at a time: piece p of 256.  The cluster
+// barrier that follows publishes it.
+__device__ __forceinline__ void nc_send(const float* tile, bool transposed, float* matrix, int ld, int r, int c, uint32_t mask, int p) {
+  const int row = p >> 3, col = 4 * (p & 7);
+  float4 v;
+  if (transposed) {
+    v.x = tile[col * NC_LD_TILE + row]; v.y = tile[(col + 1) * NC_LD_TILE + row];
+    v.z = tile[(col + 2) * NC_LD_TILE + row]; v.w = tile[(col + 3) * NC_LD_TILE + row];
   } else {
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      if (c + j < d) p[j] = v[j];
+    v = *reinterpret_cast<const float4*>(tile + row * NC_LD_TILE + col);
   }
-  if (mirror) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      if (c + j < d) P[(size_t)(c + j) * d + r] = v[j];
+  const uint32_t here = nc_smem_u32(matrix + (32 * r + row) * ld + 32 * c + col);
+  for (; mask; mask &= mask - 1) {
+    uint32_t there;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(here), "r"(__ffs((int)mask) - 1));
+    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(there), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
   }
 }
 
@@ -129,8 +145,8 @@ __device__ __forceinline__ void nc_st4(float* P, int d, int r, int c, const floa
 __device__ __forceinline__ void nc_tell(double v, double* slots, int from) {
   const int lane = threadIdx.x & 31;
   if (lane < NC_CTAS) {
-    uint32_t a, r;
-    asm("{ .reg .u64 t; cvta.to.shared.u64 t, %1; cvt.u32.u64 %0, t; }" : "=r"(a) : "l"(slots + from));
+    uint32_t r;
+    const uint32_t a = nc_smem_u32(slots + from);
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(lane));
     asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(r), "d"(v) : "memory");
   }
@@ -150,14 +166,37 @@ __global__ void __launch_bounds__(NC_THREADS, 1) ns_cluster_kernel(const NcArgs 
   __shared__ double sums[2][NC_CTAS], maxima[2][NC_CTAS];     // what the CTAs tell each other, alternating
   __shared__ float coef[4];
   __shared__ int done_s;
+  __shared__ uint32_t by_col[NC_MAX_TILES], by_row[NC_MAX_TILES], by_factor[NC_MAX_TILES];    // who reads what, see below
   __shared__ SchedEntry sched[NS_SCHED_MAX];
-  const int cta = (int)blockIdx.x, t = threadIdx.x, d = g.d, tiles = (d + 31) / 32;
+  const int cta = (int)blockIdx.x, t = threadIdx.x, d = g.d, kp = (d + 3) / 4 * 4;
+  const int tiles = (d + 31) / 32, ld = nc_ld(tiles), sym_tiles = tiles * (tiles + 1) / 2;
+  const bool in_place = nc_matrices(tiles) == 2;
+  float* X = nc_smem;
+  float* E = X + nc_matrix_floats(tiles);
+  float* Bm = in_place ? E : E + nc_matrix_floats(tiles);
+  float* const tile = nc_smem + nc_matrices(tiles) * nc_matrix_floats(tiles);
   const size_t dd = (size_t)d * d;
-  const bool vec = (d & 3) == 0;
   DevState* st = g.st;
+  auto sym_coords = [&](int i, int& tm, int& tn) { tn = 0; while ((tn + 1) * (tn + 2) / 2 <= i) ++tn; tm = i - tn * (tn + 1) / 2; };
   for (int i = t; i < g.c.n_sched && i < NS_SCHED_MAX; i += NC_THREADS) sched[i] = g.c.sched[i];
   NsControlParams c = g.c;
   c.sched = sched;
+  for (int i = t; i < nc_matrices(tiles) * nc_matrix_floats(tiles) / 4; i += NC_THREADS)
+    reinterpret_cast<float4*>(nc_smem)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (t < tiles) {
+    // symmetric products read columns of X or of the residual; the last product rows of X and columns of the polynomial
+    uint32_t col = 0, row = 0, factor = 0;
+    for (int i = 0; i < sym_tiles; ++i) {
+      int tm, tn;
+      sym_coords(i, tm, tn);
+      if (t == tm || t == tn) col |= 1u << (i % NC_CTAS);
+    }
+    for (int i = 0; i < tiles * tiles; ++i) {
+      if (t == i / tiles) row |= 1u << (i % NC_CTAS);
+      if (t == i % tiles) factor |= 1u << (i % NC_CTAS);
+    }
+    by_col[t] = col; by_row[t] = row; by_factor[t] = factor;
+  }
   int slot = 0;
   auto sumsq = [&](float lam) {                  // ||M + lam R||_F^2
     double v = 0.0;
@@ -192,47 +231,54 @@ __global__ void __launch_bounds__(NC_THREADS, 1) ns_cluster_kernel(const NcArgs 
     st->ns_done = ok ? 0 : NS_DONE_FAILED;
     st->ns_steps_used = 0; st->ns_final_buf = 0; st->seg_x = 2; st->seg_e = 3; st->tau = 1.0f;
   }
+  // every CTA forms the whole first iterate: it reads most of it, and M and R are in the L2
+  if ((d & 3) == 0) {
 #pragma unroll 4
-  for (size_t i = (size_t)cta * NC_THREADS + t; i < dd; i += (size_t)NC_CTAS * NC_THREADS) g.Xa[i] = fmaf(lam, g.R[i], g.M[i]) * x0_scale;
-  nc_cluster_sync();
-  NsCtl ctl;                                     // thread 0 of every CTA takes the same decisions
-  if (t == 0) {
+    for (int i = t; i < d * (d / 4); i += NC_THREADS) {
+      const float4 m = reinterpret_cast<const float4*>(g.M)[i], q = reinterpret_cast<const float4*>(g.R)[i];
+      const int r = i / (d / 4), c4 = i - r * (d / 4);
+      *reinterpret_cast<float4*>(X + r * ld + 4 * c4) = make_float4(fmaf(lam, q.x, m.x) * x0_scale, fmaf(lam, q.y, m.y) * x0_scale,
+                                                                    fmaf(lam, q.z, m.z) * x0_scale, fmaf(lam, q.w, m.w) * x0_scale);
+    }
+  } else {
+#pragma unroll 4
+    for (int i = t; i < d * d; i += NC_THREADS) {
+      const int r = i / d;
+      X[r * ld + i - r * d] = fmaf(lam, g.R[i], g.M[i]) * x0_scale;
+    }
+  }
+  nc_cluster_sync();                             // (the state above is there for all, and nobody's matrices are still being cleared)
+  NsCtl ctl;                                     // one thread of every CTA, not one that multiplies, takes the same decisions
+  const bool decides = t == NC_WORK;
+  if (decides) {
     ns_ctl_load(ctl, st);
     done_s = ctl.ns_done;
   }
   __syncthreads();
-  const int sym_tiles = tiles * (tiles + 1) / 2;
-  auto sym_coords = [&](int i, int& tm, int& tn) { tn = 0; while ((tn + 1) * (tn + 2) / 2 <= i) ++tn; tm = i - tn * (tn + 1) / 2; };
-  const int r = 4 * (t >> 3), c4 = (t & 7) * 4;  // this thread's piece of a tile (t < NC_WORK)
-  const float* const slab_a = nc_smem;
-  const float* const slab_b = nc_smem + (d + 3) / 4 * 4 * NC_LD;
+  int tm = 0, tn = 0;                            // this CTA's tile of a symmetric product
+  const bool has_sym = cta < sym_tiles;
+  if (has_sym) sym_coords(cta, tm, tn);
+  const int r4 = 4 * (t >> 3), c4 = 4 * (t & 7); // this thread's piece of it (t < NC_WORK)
   float v[4][4];
   int k = 0, cur = 0;
   for (; done_s == 0; ++k, cur ^= 1) {
-    const float* X = cur ? g.Xb : g.Xa;
-    float* Xn = cur ? g.Xa : g.Xb;
     // E = X^T X - I and its norms
     float mx = 0.f;
     double sq = 0.0;
-    for (int i = cta; i < sym_tiles; i += NC_CTAS) {
-      int tm, tn;
-      sym_coords(i, tm, tn);
-      nc_tile<false>(X, X, d, tm * 32, tn * 32, vec, nc_smem, v);
-      if (t < NC_WORK) {
+    if (has_sym && t < NC_WORK) {
+      nc_tile<false>(X, X, ld, kp, tm * 32, tn * 32, v);
 #pragma unroll
-        for (int h = 0; h < 4; ++h) {
-          const int row = tm * 32 + r + h, col = tn * 32 + c4;
+      for (int h = 0; h < 4; ++h) {
+        const int row = tm * 32 + r4 + h, col = tn * 32 + c4;
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            if (row >= d || col + j >= d) continue;
-            if (row == col + j) v[h][j] -= 1.f;
-            mx = fmaxf(mx, fabsf(v[h][j]));
-            sq += (tm != tn ? 2.0 : 1.0) * ((double)v[h][j] * (double)v[h][j]);
-          }
-          nc_st4(g.E, d, row, col, v[h], vec, tm != tn);
+        for (int j = 0; j < 4; ++j) {
+          if (row >= d || col + j >= d) continue;
+          if (row == col + j) v[h][j] -= 1.f;
+          mx = fmaxf(mx, fabsf(v[h][j]));
+          sq += (tm != tn ? 2.0 : 1.0) * ((double)v[h][j] * (double)v[h][j]);
         }
       }
-      __syncthreads();                           // the slabs are free
+      nc_put(tile, r4, 1, v);
     }
     if (t < NC_WORK) {
       sq = warp_sum_d(sq);
@@ -244,8 +290,14 @@ __global__ void __launch_bounds__(NC_THREADS, 1) ns_cluster_kernel(const NcArgs 
       nc_tell(sq + redd[0], sums[slot], cta);
       nc_tell((double)fmaxf(mx, redf[0]), maxima[slot], cta);
     }
+    if (has_sym) {
+      nc_send(tile, false, E, ld, tm, tn, by_col[tn], t);
+      if (tm != tn) nc_send(tile, true, E, ld, tn, tm, by_col[tm], t);
+    }
     nc_cluster_sync();
-    if (t == 0) {
+    // B = beta2 E E + beta1 E, whose product does not wait for the decision
+    if (has_sym && t < NC_WORK) nc_tile<false>(E, E, ld, kp, tm * 32, tn * 32, v);
+    if (decides) {
       const double tsq = nc_total(sums[slot]);
       double tmx = 0.0;
 #pragma unroll
@@ -259,53 +311,63 @@ __global__ void __launch_bounds__(NC_THREADS, 1) ns_cluster_kernel(const NcArgs 
     slot ^= 1;
     __syncthreads();
     if (done_s != 0) break;
-    // B = beta2 E E + beta1 E
-    for (int i = cta; i < sym_tiles; i += NC_CTAS) {
-      int tm, tn;
-      sym_coords(i, tm, tn);
-      nc_tile<false>(g.E, g.E, d, tm * 32, tn * 32, vec, nc_smem, v);
-      if (t < NC_WORK) {
+    if (has_sym && t < NC_WORK) {
 #pragma unroll
-        for (int h = 0; h < 4; ++h) {
-          const int row = tm * 32 + r + h, col = tn * 32 + c4;
-          if (row >= d) continue;
+      for (int h = 0; h < 4; ++h)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) v[h][j] = fmaf(coef[2], v[h][j], coef[1] * slab_b[row * NC_LD + c4 + j]);     // E(row, col + j)
-          nc_st4(g.B, d, row, col, v[h], vec, tm != tn);
-        }
-      }
-      __syncthreads();
+        for (int j = 0; j < 4; ++j) v[h][j] = fmaf(coef[2], v[h][j], coef[1] * E[(tm * 32 + r4 + h) * ld + tn * 32 + c4 + j]);
+      nc_put(tile, r4, 1, v);
+    }
+    if (in_place) nc_cluster_sync(); else __syncthreads();
+    if (has_sym) {
+      nc_send(tile, false, Bm, ld, tm, tn, by_factor[tn], t);
+      if (tm != tn) nc_send(tile, true, Bm, ld, tn, tm, by_factor[tm], t);
     }
     nc_cluster_sync();
-    // X_next = X B + gamma X
-    for (int i = cta; i < tiles * tiles; i += NC_CTAS) {
-      const int tm = i / tiles, tn = i - tm * tiles;
-      nc_tile<true>(X, g.B, d, tm * 32, tn * 32, vec, nc_smem, v);
-      if (t < NC_WORK) {
+    // X_next = X B + gamma X, into the residual's place (nobody reads it any more) or X's
+    float* const Xn = in_place ? X : E;
+    float w[4][4];                               // a second tile's, where there are more than sixteen
+    auto next = [&](int f, float (&o)[4][4]) {
+      const int fm = f / tiles, fn = f - fm * tiles;
+      nc_tile<true>(X, Bm, ld, kp, fm * 32, fn * 32, o);
 #pragma unroll
-        for (int h = 0; h < 4; ++h) {
-          const int row = tm * 32 + r + h, col = tn * 32 + c4;
-          if (row >= d) continue;
+      for (int h = 0; h < 4; ++h)
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (col + j < d) v[h][j] = fmaf(coef[0], slab_a[(col + j) * NC_LD + r + h], v[h][j]);                   // X(row, col + j)
-          nc_st4(Xn, d, row, col, v[h], vec, false);
-        }
-      }
+        for (int j = 0; j < 4; ++j) o[h][j] = fmaf(coef[0], X[(fm * 32 + (t >> 3) + 8 * h) * ld + fn * 32 + c4 + j], o[h][j]);
+    };
+    const int f1 = cta + NC_CTAS;
+    if (t < NC_WORK) {
+      if (cta < tiles * tiles) { next(cta, v); nc_put(tile, t >> 3, 8, v); }
+      if (f1 < tiles * tiles) next(f1, w);
+    }
+    if (in_place) nc_cluster_sync(); else __syncthreads();
+    if (cta < tiles * tiles) {
+      const int fm = cta / tiles, fn = cta - fm * tiles;
+      nc_send(tile, false, Xn, ld, fm, fn, by_col[fn] | by_row[fm], t);
+    }
+    if (f1 < tiles * tiles) {
+      const int fm = f1 / tiles, fn = f1 - fm * tiles;
       __syncthreads();
+      if (t < NC_WORK) nc_put(tile, t >> 3, 8, w);
+      __syncthreads();
+      nc_send(tile, false, Xn, ld, fm, fn, by_col[fn] | by_row[fm], t);
     }
     nc_cluster_sync();
+    if (!in_place) { E = X; X = Xn; }
   }
-  // accept or reject (see ns_commit_kernel, ns_commit_state_kernel)
+  // accept or reject (see ns_commit_kernel, ns_commit_state_kernel): each CTA holds the rows of X that its tiles of the last product read
   if (done_s == NS_DONE_CONVERGED) {
-    const float* X = cur ? g.Xb : g.Xa;
-#pragma unroll 4
-    for (size_t i = (size_t)cta * NC_THREADS + t; i < dd; i += (size_t)NC_CTAS * NC_THREADS) {
-      g.R[i] = __ldcg(X + i);
-      g.M[i] = 0.f;
+    for (int f = cta; f < tiles * tiles; f += NC_CTAS) {
+      const int row = (f / tiles) * 32 + (t >> 3), col = (f % tiles) * 32 + c4;
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (row < d && col + j < d) {
+          g.R[(size_t)row * d + col + j] = X[row * ld + col + j];
+          g.M[(size_t)row * d + col + j] = 0.f;
+        }
     }
   }
-  if (cta == 0 && t == 0) {
+  if (cta == 0 && decides) {
     ns_ctl_store(ctl, st);
     ns_commit_state(st, g.n_endgame);
   }
