@@ -371,9 +371,10 @@ int step_pieces(conqur_ctx* c, const TIn* X, int64_t n, int64_t ld) {
   float* rnorm = c->at<float>(c->L.rnorm);
   float* rs = c->at<float>(L.rs);
   double* part = c->at<double>(c->L.part_d);
+  unsigned* ranges = g.quant_bits || g.diagnostics ? c->at<unsigned>(c->L.rowmax) : nullptr;      // rows' maxima, then minima
   const int64_t xpiece = n * L.ldp;                       // the pieces of this step's rows lie one behind another
   sp_stage_kernel<TIn, true><<<(unsigned)n, 128, 0, c->stream>>>(X, n, d, ld, rnorm, rs, sp_ptr(c, L.Xp), L.ldp, xpiece, c->state(),
-                                                                 c->at<unsigned>(L.arrived));
+                                                                 c->at<unsigned>(L.arrived), ranges, ranges ? ranges + g.n_max : nullptr);
   CQ_LAUNCHED(c, K_ROWNORM);
   const int bm = sp_pick_bn(d, d, c->sp_pairs);
   CUtensorMap xk, rk, xm, sm;
@@ -398,10 +399,8 @@ int step_pieces(conqur_ctx* c, const TIn* X, int64_t n, int64_t ld) {
     c->prof.count(K_ROTATE);
     per_problem = (int)(16 * sp_tiles(n, d, SP_ROT_BN));
   } else {
-    a.rowmax = c->at<unsigned>(c->L.rowmax); a.rowmin = a.rowmax + g.n_max;
+    a.rowmax = ranges; a.rowmin = ranges + g.n_max;
     a.outF = c->at<float>(c->L.C); a.ldo = d;
-    CQ_CUDA(cudaMemsetAsync(a.rowmax, 0, sizeof(unsigned) * n, c->stream));
-    CQ_CUDA(cudaMemsetAsync(a.rowmin, 0xff, sizeof(unsigned) * n, c->stream));
     rc = sp_launch_bn<SP_ROT_BN, SP_EPI_ROTATE_Q>(c->device, c->sp_pairs, c->stream, xk, rk, a);
     if (rc) return rc;
     c->prof.count(K_ROTATE);
@@ -410,14 +409,12 @@ int step_pieces(conqur_ctx* c, const TIn* X, int64_t n, int64_t ld) {
     CQ_LAUNCHED(c, K_OTHER);
     per_problem = cdiv(n, 8);
   }
-  finalize_step_kernel<<<1, 256, 0, c->stream>>>(c->state(), part, per_problem, n, 1.0 / std::sqrt((double)d), pdiag,
-                                                 pdiag ? cdiv(n, 8) : 0);
-  CQ_LAUNCHED(c, K_OTHER);
   SpArgs m{};
+  m.step = StepSums{part, per_problem, n, 1.0 / std::sqrt((double)d), pdiag, pdiag ? cdiv(n, 8) : 0};
   m.M = d; m.N = d; m.K = (int)n; m.st = c->state();
   m.outF = c->at<float>(c->L.M); m.ldo = d;
   sp_stage_kernel<TIn, false><<<(unsigned)n, 128, 0, c->stream>>>(X, n, d, ld, rnorm, rs, sp_ptr(c, L.Xp), L.ldp, xpiece, c->state(),
-                                                                  nullptr);
+                                                                  nullptr, nullptr, nullptr);
   CQ_LAUNCHED(c, K_ROWNORM);
   rc = bm == 256 ? sp_launch_bn<256, SP_EPI_ACCUM>(c->device, c->sp_pairs, c->stream, xm, sm, m)
                  : sp_launch_bn<128, SP_EPI_ACCUM>(c->device, c->sp_pairs, c->stream, xm, sm, m);
@@ -440,7 +437,9 @@ int step_exact(conqur_ctx* c, const TIn* X, int64_t n, int64_t ld, int64_t pstri
   float* C = c->at<float>(c->L.C);
   double* part = c->at<double>(c->L.part_d);
   const int64_t c_ps = (int64_t)g.n_max * d;
-  rownorm_kernel<TIn><<<dim3(cdiv(n, 8), P), 256, 0, c->stream>>>(X, n, d, ld, pstride, rnorm, g.n_max, st, 1);
+  unsigned* rowmax = g.quant_bits || g.diagnostics ? c->at<unsigned>(c->L.rowmax) : nullptr;
+  unsigned* rowmin = rowmax ? rowmax + g.n_max * g.P : nullptr;
+  rownorm_kernel<TIn><<<dim3(cdiv(n, 8), P), 256, 0, c->stream>>>(X, n, d, ld, pstride, rnorm, g.n_max, st, 1, rowmax, rowmin);
   CQ_LAUNCHED(c, K_ROWNORM);
   const int rt = sg_pick(n, d, P, c->L.max_partials);
   int per_problem;
@@ -455,10 +454,6 @@ int step_exact(conqur_ctx* c, const TIn* X, int64_t n, int64_t ld, int64_t pstri
     });
     CQ_LAUNCHED(c, K_ROTATE);
   } else {
-    unsigned* rowmax = c->at<unsigned>(c->L.rowmax);
-    unsigned* rowmin = rowmax + g.n_max * g.P;
-    CQ_CUDA(cudaMemsetAsync(rowmax, 0, sizeof(unsigned) * g.n_max * P, c->stream));
-    CQ_CUDA(cudaMemsetAsync(rowmin, 0xff, sizeof(unsigned) * g.n_max * P, c->stream));
     sg_with_tile(rt, [&](auto tile) {
       using Tile = decltype(tile);
       rotate_target_exact_kernel<Tile, TIn, true><<<sg_grid<Tile>(n, d, P), Tile::NT, 0, c->stream>>>(
@@ -470,9 +465,7 @@ int step_exact(conqur_ctx* c, const TIn* X, int64_t n, int64_t ld, int64_t pstri
     CQ_LAUNCHED(c, K_OTHER);
     per_problem = cdiv(n, 8);
   }
-  finalize_step_kernel<<<P, 256, 0, c->stream>>>(st, part, per_problem, n, 1.0 / std::sqrt((double)d), pdiag,
-                                                 pdiag ? cdiv(n, 8) : 0);
-  CQ_LAUNCHED(c, K_OTHER);
+  const StepSums sums{part, per_problem, n, 1.0 / std::sqrt((double)d), pdiag, pdiag ? cdiv(n, 8) : 0};
   const int S = c->L.acc_splits;
   sg_with_tile(sg_pick(d, d, (int64_t)P * S), [&](auto tile) {
     using Tile = decltype(tile);
@@ -483,9 +476,11 @@ int step_exact(conqur_ctx* c, const TIn* X, int64_t n, int64_t ld, int64_t pstri
   CQ_LAUNCHED(c, K_ACCUM);
   if (S > 1) {
     splitk_reduce_add_kernel<<<dim3(ew_blocks((int64_t)d * d), P), 256, 0, c->stream>>>(
-        c->at<float>(c->L.M) + pdd, c->at<float>(c->L.splitk), (int64_t)d * d, S);
-    CQ_LAUNCHED(c, K_OTHER);
+        c->at<float>(c->L.M) + pdd, c->at<float>(c->L.splitk), (int64_t)d * d, S, st, sums);
+  } else {
+    finalize_step_kernel<<<P, 256, 0, c->stream>>>(st, sums);
   }
+  CQ_LAUNCHED(c, K_OTHER);
   return CONQUR_OK;
 }
 

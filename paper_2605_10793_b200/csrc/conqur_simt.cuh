@@ -112,7 +112,8 @@ __device__ __forceinline__ RowQuant row_quant(const QuantSpec q, float vmax, flo
 template <typename TIn>
 __global__ void __launch_bounds__(256) rownorm_kernel(const TIn* __restrict__ X, int64_t n, int d, int64_t ld,
                                                       int64_t problem_stride, float* __restrict__ rnorm,
-                                                      int64_t rnorm_stride, DevState* st, int state_stride_problems) {
+                                                      int64_t rnorm_stride, DevState* st, int state_stride_problems,
+                                                      unsigned* rowmax = nullptr, unsigned* rowmin = nullptr) {
   const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   const int p = blockIdx.y;
@@ -143,6 +144,7 @@ __global__ void __launch_bounds__(256) rownorm_kernel(const TIn* __restrict__ X,
       if (!(ss == 0.f)) atomicOr(&s->status_flags, STATUS_FLAG_NONFINITE);
     }
     rnorm[(int64_t)p * rnorm_stride + row] = r;
+    if (rowmax) { rowmax[(int64_t)p * rnorm_stride + row] = 0u; rowmin[(int64_t)p * rnorm_stride + row] = ~0u; }   // the row's range starts empty
   }
 }
 
@@ -549,40 +551,61 @@ __global__ void __launch_bounds__(Tile::NT, Tile::MINB) accumulate_exact_kernel(
   }
 }
 
+// What a step adds to a problem's running sums: its objective partials (fixed order; none where `partials` is null), the Section-4
+// diagnostics' (null: none) and token counts.
+struct StepSums {
+  const double* partials;
+  int count;                                     // partials of a problem
+  int64_t n;                                     // rows of the step
+  double inv_sqrt_d;
+  const double* diag;
+  int diag_blocks;
+};
+// Takes them over, 256 threads (tid 0 .. 255) with eight doubles of shared memory; sync: a barrier of just these threads.  A launch of its
+// own for this took 3 to 4 us of a step, and clearing the rows' ranges of a quantised one by two fills as much, so a kernel that runs
+// behind the targets' takes them over beside its own work and the row norms' kernel clears the ranges (step of 2048 x 4096 209 -> 206 us,
+// 32 per-head problems of 4001 rows 83 -> 80.5 with the calls around it; quantised steps of a few hundred rows 116 -> 109).
+template <typename Sync>
+__device__ __forceinline__ void finalize_step(DevState* s, int p, const StepSums& f, int tid, double* red, Sync sync) {
+  auto total = [&](const double* part, int count) -> double {      // valid in thread 0
+    double v = 0.0;
+    if (part)
+      for (int i = tid; i < count; i += 256) v += part[i];
+    v = warp_sum_d(v);
+    if ((tid & 31) == 0) red[tid >> 5] = v;
+    sync();
+    double r = 0.0;
+    if (tid < 32) r = warp_sum_d(tid < 8 ? red[tid] : 0.0);
+    sync();
+    return r;
+  };
+  const double tot = total(f.partials ? f.partials + (int64_t)p * f.count : nullptr, f.count);
+  double dsum[4] = {0.0, 0.0, 0.0, 0.0};
+  if (f.diag)
+    for (int k = 0; k < 4; ++k) dsum[k] = total(f.diag + ((int64_t)p * 4 + k) * f.diag_blocks, f.diag_blocks);
+  if (tid == 0) {
+    s->J += tot * f.inv_sqrt_d;
+    s->N += f.n - s->step_skipped;
+    s->n_skipped += s->step_skipped;
+    s->step_skipped = 0;
+    if (f.diag) { s->diag_pr += dsum[0]; s->diag_rho += dsum[1]; s->diag_qnum += dsum[2]; s->diag_qden += dsum[3]; }
+  }
+}
+static __global__ void finalize_step_kernel(DevState* st, const StepSums f) {
+  __shared__ double red[8];
+  finalize_step(st + blockIdx.x, (int)blockIdx.x, f, (int)threadIdx.x, red, [] { __syncthreads(); });
+}
+
+// M += its splits' partials in order; the first block of a problem finalizes the step besides.
 static __global__ void splitk_reduce_add_kernel(float* __restrict__ M, const float* __restrict__ partial, int64_t dd,
-                                         int splits) {
+                                         int splits, DevState* st, const StepSums f) {
+  __shared__ double red[8];
   const int p = blockIdx.y;
+  if (blockIdx.x == 0) finalize_step(st + p, p, f, (int)threadIdx.x, red, [] { __syncthreads(); });
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < dd; i += (int64_t)gridDim.x * blockDim.x) {
     float v = M[p * dd + i];
     for (int s = 0; s < splits; ++s) v += partial[((int64_t)p * splits + s) * dd + i];
     M[p * dd + i] = v;
-  }
-}
-
-// Adds the step's objective partials (fixed order; none when `partials` is null) and token counts to the running sums.
-static __global__ void finalize_step_kernel(DevState* st, const double* __restrict__ partials, int per_problem, int64_t n,
-                                     double inv_sqrt_d, const double* __restrict__ part_diag = nullptr, int diag_blocks = 0) {
-  const int p = blockIdx.x;
-  __shared__ double red[8];
-  double v = 0.0;
-  if (partials)
-    for (int i = threadIdx.x; i < per_problem; i += 256) v += partials[(int64_t)p * per_problem + i];
-  const double tot = block_sum_d<256>(v, red);
-  double dsum[4] = {0.0, 0.0, 0.0, 0.0};
-  if (part_diag) {
-    for (int k = 0; k < 4; ++k) {
-      double w = 0.0;
-      for (int i = threadIdx.x; i < diag_blocks; i += 256) w += part_diag[((int64_t)p * 4 + k) * diag_blocks + i];
-      dsum[k] = block_sum_d<256>(w, red);
-    }
-  }
-  if (threadIdx.x == 0) {
-    DevState* s = st + p;
-    s->J += tot * inv_sqrt_d;
-    s->N += n - s->step_skipped;
-    s->n_skipped += s->step_skipped;
-    s->step_skipped = 0;
-    if (part_diag) { s->diag_pr += dsum[0]; s->diag_rho += dsum[1]; s->diag_qnum += dsum[2]; s->diag_qden += dsum[3]; }
   }
 }
 

@@ -42,6 +42,7 @@ struct SpArgs {
   __nv_bfloat16* outS; long long lds;                    // targets
   const float* rs;                                       // 1, or 0 for rows that are left out
   unsigned *rowmax, *rowmin;
+  StepSums step;                                         // ACCUM: what the step adds to the running sums
   double* part_d;                                        // objective partials: sixteen per tile (a warp's of either CTA)
   DevState* st;
   // rotate: tiles from `whole` on are shared out over k, `share` accumulators of them in a row to each pair (see sp_share_tail)
@@ -54,6 +55,7 @@ struct SpAux {
   uint64_t full[SP_STAGES_MAX], empty[SP_STAGES_MAX], tfull[2], tempty[2];
   uint32_t tmem_base;
   int abort_flag;
+  double red_d[8];
 };
 static_assert(sizeof(SpAux) <= 1024, "reserved behind the ring");
 
@@ -298,6 +300,9 @@ sp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     uint8_t* stg = smem + SP_RING_BYTES + 1024 + ew * 4096;
     const uint32_t tempty0 = ptx::mapa_u32(ptx::smem_u32(&aux->tempty[0]), 0);
     const uint32_t t_lane = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * HALF);
+    // (these warps have nothing to add up yet)
+    if (MN && worker == 0 && rank == 1)
+      finalize_step(g.st, 0, g.step, (int)threadIdx.x - 128, aux->red_d, [] { asm volatile("bar.sync 1, 256;" ::: "memory"); });
     uint32_t n_acc = 0;
     bool ok = true;
     Item w;
@@ -446,7 +451,8 @@ constexpr int SP_ARRIVED = 2048;                         // counters: sixteen wa
 template <typename TIn, bool GRID>
 __global__ void __launch_bounds__(128) sp_stage_kernel(const TIn* __restrict__ X, int64_t n, int d, int64_t ld, float* __restrict__ rnorm,
                                                        float* __restrict__ rs, __nv_bfloat16* __restrict__ Xp, int64_t ldp,
-                                                       int64_t piece, DevState* st, unsigned* arrived) {
+                                                       int64_t piece, DevState* st, unsigned* arrived, unsigned* rowmax,
+                                                       unsigned* rowmin) {
   if (GRID && blockIdx.x == 0)                           // (the rotate product that follows counts its shared tiles' parts there)
     for (int i = threadIdx.x; i < SP_ARRIVED; i += 128) arrived[i] = 0u;
   __shared__ float part[8];
@@ -488,6 +494,7 @@ __global__ void __launch_bounds__(128) sp_stage_kernel(const TIn* __restrict__ X
       }
       rnorm[row] = r;
       rs[row] = good ? 1.f : 0.f;
+      if (rowmax) { rowmax[row] = 0u; rowmin[row] = ~0u; }
     }
   } else {
     r = rnorm[row];

@@ -263,6 +263,7 @@ struct TcGemmArgs {
   const double* x2_part; int n_x2;   // residual: the sums of squares the last next-iterate product left (n_x2 == 0: tau is in the state)
   DevState* st;
   int check_done;
+  StepSums step;                // accumulate: what the step adds to the running sums
 };
 
 // Tiles (TM x BN) of a symmetric product, column by column: column tn holds the row tiles 0 .. (tn+1)*BN/TM - 1.
@@ -662,6 +663,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (worker == 0 && rank == 0 && ew == 0 && lane == 0) g.st->tau = c_tau;      // (for the decision that follows this launch)
       }
     }
+    // (these warps have no accumulator to read yet)
+    if (EPI == TC_EPI_ACCUM && worker == 0 && rank == (PAIR ? 1u : 0u))
+      finalize_step(g.st, 0, g.step, (int)threadIdx.x - 64, aux->red_d, [] { asm volatile("bar.sync 1, 256;" ::: "memory"); });
     int local = 0;
     bool ok = true;
     const uint32_t tempty_addr0 = PAIR ? ptx::mapa_u32(ptx::smem_u32(&aux->tempty[0]), 0) : 0u;
@@ -892,7 +896,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 template <typename TIn, int W>
 __global__ void __launch_bounds__(256) rownorm_stage_kernel(const TIn* __restrict__ X, int64_t n, int d, int64_t ld,
                                                             float* __restrict__ rnorm,
-                                                            __nv_bfloat16* __restrict__ Xs, DevState* st) {
+                                                            __nv_bfloat16* __restrict__ Xs, DevState* st,
+                                                            unsigned* rowmax, unsigned* rowmin) {
   __shared__ float part_ss[8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t row = (int64_t)blockIdx.x * (8 / W) + warp / W;
@@ -976,6 +981,7 @@ __global__ void __launch_bounds__(256) rownorm_stage_kernel(const TIn* __restric
       if (!(ss == 0.f)) atomicOr(&st->status_flags, STATUS_FLAG_NONFINITE);
     }
     rnorm[row] = good ? 1.0f / sqrtf(ss) : 0.f;
+    if (rowmax) { rowmax[row] = 0u; rowmin[row] = ~0u; }                // (quantised targets: the row's range starts empty)
   }
 }
 
@@ -1410,13 +1416,15 @@ inline TcGemmArgs tc_args(const TcHost& h, int M, int N, int K) {
 inline int tc_stage(TcHost& h, cudaStream_t s, const void* X, int in_dtype, int64_t n, int64_t ld, int64_t row0) {
   const int d = h.d;
   __nv_bfloat16* Xs = reinterpret_cast<__nv_bfloat16*>(h.ws + h.L.Xs) + row0 * d;
+  unsigned* rowmax = h.quant_bits || h.diagnostics ? h.rowmax + row0 : nullptr;
+  unsigned* rowmin = rowmax ? rowmax + h.n_max : nullptr;
   auto launch = [&](auto w) {                              // W warps a row: at most 4096 elements each
     constexpr int W = decltype(w)::value;
     const int rb = (int)((n + 8 / W - 1) / (8 / W));
     if (in_dtype == CONQUR_F32)
-      rownorm_stage_kernel<float, W><<<rb, 256, 0, s>>>(static_cast<const float*>(X), n, d, ld, h.rnorm + row0, Xs, h.st);
+      rownorm_stage_kernel<float, W><<<rb, 256, 0, s>>>(static_cast<const float*>(X), n, d, ld, h.rnorm + row0, Xs, h.st, rowmax, rowmin);
     else
-      rownorm_stage_kernel<__nv_bfloat16, W><<<rb, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(X), n, d, ld, h.rnorm + row0, Xs, h.st);
+      rownorm_stage_kernel<__nv_bfloat16, W><<<rb, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(X), n, d, ld, h.rnorm + row0, Xs, h.st, rowmax, rowmin);
   };
   if (d <= 4096) launch(std::integral_constant<int, 1>{});
   else if (d <= 8192) launch(std::integral_constant<int, 2>{});
@@ -1451,8 +1459,6 @@ inline int tc_process(TcHost& h, cudaStream_t s, int64_t n) {
     per_problem = tc_part_slots(h, tc_variant(h, d, tc_small_step(n, d, d)), (int)n, d, 0);
   } else {
     unsigned* rowmin = h.rowmax + h.n_max;
-    if (cudaMemsetAsync(h.rowmax, 0, sizeof(unsigned) * n, s) != cudaSuccess) return CONQUR_ERR_CUDA;
-    if (cudaMemsetAsync(rowmin, 0xff, sizeof(unsigned) * n, s) != cudaSuccess) return CONQUR_ERR_CUDA;
     g.outF = h.Y; g.ldo = d; g.rowmax = h.rowmax; g.rowmin = rowmin;
     rc = tc_launch_n<false, true, TC_EPI_ROTATE_Q>(h, s, tmXs_k, h.tmRb_mn, g);
     if (rc) return rc;
@@ -1462,10 +1468,8 @@ inline int tc_process(TcHost& h, cudaStream_t s, int64_t n) {
     if (h.prof) h.prof->count(K_OTHER);
     per_problem = rb;
   }
-  finalize_step_kernel<<<1, 256, 0, s>>>(h.st, h.part_d, per_problem, n, isd, h.diagnostics ? h.part_diag : nullptr, rb);
-  if (cudaGetLastError() != cudaSuccess) return CONQUR_ERR_CUDA;
-  if (h.prof) h.prof->count(K_OTHER);
   TcGemmArgs a = tc_args(h, d, d, (int)n);
+  a.step = StepSums{h.part_d, per_problem, n, isd, h.diagnostics ? h.part_diag : nullptr, rb};
   a.outF = h.M; a.ldo = d;
   return tc_launch_n<true, true, TC_EPI_ACCUM>(h, s, tmXs_mn, tmCp_mn, a);
 }

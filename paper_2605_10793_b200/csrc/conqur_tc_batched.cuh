@@ -869,9 +869,12 @@ inline int tcb_refresh_objective(TcHost& h, cudaStream_t s) {
   return CONQUR_OK;
 }
 
-// M[p] += partial[p * S + 0] + ... + partial[p * S + S - 1], in that order.  grid (16, problems), 256 threads.
-static __global__ void tcb_sum_partials_kernel(float* __restrict__ M, const float* __restrict__ part, int S) {
+// M[p] += partial[p * S + 0] + ... + partial[p * S + S - 1], in that order.  grid (16, problems), 256 threads; the first block of a
+// problem finalizes the step besides.
+static __global__ void tcb_sum_partials_kernel(float* __restrict__ M, const float* __restrict__ part, int S, DevState* st, const StepSums f) {
+  __shared__ double red[8];
   const int p = blockIdx.y;
+  if (blockIdx.x == 0) finalize_step(st + p, p, f, (int)threadIdx.x, red, [] { __syncthreads(); });
   const int i = (blockIdx.x * 256 + threadIdx.x) * 4;
   float4 m = *reinterpret_cast<const float4*>(M + (size_t)p * TCB_D * TCB_D + i);
   for (int sp = 0; sp < S; ++sp) {
@@ -975,12 +978,9 @@ inline int tcb_step(TcHost& h, cudaStream_t s, const void* X, int in_dtype, int6
   if (timed) { cudaEventRecord(rec.e1, s); h.prof->open.push_back(rec); }
   if (cudaGetLastError() != cudaSuccess) return CONQUR_ERR_CUDA;
   if (h.prof) h.prof->count(K_ROTATE);
-  if (S > 1) {
-    tcb_sum_partials_kernel<<<dim3(16, np), 256, 0, s>>>(g.M, g.Mpart, S);
-    if (cudaGetLastError() != cudaSuccess) return CONQUR_ERR_CUDA;
-    if (h.prof) h.prof->count(K_OTHER);
-  }
-  finalize_step_kernel<<<np, 256, 0, s>>>(g.st, h.qs.bits > 0 ? h.part_d : nullptr, S * TCB_PARTS, n, 1.0 / std::sqrt((double)TCB_D));
+  const StepSums sums{h.qs.bits > 0 ? h.part_d : nullptr, S * TCB_PARTS, n, 1.0 / std::sqrt((double)TCB_D), nullptr, 0};
+  if (S > 1) tcb_sum_partials_kernel<<<dim3(16, np), 256, 0, s>>>(g.M, g.Mpart, S, g.st, sums);
+  else finalize_step_kernel<<<np, 256, 0, s>>>(g.st, sums);
   if (cudaGetLastError() != cudaSuccess) return CONQUR_ERR_CUDA;
   if (h.prof) h.prof->count(K_OTHER);
   return CONQUR_OK;
