@@ -253,12 +253,10 @@ __global__ void clear_flags_kernel(DevState* st, int P, int* agg) {
   for (int i = threadIdx.x; i < P; i += blockDim.x) st[i].status_flags = 0;
   if (threadIdx.x == 0) *agg = 0;
 }
-__global__ void arm_check_kernel(DevState* st, int P) {
-  for (int i = threadIdx.x; i < P; i += blockDim.x) { st[i].ns_done = 0; st[i].ns_steps_used = 0; st[i].seg_e = 3; }
-}
-// max|G - I| and sum (G - I)^2 over the partials of a residual product (one block).  st: state of the tensor-core product
-// that left them, or null.
-__global__ void check_reduce_kernel(const DevState* st, const float* pmax, const double* psq, int n, double* out) {
+// max|G - I| and sum (G - I)^2 over the partials of a residual product (one block); the problems' states as before an update's first
+// step.  st: state of the tensor-core product that left the partials, or null.
+__global__ void check_reduce_kernel(const DevState* st, const float* pmax, const double* psq, int n, double* out, DevState* all, int P) {
+  for (int i = threadIdx.x; i < P; i += 256) ns_arm_check(all + i);
   __shared__ double redd[8];
   __shared__ float redf[8];
   float mx = 0.f;
@@ -914,7 +912,7 @@ extern "C" int conqur_destroy(conqur_ctx* ctx) {
 // any entry is; infinite where the tensor-core product of state `st` gave up).
 static int check_read(conqur_ctx* c, const DevState* st, int n, double (&h)[2]) {
   double* out = result_area(c, sizeof(h), c->at<double>(c->L.obj_out));
-  check_reduce_kernel<<<1, 256, 0, c->stream>>>(st, c->at<float>(c->L.part_f), c->at<double>(c->L.part_d), n, out);
+  check_reduce_kernel<<<1, 256, 0, c->stream>>>(st, c->at<float>(c->L.part_f), c->at<double>(c->L.part_d), n, out, c->state(), c->cfg.P);
   CQ_LAUNCHED(c, K_OTHER);
   return take_results(c, out, h, sizeof(h));
 }
@@ -924,8 +922,16 @@ extern "C" int conqur_set_R(conqur_ctx* c, const float* R_dev) {
   const Cfg& g = c->cfg;
   const int64_t dd = (int64_t)g.d * g.d;
   { const int frc = flush_pending(c); if (frc) return frc; }      // queued rows belong to the rotation being replaced
-  arm_check_kernel<<<1, 256, 0, c->stream>>>(c->state(), g.P);
-  CQ_LAUNCHED(c, K_OTHER);
+  if (c->one_cluster) {                                            // narrow: product, decision and copy in one kernel
+    double* out = result_area(c, 2 * sizeof(double), c->at<double>(c->L.obj_out));
+    const int lrc = nc_check_launch(NcCheckArgs{R_dev, c->at<float>(c->L.R), c->state(), out, g.d}, c->stream);
+    if (lrc) return lrc;
+    c->prof.count(K_OTHER);
+    double h[2];
+    const int rc = take_results(c, out, h, sizeof(h));
+    if (rc) return rc;
+    return nc_accepts(h[0], h[1]) ? CONQUR_OK : CONQUR_ERR_NOT_ORTHOGONAL_INPUT;
+  }
   bool decided = false;
   const bool aligned = (reinterpret_cast<uintptr_t>(R_dev) & 15) == 0;
   // The decision max|R^T R - I| <= 1e-3 on the tensor cores first, by the three-pass product of R's bf16 pair.  How far an
@@ -947,7 +953,7 @@ extern "C" int conqur_set_R(conqur_ctx* c, const float* R_dev) {
     if (g.P > 1) {
       rc = tcb_check(c->tc, c->stream, R_dev, pf, pd);
     } else {
-      split_bf16_kernel<<<ew_blocks(dd / 4), 256, 0, c->stream>>>(R_dev, tc_iterate_ptr(c->tc, 0), dd, dd);
+      split_bf16_kernel<<<ew_blocks(dd / 4), 256, 0, c->stream>>>(R_dev, tc_iterate_ptr(c->tc, 0), dd, dd, c->state());
       CQ_LAUNCHED(c, K_OTHER);
       rc = tc_ns_residual(c->tc, c->stream, 0);
     }
@@ -968,7 +974,7 @@ extern "C" int conqur_set_R(conqur_ctx* c, const float* R_dev) {
     const int rc = check_read(c, nullptr, ns_exact_parts(c) * g.P, h);
     if (rc) return rc;
     // (the maximum drops NaN, the sum keeps it)
-    if (!((float)h[0] <= 1e-3f) || !std::isfinite(h[1])) return CONQUR_ERR_NOT_ORTHOGONAL_INPUT;
+    if (!nc_accepts(h[0], h[1])) return CONQUR_ERR_NOT_ORTHOGONAL_INPUT;
   }
   if (g.mode == CONQUR_TC_BF16 && aligned) return tc_take_R(c->tc, c->stream, R_dev);
   CQ_CUDA(cudaMemcpyAsync(c->at<float>(c->L.R), R_dev, sizeof(float) * dd * g.P, cudaMemcpyDeviceToDevice, c->stream));

@@ -374,6 +374,81 @@ __global__ void __launch_bounds__(NC_THREADS, 1) ns_cluster_kernel(const NcArgs 
   nc_cluster_sync();                             // no CTA leaves while another may still write into its shared memory
 }
 
+// conqur_set_R's check of one narrow matrix, whose product is the launches' (the same chains), with the copy of what is accepted: one
+// kernel where the product, the reduction of its partials and, behind the host's decision, the copy took three launches (whole call at
+// d = 128 26 -> 21 us).
+inline int nc_check_smem_bytes(int d) {              // (a matrix, and four rows that the product's last reads fetch past it)
+  const int tiles = (d + 31) / 32;
+  return (nc_matrix_floats(tiles) + 4 * nc_ld(tiles)) * (int)sizeof(float);
+}
+struct NcCheckArgs { const float* src; float* R; DevState* st; double* out; int d; };
+// max|R^T R - I| (which drops NaN) and the sum of squares (which keeps it)
+__host__ __device__ inline bool nc_accepts(double mx, double sq) { return (float)mx <= 1e-3f && sq - sq == 0.0; }
+
+__global__ void __launch_bounds__(NC_THREADS, 1) nc_check_kernel(const NcCheckArgs g) {
+  extern __shared__ __align__(16) float nc_smem[];
+  __shared__ double redd[2];
+  __shared__ float redf[2];
+  __shared__ double sums[NC_CTAS], maxima[NC_CTAS];
+  const int cta = (int)blockIdx.x, t = threadIdx.x, d = g.d, kp = (d + 3) / 4 * 4;
+  const int tiles = (d + 31) / 32, ld = nc_ld(tiles), sym_tiles = tiles * (tiles + 1) / 2;
+  float* X = nc_smem;
+  for (int i = t; i < nc_matrix_floats(tiles); i += NC_THREADS) {
+    const int r = i / ld, col = i - r * ld;
+    X[i] = r < d && col < d ? g.src[(size_t)r * d + col] : 0.f;
+  }
+  __syncthreads();
+  float mx = 0.f, v[4][4];
+  double sq = 0.0;
+  if (cta < sym_tiles && t < NC_WORK) {
+    int tn = 0;
+    while ((tn + 1) * (tn + 2) / 2 <= cta) ++tn;
+    const int tm = cta - tn * (tn + 1) / 2;
+    nc_tile<false>(X, X, ld, kp, tm * 32, tn * 32, v);
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const int row = tm * 32 + 4 * (t >> 3) + h, col = tn * 32 + 4 * (t & 7);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (row >= d || col + j >= d) continue;
+        if (row == col + j) v[h][j] -= 1.f;
+        mx = fmaxf(mx, fabsf(v[h][j]));
+        sq += (tm != tn ? 2.0 : 1.0) * ((double)v[h][j] * (double)v[h][j]);
+      }
+    }
+  }
+  if (t < NC_WORK) {
+    sq = warp_sum_d(sq);
+    mx = warp_max(mx);
+    if ((t & 31) == 0) { redd[t >> 5] = sq; redf[t >> 5] = mx; }
+  }
+  nc_cluster_sync();                             // (the sums of this CTA, and every CTA runs before anything is written into its memory)
+  if (t < 32) {
+    nc_tell(redd[0] + redd[1], sums, cta);
+    nc_tell((double)fmaxf(redf[0], redf[1]), maxima, cta);
+  }
+  nc_cluster_sync();
+  const double tsq = nc_total(sums);
+  double tmx = 0.0;
+#pragma unroll
+  for (int i = 0; i < NC_CTAS; ++i) tmx = fmax(tmx, maxima[i]);
+  if (cta == 0 && t == 0) {
+    ns_arm_check(g.st);
+    g.out[0] = tmx; g.out[1] = tsq;
+  }
+  if (nc_accepts(tmx, tsq))
+    for (int i = cta * NC_THREADS + t; i < d * d; i += NC_CTAS * NC_THREADS) g.R[i] = X[i / d * ld + i % d];
+}
+inline int nc_check_launch(const NcCheckArgs& a, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(NC_CTAS); cfg.blockDim = dim3(NC_THREADS); cfg.dynamicSmemBytes = (size_t)nc_check_smem_bytes(a.d); cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = NC_CTAS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, nc_check_kernel, a) == cudaSuccess ? CONQUR_OK : CONQUR_ERR_CUDA;
+}
+
 // Whether a cluster of NC_CTAS can be resident on the device (asked once per device, under a lock).
 inline bool nc_available(int dev) {
   static std::mutex mu;
@@ -390,6 +465,8 @@ inline bool nc_available(int dev) {
     cfg.attrs = at; cfg.numAttrs = 1;
     const bool yes = cudaFuncSetAttribute(ns_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, nc_smem_bytes(NC_MAX_D)) == cudaSuccess &&
                      cudaFuncSetAttribute(ns_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                     cudaFuncSetAttribute(nc_check_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, nc_check_smem_bytes(NC_MAX_D)) == cudaSuccess &&
+                     cudaFuncSetAttribute(nc_check_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
                      cudaOccupancyMaxActiveClusters(&n, ns_cluster_kernel, &cfg) == cudaSuccess && n > 0;
     if (!yes) cudaGetLastError();
     known[dev] = yes ? 1 : 2;

@@ -630,7 +630,7 @@ __global__ void __launch_bounds__(Tile::NT, Tile::MINB) ns_gemm_exact_kernel(con
   static_assert(Tile::TN % Tile::TM == 0, "see the mirrored tiles");
   const int p = blockIdx.z;
   const DevState* s = st + p;
-  if (s->ns_done) return;
+  if (D != nullptr && s->ns_done) return;                                 // (a check is no step of an iteration)
   const int64_t off = (int64_t)p * d * d;
   const int m0 = blockIdx.y * Tile::TM, n0 = blockIdx.x * Tile::TN;
   const int64_t slot = ((int64_t)p * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
@@ -1029,6 +1029,8 @@ static __global__ void ns_commit_kernel(DevState* st, const float* __restrict__ 
     M[p * dd + i] = 0.f;
   }
 }
+// ... and after the check of a rotation that conqur_set_R was given: as before the first step, with the product of all three passes.
+__device__ __forceinline__ void ns_arm_check(DevState* s) { s->ns_done = 0; s->ns_steps_used = 0; s->seg_e = 3; }
 // The problem's state after an update (one thread).
 __device__ __forceinline__ void ns_commit_state(DevState* s, int n_endgame) {
   ns_adapt_lift_plan(s, n_endgame, s->ns_done == NS_DONE_CONVERGED);

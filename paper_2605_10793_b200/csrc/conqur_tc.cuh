@@ -985,9 +985,10 @@ __global__ void __launch_bounds__(256) rownorm_stage_kernel(const TIn* __restric
   }
 }
 
-// fp32 -> bf16 (hi only, lo_elems == 0) or the two-term split [hi; lo]
+// fp32 -> bf16 (hi only, lo_elems == 0) or the two-term split [hi; lo].  check: state to arm for a residual product that follows (or null).
 __global__ void split_bf16_kernel(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst, int64_t count,
-                                  int64_t lo_elems) {
+                                  int64_t lo_elems, DevState* check = nullptr) {
+  if (check != nullptr && blockIdx.x == 0 && threadIdx.x == 0) ns_arm_check(check);
   for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; i < count;
        i += (int64_t)gridDim.x * blockDim.x * 4) {
     const float4 t = *reinterpret_cast<const float4*>(src + i);

@@ -92,3 +92,38 @@ def test_same_steps_from_the_same_scale_give_the_same_bits(d, kind):
         # sqrt of a sum of d^2 squares in double, whatever its grouping, then one rounding to fp32
         assert abs(s1 - s2) <= 2.0 ** -23 * s2 and n1 == n2
         assert s1 != s2 or torch.equal(r1, r2)
+
+
+@pytest.mark.parametrize("d", WIDTHS)
+def test_set_R_accepts_and_refuses_as_the_launches_do(d):
+    """Columns off norm 1 by just under and just over the limit, one entry off, NaN and infinities; a matrix off 16-byte boundaries."""
+    q = torch.linalg.qr(_rand(d, d, d).double())[0].float().contiguous()
+    off = torch.empty(d * d + 1, device="cuda")[1:].view(d, d)
+    off.copy_(q)
+    cases = [q, off]
+    for e in (4.99e-4, 4.998e-4, 4.9985e-4, 5e-4, 5.01e-4):
+        w = q.clone()
+        w[:, d // 2] *= 1.0 + e
+        cases.append(w)
+    for bad in (float("nan"), float("inf"), 1e20):
+        w = q.clone()
+        w[d - 1, 0] = bad
+        cases.append(w)
+    ctx = [B.Context(d, 16, in_dtype="f32", mode="exact", debug_flags=f) for f in (0, B.CONQUR_DEBUG_NO_GRAPH)]
+    refused = 0
+    for w in cases:
+        took = []
+        for c in ctx:
+            c.set_R(q)
+            try:
+                c.set_R(w)
+                took.append(True)
+                assert torch.equal(c.get_R(), w)
+            except B.ConqurError:
+                took.append(False)
+                assert torch.equal(c.get_R(), q)
+        assert took[0] == took[1]
+        refused += not took[0]
+    # 5.01e-4 and the three bad ones for certain, 4.99e-4 never; the others lie within the entries' rounding (twice 2^-23 of a norm) and the
+    # product's (d 2^-24) of the limit and go the same way for both, whichever that is
+    assert 4 <= refused <= 7 and took[0] is False
