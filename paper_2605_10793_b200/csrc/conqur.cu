@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
+#include <chrono>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -144,7 +146,8 @@ bool make_layout(int d, const conqur_config* c, Layout* L) {
 // Page-locked host memory that a context's synchronising calls exchange small results through: kernels write (or read) it
 // directly, where a copy through pageable memory costs a node of its own and about 8 us more.  Slots go back to a small pool
 // (allocating and freeing one takes ~0.1 ms and may wait for the device); at most MAIL_KEPT idle ones are held.
-constexpr size_t MAIL_BYTES = 32768;
+constexpr size_t MAIL_BYTES = 32768;                    // results; behind them the word that says they are there
+constexpr size_t MAIL_ALLOC = MAIL_BYTES + 64;
 constexpr size_t MAIL_KEPT = 8;
 struct RelaxedCapture {                                 // (a stream that another thread captures is not disturbed by the allocation)
   cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
@@ -161,7 +164,8 @@ struct MailPool {
     }
     RelaxedCapture relaxed;
     void* p = nullptr;
-    if (cudaHostAlloc(&p, MAIL_BYTES, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    if (cudaHostAlloc(&p, MAIL_ALLOC, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    std::memset(p, 0, MAIL_ALLOC);
     return p;
   }
   void give(void* p) {
@@ -183,7 +187,8 @@ struct conqur_ctx {
   Layout L;
   char* ws;
   cudaStream_t stream;
-  unsigned char* mail = nullptr;   // MAIL_BYTES of page-locked memory, used between a call's launch and its synchronise only
+  unsigned char* mail = nullptr;   // page-locked memory, used between a call's launch and its wait only
+  unsigned mail_seq = 0;           // what the last such call waited for
   std::vector<int64_t> tokens;   // per problem: rows enqueued since the last update
   std::vector<int64_t> tokens_at_update;   // ... as they stood when the last update was enqueued (restored if it is rejected)
   int64_t last_n;            // rows per problem of the last step (for debug_get_signs)
@@ -234,8 +239,18 @@ int cuda_fail(const char* what, cudaError_t e) {
     (c)->prof.count(cls);            \
   } while (0)
 
+// ... where several blocks work: `count` says how many have finished; the last one tells, so that all of the kernel's work is done.
+__device__ __forceinline__ void post_mail_last(const MailPost& post, unsigned* count) {
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  if (blockIdx.x == 0) __threadfence_system(); else __threadfence();      // (the first block's results go to the host)
+  if (atomicAdd(count, 1u) != gridDim.x - 1) return;
+  *count = 0u;
+  post_mail(post);
+}
+
 // The latched status of all problems (one block) and, where J is given, their sums: what a read-out copies to the host.
-__global__ void read_out_kernel(const DevState* st, int P, int* agg, double* J, long long* N) {
+__global__ void read_out_kernel(const DevState* st, int P, int* agg, double* J, long long* N, const MailPost post) {
   __shared__ int all;
   if (threadIdx.x == 0) all = 0;
   __syncthreads();
@@ -247,7 +262,7 @@ __global__ void read_out_kernel(const DevState* st, int P, int* agg, double* J, 
   f = __reduce_or_sync(0xffffffffu, f);
   if ((threadIdx.x & 31) == 0 && f) atomicOr(&all, f);
   __syncthreads();
-  if (threadIdx.x == 0) *agg = all;
+  if (threadIdx.x == 0) { *agg = all; post_mail(post); }
 }
 __global__ void clear_flags_kernel(DevState* st, int P, int* agg) {
   for (int i = threadIdx.x; i < P; i += blockDim.x) st[i].status_flags = 0;
@@ -255,7 +270,8 @@ __global__ void clear_flags_kernel(DevState* st, int P, int* agg) {
 }
 // max|G - I| and sum (G - I)^2 over the partials of a residual product (one block); the problems' states as before an update's first
 // step.  st: state of the tensor-core product that left the partials, or null.
-__global__ void check_reduce_kernel(const DevState* st, const float* pmax, const double* psq, int n, double* out, DevState* all, int P) {
+__global__ void check_reduce_kernel(const DevState* st, const float* pmax, const double* psq, int n, double* out, DevState* all, int P,
+                                    const MailPost post) {
   for (int i = threadIdx.x; i < P; i += 256) ns_arm_check(all + i);
   __shared__ double redd[8];
   __shared__ float redf[8];
@@ -265,15 +281,17 @@ __global__ void check_reduce_kernel(const DevState* st, const float* pmax, const
   const double tsq = block_sum_d<256>(sq, redd);
   const float tmx = block_max_f<256>(mx, redf);
   const bool gave_up = st != nullptr && (st->status_flags & STATUS_FLAG_TIMEOUT) != 0;   // the product is not to be trusted
-  if (threadIdx.x == 0) { out[0] = (double)tmx; out[1] = gave_up ? (double)INFINITY : tsq; }
+  if (threadIdx.x == 0) { out[0] = (double)tmx; out[1] = gave_up ? (double)INFINITY : tsq; post_mail(post); }
 }
 __global__ void export_sums_kernel(const DevState* st, double* J, long long* N, int P) {
   for (int i = threadIdx.x; i < P; i += blockDim.x) { J[i] = st[i].J; N[i] = st[i].N; }
 }
 // dst = src * f; block 0 besides takes the sums over (J given; set_M) or reads the latched status of all problems out (agg
 // given; get_M, get_R), which the copies of the other blocks hide.
+template <bool POST>
 __global__ void __launch_bounds__(256) scale_copy_kernel(const float* __restrict__ src, float* __restrict__ dst, int64_t count, float f,
-                                                         DevState* st, int P, int* agg, const double* J, const long long* N) {
+                                                         DevState* st, int P, int* agg, const double* J, const long long* N,
+                                                         const MailPost post, unsigned* count_done) {
   __shared__ int all;
   if (blockIdx.x == 0) {
     if (threadIdx.x == 0) all = 0;
@@ -299,6 +317,7 @@ __global__ void __launch_bounds__(256) scale_copy_kernel(const float* __restrict
   } else {
     for (int64_t i = first; i < count; i += step) dst[i] = src[i] * f;
   }
+  if (POST) post_mail_last(post, count_done);
 }
 
 int flags_to_status(int f) {
@@ -314,31 +333,63 @@ int ew_blocks(int64_t count) { return (int)std::min<int64_t>(148 * 8, (count + 2
 template <typename T> T* result_area(conqur_ctx* c, size_t bytes, T* dev) {
   return c->mail && bytes <= MAIL_BYTES ? reinterpret_cast<T*>(c->mail) : dev;
 }
-// Synchronise and take them over.
-int take_results(conqur_ctx* c, const void* area, void* host, size_t bytes) {
-  if (area != c->mail) CQ_CUDA(cudaMemcpyAsync(host, area, bytes, cudaMemcpyDeviceToHost, c->stream));
+template <typename T> bool in_mail(const conqur_ctx* c, const T* area) { return reinterpret_cast<const unsigned char*>(area) == c->mail; }
+// What a call's last kernel is given to tell that they are there.
+MailPost mail_post(conqur_ctx* c, bool posted) {
+  return posted ? MailPost{reinterpret_cast<unsigned*>(c->mail + MAIL_BYTES), ++c->mail_seq} : MailPost{nullptr, 0};
+}
+// Wait for everything enqueued; posted: its last kernel tells.  Its word is seen 2 us before the driver reports the kernel's end (an empty
+// kernel 10.3 -> 8.7 us from launch to return), so the call looks out for it as long as a short one takes; then, and for whatever
+// failed, the driver is asked.
+int wait_stream(conqur_ctx* c, bool posted) {
+  if (posted) {
+    const volatile unsigned* flag = reinterpret_cast<const volatile unsigned*>(c->mail + MAIL_BYTES);
+    const auto t0 = std::chrono::steady_clock::now();
+    do {
+      for (int i = 0; i < 64; ++i) {
+        if (*flag == c->mail_seq) { std::atomic_thread_fence(std::memory_order_acquire); return CONQUR_OK; }
+#if defined(__x86_64__)
+        __builtin_ia32_pause();
+#endif
+      }
+    } while (std::chrono::steady_clock::now() - t0 < std::chrono::microseconds(200));
+  }
   CQ_CUDA(cudaStreamSynchronize(c->stream));
-  if (area == c->mail) std::memcpy(host, area, bytes);
   return CONQUR_OK;
 }
+// Wait for the results and take them over.
+int take_results(conqur_ctx* c, const void* area, void* host, size_t bytes, bool posted) {
+  if (!in_mail(c, area)) CQ_CUDA(cudaMemcpyAsync(host, area, bytes, cudaMemcpyDeviceToHost, c->stream));
+  const int rc = wait_stream(c, posted);
+  if (rc == CONQUR_OK && in_mail(c, area)) std::memcpy(host, area, bytes);
+  return rc;
+}
+// Whether a copy of this many blocks tells: with the code that finds the last of them it takes 40 registers instead of 32, and 5 us longer
+// for 64 MB; up to 2 MB the word gains more (32 per-head problems: set_M, step and the read-outs 80.6 -> 77.7 us).
+bool copy_posts(const conqur_ctx* c, const void* area, int blocks) { return in_mail(c, area) && blocks <= 4 * 148; }
+unsigned* blocks_done(const conqur_ctx* c) { return c->at<unsigned>(c->L.flags_agg) + 2; }      // (zero between launches)
 
 // Synchronise and return the latched device status (not cleared).
 int sync_status(conqur_ctx* c) {
   int* agg = result_area(c, sizeof(int), c->at<int>(c->L.flags_agg));
-  read_out_kernel<<<1, c->cfg.P > 32 ? 256 : 32, 0, c->stream>>>(c->state(), c->cfg.P, agg, nullptr, nullptr);
+  read_out_kernel<<<1, c->cfg.P > 32 ? 256 : 32, 0, c->stream>>>(c->state(), c->cfg.P, agg, nullptr, nullptr,
+                                                                    mail_post(c, in_mail(c, agg)));
   CQ_LAUNCHED(c, K_OTHER);
   int f = 0;
-  const int rc = take_results(c, agg, &f, sizeof(int));
+  const int rc = take_results(c, agg, &f, sizeof(int), in_mail(c, agg));
   return rc ? rc : flags_to_status(f);
 }
 // dst = src * f over all problems' matrices, then synchronise and return the latched device status.
 int copy_out(conqur_ctx* c, const float* src, float* dst, float f) {
   const int64_t count = (int64_t)c->cfg.d * c->cfg.d * c->cfg.P;
   int* agg = result_area(c, sizeof(int), c->at<int>(c->L.flags_agg));
-  scale_copy_kernel<<<ew_blocks((count + 3) / 4), 256, 0, c->stream>>>(src, dst, count, f, c->state(), c->cfg.P, agg, nullptr, nullptr);
+  const int blocks = ew_blocks((count + 3) / 4);
+  const bool posted = copy_posts(c, agg, blocks);
+  (posted ? scale_copy_kernel<true> : scale_copy_kernel<false>)<<<blocks, 256, 0, c->stream>>>(src, dst, count, f, c->state(), c->cfg.P, agg, nullptr, nullptr,
+                                                   mail_post(c, posted), blocks_done(c));
   CQ_LAUNCHED(c, K_OTHER);
   int flags = 0;
-  const int rc = take_results(c, agg, &flags, sizeof(int));
+  const int rc = take_results(c, agg, &flags, sizeof(int), posted);
   return rc ? rc : flags_to_status(flags);
 }
 
@@ -894,6 +945,7 @@ extern "C" int conqur_init(conqur_ctx** out, int32_t d, const conqur_config* cfg
   }
   if (cudaStreamSynchronize(c->stream) != cudaSuccess) return fail(CONQUR_ERR_CUDA);   // coef is a local
   c->mail = static_cast<unsigned char*>(mail_pool().take());   // (none: results are copied)
+  if (c->mail) std::memcpy(&c->mail_seq, c->mail + MAIL_BYTES, sizeof(unsigned));        // (where its last user left off)
   *out = c;
   return CONQUR_OK;
 }
@@ -912,9 +964,10 @@ extern "C" int conqur_destroy(conqur_ctx* ctx) {
 // any entry is; infinite where the tensor-core product of state `st` gave up).
 static int check_read(conqur_ctx* c, const DevState* st, int n, double (&h)[2]) {
   double* out = result_area(c, sizeof(h), c->at<double>(c->L.obj_out));
-  check_reduce_kernel<<<1, 256, 0, c->stream>>>(st, c->at<float>(c->L.part_f), c->at<double>(c->L.part_d), n, out, c->state(), c->cfg.P);
+  check_reduce_kernel<<<1, 256, 0, c->stream>>>(st, c->at<float>(c->L.part_f), c->at<double>(c->L.part_d), n, out, c->state(), c->cfg.P,
+                                              mail_post(c, in_mail(c, out)));
   CQ_LAUNCHED(c, K_OTHER);
-  return take_results(c, out, h, sizeof(h));
+  return take_results(c, out, h, sizeof(h), in_mail(c, out));
 }
 
 extern "C" int conqur_set_R(conqur_ctx* c, const float* R_dev) {
@@ -924,11 +977,11 @@ extern "C" int conqur_set_R(conqur_ctx* c, const float* R_dev) {
   { const int frc = flush_pending(c); if (frc) return frc; }      // queued rows belong to the rotation being replaced
   if (c->one_cluster) {                                            // narrow: product, decision and copy in one kernel
     double* out = result_area(c, 2 * sizeof(double), c->at<double>(c->L.obj_out));
-    const int lrc = nc_check_launch(NcCheckArgs{R_dev, c->at<float>(c->L.R), c->state(), out, g.d}, c->stream);
+    const int lrc = nc_check_launch(NcCheckArgs{R_dev, c->at<float>(c->L.R), c->state(), out, mail_post(c, in_mail(c, out)), g.d}, c->stream);
     if (lrc) return lrc;
     c->prof.count(K_OTHER);
     double h[2];
-    const int rc = take_results(c, out, h, sizeof(h));
+    const int rc = take_results(c, out, h, sizeof(h), in_mail(c, out));
     if (rc) return rc;
     return nc_accepts(h[0], h[1]) ? CONQUR_OK : CONQUR_ERR_NOT_ORTHOGONAL_INPUT;
   }
@@ -1068,10 +1121,10 @@ extern "C" int conqur_get_objective(conqur_ctx* c, double* J_sum, int64_t* n_tok
   double* dJ = result_area(c, bytes, c->at<double>(c->L.part_d));
   long long* dN = reinterpret_cast<long long*>(dJ + P);
   int* df = reinterpret_cast<int*>(dN + P);
-  read_out_kernel<<<1, P > 32 ? 256 : 32, 0, c->stream>>>(c->state(), P, df, dJ, dN);
+  read_out_kernel<<<1, P > 32 ? 256 : 32, 0, c->stream>>>(c->state(), P, df, dJ, dN, mail_post(c, in_mail(c, dJ)));
   CQ_LAUNCHED(c, K_OTHER);
   std::vector<unsigned char> h(bytes);
-  const int rc = take_results(c, dJ, h.data(), bytes);
+  const int rc = take_results(c, dJ, h.data(), bytes, in_mail(c, dJ));
   if (rc) return rc;
   std::memcpy(J_sum, h.data(), 8 * (size_t)P);
   std::memcpy(n_tokens, h.data() + 8 * (size_t)P, 8 * (size_t)P);
@@ -1130,10 +1183,13 @@ extern "C" int conqur_set_M(conqur_ctx* c, const float* M_dev, const double* J_s
   std::memcpy(to, J_sum, 8 * (size_t)P);
   std::memcpy(to + 8 * (size_t)P, n_tokens, 8 * (size_t)P);
   if (to != c->mail) CQ_CUDA(cudaMemcpyAsync(dJ, to, bytes, cudaMemcpyHostToDevice, c->stream));
-  scale_copy_kernel<<<ew_blocks((count + 3) / 4), 256, 0, c->stream>>>(M_dev, c->at<float>(c->L.M), count, (float)std::sqrt((double)c->cfg.d),
-                                                                       c->state(), P, nullptr, dJ, reinterpret_cast<const long long*>(dJ + P));
+  const int blocks = ew_blocks((count + 3) / 4);
+  const bool posted = copy_posts(c, dJ, blocks);
+  (posted ? scale_copy_kernel<true> : scale_copy_kernel<false>)<<<blocks, 256, 0, c->stream>>>(M_dev, c->at<float>(c->L.M), count, (float)std::sqrt((double)c->cfg.d),
+                                                   c->state(), P, nullptr, dJ, reinterpret_cast<const long long*>(dJ + P),
+                                                   mail_post(c, posted), blocks_done(c));
   CQ_LAUNCHED(c, K_OTHER);
-  CQ_CUDA(cudaStreamSynchronize(c->stream));
+  { const int wrc = wait_stream(c, posted); if (wrc) return wrc; }
   for (int p = 0; p < P; ++p) c->tokens[p] = n_tokens[p];
   return CONQUR_OK;
 }
@@ -1346,21 +1402,29 @@ extern "C" int conqur_fold_weight(const float* W_dev, int64_t ldw, int32_t rows,
     DevState* st = reinterpret_cast<DevState*>(base);
     __nv_bfloat16* Ws = reinterpret_cast<__nv_bfloat16*>(base + 512);
     __nv_bfloat16* Rs = reinterpret_cast<__nv_bfloat16*>(base + 512 + align_up((size_t)rows * cols * 4));
-    CQ_CUDA(cudaMemsetAsync(st, 0, sizeof(DevState), s));
+    // the product's status: in page-locked memory (cleared and read here), or in the scratch where there is none
+    void* const slot = mail_pool().take();
+    struct GiveBack { void* p; ~GiveBack() { mail_pool().give(p); } } give_back{slot};
+    if (slot) {
+      st = static_cast<DevState*>(slot);
+      std::memset(slot, 0, sizeof(DevState));
+    } else {
+      CQ_CUDA(cudaMemsetAsync(st, 0, sizeof(DevState), s));
+    }
     split_bf16_2d_kernel<<<ew_blocks((int64_t)rows * cols / 4), 256, 0, s>>>(W_dev, ldw, rows, cols, Ws);
-    CQ_LAUNCH_CHECK();
     split_bf16_2d_kernel<<<ew_blocks((int64_t)d * d / 4), 256, 0, s>>>(R_dev, d, d, d, Rs);
-    CQ_LAUNCH_CHECK();
-    int rc;
-    if (side == CONQUR_FOLD_INPUT)     // out (rows x d) = W R: A = W, K-major; B(n, k) = R[k][n], MN-major
-      rc = tc_plain_gemm(Ws, Rs, out_dev, rows, d, d, 0, 1, 1, st, s, ldo);
-    else                               // out (d x cols) = R^T W: A(m, k) = R[k][m] and B(n, k) = W[k][n], both MN-major
-      rc = tc_plain_gemm(Rs, Ws, out_dev, d, cols, d, 1, 1, 1, st, s, ldo);
+    int rc = cudaGetLastError() == cudaSuccess ? CONQUR_OK : CONQUR_ERR_CUDA;
+    if (rc == CONQUR_OK)
+      rc = side == CONQUR_FOLD_INPUT
+               ? tc_plain_gemm(Ws, Rs, out_dev, rows, d, d, 0, 1, 1, st, s, ldo)      // out (rows x d) = W R: A = W, K-major; B(n, k) = R[k][n], MN-major
+               : tc_plain_gemm(Rs, Ws, out_dev, d, cols, d, 1, 1, 1, st, s, ldo);     // out (d x cols) = R^T W: A(m, k) = R[k][m] and B(n, k) = W[k][n], both MN-major
+    int flags = 0;
+    if (rc == CONQUR_OK && !slot) CQ_CUDA(cudaMemcpyAsync(&flags, &st->status_flags, sizeof(int), cudaMemcpyDeviceToHost, s));
+    const cudaError_t e = cudaStreamSynchronize(s);     // (whatever happened: the kernels enqueued may still write into the slot)
     if (rc) return rc;
-    DevState h;
-    CQ_CUDA(cudaMemcpyAsync(&h, st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
-    CQ_CUDA(cudaStreamSynchronize(s));
-    return flags_to_status(h.status_flags);
+    CQ_CUDA(e);
+    if (slot) flags = st->status_flags;
+    return flags_to_status(flags);
   }
   int dev = 0;
   TcDevFacts facts;

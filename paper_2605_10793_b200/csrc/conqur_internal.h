@@ -54,6 +54,9 @@ struct DevState {
 
 static_assert(sizeof(DevState) <= 512, "scratch buffers of the test hooks are documented as 512 bytes");
 
+// How a kernel tells a waiting call that its results are in page-locked memory (flag null: it does not).
+struct MailPost { unsigned* flag; unsigned seq; };
+
 // One entry of the device copy of the polynomial schedule.
 struct SchedEntry { float a, b, c, l; int lift, seg_x; };
 constexpr int NS_SCHED_MAX = 128;

@@ -27,6 +27,13 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
+// Tells a waiting call that its results are there (one thread, once the block's are written).
+__device__ __forceinline__ void post_mail(const MailPost& post) {
+  if (post.flag == nullptr) return;
+  __threadfence_system();
+  *reinterpret_cast<volatile unsigned*>(post.flag) = post.seq;
+}
+
 // Block-wide sum in double, fixed order (lane tree, then warp 0 over the warp results).
 template <int THREADS>
 __device__ __forceinline__ double block_sum_d(double v, double* smem /* THREADS/32 */) {
