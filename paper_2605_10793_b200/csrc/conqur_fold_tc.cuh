@@ -7,9 +7,11 @@
 // half a k at a time (three 32 KB buffers); eight warps split it into pieces in the swizzled operand layout, one half while the
 // products read the other; one warp issues the six products of each half into an accumulator of its own (64 terms, small pieces
 // first); eight warps add the two halves in fp32 and write the tile (on SIDE 0 a TMEM lane is a column of the output, so a warp's
-// stores are whole lines as they are).  W is read once and out written once: bound by that (128 KB a tile, 5.7 k cycles of an SM's
-// share of the HBM rate; the products take 3.1 k).  32 blocks of 128, W 4096 x 4096: 90 -> 42 us, of which half is each CTA's
-// rotation (4 k cycles, once or twice) and the pipeline's fill; 4096 x 14336 4.4 TB/s.
+// stores are turned into whole 16-byte pieces first).  W is read once and out written once: bound by that (128 KB a tile, 5.7 k cycles of
+// an SM's share of the HBM rate; splitting takes 5 k, the products 3.1 k, writing 4.5 k).  A rotation comes through the copy engine into
+// the pieces' place, ahead of W, and is split from there in 3 k cycles, once or twice a CTA (with single loads from memory, behind W's
+// copies, 11 k).  32 blocks of 128, W 4096 x 4096, whole call: CUDA cores 111 us, this 57.5 (65 with single loads); 64 blocks 4096 wide
+// INPUT 66 -> 58, where a thread's 4-byte stores had set the pace.
 // Error against 64 bits, in 2^-24 of the result's norm, fp32 chain / this: 128-blocks 3.4 / 1.4, 64-blocks 2.4 / 1.3.
 //
 // Both operands are split after a multiplication by 2^32, so that no piece of any fp32 number is subnormal (its last bit is worth
@@ -47,11 +49,11 @@ struct FbArgs {
   int64_t ldw, ldo;
   int logdb, rows, cols;            // blocks of 1 << logdb
   int n_super, tiles;               // 128-wide groups of blocks; W tiles along the other dimension
-  int copied;                       // 1: W's rows suit the copy engine (16-byte aligned)
+  int copied, r_copied;             // 1: W's rows, R suit the copy engine (16-byte aligned)
   int* status;                      // page-locked host memory, two words cleared by the caller: flags, and whether a value was unfit
 };
 struct FbAux {
-  uint64_t raw_full[FB_RAW], raw_free[FB_RAW], full[2], free_[2], tfull, tempty;
+  uint64_t raw_full[FB_RAW], raw_free[FB_RAW], full[2], free_[2], tfull, tempty, rfull, rread;
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -67,7 +69,8 @@ struct FbRange {
 };
 
 template <int SIDE>
-__global__ void __launch_bounds__(FB_THREADS, 1) fold_blocks_kernel(const __grid_constant__ CUtensorMap tmW, const FbArgs g) {
+__global__ void __launch_bounds__(FB_THREADS, 1) fold_blocks_kernel(const __grid_constant__ CUtensorMap tmW,
+                                                                     const __grid_constant__ CUtensorMap tmR, const FbArgs g) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sW = smem;                                    // pieces: two 64-column chunks of 128 rows x 128 bytes each, swizzled by the row
@@ -80,14 +83,23 @@ __global__ void __launch_bounds__(FB_THREADS, 1) fold_blocks_kernel(const __grid
   const int folded = SIDE == 0 ? g.cols : g.rows;       // length of the folded dimension
   const int db = 1 << g.logdb;
 
+  // a group's rotation, 64 rows of one block either way, into the pieces' place while that is idle (one thread)
+  auto copy_r = [&](int sb) {
+    ptx::mbar_expect_tx(&aux->rfull, 2u * 64u * 4u << g.logdb);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) ptx::tma_load_2d(sW + h * FB_PIECE, &tmR, &aux->rfull, 0, sb * 128 + 64 * h);
+  };
   if (threadIdx.x == 0) {
     for (int s = 0; s < FB_RAW; ++s) { ptx::mbar_init(&aux->raw_full[s], 1); ptx::mbar_init(&aux->raw_free[s], FB_CONV / 32); }
     for (int b = 0; b < 2; ++b) { ptx::mbar_init(&aux->full[b], FB_CONV / 32); ptx::mbar_init(&aux->free_[b], 1); }
     ptx::mbar_init(&aux->tfull, 1);
     ptx::mbar_init(&aux->tempty, 8);
+    ptx::mbar_init(&aux->rfull, 1);
+    ptx::mbar_init(&aux->rread, FB_CONV / 32);
     aux->abort_flag = 0;
     ptx::fence_barrier_init();
     ptx::fence_proxy_async();
+    if (g.r_copied) copy_r(t0 / g.tiles);                // (the first, before the copies of W fill the queues)
     if (g.copied) ptx::prefetch_tmap(&tmW);
   }
   if (warp == FB_CONV / 32 + 1) { ptx::tmem_alloc(&aux->tmem_base, 512); ptx::tmem_relinquish(); }
@@ -101,7 +113,7 @@ __global__ void __launch_bounds__(FB_THREADS, 1) fold_blocks_kernel(const __grid
     // ---- splitting, one half of k after the other (64 rows of the tile on SIDE 1, 64 columns on SIDE 0): 4 elements eight times a thread
     int cur_sb = -1;
     bool bad = false;
-    uint32_t n = 0, it = 0;
+    uint32_t n = 0, it = 0, nr = 0;
     bool ok = true;
     for (int t = t0; t < t1 && ok; ++t, ++n) {
       const int sb = t / g.tiles, j = t - sb * g.tiles;
@@ -110,33 +122,49 @@ __global__ void __launch_bounds__(FB_THREADS, 1) fold_blocks_kernel(const __grid
         // R^T into TMEM: lane = its row, two consecutive k per column.  (The products of the tile before read the old one last.)
         if (!tc_wait_warp(&aux->free_[0], ph, abort_flag) || !tc_wait_warp(&aux->free_[1], ph, abort_flag)) { timeout_site = 1; break; }
         ptx::tc_fence_after();
+        if (g.r_copied && cur_sb >= 0 && threadIdx.x == 0) copy_r(sb);
         cur_sb = sb;
         FbRange rr;
-        const int a = (warp & 3) * 32 + lane, ag = sb * 128 + a;
-        const uint32_t ta = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + FB_TM_A;
-#pragma unroll 1
-        for (int c = 0; c < 4; ++c) {                    // 16 k, 8 columns of each piece
-          const int k0 = (warp >> 2) * 64 + c * 16;
-          float v[16];
+        // a warp's 32 lanes and half of k lie in one block: its own where their block numbers agree, or there are zeros (two blocks side by
+        // side, or one past the last).  Sixteen k at a time (8 columns of each piece), the next sixteen on their way meanwhile.
+        const int a = (warp & 3) * 32 + lane, kh = warp >> 2;
+        const bool in = sb * 128 + kh * 64 < folded && (kh * 64 >> g.logdb) == ((warp & 3) * 32 >> g.logdb);
+        const float* src = (g.r_copied ? reinterpret_cast<const float*>(sW + kh * FB_PIECE) : g.R + ((int64_t)(sb * 128 + kh * 64) << g.logdb)) +
+                           (a & (db - 1));
+        if (g.r_copied && !tc_wait_warp(&aux->rfull, nr & 1u, abort_flag)) { timeout_site = 7; break; }
+        const uint32_t ta = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(FB_TM_A + kh * 32);
+        float v[2][16];
+        auto fetch = [&](int c, float (&x)[16]) {
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const int k = k0 + i, kg = sb * 128 + k;
-            // (two or more blocks side by side: element (k, a) lies in one of them where their block numbers agree)
-            v[i] = (kg < folded && ag < folded && (k >> g.logdb) == (a >> g.logdb))
-                       ? __ldg(g.R + ((int64_t)kg << g.logdb) + (a & (db - 1))) : 0.f;
-          }
+          for (int i = 0; i < 16; ++i) x[i] = in ? src[(c * 16 + i) << g.logdb] : 0.f;
+        };
+        auto split = [&](int c, const float (&x)[16]) {
           uint32_t w[3][8];
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
-            rr.see(v[2 * i]); rr.see(v[2 * i + 1]);
-            sp_split2(v[2 * i] * FB_UP, v[2 * i + 1] * FB_UP, w[0][i], w[1][i], w[2][i]);
+            rr.see(x[2 * i]); rr.see(x[2 * i + 1]);
+            sp_split2(x[2 * i] * FB_UP, x[2 * i + 1] * FB_UP, w[0][i], w[1][i], w[2][i]);
           }
 #pragma unroll
-          for (int p = 0; p < 3; ++p) ptx::tmem_st8(ta + (uint32_t)(p * 64 + k0 / 2), w[p]);
+          for (int p = 0; p < 3; ++p) ptx::tmem_st8(ta + (uint32_t)(p * 64 + c * 8), w[p]);
+        };
+        fetch(0, v[0]);
+#pragma unroll 1
+        for (int c = 0; c < 4; c += 2) {
+          fetch(c + 1, v[1]);
+          split(c, v[0]);
+          if (c == 0) fetch(2, v[0]);
+          split(c + 1, v[1]);
         }
         bad |= !rr.within(FB_R_LIMIT);
         ptx::tmem_st_wait();
         ptx::tc_fence_before();
+        if (g.r_copied) {                                // (nobody's pieces go there before all have read it)
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive(&aux->rread);
+          if (!tc_wait_warp(&aux->rread, nr & 1u, abort_flag)) { timeout_site = 7; break; }
+          ++nr;
+        }
       }
 #pragma unroll 1
       for (int h = 0; h < 2; ++h, ++it) {
@@ -181,6 +209,10 @@ __global__ void __launch_bounds__(FB_THREADS, 1) fold_blocks_kernel(const __grid
           ptx::mbar_arrive(&aux->full[h]);
         }
       }
+    }
+    if (*abort_flag && threadIdx.x == 0) {                 // let the rotation's copy land before the CTA's shared memory goes
+      const long long c0 = clock64();
+      while (clock64() - c0 < 4000000ll) {}
     }
     if (bad) reinterpret_cast<volatile int*>(g.status)[1] = 1;
   } else if (warp < FB_CONV / 32 + 4) {
@@ -260,11 +292,31 @@ __global__ void __launch_bounds__(FB_THREADS, 1) fold_blocks_kernel(const __grid
       const int f = sb * 128 + q * 32 + lane, o0 = j * 128 + half * 64;
       const int other = SIDE == 0 ? g.rows : g.cols;
       if (SIDE == 0) {
-        if (f < folded) {
-          float* p = g.out + (int64_t)o0 * g.ldo + f;
+        // 32 rows of 32 columns at a time, turned in the warp's buffer into 16-byte pieces of a row where out's rows allow them (64 stores of
+        // 4 bytes a thread took 6.3 k cycles a tile and set its pace, sixteen of 16 bytes take 4.5 k)
+        const int c0 = sb * 128 + q * 32;
+        const bool whole = c0 + 32 <= folded && (g.ldo & 3) == 0 && (reinterpret_cast<uintptr_t>(g.out) & 15) == 0;
 #pragma unroll
-          for (int i = 0; i < 64; ++i)
-            if (o0 + i < other) __stcs(p + (int64_t)i * g.ldo, v[i] * FB_DOWN);
+        for (int c = 0; c < 2; ++c) {
+          const int r0 = o0 + c * 32;
+          if (whole) {
+            float* const sf = reinterpret_cast<float*>(stg);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) sf[i * 32 + (lane ^ ((i & 7) << 2))] = v[c * 32 + i] * FB_DOWN;
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const int r = i * 4 + (lane >> 3), piece = lane & 7;
+              const float4 t4 = *reinterpret_cast<const float4*>(sf + r * 32 + ((piece ^ (r & 7)) << 2));
+              if (r0 + r < other) __stcs(reinterpret_cast<float4*>(g.out + (int64_t)(r0 + r) * g.ldo + c0 + piece * 4), t4);
+            }
+            __syncwarp();
+          } else if (f < folded) {
+            float* p = g.out + (int64_t)r0 * g.ldo + f;
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+              if (r0 + i < other) __stcs(p + (int64_t)i * g.ldo, v[c * 32 + i] * FB_DOWN);
+          }
         }
       } else {
         const int m0 = sb * 128 + q * 32, rows_ok = min(32, max(0, g.rows - m0));
@@ -309,11 +361,12 @@ inline int tc_make_tmap_f32(CUtensorMap* tm, const void* ptr, uint64_t rows, uin
 // Folds that take this kernel: several blocks of 64 or 128, enough of W, and tiles that are not mostly empty (each group of blocks
 // costs its rotation's splitting, however short the other side is).  Whole call (as timed in a row), fp32 CUDA cores -> this, us,
 // blocks x other side:
-//   of 128         8 x 1024 35 -> 34, 64 x 96 35 -> 34, 64 x 512 52 -> 42, 64 x 2048 118 -> 67, 256 x 128 52 -> 42, 1024 x 96 116 -> 93;
+//   of 128         8 x 1024 35 -> 33, 64 x 96 35 -> 36, 64 x 512 52 -> 39, 64 x 2048 118 -> 58, 256 x 128 52 -> 40, 1024 x 96 116 -> 75;
 //                  not 32 x 160 31.5 -> 34, 64 x 64 30 -> 33, 128 x 32 30 -> 33, 512 x 64 53 -> 55, 1024 x 1 57 -> 82, 1024 x 64 75 -> 91
-//   of 64, INPUT   64 x 1024 42 -> 42, 512 x 256 61 -> 53, 1024 x 256 97 -> 84;  not 512 x 160 48 -> 52, 1024 x 1 33 -> 54
-//   of 64, OUTPUT  64 x 2048 48 -> 47, 512 x 512 71 -> 69, 256 x 2048 114 -> 91; not 64 x 1024 38 -> 40, 1024 x 256 71 -> 77
-// (the CUDA cores give an element the same bits in a call of any shape; this kernel gives it its own)
+//   of 64, INPUT   64 x 1024 42 -> 39, 512 x 256 61 -> 49, 1024 x 256 97 -> 65;  not 512 x 160 48 -> 52, 1024 x 1 33 -> 54
+//   of 64, OUTPUT  64 x 2048 48 -> 44, 512 x 512 71 -> 58, 256 x 2048 114 -> 77; not 64 x 1024 38 -> 40, 1024 x 256 71 -> 77
+// (the shapes that are "not" with the rotation loaded singly: up to a tenth less now, and the line has stayed; the CUDA cores give an
+// element the same bits in a call of any shape, this kernel gives it its own)
 inline bool fold_blocks_takes(int64_t rows, int64_t cols, int block, int side) {
   const bool in = side == CONQUR_FOLD_INPUT;
   const int64_t folded = in ? cols : rows, other = in ? rows : cols;
@@ -334,7 +387,7 @@ inline int fold_blocks_launch(const float* W, int64_t ldw, int rows, int cols, c
     }
     attr_dev_mask.fetch_or(dev_bit, std::memory_order_release);
   }
-  FbArgs g{W, R, out, ldw, ldo, block == 64 ? 6 : 7, rows, cols, 0, 0, 0, status};
+  FbArgs g{W, R, out, ldw, ldo, block == 64 ? 6 : 7, rows, cols, 0, 0, 0, 0, status};
   const bool in = side == CONQUR_FOLD_INPUT;
   g.n_super = ((in ? cols : rows) + 127) / 128;
   g.tiles = ((in ? rows : cols) + 127) / 128;
@@ -343,10 +396,15 @@ inline int fold_blocks_launch(const float* W, int64_t ldw, int rows, int cols, c
     if (tc_make_tmap_f32(&tm, W, (uint64_t)rows, (uint64_t)cols, (uint64_t)ldw, in ? 64 : 128, in ? 128 : 64) != CONQUR_OK) return CONQUR_ERR_CUDA;
     g.copied = 1;
   }
+  CUtensorMap tr = {};
+  if ((reinterpret_cast<uintptr_t>(R) & 15) == 0) {
+    if (tc_make_tmap_f32(&tr, R, (uint64_t)(in ? cols : rows), (uint64_t)block, (uint64_t)block, (uint32_t)block, 64) != CONQUR_OK) return CONQUR_ERR_CUDA;
+    g.r_copied = 1;
+  }
   const int64_t total = (int64_t)g.n_super * g.tiles;
   const unsigned grid = (unsigned)(total < sms ? total : sms);
-  if (in) fold_blocks_kernel<0><<<grid, FB_THREADS, FB_SMEM_BYTES, s>>>(tm, g);
-  else fold_blocks_kernel<1><<<grid, FB_THREADS, FB_SMEM_BYTES, s>>>(tm, g);
+  if (in) fold_blocks_kernel<0><<<grid, FB_THREADS, FB_SMEM_BYTES, s>>>(tm, tr, g);
+  else fold_blocks_kernel<1><<<grid, FB_THREADS, FB_SMEM_BYTES, s>>>(tm, tr, g);
   return cudaGetLastError() == cudaSuccess ? CONQUR_OK : CONQUR_ERR_CUDA;
 }
 

@@ -152,3 +152,23 @@ def test_short_and_small_folds_stay_on_the_cuda_cores(k, b, other, side):
     for i in range(0, k, max(1, k // 16)):
         cut = (slice(None), slice(i * b, (i + 1) * b)) if side == "input" else (slice(i * b, (i + 1) * b), slice(None))
         assert torch.equal(got[cut], B.conqur_fold_weight(w[cut], r[i], side, "exact"))
+
+
+# one group of blocks and several a block of threads, an odd number of 64-blocks, remainders of a tile
+@pytest.mark.parametrize("k,b,other", [(3, 128, 2690), (241, 64, 512), (256, 128, 97)])
+@pytest.mark.parametrize("side", ["input", "output"])
+def test_rotations_and_results_off_16_byte_boundaries(k, b, other, side):
+    """R that the copy engine does not take, and out whose rows 16-byte stores do not: the same bits."""
+    w = _rand(other, *((other, k * b) if side == "input" else (k * b, other)))
+    r = _rand(k, k, b, b) / b ** 0.5
+    odd = torch.empty(r.numel() + 1, device="cuda")[1:].view(k, b, b)
+    odd.copy_(r)
+    ref = B.conqur_fold_weight(w, r, side, "exact")
+    assert torch.equal(B.conqur_fold_weight(w, odd, side, "exact"), ref)
+    rows, cols = w.shape
+    wide = torch.full((rows, cols + 1), 7.0, device="cuda")
+    scratch = torch.empty(4096, dtype=torch.uint8, device="cuda")
+    code = B.CONQUR_FOLD_INPUT if side == "input" else B.CONQUR_FOLD_OUTPUT
+    rc = B.load().conqur_fold_weight(w.data_ptr(), w.stride(0), rows, cols, r.data_ptr(), b, code, B.CONQUR_EXACT_F32, wide.data_ptr(),
+                                     wide.stride(0), scratch.data_ptr(), 4096, torch.cuda.current_stream().cuda_stream)
+    assert rc == 0 and torch.equal(wide[:, :cols], ref) and bool((wide[:, cols] == 7.0).all())
