@@ -3,17 +3,18 @@
 // At these widths a launch of the iteration costs more than its work: 128^3 multiply-adds are 0.1 us of the chip, a launch with
 // the load latency of its operands about 6 us, and a step takes three of them and the control decision.  Sixteen CTAs of one
 // cluster share the 32 x 32 tiles of every product instead, and every CTA takes the decision itself from the same sums.  The matrices
-// live in shared memory: a finished tile is written straight into that of the CTAs whose next products read it, so that between
-// two products stands one cluster barrier with no trip to the L2 in front of or behind it.  An element of a product is the same chain
-// of multiply-adds as in the launches' kernels, and the coefficients of a step depend on its place in the plan alone: the same bits
-// wherever the start scale rounds to the same number and the decisions agree.  (The squares behind these are added in another
-// grouping, sixteen CTAs' instead of a block's per 1024 elements or per tile: double sums rounded to fp32, so a last bit may differ.)
-// What a step takes (d = 128, SM cycles, clock stamps): products 3.3 k to 4.2 k each (a warp's packed multiply-adds, two cycles each, and
-// its 16-byte reads share their time unevenly: 16 would do per k, 26 to 32 are taken), sending 1.3 k (32 KB a CTA at 25 bytes a cycle) and
-// the barrier behind it 1.7 k to 2 k, norms 0.6 k; the decision runs beside the next product.  22 k in all; 29 k with the matrices in the
-// L2 between the products.  Whole update of given statistics once its step count is learnt, from an idle stream, matrices in the L2 -> this,
-// us (one B200): d = 16, 4 steps 36 -> 26;  64, 4 steps 49 -> 36;  128, 4 steps 70 -> 61;  160, 5 steps 121 -> 110 (as a graph of launches the
-// first took 139, with 8 steps, and 128 with 9 steps 223).  192 (three tiles a CTA) has no room for its matrices.
+// live in shared memory: a finished tile is written straight into that of the CTAs whose next products read it.  Up to d = 128 a CTA
+// waits for the bytes it reads and nothing else (beyond, where there is no room to keep what others still read, for barriers of
+// the cluster).  An element of a product is the same chain of multiply-adds as in the launches' kernels, and the coefficients of a
+// step depend on its place in the plan alone: the same bits wherever the start scale rounds to the same number and the decisions
+// agree.  (The squares behind these are added in another grouping, sixteen CTAs' instead of a block's per 1024 elements or per tile:
+// double sums rounded to fp32, so a last bit may differ.)
+// What a step takes (d = 128, SM cycles, clock stamps): products 3.3 k each, bound by their reads of shared memory, sending 1.3 k (32 KB a
+// CTA at 25 bytes a cycle), the way there 0.6 k, norms 0.4 k; the decision runs beside the next product.  Whole update of given statistics
+// once its step count is learnt, from an idle stream, us (one B200): matrices in the L2 between the products -> in shared memory with two
+// multiplying warps and cluster barriers -> waiting for bytes -> this, with four warps
+//   d = 16, 4 steps 36 -> 26 -> 23 -> 24;  64, 4 steps 49 -> 36 -> 35 -> 34;  128, 4 steps 70 -> 61 -> 59 -> 55;  160, 5 steps 121 -> 110 -> - -> 103
+// (as a graph of launches the first took 139, with 8 steps, and 128 with 9 steps 223).  192 has no room for its matrices.
 #pragma once
 #include <mutex>
 
@@ -24,9 +25,10 @@ namespace conqur {
 
 constexpr int NC_MAX_TILES = 5;                  // tiles of 32 along a side: one or two of a product's 25 a CTA
 constexpr int NC_MAX_D = 32 * NC_MAX_TILES;
+constexpr int NC_SMALL_D = 128;                  // up to here three matrices fit
 constexpr int NC_THREADS = 256;
 constexpr int NC_CTAS = 16;
-constexpr int NC_WORK = 64;                      // threads that multiply: a 4 x 4 piece of the tile each
+constexpr int NC_WORK = 128;                     // threads that multiply: a 2 x 4 piece of the tile each
 constexpr int NC_LD_TILE = 36;                   // rows of the tile on its way out: 32 columns and 4 floats against bank conflicts
 
 struct NcArgs {
@@ -38,11 +40,11 @@ struct NcArgs {
 };
 
 // A matrix in shared memory: 32 T rows of 32 T columns and 4 floats against bank conflicts, zeros past d.  Up to four tiles a side three
-// of them fit: the next iterate then takes the residual's place and never one that another CTA still reads.  With five tiles there are
-// two, written in place, and a barrier more in front of each write.
+// of them fit, and a tile never goes where another CTA still reads.  With five there are two, written in place, and a barrier of the
+// cluster stands in front of and behind each write.
 __host__ __device__ inline int nc_ld(int tiles) { return 32 * tiles + 4; }
 __host__ __device__ inline int nc_matrix_floats(int tiles) { return 32 * tiles * nc_ld(tiles); }
-__host__ __device__ inline int nc_matrices(int tiles) { return tiles <= 4 ? 3 : 2; }
+__host__ __device__ inline int nc_matrices(int tiles) { return 32 * tiles <= NC_SMALL_D ? 3 : 2; }
 inline int nc_smem_bytes(int d) {
   const int tiles = (d + 31) / 32;
   return (nc_matrices(tiles) * nc_matrix_floats(tiles) + 32 * NC_LD_TILE) * (int)sizeof(float);
@@ -54,54 +56,59 @@ __device__ __forceinline__ void nc_cluster_sync() {
 }
 
 // Tile (m0, n0) of sum_k A(m, k) B(k, n), each sum one chain in the order of k as sg_mainloop's; k runs to kp, d rounded up to four.
-// A(m, k) = A[k][m]: thread t < NC_WORK returns rows 4 (t / 8) .. +3; A[m][k] with TRANS: rows t / 8 + 8 i (neighbouring rows of A lie
-// four banks apart).  Columns 4 (t % 8) .. +3 either way.  A 16-byte read takes the shared memory four cycles a warp whatever is equal
-// in it and a multiply-add the lanes two, packed or not: two warps with 4 x 4 pieces in packed pairs need 16 cycles of either per k.
+// A(m, k) = A[k][m]: thread t < NC_WORK returns rows 2 (t / 8) and the next; A[m][k] with TRANS: rows t / 8 and + 16 (neighbouring rows of
+// A lie four banks apart).  Columns 4 (t % 8) .. +3 either way.  A warp's read of 8 or 16 bytes a lane takes the shared memory two or
+// four cycles whatever is equal in it, a packed multiply-add the lanes two: four warps with 2 x 4 pieces need 24 and 8 cycles per k (two
+// with 4 x 4 16 of either, and took 26 to 32, with nobody to hide a warp's waits behind).
 template <bool TRANS>
-__device__ __forceinline__ void nc_tile(const float* A, const float* B, int ld, int kp, int m0, int n0, float (&out)[4][4]) {
+__device__ __forceinline__ void nc_tile(const float* A, const float* B, int ld, int kp, int m0, int n0, float (&out)[2][4]) {
   const int ty = (int)threadIdx.x >> 3, tx = (int)threadIdx.x & 7;
   const float* pb = B + n0 + 4 * tx;
-  const float* pa = TRANS ? A + (m0 + ty) * ld : A + m0 + 4 * ty;
-  unsigned long long acc[4][2] = {};
-  auto step = [&](const float (&a)[4], const float4& b) {
-    const unsigned long long b0 = f32x2_pack(b.x, b.y), b1 = f32x2_pack(b.z, b.w);
+  const float* pa = TRANS ? A + (m0 + ty) * ld : A + m0 + 2 * ty;
+  unsigned long long acc[2][2] = {};
+  // (four k ahead in registers.  The last reads go past the matrix, into its row padding or what lies behind it, and go unused.)
+  struct Four { float a[2][4]; float4 b[4]; };   // a[row][k]
+  auto fetch = [&](int k, Four& f) {
+    if (TRANS) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const unsigned long long a2 = f32x2_pack(a[i], a[i]);
-      f32x2_fma(acc[i][0], a2, b0);
-      f32x2_fma(acc[i][1], a2, b1);
-    }
-  };
-  // (four k ahead in registers: a warp has nobody to hide its loads behind.  The last ones read past the matrix, into its row padding or
-  // what lies behind it, and go unused.)
-  float4 a[2][4], b[2][4];
-  auto fetch = [&](int k, float4 (&fa)[4], float4 (&fb)[4]) {
+      for (int i = 0; i < 2; ++i) {
+        const float4 v = *reinterpret_cast<const float4*>(pa + 16 * i * ld + k);
+        f.a[i][0] = v.x; f.a[i][1] = v.y; f.a[i][2] = v.z; f.a[i][3] = v.w;
+      }
+    } else {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      fa[i] = *reinterpret_cast<const float4*>(TRANS ? pa + 8 * i * ld + k : pa + (k + i) * ld);
-      fb[i] = *reinterpret_cast<const float4*>(pb + (k + i) * ld);
+      for (int j = 0; j < 4; ++j) {
+        const float2 v = *reinterpret_cast<const float2*>(pa + (k + j) * ld);
+        f.a[0][j] = v.x; f.a[1][j] = v.y;
+      }
     }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) f.b[j] = *reinterpret_cast<const float4*>(pb + (k + j) * ld);
   };
-  auto multiply = [&](const float4 (&fa)[4], const float4 (&fb)[4]) {
-    const float m[4][4] = {{fa[0].x, fa[0].y, fa[0].z, fa[0].w}, {fa[1].x, fa[1].y, fa[1].z, fa[1].w},
-                           {fa[2].x, fa[2].y, fa[2].z, fa[2].w}, {fa[3].x, fa[3].y, fa[3].z, fa[3].w}};
+  auto multiply = [&](const Four& f) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const float col[4] = {TRANS ? m[0][j] : m[j][0], TRANS ? m[1][j] : m[j][1], TRANS ? m[2][j] : m[j][2], TRANS ? m[3][j] : m[j][3]};
-      step(col, fb[j]);
+      const unsigned long long b0 = f32x2_pack(f.b[j].x, f.b[j].y), b1 = f32x2_pack(f.b[j].z, f.b[j].w);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const unsigned long long a2 = f32x2_pack(f.a[i][j], f.a[i][j]);
+        f32x2_fma(acc[i][0], a2, b0);
+        f32x2_fma(acc[i][1], a2, b1);
+      }
     }
   };
-  fetch(0, a[0], b[0]);
+  Four f0, f1;
+  fetch(0, f0);
   int k = 0;
   for (; k + 8 <= kp; k += 8) {
-    fetch(k + 4, a[1], b[1]);
-    multiply(a[0], b[0]);
-    fetch(k + 8, a[0], b[0]);
-    multiply(a[1], b[1]);
+    fetch(k + 4, f1);
+    multiply(f0);
+    fetch(k + 8, f0);
+    multiply(f1);
   }
-  if (k < kp) multiply(a[0], b[0]);
+  if (k < kp) multiply(f0);
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       out[i][2 * j] = __uint_as_float((uint32_t)acc[i][j]);
@@ -110,9 +117,9 @@ __device__ __forceinline__ void nc_tile(const float* A, const float* B, int ld, 
 }
 
 // This thread's piece of a tile into the tile's buffer (row r0 + step i).
-__device__ __forceinline__ void nc_put(float* tile, int r0, int step, const float (&v)[4][4]) {
+__device__ __forceinline__ void nc_put(float* tile, int r0, int step, const float (&v)[2][4]) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 2; ++i)
     *reinterpret_cast<float4*>(tile + (r0 + step * i) * NC_LD_TILE + 4 * ((int)threadIdx.x & 7)) = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
 }
 
@@ -140,6 +147,55 @@ __device__ __forceinline__ void nc_send(const float* tile, bool transposed, floa
   }
 }
 
+// The same for up to four tiles a side, where nothing but the data itself is waited for: the bytes are counted on a barrier in each CTA that
+// gets them.  No copy or barrier of the whole cluster stands between two products then.
+__device__ __forceinline__ void nc_send_async(const float* tile, bool transposed, float* matrix, int ld, int r, int c, uint32_t mask, int p,
+                                              uint64_t* bar) {
+  const int row = p >> 3, col = 4 * (p & 7);
+  float4 v;
+  if (transposed) {
+    v.x = tile[col * NC_LD_TILE + row]; v.y = tile[(col + 1) * NC_LD_TILE + row];
+    v.z = tile[(col + 2) * NC_LD_TILE + row]; v.w = tile[(col + 3) * NC_LD_TILE + row];
+  } else {
+    v = *reinterpret_cast<const float4*>(tile + row * NC_LD_TILE + col);
+  }
+  const uint32_t here = nc_smem_u32(matrix + (32 * r + row) * ld + 32 * c + col), bar_here = nc_smem_u32(bar);
+  for (; mask; mask &= mask - 1) {
+    const int to = __ffs((int)mask) - 1;
+    uint32_t there, bar_there;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(here), "r"(to));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(bar_there) : "r"(bar_here), "r"(to));
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(there), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar_there) : "memory");
+  }
+}
+__device__ __forceinline__ void nc_bar_init(uint64_t* bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(nc_smem_u32(bar)) : "memory");
+}
+// The barrier's next phase: `bytes` will come (one thread).
+__device__ __forceinline__ void nc_expect(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(nc_smem_u32(bar)), "r"(bytes) : "memory");
+}
+// Waits for a phase's bytes, for two seconds at most; gave_up ends every wait of the CTA.
+__device__ __forceinline__ void nc_wait(uint64_t* bar, uint32_t parity, volatile int* gave_up) {
+  const uint32_t at = nc_smem_u32(bar);
+  const long long t0 = clock64();
+  for (uint32_t spins = 0;; ++spins) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.b32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(at), "r"(parity) : "memory");
+    if (ok) return;
+    if ((spins & 255u) == 255u && (*gave_up || clock64() - t0 > 4000000000ll)) { *gave_up = 1; return; }
+  }
+}
+
+// The multiplying warps' sums and maxima.
+__device__ __forceinline__ double nc_all_of(const double* s) { return (s[0] + s[1]) + (s[2] + s[3]); }
+__device__ __forceinline__ float nc_most_of(const float* m) { return fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3])); }
+
 // Leaves a value in every CTA of the cluster (slot `from` of `slots`, the same place in each one's shared memory); one warp.
 // The cluster barrier that follows publishes it.
 __device__ __forceinline__ void nc_tell(double v, double* slots, int from) {
@@ -151,6 +207,17 @@ __device__ __forceinline__ void nc_tell(double v, double* slots, int from) {
     asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(r), "d"(v) : "memory");
   }
 }
+// Two values, counted on a barrier there.
+__device__ __forceinline__ void nc_tell_async(double a, double b, double (*slots)[2], int from, uint64_t* bar) {
+  const int lane = threadIdx.x & 31;
+  if (lane < NC_CTAS) {
+    uint32_t there, bar_there;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(nc_smem_u32(slots + from)), "r"(lane));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(bar_there) : "r"(nc_smem_u32(bar)), "r"(lane));
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%0], {%1, %2}, [%3];"
+                 ::"r"(there), "d"(a), "d"(b), "r"(bar_there) : "memory");
+  }
+}
 // The sixteen values, added in order (every CTA gets the same sum).
 __device__ __forceinline__ double nc_total(const double* slots) {
   double s = 0.0;
@@ -159,6 +226,7 @@ __device__ __forceinline__ double nc_total(const double* slots) {
   return s;
 }
 
+template <bool SMALL>
 __global__ void __launch_bounds__(NC_THREADS, 1) ns_cluster_kernel(const NcArgs g) {
   extern __shared__ __align__(16) float nc_smem[];
   __shared__ double redd[NC_THREADS / 32];
@@ -168,12 +236,14 @@ __global__ void __launch_bounds__(NC_THREADS, 1) ns_cluster_kernel(const NcArgs 
   __shared__ int done_s;
   __shared__ uint32_t by_col[NC_MAX_TILES], by_row[NC_MAX_TILES], by_factor[NC_MAX_TILES];    // who reads what, see below
   __shared__ SchedEntry sched[NS_SCHED_MAX];
+  __shared__ __align__(16) double told[2][NC_CTAS][2];        // SMALL: what the CTAs tell each other, alternating
+  __shared__ __align__(8) uint64_t bar_e, bar_b, bar_x, bar_t[2];
+  __shared__ int gave_up;
   const int cta = (int)blockIdx.x, t = threadIdx.x, d = g.d, kp = (d + 3) / 4 * 4;
   const int tiles = (d + 31) / 32, ld = nc_ld(tiles), sym_tiles = tiles * (tiles + 1) / 2;
-  const bool in_place = nc_matrices(tiles) == 2;
   float* X = nc_smem;
   float* E = X + nc_matrix_floats(tiles);
-  float* Bm = in_place ? E : E + nc_matrix_floats(tiles);
+  float* Bm = SMALL ? E + nc_matrix_floats(tiles) : E;
   float* const tile = nc_smem + nc_matrices(tiles) * nc_matrix_floats(tiles);
   const size_t dd = (size_t)d * d;
   DevState* st = g.st;
@@ -196,6 +266,20 @@ __global__ void __launch_bounds__(NC_THREADS, 1) ns_cluster_kernel(const NcArgs 
       if (t == i % tiles) factor |= 1u << (i % NC_CTAS);
     }
     by_col[t] = col; by_row[t] = row; by_factor[t] = factor;
+  }
+  // this CTA's tiles, and the bytes of a step's residual, polynomial and iterate that come to it
+  int tm = 0, tn = 0;
+  const bool has_sym = cta < sym_tiles, has_full = cta < tiles * tiles;
+  if (has_sym) sym_coords(cta, tm, tn);
+  const uint32_t n_cols = has_sym ? (tm == tn ? 1u : 2u) : 0u;
+  const uint32_t e_bytes = 4096u * tiles * n_cols, b_bytes = has_full ? 4096u * tiles : 0u;
+  const uint32_t x_bytes = e_bytes + (has_full ? 4096u * (tiles - n_cols) : 0u);
+  if (SMALL && t == 0) {
+    nc_bar_init(&bar_e); nc_bar_init(&bar_b); nc_bar_init(&bar_x); nc_bar_init(&bar_t[0]); nc_bar_init(&bar_t[1]);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    nc_expect(&bar_e, e_bytes); nc_expect(&bar_b, b_bytes); nc_expect(&bar_x, x_bytes);
+    nc_expect(&bar_t[0], NC_CTAS * 16u); nc_expect(&bar_t[1], NC_CTAS * 16u);
+    gave_up = 0;
   }
   int slot = 0;
   auto sumsq = [&](float lam) {                  // ||M + lam R||_F^2
@@ -255,105 +339,174 @@ __global__ void __launch_bounds__(NC_THREADS, 1) ns_cluster_kernel(const NcArgs 
     done_s = ctl.ns_done;
   }
   __syncthreads();
-  int tm = 0, tn = 0;                            // this CTA's tile of a symmetric product
-  const bool has_sym = cta < sym_tiles;
-  if (has_sym) sym_coords(cta, tm, tn);
-  const int r4 = 4 * (t >> 3), c4 = 4 * (t & 7); // this thread's piece of it (t < NC_WORK)
-  float v[4][4];
+  const int r2 = 2 * (t >> 3), c4 = 4 * (t & 7); // this thread's piece of it (t < NC_WORK)
+  float v[2][4];
   int k = 0, cur = 0;
-  for (; done_s == 0; ++k, cur ^= 1) {
-    // E = X^T X - I and its norms
-    float mx = 0.f;
-    double sq = 0.0;
-    if (has_sym && t < NC_WORK) {
-      nc_tile<false>(X, X, ld, kp, tm * 32, tn * 32, v);
+  // E = X^T X - I, this thread's piece, and its norms
+  auto residual = [&](float& mx, double& sq) {
+    nc_tile<false>(X, X, ld, kp, tm * 32, tn * 32, v);
 #pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        const int row = tm * 32 + r4 + h, col = tn * 32 + c4;
+    for (int h = 0; h < 2; ++h) {
+      const int row = tm * 32 + r2 + h, col = tn * 32 + c4;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          if (row >= d || col + j >= d) continue;
-          if (row == col + j) v[h][j] -= 1.f;
-          mx = fmaxf(mx, fabsf(v[h][j]));
-          sq += (tm != tn ? 2.0 : 1.0) * ((double)v[h][j] * (double)v[h][j]);
+      for (int j = 0; j < 4; ++j) {
+        if (row >= d || col + j >= d) continue;
+        if (row == col + j) v[h][j] -= 1.f;
+        mx = fmaxf(mx, fabsf(v[h][j]));
+        sq += (tm != tn ? 2.0 : 1.0) * ((double)v[h][j] * (double)v[h][j]);
+      }
+    }
+  };
+  auto polynomial = [&] {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[h][j] = fmaf(coef[2], v[h][j], coef[1] * E[(tm * 32 + r2 + h) * ld + tn * 32 + c4 + j]);
+  };
+  auto next = [&](int f, float (&o)[2][4]) {     // X B + gamma X
+    const int fm = f / tiles, fn = f - fm * tiles;
+    nc_tile<true>(X, Bm, ld, kp, fm * 32, fn * 32, o);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) o[h][j] = fmaf(coef[0], X[(fm * 32 + (t >> 3) + 16 * h) * ld + fn * 32 + c4 + j], o[h][j]);
+  };
+  auto decide = [&](double tsq, double tmx) {
+    const unsigned char entry = ns_control_decide(&ctl, (float)tmx, tsq, 0.0, k, cur, c);
+    if (cta == 0 && entry && k < 128) st->seg_log[k] = entry;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) coef[j] = ctl.coef[j];
+    done_s = ctl.ns_done;
+  };
+  // Up to sixteen tiles.  A phase begins when what it reads has come.  What may still be read is not written over: the residual goes where
+  // the polynomial before it was, the polynomial where the iterate before that was, the next iterate where the residual was, and whoever
+  // sends a tile to one of these places has waited, by way of its operands, for what the receiver made of the tile that stands there (a
+  // receiver reads columns tm and tn of X and of the residual, column fn of the polynomial and row fm of X; the products behind a tile of
+  // column c have read all of column c, and behind every tile of a step stand all CTAs' norms of that step).  Likewise no phase of a
+  // barrier gets bytes of the one after the next, and the norms, which not every tile waits for, alternate between two.
+  if constexpr (SMALL) {
+    const int fm = cta / tiles, fn = cta - fm * tiles;
+    for (; done_s == 0; ++k, cur ^= 1) {
+      float mx = 0.f;
+      double sq = 0.0;
+      if (t < NC_WORK) {
+        if (k > 0 && x_bytes) {
+          nc_wait(&bar_x, (uint32_t)(k - 1) & 1u, &gave_up);
+          if (t == 0) nc_expect(&bar_x, x_bytes);
+        }
+        if (has_sym) residual(mx, sq);
+        sq = warp_sum_d(sq);
+        mx = warp_max(mx);
+        if ((t & 31) == 0) { redd[t >> 5] = sq; redf[t >> 5] = mx; }
+      }
+      __syncthreads();                           // (and the tile before has been sent)
+      if (has_sym && t < NC_WORK) nc_put(tile, r2, 1, v);
+      if (t < 32) nc_tell_async(nc_all_of(redd), (double)nc_most_of(redf), told[k & 1], cta, &bar_t[k & 1]);
+      __syncthreads();
+      if (has_sym) {
+        nc_send_async(tile, false, E, ld, tm, tn, by_col[tn], t, &bar_e);
+        if (tm != tn) nc_send_async(tile, true, E, ld, tn, tm, by_col[tm], t, &bar_e);
+        if (t < NC_WORK) {
+          nc_wait(&bar_e, (uint32_t)k & 1u, &gave_up);
+          if (t == 0) nc_expect(&bar_e, e_bytes);
+          nc_tile<false>(E, E, ld, kp, tm * 32, tn * 32, v);      // does not wait for the decision
         }
       }
-      nc_put(tile, r4, 1, v);
+      if (decides) {
+        nc_wait(&bar_t[k & 1], (uint32_t)(k >> 1) & 1u, &gave_up);
+        nc_expect(&bar_t[k & 1], NC_CTAS * 16u);
+        double tsq = 0.0, tmx = 0.0;
+#pragma unroll
+        for (int i = 0; i < NC_CTAS; ++i) { tsq += told[k & 1][i][0]; tmx = fmax(tmx, told[k & 1][i][1]); }
+        decide(tsq, tmx);
+      }
+      __syncthreads();
+      if (done_s != 0 || gave_up) break;
+      if (has_sym && t < NC_WORK) { polynomial(); nc_put(tile, r2, 1, v); }
+      __syncthreads();
+      if (has_sym) {
+        nc_send_async(tile, false, Bm, ld, tm, tn, by_factor[tn], t, &bar_b);
+        if (tm != tn) nc_send_async(tile, true, Bm, ld, tn, tm, by_factor[tm], t, &bar_b);
+      }
+      if (has_full && t < NC_WORK) {
+        nc_wait(&bar_b, (uint32_t)k & 1u, &gave_up);
+        if (t == 0) nc_expect(&bar_b, b_bytes);
+        next(cta, v);
+      }
+      __syncthreads();
+      if (has_full && t < NC_WORK) nc_put(tile, t >> 3, 16, v);
+      __syncthreads();
+      if (has_full) nc_send_async(tile, false, E, ld, fm, fn, by_col[fn] | by_row[fm], t, &bar_x);
+      float* const old = X;
+      X = E; E = Bm; Bm = old;
     }
+    if (gave_up) {                               // let what is on its way land before the memory goes
+      const long long t0 = clock64();
+      while (clock64() - t0 < 4000000ll) {}
+      if (decides) {
+        ctl.ns_done = NS_DONE_FAILED;
+        atomicOr(&st->status_flags, STATUS_FLAG_TIMEOUT);
+        st->timeout_site = 50;
+      }
+    }
+  } else {
+  for (; done_s == 0; ++k, cur ^= 1) {
+    float mx = 0.f;
+    double sq = 0.0;
     if (t < NC_WORK) {
+      if (has_sym) { residual(mx, sq); nc_put(tile, r2, 1, v); }
       sq = warp_sum_d(sq);
       mx = warp_max(mx);
-      if (t == 32) { redd[0] = sq; redf[0] = mx; }
+      if ((t & 31) == 0) { redd[t >> 5] = sq; redf[t >> 5] = mx; }
     }
     __syncthreads();
     if (t < 32) {
-      nc_tell(sq + redd[0], sums[slot], cta);
-      nc_tell((double)fmaxf(mx, redf[0]), maxima[slot], cta);
+      nc_tell(nc_all_of(redd), sums[slot], cta);
+      nc_tell((double)nc_most_of(redf), maxima[slot], cta);
     }
     if (has_sym) {
       nc_send(tile, false, E, ld, tm, tn, by_col[tn], t);
       if (tm != tn) nc_send(tile, true, E, ld, tn, tm, by_col[tm], t);
     }
     nc_cluster_sync();
-    // B = beta2 E E + beta1 E, whose product does not wait for the decision
-    if (has_sym && t < NC_WORK) nc_tile<false>(E, E, ld, kp, tm * 32, tn * 32, v);
+    if (has_sym && t < NC_WORK) nc_tile<false>(E, E, ld, kp, tm * 32, tn * 32, v);      // does not wait for the decision
     if (decides) {
-      const double tsq = nc_total(sums[slot]);
       double tmx = 0.0;
 #pragma unroll
       for (int i = 0; i < NC_CTAS; ++i) tmx = fmax(tmx, maxima[slot][i]);
-      const unsigned char entry = ns_control_decide(&ctl, (float)tmx, tsq, 0.0, k, cur, c);
-      if (cta == 0 && entry && k < 128) st->seg_log[k] = entry;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) coef[j] = ctl.coef[j];
-      done_s = ctl.ns_done;
+      decide(nc_total(sums[slot]), tmx);
     }
     slot ^= 1;
     __syncthreads();
     if (done_s != 0) break;
-    if (has_sym && t < NC_WORK) {
-#pragma unroll
-      for (int h = 0; h < 4; ++h)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) v[h][j] = fmaf(coef[2], v[h][j], coef[1] * E[(tm * 32 + r4 + h) * ld + tn * 32 + c4 + j]);
-      nc_put(tile, r4, 1, v);
-    }
-    if (in_place) nc_cluster_sync(); else __syncthreads();
+    if (has_sym && t < NC_WORK) { polynomial(); nc_put(tile, r2, 1, v); }
+    nc_cluster_sync();                           // (the residual has been read everywhere)
     if (has_sym) {
       nc_send(tile, false, Bm, ld, tm, tn, by_factor[tn], t);
       if (tm != tn) nc_send(tile, true, Bm, ld, tn, tm, by_factor[tm], t);
     }
     nc_cluster_sync();
-    // X_next = X B + gamma X, into the residual's place (nobody reads it any more) or X's
-    float* const Xn = in_place ? X : E;
-    float w[4][4];                               // a second tile's, where there are more than sixteen
-    auto next = [&](int f, float (&o)[4][4]) {
-      const int fm = f / tiles, fn = f - fm * tiles;
-      nc_tile<true>(X, Bm, ld, kp, fm * 32, fn * 32, o);
-#pragma unroll
-      for (int h = 0; h < 4; ++h)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) o[h][j] = fmaf(coef[0], X[(fm * 32 + (t >> 3) + 8 * h) * ld + fn * 32 + c4 + j], o[h][j]);
-    };
+    float w[2][4];                               // a second tile's
     const int f1 = cta + NC_CTAS;
     if (t < NC_WORK) {
-      if (cta < tiles * tiles) { next(cta, v); nc_put(tile, t >> 3, 8, v); }
+      next(cta, v);
+      nc_put(tile, t >> 3, 16, v);
       if (f1 < tiles * tiles) next(f1, w);
     }
-    if (in_place) nc_cluster_sync(); else __syncthreads();
-    if (cta < tiles * tiles) {
+    nc_cluster_sync();                           // (and so has X)
+    {
       const int fm = cta / tiles, fn = cta - fm * tiles;
-      nc_send(tile, false, Xn, ld, fm, fn, by_col[fn] | by_row[fm], t);
+      nc_send(tile, false, X, ld, fm, fn, by_col[fn] | by_row[fm], t);
     }
     if (f1 < tiles * tiles) {
       const int fm = f1 / tiles, fn = f1 - fm * tiles;
       __syncthreads();
-      if (t < NC_WORK) nc_put(tile, t >> 3, 8, w);
+      if (t < NC_WORK) nc_put(tile, t >> 3, 16, w);
       __syncthreads();
-      nc_send(tile, false, Xn, ld, fm, fn, by_col[fn] | by_row[fm], t);
+      nc_send(tile, false, X, ld, fm, fn, by_col[fn] | by_row[fm], t);
     }
     nc_cluster_sync();
-    if (!in_place) { E = X; X = Xn; }
+  }
   }
   // accept or reject (see ns_commit_kernel, ns_commit_state_kernel): each CTA holds the rows of X that its tiles of the last product read
   if (done_s == NS_DONE_CONVERGED) {
@@ -387,8 +540,8 @@ __host__ __device__ inline bool nc_accepts(double mx, double sq) { return (float
 
 __global__ void __launch_bounds__(NC_THREADS, 1) nc_check_kernel(const NcCheckArgs g) {
   extern __shared__ __align__(16) float nc_smem[];
-  __shared__ double redd[2];
-  __shared__ float redf[2];
+  __shared__ double redd[NC_WORK / 32];
+  __shared__ float redf[NC_WORK / 32];
   __shared__ double sums[NC_CTAS], maxima[NC_CTAS];
   const int cta = (int)blockIdx.x, t = threadIdx.x, d = g.d, kp = (d + 3) / 4 * 4;
   const int tiles = (d + 31) / 32, ld = nc_ld(tiles), sym_tiles = tiles * (tiles + 1) / 2;
@@ -398,7 +551,7 @@ __global__ void __launch_bounds__(NC_THREADS, 1) nc_check_kernel(const NcCheckAr
     X[i] = r < d && col < d ? g.src[(size_t)r * d + col] : 0.f;
   }
   __syncthreads();
-  float mx = 0.f, v[4][4];
+  float mx = 0.f, v[2][4];
   double sq = 0.0;
   if (cta < sym_tiles && t < NC_WORK) {
     int tn = 0;
@@ -406,8 +559,8 @@ __global__ void __launch_bounds__(NC_THREADS, 1) nc_check_kernel(const NcCheckAr
     const int tm = cta - tn * (tn + 1) / 2;
     nc_tile<false>(X, X, ld, kp, tm * 32, tn * 32, v);
 #pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      const int row = tm * 32 + 4 * (t >> 3) + h, col = tn * 32 + 4 * (t & 7);
+    for (int h = 0; h < 2; ++h) {
+      const int row = tm * 32 + 2 * (t >> 3) + h, col = tn * 32 + 4 * (t & 7);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         if (row >= d || col + j >= d) continue;
@@ -424,8 +577,8 @@ __global__ void __launch_bounds__(NC_THREADS, 1) nc_check_kernel(const NcCheckAr
   }
   nc_cluster_sync();                             // (the sums of this CTA, and every CTA runs before anything is written into its memory)
   if (t < 32) {
-    nc_tell(redd[0] + redd[1], sums, cta);
-    nc_tell((double)fmaxf(redf[0], redf[1]), maxima, cta);
+    nc_tell(nc_all_of(redd), sums, cta);
+    nc_tell((double)nc_most_of(redf), maxima, cta);
   }
   nc_cluster_sync();
   const double tsq = nc_total(sums);
@@ -464,11 +617,13 @@ inline bool nc_available(int dev) {
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = NC_CTAS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.attrs = at; cfg.numAttrs = 1;
-    const bool yes = cudaFuncSetAttribute(ns_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, nc_smem_bytes(NC_MAX_D)) == cudaSuccess &&
-                     cudaFuncSetAttribute(ns_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+    const bool yes = cudaFuncSetAttribute(ns_cluster_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, nc_smem_bytes(NC_MAX_D)) == cudaSuccess &&
+                     cudaFuncSetAttribute(ns_cluster_kernel<false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                     cudaFuncSetAttribute(ns_cluster_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, nc_smem_bytes(NC_SMALL_D)) == cudaSuccess &&
+                     cudaFuncSetAttribute(ns_cluster_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
                      cudaFuncSetAttribute(nc_check_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, nc_check_smem_bytes(NC_MAX_D)) == cudaSuccess &&
                      cudaFuncSetAttribute(nc_check_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-                     cudaOccupancyMaxActiveClusters(&n, ns_cluster_kernel, &cfg) == cudaSuccess && n > 0;
+                     cudaOccupancyMaxActiveClusters(&n, ns_cluster_kernel<false>, &cfg) == cudaSuccess && n > 0;
     if (!yes) cudaGetLastError();
     known[dev] = yes ? 1 : 2;
   }
@@ -481,7 +636,7 @@ inline int nc_launch(const NcArgs& a, cudaStream_t s) {
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = NC_CTAS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
   cfg.attrs = at; cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, ns_cluster_kernel, a) == cudaSuccess ? CONQUR_OK : CONQUR_ERR_CUDA;
+  return cudaLaunchKernelEx(&cfg, a.d <= NC_SMALL_D ? ns_cluster_kernel<true> : ns_cluster_kernel<false>, a) == cudaSuccess ? CONQUR_OK : CONQUR_ERR_CUDA;
 }
 
 }  // namespace conqur

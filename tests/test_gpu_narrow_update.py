@@ -127,3 +127,18 @@ def test_set_R_accepts_and_refuses_as_the_launches_do(d):
     # 5.01e-4 and the three bad ones for certain, 4.99e-4 never; the others lie within the entries' rounding (twice 2^-23 of a norm) and the
     # product's (d 2^-24) of the limit and go the same way for both, whichever that is
     assert 4 <= refused <= 7 and took[0] is False
+
+
+# one tile to sixteen, remainders, and the wider ones whose matrices are written in place
+@pytest.mark.parametrize("d", [2, 32, 33, 64, 97, 128, 129, 160])
+def test_repeated_updates_give_the_same_bits(d):
+    """Blocks of threads write into each other's operands: whatever their pace, the same statistics give the same rotation."""
+    m = _spectrum(d, "flat")
+    c = B.Context(d, 4096, in_dtype="f32", mode="exact")
+    seen = {}                                                # by the lifting count the update started with (learnt as they go) and its steps
+    for _ in range(150):
+        plan = c.get_stats().ns_lift_plan
+        c.set_M(m, 1.0, 4096)
+        c.update()
+        assert torch.equal(c.get_R(), seen.setdefault((plan, c.get_stats().ns_steps_used), c.get_R()))
+    assert len(seen) < 30
