@@ -202,7 +202,7 @@ hadamard_tc_kernel(const __grid_constant__ CUtensorMap tmX, TOut* Y, long long N
         ptx::tmem_ld32(t_addr, v0);
         ptx::tmem_ld32(t_addr + 32u, v1);
 #pragma unroll
-        for (int k = 0; k < 32; ++k) { const float a = v0[k], b = v1[k]; v0[k] = a + b; v1[k] = a - b; }
+        for (int k = 0; k < 32; k += 2) had_pair(v0[k], v0[k + 1], v1[k], v1[k + 1]);
         finish32(v0, chunk0);
         finish32(v1, chunk0 + 32);
       } else {
