@@ -62,12 +62,14 @@ struct Cfg {
   bool simt_ns;             // the Newton-Schulz products run on the fp32 CUDA-core kernels (exact mode)
 };
 
+// How many ranges of rows an exact step's accumulate product is shared out to, where the tiles of M alone leave most of the chip idle: a
+// chain of 256 rows takes 6 us whatever else runs.  Ranges of 128 rows, shorter ones up to eight of them; more partials take longer to add up
+// than they save.  Whole step, ranges of 256 rows -> these, us: d = 32  n = 256 25 -> 19, 700 31 -> 21, 2048 28 -> 24;  128  256 28 -> 22,
+// 1024 31 -> 25, 2048 31 -> 27;  512  700 56 -> 50, 2048 85 -> 80 (4 us of each is the launch that splitk_reduce_add_kernel took over)
 int pick_acc_splits(int d, int P, int64_t n_max) {
-  const int tiles = cdiv(d, SG_BM) * cdiv(d, SG_BN) * P;
-  if (tiles >= 148) return 1;
-  int s = std::min<int64_t>(16, std::max<int64_t>(1, 148 / tiles));
-  s = (int)std::min<int64_t>(s, std::max<int64_t>(1, n_max / 256));
-  return std::max(1, s);
+  const int64_t tiles = (int64_t)cdiv(d, SG_BM) * cdiv(d, SG_BN) * P;
+  const int64_t ranges = std::max<int64_t>(n_max / 128, std::min<int64_t>(8, n_max / 64));
+  return (int)std::max<int64_t>(1, std::min<int64_t>({16, 148 / tiles, ranges}));
 }
 
 bool make_layout(int d, const conqur_config* c, Layout* L) {
