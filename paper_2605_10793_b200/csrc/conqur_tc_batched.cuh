@@ -72,7 +72,7 @@ struct TcbStepArgs {
   QuantSpec qs;               // tcb_step_kernel: the per-token fake-quantisation
   float* M;                   // P x 128 x 128 fp32 (without the 1/sqrt(d))
   int S;                      // token splits per problem: work item i = (problem i / S, tiles [T (i % S) / S, T (i % S + 1) / S))
-  float* Mpart;               // S > 1: P * S partial cross-covariances (item order), summed into M by tcb_finish_kernel
+  float* Mpart;               // S > 1: P * S partial cross-covariances (item order), summed into M by tcb_sum_partials_kernel
   double* part_d;             // tcb_step_kernel: P * S * TCB_PARTS objective partials (one per epilogue warp), item order
   DevState* st;               // P
   long long* trace;           // measurement hook: when set, CTA 0 records SM-clock timestamps of its first TCB_TRACE_TILES tiles
@@ -320,7 +320,9 @@ tcb_step_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         // product uses.  It differs from ||x|| by at most ||R~ R~^T - I||_2 / 2 (about 1e-4 for a typical row at
         // d = 128), an order below the rounding of the scale itself to bf16 in the target tile, and costs no pass
         // over the input tile in shared memory, whose bandwidth bounds this kernel.  Every warp reads the whole
-        // row (both warps of a row pair get the same sum); the same pass finds the row's range.
+        // row (both warps of a row pair get the same sum); the same pass finds the row's range.  (Half a row each and an exchange
+        // through the target buffer: its latency is on every tile's path; 1024 problems x 4096 rows, symmetric 386 -> 406 us, zero-point
+        // 443 -> 433.)
         if (tr_epi) TCB_TR(it, TCB_EV_NORM_BEGIN);
         float ss;
         float vmax = sym ? 0.f : -3.0e38f, vmin = 3.0e38f;
@@ -755,8 +757,14 @@ tcb_step_plain_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         nonfinite |= __shfl_xor_sync(0xffffffffu, nonfinite, o);
       }
       if (lane == 0) {
-        if (skipped) atomicAdd(reinterpret_cast<unsigned long long*>(&g.st[p].step_skipped), (unsigned long long)skipped);
-        if (nonfinite) atomicOr(&g.st[p].status_flags, STATUS_FLAG_NONFINITE);
+        DevState* sp = g.st + p;
+        if (g.S == 1) {                            // the problem is this CTA's alone: its rows are counted here, not by a launch
+                                                   // behind (1024 problems: 6 us and the gap before it)
+          const int add = (warp == TCBT_NORM_WARP0 ? g.n : 0) - skipped;
+          if (add) atomicAdd(reinterpret_cast<unsigned long long*>(&sp->N), (unsigned long long)(long long)add);
+          if (skipped) atomicAdd(reinterpret_cast<unsigned long long*>(&sp->n_skipped), (unsigned long long)skipped);
+        } else if (skipped) atomicAdd(reinterpret_cast<unsigned long long*>(&sp->step_skipped), (unsigned long long)skipped);
+        if (nonfinite) atomicOr(&sp->status_flags, STATUS_FLAG_NONFINITE);
       }
     }
   } else {
@@ -1012,7 +1020,8 @@ inline int tcb_step(TcHost& h, cudaStream_t s, const void* X, int in_dtype, int6
   if (h.prof) h.prof->count(K_ROTATE);
   const StepSums sums{h.qs.bits > 0 ? h.part_d : nullptr, S * TCB_PARTS, n, 1.0 / std::sqrt((double)TCB_D), nullptr, 0};
   if (S > 1) tcb_sum_partials_kernel<<<dim3(16, np), 256, 0, s>>>(g.M, g.Mpart, S, g.st, sums);
-  else finalize_step_kernel<<<np, 256, 0, s>>>(g.st, sums);
+  else if (h.qs.bits > 0) finalize_step_kernel<<<np, 256, 0, s>>>(g.st, sums);      // plain steps have counted their rows themselves
+  else return CONQUR_OK;
   if (cudaGetLastError() != cudaSuccess) return CONQUR_ERR_CUDA;
   if (h.prof) h.prof->count(K_OTHER);
   return CONQUR_OK;

@@ -64,3 +64,23 @@ def test_codes_beyond_what_an_addition_rounds():
     assert torch.equal(signs.float(), torch.sign(x))
     # every coordinate is quantised to within half a step of 2^-20 / 15: sum |y| / (||y|| sqrt(d)) = 1
     assert ((j - n).abs() <= 1e-5 * n).all()
+
+
+# rows counted and skipped (zero, NaN) over three steps: a problem of one tile or more on one CTA, or shared out over several
+@pytest.mark.parametrize("bits", [0, 4])
+@pytest.mark.parametrize("problems,n", [(2, 1), (3, 200), (3, 700), (150, 300)])
+def test_rows_counted(problems, n, bits):
+    d = 128
+    g = torch.Generator(device="cuda").manual_seed(problems + n)
+    x = torch.randn(problems, n, d, generator=g, device="cuda").bfloat16()
+    bad = torch.zeros(problems, n, dtype=torch.bool, device="cuda")
+    bad[0, 0] = bad[-1, n // 2] = bad[-1, n - 1] = True
+    x[0, 0] = 0
+    x[-1, n // 2] = float("nan")
+    x[-1, n - 1] = 0
+    c = B.Context(d, n, in_dtype="bf16", batch=problems, quant_bits=bits)
+    for _ in range(3):
+        c.step_batched(x, n, d, n * d)
+    _, cnt = c.get_objective(check=False)
+    assert cnt.tolist() == (3 * (n - bad.sum(dim=1))).tolist()
+    assert c.get_stats().n_skipped == 3 * int(bad.sum())
