@@ -16,7 +16,8 @@
  *
  * Ordering: conqur_step / conqur_step_batched(_range) / conqur_update only ENQUEUE work on
  * the context's stream and return; X must stay valid until that work has run.
- * The conqur_get_* calls synchronise the stream.  A context is not thread-safe.
+ * The conqur_get_* calls synchronise the stream: everything enqueued on it before has done its work when they return (the
+ * driver may report their own last, short kernel as running for a few microseconds more).  A context is not thread-safe.
  *
  * Errors: every call returns CONQUR_OK (0) or a negative conqur_status.  Errors
  * found on the host change nothing.  Conditions found on the device (non-finite
