@@ -66,9 +66,10 @@ def test_codes_beyond_what_an_addition_rounds():
     assert ((j - n).abs() <= 1e-5 * n).all()
 
 
-# rows counted and skipped (zero, NaN) over three steps: a problem of one tile or more on one CTA, or shared out over several
+# rows counted and skipped (zero, NaN) over three steps: a problem of one tile or more on one CTA, or shared out over several; more problems
+# than a read's results fit in page-locked memory
 @pytest.mark.parametrize("bits", [0, 4])
-@pytest.mark.parametrize("problems,n", [(2, 1), (3, 200), (3, 700), (150, 300)])
+@pytest.mark.parametrize("problems,n", [(2, 1), (3, 200), (3, 700), (150, 300), (2100, 2)])
 def test_rows_counted(problems, n, bits):
     d = 128
     g = torch.Generator(device="cuda").manual_seed(problems + n)
@@ -81,6 +82,13 @@ def test_rows_counted(problems, n, bits):
     c = B.Context(d, n, in_dtype="bf16", batch=problems, quant_bits=bits)
     for _ in range(3):
         c.step_batched(x, n, d, n * d)
-    _, cnt = c.get_objective(check=False)
-    assert cnt.tolist() == (3 * (n - bad.sum(dim=1))).tolist()
+    for _ in range(2):                                   # a second read finds the same, and the same status
+        j, cnt = c.get_objective(check=False)
+        assert cnt.tolist() == (3 * (n - bad.sum(dim=1))).tolist()
+        if bool(x.isnan().any()):
+            with pytest.raises(RuntimeError):
+                c.get_objective()
+    if bits == 0:                                        # <R, M> in double, M as read out (rounded to fp32 once more)
+        part = c.get_R(check=False).double() * c.get_M(check=False).double()
+        assert ((torch.from_numpy(j).cuda() - part.sum(dim=(1, 2))).abs() <= 2.0 ** -23 * part.abs().sum(dim=(1, 2))).all()
     assert c.get_stats().n_skipped == 3 * int(bad.sum())
