@@ -681,7 +681,7 @@ int update_impl(conqur_ctx* c) {
   if (g.mode == CONQUR_TC_BF16 && g.P > 1) {
     // many small problems: the whole iteration of a problem runs inside one CTA
     const NsControlParams ncp{c->at<SchedEntry>(c->L.sched), c->n_sched, c->n_lift_init, g.ns_max_steps, g.d, 1,
-                              g.orth_tol, g.fro_tol, g.margin, g.lo_budget, 1.0 / (double)g.d, 1, 1.f / 2048.f};
+                              g.orth_tol, g.fro_tol, g.margin, g.lo_budget, 1.0 / (double)g.d, 0, 1.f / 256.f};
     return tcb_update(c->tc, c->stream, ncp, g.prior_rel, g.margin);
   }
   if (c->one_cluster) {

@@ -873,7 +873,7 @@ struct NsControlParams {
   float lo_budget;          // tensor-core mode: the iterate enters the last product as hi + lo while d lo_unit / growth exceeds this
   double inv_d;             // 1 / d (the decision runs on one thread between two products: no divisions there)
   int full_check;           // 1: a rotation is accepted only on a residual of all three passes (seg_e == 3)
-  float lo_unit;            // rounding of the operand of the one-pass form: 2^-11 (fp16)
+  float lo_unit;            // rounding of the one-pass form's operand: 2^-8 where it is the bf16 hi part, 2^-11 for the fp16 copy
 };
 
 // The decision itself (one thread): tmx = max|G - I|, tsq = ||G - I||_F^2, ttr = tr G of step k.
@@ -974,8 +974,7 @@ __device__ __forceinline__ unsigned char ns_control_decide(NsCtl* s, float tmx, 
 // to X^T X - I.  One over the fp16 copy otherwise (see tc_ns_residual), except that a caller's threshold (e1_tau > 0, ns_tau_kernel)
 // asks for three wherever tau has reached it.  (max|X^T X - I| of accepted rotations, d = 1280 .. 4096: 4e-5 .. 9e-5 with one
 // pass in that last step, 6e-6 .. 1e-5 with three; at d = 512 one pass cost every update a step more.)
-template <typename State>
-__device__ __forceinline__ bool ns_full_residual(const State* s, int n_sched, int max_steps) {
+__device__ __forceinline__ bool ns_full_residual(const DevState* s, int n_sched, int max_steps) {
   return s->ns_idx >= n_sched - 1 || s->ns_steps_used >= max_steps;
 }
 

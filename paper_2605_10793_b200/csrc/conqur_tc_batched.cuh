@@ -1029,45 +1029,21 @@ inline int tcb_step(TcHost& h, cudaStream_t s, const void* X, int in_dtype, int6
 
 // ------------------------------------------------------------------ fused polar update of many 128 x 128 problems
 // One CTA runs the whole Newton-Schulz iteration of one problem at a time with everything on chip: the iterate as
-// an fp16 (hi, lo) pair in shared memory, G = X^T X and the products in TMEM, the scalar control in one thread.
+// a bf16 (hi, lo) pair in shared memory, G = X^T X and the products in TMEM, the scalar control in one thread.
 // Per step (phases are strictly sequential; 128 threads = 128 rows):
-//   G = X^T X (hi hi; + hi lo + lo hi where the rotation may be accepted)   -> TMEM [0,128)
-//   statistics of G - I, control decision, E = G - tau I as fp16           -> shared memory
+//   G = X^T X (hi hi + hi lo + lo hi)      -> TMEM [0,128)
+//   statistics of G - I, control decision, E = G - tau I as bf16           -> shared memory
 //   E E                                     -> TMEM [128,256)
-//   B = beta2 E E + beta1 E - kappa I as fp16                              -> shared memory (over E)
+//   B = beta2 E E + beta1 E - kappa I as bf16                              -> shared memory (over E)
 //   X B (hi, + lo while the schedule asks)  -> TMEM [0,128)
 //   X <- (gamma + kappa) X + X B, tau = ||X||_F^2 / d, split into (hi, lo) -> shared memory
 // Two CTAs fit one SM (96 KB of shared memory and 256 TMEM columns each), so one problem's element-wise phases
-// overlap the other's products.  With a bf16 pair, E and B in bf16 and three-pass G throughout 1024 problems took 297 us for 280 (kernel
-// time in a profile), and the rotation lay 3 to 6 times as far from the 64-bit polar factor (statistics of 16 d rows 1.5e-3 of its norm for
-// 0.5e-3, condition 1e4 5.4e-3 for 1.0e-3, 1e6 3.2e-2 for 0.7e-2).
+// overlap the other's products.
+// The pair is bf16, although an fp16 one (times 2^12, the lower half times 2^12 more), which takes one-pass G between the steps, ran 1024 problems in
+// 280 us for 297 and lay 3 to 8 times closer to the polar factor on ordinary statistics: its least unit is 2^-48 of the norm, and rows or columns of M that
+// lie 1e-10 and further below the others came out wrong without an error (a third of the rows at 1e-11, 1e-12, 1e-13: off by 0.20, 0.25, 0.65
+// of the rotation's norm, by 0.019 to 0.020 in this form), or were gone.
 constexpr int TCBU_THREADS = 256;            // 128 rows x 2 column halves
-// The iterate is an fp16 pair, X = (hi + lo / LO) / F: hi alone (2^-12) serves the products between the steps, the pair (2^-24 of an entry, or
-// 2^-49 where that is more) those that small singular values or the rotation's acceptance hang on.  The products bring lo's share down by
-// themselves: an instruction scales the accumulator it adds to by 2^-12.
-constexpr float TCBU_F = TC_F16_SCALE, TCBU_LO = 4096.f, TCBU_B = TC_B16_SCALE;
-constexpr float TCBU_G = 1.f / (TCBU_F * TCBU_F);       // what X^T X and E E come out multiplied by, undone
-namespace ptx {
-// D(tmem) = A * B + D 2^-12 (fp16 operands in shared memory), as the form of umma_bf16_by for one CTA
-__device__ __forceinline__ void umma_f16_onto_scaled_by(uint32_t leader, uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc) {
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.eq.b32 p, 0, 0;\n\tsetp.ne.b32 q, %4, 0;\n\t"
-      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %5, %5, %5}, p, 12;\n\t}"
-      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(leader), "r"(0u)
-      : "memory");
-}
-}  // namespace ptx
-// Two numbers (times F) as their pair.
-__device__ __forceinline__ void tcbu_split(float a, float b, uint32_t& wh, uint32_t& wl) {
-  wh = f16x2_pack(a, b);
-  const float2 h = f16x2_unpack(wh);
-  wl = f16x2_pack((a - h.x) * TCBU_LO, (b - h.y) * TCBU_LO);
-}
-__device__ __forceinline__ float2 tcbu_join(uint32_t wh, uint32_t wl) {
-  const float2 h = f16x2_unpack(wh), l = f16x2_unpack(wl);
-  return make_float2(fmaf(l.x, 1.f / TCBU_LO, h.x), fmaf(l.y, 1.f / TCBU_LO, h.y));
-}
 constexpr int TCBU_SMEM_BYTES = 3 * TCB_TILE_BYTES + 4096 + 1024;
 
 struct TcbUpdAux {
@@ -1077,7 +1053,7 @@ struct TcbUpdAux {
   int done;
   float tau, x0s, lam;
   float coef[4];
-  int seg_x, seg_e;
+  int seg_x;
   double red_d[8], red_t[8];
   float red_f[8];
   DevState state;                    // the problem's state while it is being iterated (written back once at the end)
@@ -1133,7 +1109,7 @@ __global__ void __launch_bounds__(TCBU_THREADS, 2) tcb_update_kernel(const TcbUp
   const uint32_t tmem_base = aux->tmem_base;
   const uint32_t t_row = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);      // this warp's 32 TMEM lanes
   const uint32_t aXh = ptx::smem_u32(sXh), aXl = ptx::smem_u32(sXl), aEB = ptx::smem_u32(sEB);
-  const uint32_t idesc_base = (1u << 4) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);      // fp16 operands
+  const uint32_t idesc_base = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
   const uint32_t idesc_mm = idesc_base | (1u << 15) | (1u << 16);       // both operands read "transposed" (MN-major)
   const uint32_t idesc_km = idesc_base | (1u << 16);                    // A as stored (K-major), B MN-major
   const uint32_t mbar_a = ptx::smem_u32(&aux->mbar);
@@ -1165,19 +1141,13 @@ __global__ void __launch_bounds__(TCBU_THREADS, 2) tcb_update_kernel(const TcbUp
     ptx::tc_fence_after();
     return okw;
   };
-  auto issue_gram = [&](uint32_t leader, bool full) {               // G = X^T X: hi hi, or lo hi + hi lo first
-    if (full) {
+  auto issue_gram = [&](uint32_t leader) {                          // G = X^T X (hi hi + hi lo + lo hi)
+    const uint32_t aa[3] = {aXh, aXh, aXl}, bb[3] = {aXh, aXl, aXh};
 #pragma unroll
-      for (int seg = 0; seg < 2; ++seg)
+    for (int seg = 0; seg < 3; ++seg)
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-          ptx::umma_bf16_by<false>(leader, tmem_base, desc_mn(seg ? aXh : aXl, j), desc_mn(seg ? aXl : aXh, j), idesc_mm, (seg > 0 || j > 0) ? 1u : 0u);
-      ptx::umma_f16_onto_scaled_by(leader, tmem_base, desc_mn(aXh, 0), desc_mn(aXh, 0), idesc_mm);
-    } else {
-      ptx::umma_bf16_by<false>(leader, tmem_base, desc_mn(aXh, 0), desc_mn(aXh, 0), idesc_mm, 0u);
-    }
-#pragma unroll
-    for (int j = 1; j < 8; ++j) ptx::umma_bf16_by<false>(leader, tmem_base, desc_mn(aXh, j), desc_mn(aXh, j), idesc_mm, 1u);
+      for (int j = 0; j < 8; ++j)
+        ptx::umma_bf16_by<false>(leader, tmem_base, desc_mn(aa[seg], j), desc_mn(bb[seg], j), idesc_mm, (seg > 0 || j > 0) ? 1u : 0u);
   };
 
   NsCtl ctl{};                                     // thread 0 only
@@ -1218,7 +1188,7 @@ __global__ void __launch_bounds__(TCBU_THREADS, 2) tcb_update_kernel(const TcbUp
       s->lam = lam; s->scale = fro;
       s->x0_scale = ok ? 1.0f / (fro * (1.0f + g.margin)) : 0.f;
       s->ns_done = ok ? 0 : NS_DONE_FAILED;
-      s->ns_steps_used = 0; s->ns_final_buf = 0; s->seg_x = 2; s->seg_e = 1;
+      s->ns_steps_used = 0; s->ns_final_buf = 0; s->seg_x = 2;
       ns_arm_lifting(s, g.ncp.n_lift_init);
       s->tau = 1.0f / ((1.0f + g.margin) * (1.0f + g.margin) * (float)TCB_D);
       aux->done = s->ns_done; aux->tau = s->tau; aux->x0s = s->x0_scale; aux->lam = lam;
@@ -1236,13 +1206,13 @@ __global__ void __launch_bounds__(TCBU_THREADS, 2) tcb_update_kernel(const TcbUp
           a.x = fmaf(lam, q.x, a.x); a.y = fmaf(lam, q.y, a.y); a.z = fmaf(lam, q.z, a.z); a.w = fmaf(lam, q.w, a.w);
         }
         uint32_t h0, h1, l0, l1;
-        tcbu_split(a.x * x0s * TCBU_F, a.y * x0s * TCBU_F, h0, l0);
-        tcbu_split(a.z * x0s * TCBU_F, a.w * x0s * TCBU_F, h1, l1);
+        bf16x2_split(a.x * x0s, a.y * x0s, h0, l0);
+        bf16x2_split(a.z * x0s, a.w * x0s, h1, l1);
         const uint32_t off = tcb_piece(i >> 5, (i & 31) >> 1) + (uint32_t)(i & 1) * 8u;
         *reinterpret_cast<uint2*>(sXh + off) = make_uint2(h0, h1);
         *reinterpret_cast<uint2*>(sXl + off) = make_uint2(l0, l1);
       }
-      issue_products([&](uint32_t leader) { issue_gram(leader, false); });
+      issue_products(issue_gram);
       // the next problem's matrices come into the L2 while this one is iterated (read from memory when they were needed, they took
       // 19 k of a problem's 187 k SM cycles: all blocks ask for theirs at about the same time; 1024 problems 317 -> 310 us, 600 229
       // -> 226, 320 the same)
@@ -1256,9 +1226,8 @@ __global__ void __launch_bounds__(TCBU_THREADS, 2) tcb_update_kernel(const TcbUp
         // ---- G = X^T X (issued before the loop / at the end of the previous step)
         gram_in_flight = false;
         if (!wait_products()) { timed_out = true; break; }
-        // ---- statistics of G - I; E = G - tau I (all in units of the product's: the scales are powers of two)
+        // ---- statistics of G - I; E = G - tau I
         const float tau = aux->tau;
-        constexpr float ONE = 1.f / TCBU_G;
         float mx = 0.f, tr = 0.f;
         double sq = 0.0;
         // (the diagonal lies in one 32-column chunk per warp, c_diag: only that chunk pays for finding it)
@@ -1271,13 +1240,13 @@ __global__ void __launch_bounds__(TCBU_THREADS, 2) tcb_update_kernel(const TcbUp
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
             float e1 = v[i];
-            if (decltype(has_diag)::value && i == dcol) { tr += v[i]; e1 -= ONE; v[i] -= tau * ONE; }
+            if (decltype(has_diag)::value && i == dcol) { tr += v[i]; e1 -= 1.f; v[i] -= tau; }
             mx = fmaxf(mx, fabsf(e1));
             sq32 = fmaf(e1, e1, sq32);
           }
           sq += (double)sq32;
 #pragma unroll
-          for (int i = 0; i < 16; ++i) w[i] = f16x2_pack(v[2 * i] * (1.f / TCBU_F), v[2 * i + 1] * (1.f / TCBU_F));      // E F
+          for (int i = 0; i < 16; ++i) w[i] = bf16x2_pack(v[2 * i], v[2 * i + 1]);
 #pragma unroll
           for (int q4 = 0; q4 < 4; ++q4)
             *reinterpret_cast<uint4*>(sEB + tcb_piece(r, c * 4 + q4)) = make_uint4(w[4 * q4], w[4 * q4 + 1], w[4 * q4 + 2], w[4 * q4 + 3]);
@@ -1287,8 +1256,8 @@ __global__ void __launch_bounds__(TCBU_THREADS, 2) tcb_update_kernel(const TcbUp
           if (c == c_diag) resid_chunk(c, std::true_type{}); else resid_chunk(c, std::false_type{});
         }
         {
-          const double wsq = warp_sum_d(sq) * ((double)TCBU_G * TCBU_G), wtr = warp_sum_d((double)tr) * TCBU_G;
-          const float wmx = warp_max(mx) * TCBU_G;
+          const double wsq = warp_sum_d(sq), wtr = warp_sum_d((double)tr);
+          const float wmx = warp_max(mx);
           if (lane == 0) { aux->red_d[warp] = wsq; aux->red_t[warp] = wtr; aux->red_f[warp] = wmx; }
         }
         // ---- E E, which does not depend on the control decision: issued first, the decision is taken while it runs
@@ -1307,15 +1276,12 @@ __global__ void __launch_bounds__(TCBU_THREADS, 2) tcb_update_kernel(const TcbUp
           aux->done = ctl.ns_done;
           aux->coef[0] = ctl.coef[0]; aux->coef[1] = ctl.coef[1]; aux->coef[2] = ctl.coef[2]; aux->coef[3] = ctl.coef[3];
           aux->seg_x = ctl.seg_x;
-          ctl.seg_e = ns_full_residual(&ctl, ncp.n_sched, ncp.max_steps) ? 3 : 1;
-          aux->seg_e = ctl.seg_e;
         }
         __syncthreads();
         if (!wait_products()) { timed_out = true; break; }
         if (aux->done) break;
-        const float cg = aux->coef[0], cb1 = aux->coef[1] * (TCBU_G * TCBU_B), cb2 = aux->coef[2] * (TCBU_G * TCBU_B), ck = aux->coef[3] * TCBU_B;
+        const float cg = aux->coef[0], cb1 = aux->coef[1], cb2 = aux->coef[2], ck = aux->coef[3];
         const int seg_x = aux->seg_x;
-        const bool full = aux->seg_e == 3;               // the next step's G
         // ---- B = beta2 E E + beta1 E - kappa I (over E: the product that read it has finished)
         auto poly_chunk = [&](int c, auto has_diag) {
           float gq[32], ee[32];
@@ -1326,13 +1292,13 @@ __global__ void __launch_bounds__(TCBU_THREADS, 2) tcb_update_kernel(const TcbUp
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
             const bool on_diag = decltype(has_diag)::value && i == dcol;
-            const float e = on_diag ? gq[i] - tau * ONE : gq[i];
+            const float e = on_diag ? gq[i] - tau : gq[i];
             float b = fmaf(cb2, ee[i], cb1 * e);
             if (on_diag) b -= ck;
             ee[i] = b;
           }
 #pragma unroll
-          for (int i = 0; i < 16; ++i) w[i] = f16x2_pack(ee[2 * i], ee[2 * i + 1]);                    // B times its scale
+          for (int i = 0; i < 16; ++i) w[i] = bf16x2_pack(ee[2 * i], ee[2 * i + 1]);
 #pragma unroll
           for (int q4 = 0; q4 < 4; ++q4)
             *reinterpret_cast<uint4*>(sEB + tcb_piece(r, c * 4 + q4)) = make_uint4(w[4 * q4], w[4 * q4 + 1], w[4 * q4 + 2], w[4 * q4 + 3]);
@@ -1343,15 +1309,12 @@ __global__ void __launch_bounds__(TCBU_THREADS, 2) tcb_update_kernel(const TcbUp
         }
         // ---- X B
         issue_products([&](uint32_t leader) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) ptx::umma_bf16_by<false>(leader, tmem_base, desc_k(aXh, j), desc_mn(aEB, j), idesc_km, j > 0 ? 1u : 0u);
           if (seg_x > 1) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) ptx::umma_bf16_by<false>(leader, tmem_base, desc_k(aXl, j), desc_mn(aEB, j), idesc_km, j > 0 ? 1u : 0u);
-            ptx::umma_f16_onto_scaled_by(leader, tmem_base, desc_k(aXh, 0), desc_mn(aEB, 0), idesc_km);
-          } else {
-            ptx::umma_bf16_by<false>(leader, tmem_base, desc_k(aXh, 0), desc_mn(aEB, 0), idesc_km, 0u);
+            for (int j = 0; j < 8; ++j) ptx::umma_bf16_by<false>(leader, tmem_base, desc_k(aXl, j), desc_mn(aEB, j), idesc_km, 1u);
           }
-#pragma unroll
-          for (int j = 1; j < 8; ++j) ptx::umma_bf16_by<false>(leader, tmem_base, desc_k(aXh, j), desc_mn(aEB, j), idesc_km, 1u);
         });
         if (!wait_products()) { timed_out = true; break; }
         // ---- X <- (gamma + kappa) X + X B; tau of the next step
@@ -1369,10 +1332,11 @@ __global__ void __launch_bounds__(TCBU_THREADS, 2) tcb_update_kernel(const TcbUp
             uint32_t wh[4], wl[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-              const float2 x = tcbu_join(hh[e], ll[e]);
-              const float a = fmaf(v[q4 * 8 + 2 * e], 1.f / TCBU_B, cg * x.x), b = fmaf(v[q4 * 8 + 2 * e + 1], 1.f / TCBU_B, cg * x.y);
+              const float xa = __uint_as_float(hh[e] << 16) + __uint_as_float(ll[e] << 16);
+              const float xb = __uint_as_float(hh[e] & 0xffff0000u) + __uint_as_float(ll[e] & 0xffff0000u);
+              const float a = fmaf(cg, xa, v[q4 * 8 + 2 * e]), b = fmaf(cg, xb, v[q4 * 8 + 2 * e + 1]);
               x2f = fmaf(a, a, fmaf(b, b, x2f));
-              tcbu_split(a, b, wh[e], wl[e]);
+              bf16x2_split(a, b, wh[e], wl[e]);
             }
             *reinterpret_cast<uint4*>(sXh + off) = make_uint4(wh[0], wh[1], wh[2], wh[3]);
             *reinterpret_cast<uint4*>(sXl + off) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
@@ -1380,11 +1344,11 @@ __global__ void __launch_bounds__(TCBU_THREADS, 2) tcb_update_kernel(const TcbUp
           x2 += (double)x2f;
         }
         {
-          const double wx2 = warp_sum_d(x2) * TCBU_G;
+          const double wx2 = warp_sum_d(x2);
           if (lane == 0) aux->red_d[warp] = wx2;
         }
         // ---- the next step's G needs the new iterate but not its tau: issued now, tau is summed while it runs
-        if (k < ncp.max_steps) { issue_products([&](uint32_t leader) { issue_gram(leader, full); }); gram_in_flight = true; } else { __syncthreads(); }
+        if (k < ncp.max_steps) { issue_products(issue_gram); gram_in_flight = true; } else { __syncthreads(); }
         if (threadIdx.x == 0) {
           const double tx2 = ((aux->red_d[0] + aux->red_d[1]) + (aux->red_d[2] + aux->red_d[3])) +
                              ((aux->red_d[4] + aux->red_d[5]) + (aux->red_d[6] + aux->red_d[7]));
@@ -1411,8 +1375,10 @@ __global__ void __launch_bounds__(TCBU_THREADS, 2) tcb_update_kernel(const TcbUp
         const uint32_t off = tcb_piece(i >> 5, (i & 31) >> 1) + (uint32_t)(i & 1) * 8u;
         const uint2 h2 = *reinterpret_cast<const uint2*>(sXh + off), l2 = *reinterpret_cast<const uint2*>(sXl + off);
         float4 o;
-        const float2 xa = tcbu_join(h2.x, l2.x), xb = tcbu_join(h2.y, l2.y);
-        o.x = xa.x * (1.f / TCBU_F); o.y = xa.y * (1.f / TCBU_F); o.z = xb.x * (1.f / TCBU_F); o.w = xb.y * (1.f / TCBU_F);
+        o.x = __uint_as_float(h2.x << 16) + __uint_as_float(l2.x << 16);
+        o.y = __uint_as_float(h2.x & 0xffff0000u) + __uint_as_float(l2.x & 0xffff0000u);
+        o.z = __uint_as_float(h2.y << 16) + __uint_as_float(l2.y << 16);
+        o.w = __uint_as_float(h2.y & 0xffff0000u) + __uint_as_float(l2.y & 0xffff0000u);
         Ro[i] = o;
         Rbo[i] = make_uint2(bf16x2_pack(o.x, o.y), bf16x2_pack(o.z, o.w));
         Mo[i] = make_float4(0.f, 0.f, 0.f, 0.f);
