@@ -365,6 +365,15 @@ int conqur_debug_gemm(const void* A_dev, const void* B_dev, float* D_dev, int32_
 int conqur_debug_wait_timeout(void* scratch_dev, int64_t limit_cycles, void* cuda_stream);
 
 /*
+ * The same for the one-kernel update of a narrow exact context (one problem, d <= 128; others return
+ * CONQUR_ERR_UNSUPPORTED): in every conqur_update from now on thread block `block` (0 .. 15; below 0: none, the state
+ * after conqur_init) waits in step `step` (0 .. ns_max_steps) for bytes that no other block sends, and waits end after
+ * about a millisecond.  An update that gets that far, and whose block takes part in it, keeps R, M, J, N and the learnt
+ * step count and latches CONQUR_ERR_TIMEOUT.  Enqueues nothing.
+ */
+int conqur_debug_lose_wait(conqur_ctx* ctx, int32_t block, int32_t step);
+
+/*
  * The corner objective of one batch without any device-memory allocation by anyone
  * (the paper has no counterpart; this serves callers that cannot call cudaMalloc -- e.g. code
  * running under a runtime that owns all device memory, or a plugin in a process whose device

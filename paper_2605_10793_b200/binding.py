@@ -33,7 +33,7 @@ EXPORTS = [
     "conqur_workspace_bytes", "conqur_init", "conqur_destroy", "conqur_set_R", "conqur_step",
     "conqur_step_batched", "conqur_step_batched_range", "conqur_update", "conqur_get_R", "conqur_get_objective", "conqur_get_objective_async", "conqur_get_M",
     "conqur_set_M", "conqur_debug_get_signs", "conqur_debug_capture_signs", "conqur_get_stats", "conqur_debug_check_canaries", "conqur_debug_trace_heads", "conqur_plan_schedule", "conqur_debug_gemm",
-    "conqur_set_profiling", "conqur_get_profile", "conqur_objective_noalloc", "conqur_debug_wait_timeout",
+    "conqur_set_profiling", "conqur_get_profile", "conqur_objective_noalloc", "conqur_debug_wait_timeout", "conqur_debug_lose_wait",
     "conqur_get_diagnostics", "conqur_fold_scratch_bytes", "conqur_fold_weight", "conqur_hadamard_rows", "conqur_hadamard_status",
     "conqur_strerror",
 ]
@@ -140,6 +140,8 @@ def load() -> C.CDLL:
     lib.conqur_debug_gemm.argtypes = [vp, vp, vp, i32, i32, i32, i32, i32, i32, vp, vp]
     lib.conqur_get_diagnostics.restype = C.c_int
     lib.conqur_get_diagnostics.argtypes = [vp, C.POINTER(conqur_diagnostics)]
+    lib.conqur_debug_lose_wait.restype = C.c_int
+    lib.conqur_debug_lose_wait.argtypes = [vp, i32, i32]
     lib.conqur_debug_wait_timeout.restype = C.c_int
     lib.conqur_debug_wait_timeout.argtypes = [vp, i64, vp]
     lib.conqur_fold_scratch_bytes.restype = i64
@@ -499,6 +501,10 @@ class Context:
         self._trace_buf = buf
         ptr, cap = (0, 0) if buf is None else (buf.data_ptr(), buf.numel())
         self._chk(load().conqur_debug_trace_heads(self.h, ptr, cap), "conqur_debug_trace_heads")
+
+    def debug_lose_wait(self, block: int, step: int = 0):
+        """Narrow exact contexts: from now on updates run into a bounded wait that expires (see include/conqur.h; block < 0: off)."""
+        self._chk(load().conqur_debug_lose_wait(self.h, block, step), "conqur_debug_lose_wait")
 
     def check_canaries(self) -> int:
         """Guard bands of the workspace that were overwritten (0 = intact); needs CONQUR_DEBUG_CANARIES."""

@@ -197,6 +197,7 @@ struct conqur_ctx {
   int last_np;               // problems the last step call covered
   bool last_pieces = false;  // the last step left its targets as bf16 pieces (exact mode)
   bool one_cluster = false;  // exact mode, one narrow problem: its update is one kernel (conqur_ns_cluster.cuh)
+  int nc_lose = -1;          // conqur_debug_lose_wait
   int device = 0;
   int sp_pairs = 0;          // exact contexts with pieces: CTA pairs that can be co-resident (0: CUDA cores only)
   int64_t pending_rows = 0;  // deferring context: rows staged but not yet run through the two products
@@ -692,6 +693,8 @@ int update_impl(conqur_ctx* c) {
                           g.fro_tol, g.margin, g.lo_budget, 1.0 / (double)g.d, 0, 1.f / 2048.f};
     a.d = g.d; a.n_endgame = c->n_sched - 1;
     a.prior_rel = g.prior_rel; a.inv_sqrt_d = (float)(1.0 / std::sqrt((double)g.d)); a.margin = g.margin;
+    a.lose = c->nc_lose;
+    a.wait_limit = c->nc_lose < 0 ? 4000000000ll : 2000000ll;      // two seconds, or about a millisecond
     const int rc = nc_launch(a, c->stream);
     if (rc) return rc;
     c->prof.count(K_NS_NEXT);
@@ -1345,6 +1348,13 @@ extern "C" int conqur_debug_gemm(const void* A_dev, const void* B_dev, float* D_
   CQ_CUDA(cudaMemcpyAsync(&h, scratch_dev, sizeof(DevState), cudaMemcpyDeviceToHost, s));
   CQ_CUDA(cudaStreamSynchronize(s));
   return flags_to_status(h.status_flags);
+}
+
+extern "C" int conqur_debug_lose_wait(conqur_ctx* c, int32_t block, int32_t step) {
+  if (!c || block >= NC_CTAS || (block >= 0 && (step < 0 || step > c->cfg.ns_max_steps))) return CONQUR_ERR_INVALID_ARG;
+  if (!c->one_cluster || c->cfg.d > NC_SMALL_D) return CONQUR_ERR_UNSUPPORTED;
+  c->nc_lose = block < 0 ? -1 : block + NC_CTAS * step;
+  return CONQUR_OK;
 }
 
 extern "C" int conqur_debug_wait_timeout(void* scratch_dev, int64_t limit_cycles, void* cuda_stream) {

@@ -37,6 +37,8 @@ struct NcArgs {
   NsControlParams c;
   int d, n_endgame;
   float prior_rel, inv_sqrt_d, margin;
+  long long wait_limit;                          // SM cycles a wait for bytes lasts at most
+  int lose;                                      // test hook: CTA `lose % 16` waits in step `lose / 16` for bytes that nobody sends (-1: none)
 };
 
 // A matrix in shared memory: 32 T rows of 32 T columns and 4 floats against bank conflicts, zeros past d.  Up to four tiles a side three
@@ -172,12 +174,12 @@ __device__ __forceinline__ void nc_send_async(const float* tile, bool transposed
 __device__ __forceinline__ void nc_bar_init(uint64_t* bar) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(nc_smem_u32(bar)) : "memory");
 }
-// The barrier's next phase: `bytes` will come (one thread).
+// The barrier's next phase: `bytes` will come (one thread, and only once the one before is over).
 __device__ __forceinline__ void nc_expect(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(nc_smem_u32(bar)), "r"(bytes) : "memory");
 }
-// Waits for a phase's bytes, for two seconds at most; gave_up ends every wait of the CTA.
-__device__ __forceinline__ void nc_wait(uint64_t* bar, uint32_t parity, volatile int* gave_up) {
+// Waits for a phase's bytes, for `limit` cycles at most; gave_up ends every wait of the CTA.  Whether they came.
+__device__ __forceinline__ bool nc_wait(uint64_t* bar, uint32_t parity, volatile int* gave_up, long long limit) {
   const uint32_t at = nc_smem_u32(bar);
   const long long t0 = clock64();
   for (uint32_t spins = 0;; ++spins) {
@@ -187,8 +189,8 @@ __device__ __forceinline__ void nc_wait(uint64_t* bar, uint32_t parity, volatile
         "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.b32 %0, 1, 0, p;\n\t}"
         : "=r"(ok) : "r"(at), "r"(parity) : "memory");
-    if (ok) return;
-    if ((spins & 255u) == 255u && (*gave_up || clock64() - t0 > 4000000000ll)) { *gave_up = 1; return; }
+    if (ok) return true;
+    if ((spins & 255u) == 255u && (*gave_up || clock64() - t0 > limit)) { *gave_up = 1; return false; }
   }
 }
 
@@ -238,7 +240,7 @@ __global__ void __launch_bounds__(NC_THREADS, 1) ns_cluster_kernel(const NcArgs 
   __shared__ SchedEntry sched[NS_SCHED_MAX];
   __shared__ __align__(16) double told[2][NC_CTAS][2];        // SMALL: what the CTAs tell each other, alternating
   __shared__ __align__(8) uint64_t bar_e, bar_b, bar_x, bar_t[2];
-  __shared__ int gave_up;
+  __shared__ int gave_up, lost;                               // this CTA gave a wait up, any CTA did
   const int cta = (int)blockIdx.x, t = threadIdx.x, d = g.d, kp = (d + 3) / 4 * 4;
   const int tiles = (d + 31) / 32, ld = nc_ld(tiles), sym_tiles = tiles * (tiles + 1) / 2;
   float* X = nc_smem;
@@ -274,10 +276,11 @@ __global__ void __launch_bounds__(NC_THREADS, 1) ns_cluster_kernel(const NcArgs 
   const uint32_t n_cols = has_sym ? (tm == tn ? 1u : 2u) : 0u;
   const uint32_t e_bytes = 4096u * tiles * n_cols, b_bytes = has_full ? 4096u * tiles : 0u;
   const uint32_t x_bytes = e_bytes + (has_full ? 4096u * (tiles - n_cols) : 0u);
+  if (t == 0) lost = 0;
   if (SMALL && t == 0) {
     nc_bar_init(&bar_e); nc_bar_init(&bar_b); nc_bar_init(&bar_x); nc_bar_init(&bar_t[0]); nc_bar_init(&bar_t[1]);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    nc_expect(&bar_e, e_bytes); nc_expect(&bar_b, b_bytes); nc_expect(&bar_x, x_bytes);
+    nc_expect(&bar_e, e_bytes + (g.lose == cta ? 16u : 0u)); nc_expect(&bar_b, b_bytes); nc_expect(&bar_x, x_bytes);
     nc_expect(&bar_t[0], NC_CTAS * 16u); nc_expect(&bar_t[1], NC_CTAS * 16u);
     gave_up = 0;
   }
@@ -391,8 +394,8 @@ __global__ void __launch_bounds__(NC_THREADS, 1) ns_cluster_kernel(const NcArgs 
       double sq = 0.0;
       if (t < NC_WORK) {
         if (k > 0 && x_bytes) {
-          nc_wait(&bar_x, (uint32_t)(k - 1) & 1u, &gave_up);
-          if (t == 0) nc_expect(&bar_x, x_bytes);
+          const bool came = nc_wait(&bar_x, (uint32_t)(k - 1) & 1u, &gave_up, g.wait_limit);
+          if (t == 0 && came) nc_expect(&bar_x, x_bytes);
         }
         if (has_sym) residual(mx, sq);
         sq = warp_sum_d(sq);
@@ -407,13 +410,12 @@ __global__ void __launch_bounds__(NC_THREADS, 1) ns_cluster_kernel(const NcArgs 
         nc_send_async(tile, false, E, ld, tm, tn, by_col[tn], t, &bar_e);
         if (tm != tn) nc_send_async(tile, true, E, ld, tn, tm, by_col[tm], t, &bar_e);
         if (t < NC_WORK) {
-          nc_wait(&bar_e, (uint32_t)k & 1u, &gave_up);
-          if (t == 0) nc_expect(&bar_e, e_bytes);
+          const bool came = nc_wait(&bar_e, (uint32_t)k & 1u, &gave_up, g.wait_limit);
+          if (t == 0 && came) nc_expect(&bar_e, e_bytes + (g.lose == cta + NC_CTAS * (k + 1) ? 16u : 0u));
           nc_tile<false>(E, E, ld, kp, tm * 32, tn * 32, v);      // does not wait for the decision
         }
       }
-      if (decides) {
-        nc_wait(&bar_t[k & 1], (uint32_t)(k >> 1) & 1u, &gave_up);
+      if (decides && nc_wait(&bar_t[k & 1], (uint32_t)(k >> 1) & 1u, &gave_up, g.wait_limit)) {
         nc_expect(&bar_t[k & 1], NC_CTAS * 16u);
         double tsq = 0.0, tmx = 0.0;
 #pragma unroll
@@ -429,8 +431,8 @@ __global__ void __launch_bounds__(NC_THREADS, 1) ns_cluster_kernel(const NcArgs 
         if (tm != tn) nc_send_async(tile, true, Bm, ld, tn, tm, by_factor[tm], t, &bar_b);
       }
       if (has_full && t < NC_WORK) {
-        nc_wait(&bar_b, (uint32_t)k & 1u, &gave_up);
-        if (t == 0) nc_expect(&bar_b, b_bytes);
+        const bool came = nc_wait(&bar_b, (uint32_t)k & 1u, &gave_up, g.wait_limit);
+        if (t == 0 && came) nc_expect(&bar_b, b_bytes);
         next(cta, v);
       }
       __syncthreads();
@@ -440,14 +442,10 @@ __global__ void __launch_bounds__(NC_THREADS, 1) ns_cluster_kernel(const NcArgs 
       float* const old = X;
       X = E; E = Bm; Bm = old;
     }
-    if (gave_up) {                               // let what is on its way land before the memory goes
-      const long long t0 = clock64();
-      while (clock64() - t0 < 4000000ll) {}
-      if (decides) {
-        ctl.ns_done = NS_DONE_FAILED;
-        atomicOr(&st->status_flags, STATUS_FLAG_TIMEOUT);
-        st->timeout_site = 50;
-      }
+    if (gave_up && t < NC_CTAS) {                // the others may have decided otherwise: tell them
+      uint32_t there;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(nc_smem_u32(&lost)), "r"(t));
+      asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(there), "r"(1) : "memory");
     }
   } else {
   for (; done_s == 0; ++k, cur ^= 1) {
@@ -508,6 +506,18 @@ __global__ void __launch_bounds__(NC_THREADS, 1) ns_cluster_kernel(const NcArgs 
     nc_cluster_sync();
   }
   }
+  // From here on nobody writes into another's shared memory, and all know whether a wait was given up: then nothing is committed anywhere.
+  nc_cluster_sync();
+  if (*(volatile int*)&lost) {
+    const long long t0 = clock64();              // (let what is on its way land before the memory goes)
+    while (clock64() - t0 < 4000000ll) {}
+    if (cta == 0 && decides) {
+      st->ns_done = NS_DONE_FAILED;
+      st->timeout_site = 50;
+      atomicOr(&st->status_flags, STATUS_FLAG_NS_FAILED | STATUS_FLAG_TIMEOUT);
+    }
+    return;
+  }
   // accept or reject (see ns_commit_kernel, ns_commit_state_kernel): each CTA holds the rows of X that its tiles of the last product read
   if (done_s == NS_DONE_CONVERGED) {
     for (int f = cta; f < tiles * tiles; f += NC_CTAS) {
@@ -524,7 +534,6 @@ __global__ void __launch_bounds__(NC_THREADS, 1) ns_cluster_kernel(const NcArgs 
     ns_ctl_store(ctl, st);
     ns_commit_state(st, g.n_endgame);
   }
-  nc_cluster_sync();                             // no CTA leaves while another may still write into its shared memory
 }
 
 // conqur_set_R's check of one narrow matrix, whose product is the launches' (the same chains), with the copy of what is accepted: one

@@ -142,3 +142,32 @@ def test_repeated_updates_give_the_same_bits(d):
         c.update()
         assert torch.equal(c.get_R(), seen.setdefault((plan, c.get_stats().ns_steps_used), c.get_R()))
     assert len(seen) < 30
+
+
+# (in the first step, in one between, and in the step that converges, where the blocks that got everything have accepted the rotation)
+@pytest.mark.parametrize("d", [33, 128])
+@pytest.mark.parametrize("block", [0, 2])
+def test_update_whose_wait_expires_changes_nothing(d, block):
+    m = _spectrum(d, "flat")
+    r0 = torch.linalg.qr(_rand(5, d, d).double())[0].float().contiguous()
+    c, ahead = [B.Context(d, 4096, in_dtype="f32", mode="exact") for _ in range(2)]
+    for x, updates in ((c, 12), (ahead, 13)):                # (the step count learnt; one more tells how many the next update takes)
+        for _ in range(updates):
+            x.set_M(m, 3.0, 4096)
+            x.update()
+    plan, steps = c.get_stats().ns_lift_plan, ahead.get_stats().ns_steps_used
+    c.set_M(m, 3.0, 4096)
+    kept = c.get_M()
+    for step in (0, steps // 2, steps):
+        c.set_R(r0)
+        c.set_M(m, 3.0, 4096)
+        c.debug_lose_wait(block, step)
+        c.update()
+        st = c.get_stats()
+        assert st.status == -8 and st.ns_lift_plan == plan
+        assert torch.equal(c.get_R(), r0) and torch.equal(c.get_M(), kept) and c.get_objective() == (3.0, 4096)
+    c.debug_lose_wait(-1)
+    c.set_M(m, 3.0, 4096)
+    c.update()
+    st = c.get_stats()
+    assert (st.status, st.ns_steps_used) == (0, steps) and torch.equal(c.get_R(), ahead.get_R())
