@@ -1263,7 +1263,9 @@ extern "C" int conqur_get_stats(conqur_ctx* c, conqur_stats* out) {
   CQ_CUDA(cudaMemcpyAsync(h.data(), c->state(), sizeof(DevState) * P, cudaMemcpyDeviceToHost, c->stream));
   const int rc = sync_status(c);
   if (rc == CONQUR_ERR_CUDA) return rc;
-  if (rc == CONQUR_ERR_NS_NOT_CONVERGED && !c->tokens_at_update.empty()) {
+  bool rejected = false;                          // (whatever other condition the status names first)
+  for (const DevState& p : h) rejected |= (p.status_flags & STATUS_FLAG_NS_FAILED) != 0;
+  if (rejected && !c->tokens_at_update.empty()) {
     // the device kept M, J and N of the rejected update: the host's row counts go back to match
     for (size_t p = 0; p < c->tokens.size(); ++p) c->tokens[p] += c->tokens_at_update[p];
     c->tokens_at_update.clear();

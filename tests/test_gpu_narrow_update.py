@@ -160,14 +160,12 @@ def test_update_whose_wait_expires_changes_nothing(d, block):
     kept = c.get_M()
     for step in (0, steps // 2, steps):
         c.set_R(r0)
-        c.set_M(m, 3.0, 4096)
         c.debug_lose_wait(block, step)
         c.update()
         st = c.get_stats()
         assert st.status == -8 and st.ns_lift_plan == plan
         assert torch.equal(c.get_R(), r0) and torch.equal(c.get_M(), kept) and c.get_objective() == (3.0, 4096)
     c.debug_lose_wait(-1)
-    c.set_M(m, 3.0, 4096)
-    c.update()
+    c.update()                                               # (of the rows counted before)
     st = c.get_stats()
     assert (st.status, st.ns_steps_used) == (0, steps) and torch.equal(c.get_R(), ahead.get_R())
