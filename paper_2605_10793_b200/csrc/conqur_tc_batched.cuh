@@ -120,7 +120,7 @@ __device__ __forceinline__ void tcb_item(int item, int T, int S, int& p, int& t_
 __device__ __noinline__ bool tcb_write_out(uint64_t* bar, uint32_t parity, volatile int* abort_flag, uint32_t t_addr, uint8_t* stg,
                                            int lane, const CUtensorMap* tmOut, int y0, bool add, int c0, int c_end, uint64_t* drained,
                                            long long* begun) {
-  if (!tc_wait(bar, parity, abort_flag)) return false;
+  if (!tc_wait_warp(bar, parity, abort_flag)) return false;
   ptx::tc_fence_after();
   if (begun) *begun = clock64();                   // timeline hook
 #pragma unroll 1
@@ -311,7 +311,8 @@ tcb_step_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         const uint32_t par3 = ((uint32_t)(it / TCB_YBUF)) & 1u, par2 = ((uint32_t)it >> 1) & 1u;
         const bool tr_epi = ew == 0;                       // the first warp of the tile's group stamps the epilogue
         if (tr_epi) TCB_TR(it, TCB_EV_EPI_BEGIN);
-        if (!tc_wait(&aux->yfull[yb], par3, abort_flag)) { ok = false; timeout_site = 32; break; }
+        // (a wait that gives up takes its whole warp out of the loop: votes, shuffles and TMEM loads follow)
+        if (!tc_wait_warp(&aux->yfull[yb], par3, abort_flag)) { ok = false; timeout_site = 32; break; }
         ptx::tc_fence_after();
         if (tr_epi) TCB_TR(it, TCB_EV_EPI_Y);
         const uint32_t t_addr = tmem_base + (uint32_t)(yb * 128) + ((uint32_t)(q * 32) << 16);
@@ -364,7 +365,7 @@ tcb_step_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         if (tr_epi) TCB_TR(it, TCB_EV_EPI_NORMS);
         const RowQuant rq = row_quant(g.qs, vmax, vmin, good);
         // the target buffer is needed only now (the second product of the tile two back has read it)
-        if (!tc_wait(&aux->cfree[cb], par2 ^ 1u, abort_flag)) { ok = false; timeout_site = 31; break; }
+        if (!tc_wait_warp(&aux->cfree[cb], par2 ^ 1u, abort_flag)) { ok = false; timeout_site = 31; break; }
         if (tr_epi) TCB_TR(it, TCB_EV_EPI_CFREE);
         const bool live = rq.inv > 0.f;
         const bool quick = __all_sync(0xffffffffu, sym ? rq.inv <= 1e36f : fmaxf(fabsf(rq.klo), fabsf(rq.khi)) <= 4194304.f);
@@ -479,7 +480,7 @@ tcb_step_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         if (ew == 0) TCB_TR(it - 1, TCB_EV_OUT_END);
         // the group's warps stay off their C' buffer until all of them have finished staging in it (bounded wait)
         if (lane == 0) ptx::mbar_arrive(&aux->pdone[grp]);
-        if (!tc_wait(&aux->pdone[grp], wo_count & 1u, abort_flag)) { ok = false; timeout_site = 36; break; }
+        if (!tc_wait_warp(&aux->pdone[grp], wo_count & 1u, abort_flag)) { ok = false; timeout_site = 36; break; }
         ++wo_count;
       }
       // every warp leaves its objective partial of the problem (summed in a fixed order by the kernel that follows)
