@@ -367,8 +367,11 @@ int take_results(conqur_ctx* c, const void* area, void* host, size_t bytes, bool
   if (rc == CONQUR_OK && in_mail(c, area)) std::memcpy(host, area, bytes);
   return rc;
 }
-// Whether a copy of this many blocks tells: with the code that finds the last of them it takes 40 registers instead of 32, and 5 us longer
-// for 64 MB; up to 2 MB the word gains more (32 per-head problems: set_M, step and the read-outs 80.6 -> 77.7 us).
+// Whether a copy of this many blocks tells (up to 2.4 MB).  With the code that finds the last block it takes 40 registers instead of 32, and what the
+// word gains depends on what the program calls next.  Never -> always, us: set_M, a step of 256 rows, get_objective and get_M, 0.07 to 2 MB 50 to 57, less by 0.4
+// to 0.8, but 1 and 2.4 MB in one problem 57.0 -> 57.4 and 59.0 -> 59.5; 4.2 MB 60.7 -> 59.7, 8.4 MB 56.0 -> 55.1, 16.8 MB 73.5 -> 73.2, 33.6 MB 92.5 -> 94.0,
+// 67 MB 131 -> 135.  32 per-head problems of 4001 rows 73.8 -> 72.8.  A row of copies alone (set_M, get_M, get_R) loses 1 us of 38 at any size up to 4 MB,
+// 2 to 3 at 8 to 17 MB, 10 of 90 at 67 MB, so the line lies below where these begin to lose more than a step gains.
 bool copy_posts(const conqur_ctx* c, const void* area, int blocks) { return in_mail(c, area) && blocks <= 4 * 148; }
 unsigned* blocks_done(const conqur_ctx* c) { return c->at<unsigned>(c->L.flags_agg) + 2; }      // (zero between launches)
 

@@ -57,3 +57,64 @@ def test_rotation_into_memory_that_is_not_this_gpus(mode, d, batch):
     odd = torch.zeros(batch * d * d + 1, device="cuda")
     assert B.conqur_get_R(c.h, odd.data_ptr() + 4) == 0
     assert torch.equal(odd[1:].view(batch, d, d), r)
+
+
+def test_objective_behind_long_and_short_work():
+    """The word that says the results are there is the call's own, whatever it waited for: sums of every step as it is read, in turn from contexts
+    that each use their slot, and from one that takes over a closed one's."""
+    d = 700
+    rows = torch.randn(16384, d, device="cuda")
+    work = [rows, rows[:3]]                                  # steps of over 1 ms and of some 40 us; a call looks out for its word for 200 us
+    contexts = [B.Context(d, 16384, in_dtype="f32", mode="exact") for _ in range(3)]
+    alone = []                                               # what either batch adds to J
+    for x in work:
+        contexts[0].step(x)
+        torch.cuda.synchronize()
+        alone.append(contexts[0].get_objective()[0])
+        contexts[0].set_M(torch.zeros(d, d, device="cuda"), 0.0, 0)
+    sums = [[0.0, 0] for _ in contexts]
+    order = [(i, w) for w in (0, 1, 1, 0, 0, 1) for i in range(3)] * 8
+    for k, (i, w) in enumerate(order):
+        if k % 17 == 16:                                     # another context, in the slot this one leaves
+            contexts[i].close()
+            contexts[i], sums[i] = B.Context(d, 16384, in_dtype="f32", mode="exact"), [0.0, 0]
+        contexts[i].step(work[w])
+        sums[i][0] += alone[w]
+        sums[i][1] += work[w].shape[0]
+        j, got = contexts[i].get_objective()
+        assert got == sums[i][1]
+        assert abs(j - sums[i][0]) <= 1e-12 * sums[i][0]     # (the same doubles, added in another order at most)
+
+
+@pytest.mark.parametrize("mode,d,batch", [("exact", 16, 1), ("exact", 778, 1), ("tc", 128, 32), ("tc", 1024, 1)])
+def test_cross_covariance_into_page_locked_memory(mode, d, batch):
+    """conqur_get_M where the host reads: what it has left is there when it returns, behind long and short work."""
+    c = B.Context(d, 4096, in_dtype="f32", mode=mode, batch=batch)
+    g = torch.Generator(device="cuda").manual_seed(d)
+    host = torch.zeros(batch, d, d).pin_memory()
+    filler = torch.empty(1 << 27, device="cuda")
+    for k in range(40):
+        m = torch.randn(batch, d, d, generator=g, device="cuda")
+        c.set_M(m if batch > 1 else m[0], [0.0] * batch if batch > 1 else 0.0, [1] * batch if batch > 1 else 1)
+        want = c.get_M().cpu().view(batch, d, d)
+        host.zero_()
+        for _ in range(k % 3):
+            filler.fill_(float(k))                           # (some 80 us each)
+        assert B.conqur_get_M(c.h, host.data_ptr()) == 0
+        assert torch.equal(host, want)
+
+
+@pytest.mark.parametrize("d", [33, 160, 640])
+def test_rotations_refused_and_taken_in_turn(d):
+    """conqur_set_R reads its decision from the same place, behind long and short work."""
+    c = B.Context(d, 4096, in_dtype="f32", mode="exact")
+    x = torch.randn(4096, d, device="cuda")
+    q = [torch.linalg.qr(torch.randn(d, d, device="cuda", dtype=torch.float64))[0].float().contiguous() for _ in range(2)]
+    for k in range(24):
+        if k % 2:
+            for _ in range(4):
+                c.step(x)
+        c.set_R(q[k % 2])
+        with pytest.raises(B.ConqurError):
+            c.set_R(1.01 * q[1 - k % 2])
+        assert torch.equal(c.get_R(), q[k % 2])
