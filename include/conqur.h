@@ -154,6 +154,8 @@ int conqur_destroy(conqur_ctx* ctx);
  * Replace the rotation(s).  R_dev: device fp32, batch x d x d, row-major, acting as
  * X_tilde @ R.  Must be orthogonal: max|R^T R - I| <= 1e-3 is checked (synchronises);
  * otherwise CONQUR_ERR_NOT_ORTHOGONAL_INPUT and the old R is kept.  Does not touch M, J, N.
+ * The call waits for the check alone: the replacement is enqueued on the context's stream and may still be reading
+ * R_dev when it returns, so R_dev must stay valid and unchanged, like X of a step, until that work has run.
  */
 int conqur_set_R(conqur_ctx* ctx, const float* R_dev);
 
@@ -168,6 +170,9 @@ int conqur_set_R(conqur_ctx* ctx, const float* R_dev);
  *          (tensor-core mode: X_dev 16-byte aligned and ld*sizeof(element) a multiple of 16)
  *   n      1..cfg.n_max (n = 0 is a no-op)
  * Single-problem contexts only (cfg.batch == 1).
+ * The order in which fp32 sums are added depends on n, cfg.n_max and the device: where rows are divided into calls in
+ * another way, the last bits of M and J may differ (in exact mode 1e-11 to 1e-9 of J between two orders, and the decision
+ * of an element that lies within fp32 rounding of zero).  The same calls give the same bits.
  */
 int conqur_step(conqur_ctx* ctx, const void* X_dev, int64_t n, int64_t ld);
 

@@ -112,8 +112,9 @@ __device__ __forceinline__ int had_pad(int i) { return i + ((i >> 6) << 2); }
 template <int E> struct HadWork { static constexpr int FLOATS = HAD_THREADS * E + HAD_THREADS * E / 16; };
 
 // Sums and differences of two pairs, each rounded as a + c and a - c are.  Half the instructions where these set the pace: 32768 x 4096 bf16
-// rows in a wider buffer 162 -> 152 us, fp32 rows 16384 x 4096 100 -> 96; 32768 x 4096 in one run 99 +- 4 either way (it settles at one of two
-// paces, by the buffers' addresses).
+// rows in a wider buffer 162 -> 152 us, fp32 rows 16384 x 4096 100 -> 96.  bf16 rows lying back to back are bound by memory and the board's power
+// (92 to 108 us for 32768 x 4096 by buffers, values and box): in turns of many passes over changing buffers 102 to 106 -> 95 to 99, in bursts of
+// thirty 98 -> 103; 4096 x 4096 20.5 -> 19.5.
 __device__ __forceinline__ void had_pair(float& a0, float& a1, float& c0, float& c1) {
   asm("{\n\t.reg .b64 a, c, s, t;\n\t"
       "mov.b64 a, {%0, %1};\n\tmov.b64 c, {%2, %3};\n\t"
