@@ -1041,7 +1041,7 @@ inline int tcb_step(TcHost& h, cudaStream_t s, const void* X, int in_dtype, int6
 // Two CTAs fit one SM (96 KB of shared memory and 256 TMEM columns each), so one problem's element-wise phases
 // overlap the other's products.
 // The pair is bf16, although an fp16 one (times 2^12, the lower half times 2^12 more), which takes one-pass G between the steps, ran 1024 problems in
-// 280 us for 297 and lay 3 to 8 times closer to the polar factor on ordinary statistics: its least unit is 2^-48 of the norm, and rows or columns of M that
+// 280 us for 297 and lay 4 to 9 times closer to the polar factor on ordinary statistics: its least unit is 2^-48 of the norm, and rows or columns of M that
 // lie 1e-10 and further below the others came out wrong without an error (a third of the rows at 1e-11, 1e-12, 1e-13: off by 0.20, 0.25, 0.65
 // of the rotation's norm, by 0.019 to 0.020 in this form), or were gone.
 constexpr int TCBU_THREADS = 256;            // 128 rows x 2 column halves
